@@ -273,7 +273,9 @@ ks_status ks_score(ks_ctx* ctx, const float* d_features, int64_t rows, const ks_
  * i the k best pairs of its candidate set ordered by (score descending, pool index
  * ascending). d_topk_idx [P, k] receives pool indices (-1 where the set has fewer than k
  * members), d_topk_score [P, k] the scores (-inf there). 1 <= k <= KS_MAX_K. The feature
- * matrix and the scores are never written to memory. `pairs` as in ks_featurize. The call
+ * matrix and the scores are never written to memory (a ranker with a layer wider than 256 units
+ * or more than two hidden layers: at most 1 M bf16 input rows and 67 M scores at a time are).
+ * `pairs` as in ks_featurize. The call
  * sizes the context's workspace (owned by the context, grown on demand, which synchronises the
  * device when it happens): partial lists, a per-call table of 16 x C records of at most 256
  * bytes, and, for a tree model on a batch of 32 problems or more, at most 256 MiB for the

@@ -165,15 +165,10 @@ void free_model(ks_model* m) {
   cudaFree(m->gbdt.d_qthr);
   cudaFree(m->gbdt.d_qfeat);
   ks::free_fast_gbdt(m->gbdt);
-  for (int l = 0; l < KS_MLP_MAX_LAYERS; ++l) {
-    cudaFree(m->mlp.d_w[l]);
-    cudaFree(m->mlp.d_b[l]);
-  }
-  cudaFree(m->mlp.d_mu);
-  cudaFree(m->mlp.d_sigma);
   cudaFree(m->mlp.d_tc_image);
   cudaFree(m->mlp.d_w1_prob);
   ks::free_fast_mlp(m->mlp);
+  ks::free_wide_mlp(m->mlp);
   ks::free_ridge(m->mlp);
   delete m;
 }
@@ -342,7 +337,7 @@ ks_status ks_model_describe(const ks_model* model, char* buf, int len) {
   } else if (model->kind == 1 && model->mlp.h_ridge) {
     std::snprintf(buf, len, "select_ridge_kernel");
   } else if (model->kind == 1) {
-    std::snprintf(buf, len, "select_generic_kernel mlp layers=%d", model->mlp.n_layers);
+    std::snprintf(buf, len, "mlp_wide_kernel layers=%d", model->mlp.n_layers);
   } else {
     std::snprintf(buf, len, "select_generic_kernel static score");
   }
@@ -424,10 +419,8 @@ ks_status ks_model_create_mlp(ks_ctx* ctx, int n_layers, const int* h_widths,
   if (n_layers < 1 || n_layers > KS_MLP_MAX_LAYERS) return KS_ERR_INVALID_ARG;
   const int in0 = h_widths[0];
   if ((in0 != KS_F_PAD && in0 != KS_F_ONEHOT) || h_widths[n_layers] != 1) return KS_ERR_INVALID_ARG;
-  int max_width = in0;
   for (int l = 1; l < n_layers; ++l) {
     if (h_widths[l] < 64 || h_widths[l] > KS_MLP_MAX_WIDTH || h_widths[l] % 64) return KS_ERR_INVALID_ARG;
-    if (h_widths[l] > max_width) max_width = h_widths[l];
   }
   for (int l = 0; l < n_layers; ++l)
     if (!h_w_bf16[l] || !h_bias[l]) return KS_ERR_INVALID_ARG;
@@ -441,17 +434,10 @@ ks_status ks_model_create_mlp(ks_ctx* ctx, int n_layers, const int* h_widths,
   m->device = ctx->device;
   m->kind = 1;
   m->mlp.n_layers = n_layers;
-  m->mlp.max_width = max_width;
   for (int l = 0; l <= n_layers; ++l) m->mlp.widths[l] = h_widths[l];
-  cudaError_t e = cudaSuccess;
-  for (int l = 0; l < n_layers && e == cudaSuccess; ++l) {
-    const size_t n = static_cast<size_t>(h_widths[l]) * h_widths[l + 1];
-    e = upload(&m->mlp.d_w[l], h_w_bf16[l], n);
-    if (e == cudaSuccess) e = upload(&m->mlp.d_b[l], h_bias[l], static_cast<size_t>(h_widths[l + 1]));
-  }
-  if (e == cudaSuccess) e = upload(&m->mlp.d_mu, h_mu, static_cast<size_t>(in0));
-  if (e == cudaSuccess) e = upload(&m->mlp.d_sigma, h_sigma, static_cast<size_t>(in0));
-  if (e == cudaSuccess) e = ks::build_fast_mlp(m->mlp, h_w_bf16, h_bias, h_mu, h_sigma);
+  cudaError_t e = ks::build_fast_mlp(m->mlp, h_w_bf16, h_bias, h_mu, h_sigma);
+  // the resident-weights kernel scores given rows in the ordinal input form only
+  if (e == cudaSuccess && !ks::score_mlp_tc_ok(m->mlp)) e = ks::build_wide_mlp(m->mlp, h_w_bf16, h_bias, h_mu, h_sigma);
   if (e == cudaSuccess) e = ks::build_ridge(m->mlp, h_w_bf16[0], h_bias[0], h_mu, h_sigma);
   if (e != cudaSuccess) {
     ks_status s = cuda_fail(ctx, e, "ks_model_create_mlp");
@@ -575,11 +561,18 @@ ks_status ks_score(ks_ctx* ctx, const float* d_features, int64_t rows, const ks_
                                             static_cast<cudaStream_t>(stream), &ctx->launches, &ctx->wait);
     return e == cudaSuccess ? KS_OK : cuda_fail(ctx, e, "ks_score");
   }
+  if (model->kind == 1 && model->mlp.wide) {
+    ks_status s = ensure_workspace(ctx, ks::score_wide_scratch_bytes(model->mlp, rows));
+    if (s != KS_OK) return s;
+    cudaError_t e = ks::launch_score_wide(model->mlp, d_features, rows, d_scores, ctx->ws, ctx->d_status,
+                                          static_cast<cudaStream_t>(stream), &ctx->launches, &ctx->wait);
+    return e == cudaSuccess ? KS_OK : cuda_fail(ctx, e, "ks_score");
+  }
   cudaError_t e =
       model->kind == 0
           ? ks::launch_score_gbdt(model->gbdt, d_features, rows, d_scores, d_leaf_idx,
                                   static_cast<cudaStream_t>(stream), &ctx->launches)
-          : ks::launch_score_mlp(model->mlp, d_features, rows, d_scores,
+          : ks::launch_score_linear(model->mlp, d_features, rows, d_scores,
                                  static_cast<cudaStream_t>(stream), &ctx->launches);
   return e == cudaSuccess ? KS_OK : cuda_fail(ctx, e, "ks_score");
 }

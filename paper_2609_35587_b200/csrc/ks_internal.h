@@ -94,31 +94,22 @@ struct GbdtModel {
   FeatQ* d_qfeat = nullptr;      // [64] rows and thresholds of each feature column
 };
 
+struct WideMlp;    // ks_mlp_wide.cu
+struct LinearRow;  // ks_kernels.cu
+
 struct MlpModel {
   int n_layers = 0;
   int widths[KS_MLP_MAX_LAYERS + 1] = {0};
-  int max_width = 0;
-  uint16_t* d_w[KS_MLP_MAX_LAYERS] = {nullptr};  // bf16 [out, in] row-major
-  float* d_b[KS_MLP_MAX_LAYERS] = {nullptr};
-  float* d_mu = nullptr;
-  float* d_sigma = nullptr;
   // one weight layer (the linear ridge scorer): fused kernel without a feature tile
   RidgeParams* h_ridge = nullptr;
-  // tensor-core path (shape 64-256-256-1 only), see ks_mlp_tc.cu
+  LinearRow* h_linear = nullptr;  // the same by input position, for ks_score
+  // tensor-core path of every other shape with a hidden layer (and of ks_score in the one-hot form), see ks_mlp_wide.cu
+  WideMlp* wide = nullptr;
+  // tensor-core path (one or two hidden layers of at most 256 units), see ks_mlp_tc.cu
   bool tc = false;
   uint16_t* d_tc_image = nullptr;      // W1 and W2 in the shared-memory operand layout
   float* d_w1_prob = nullptr;          // one-hot form: first-layer weights of the folded inputs
   MlpTcParams* h_tc_params = nullptr;  // host copy, passed by value at every launch
-};
-
-// kernel-side view of an MLP (passed by value)
-struct MlpView {
-  int n_layers;
-  int widths[KS_MLP_MAX_LAYERS + 1];
-  const uint16_t* w[KS_MLP_MAX_LAYERS];
-  const float* b[KS_MLP_MAX_LAYERS];
-  const float* mu;
-  const float* sigma;
 };
 
 }  // namespace ks
@@ -289,6 +280,21 @@ cudaError_t launch_select_mlp_tc(const ks_gpu_desc& desc, const MlpModel& m, con
                                  unsigned long long* partial, void* scratch, int* status, cudaStream_t stream,
                                  int64_t* launches, cudaEvent_t ev_begin, const FastWait* wait = nullptr);
 
+// Tensor-core path for rankers of any width (ks_mlp_wide.cu).
+cudaError_t build_wide_mlp(MlpModel& m, const uint16_t* const* h_w, const float* const* h_b, const float* h_mu,
+                           const float* h_sigma);
+void free_wide_mlp(MlpModel& m);
+int wide_rank_blocks(int64_t per_problem);
+size_t wide_scratch_bytes(const MlpModel& m, int P, int64_t pairs);
+cudaError_t launch_select_wide(const ks_gpu_desc& desc, const MlpModel& m, const ks_problem* d_p,
+                               const ks_problem* p_by_value, int P, const ks_candidate* d_c, int C, int nblk,
+                               const int64_t* seg_off, const int32_t* seg_idx, int64_t pairs, int k,
+                               unsigned long long* partial, void* scratch, int* status, cudaStream_t stream,
+                               int64_t* launches, cudaEvent_t ev_begin, const FastWait* wait);
+size_t score_wide_scratch_bytes(const MlpModel& m, int64_t rows);
+cudaError_t launch_score_wide(const MlpModel& m, const float* d_feat, int64_t rows, float* d_scores, void* scratch,
+                              int* status, cudaStream_t stream, int64_t* launches, const FastWait* wait);
+
 // k-way merge of gathered partial lists (multi-GPU candidate split).
 cudaError_t launch_merge_lists(const int32_t* d_idx, const float* d_score, int P, int n, int k, int32_t* d_out_idx,
                                float* d_out_score, cudaStream_t stream, int64_t* launches);
@@ -303,8 +309,8 @@ size_t featurize_scratch_bytes(int P);  // table of problem terms for the dense 
 cudaError_t launch_score_gbdt(const GbdtModel& m, const float* d_feat, int64_t rows, float* d_scores,
                               uint16_t* d_leaf_idx, cudaStream_t stream, int64_t* launches);
 
-cudaError_t launch_score_mlp(const MlpModel& m, const float* d_feat, int64_t rows, float* d_scores,
-                             cudaStream_t stream, int64_t* launches);
+cudaError_t launch_score_linear(const MlpModel& m, const float* d_feat, int64_t rows, float* d_scores,
+                                cudaStream_t stream, int64_t* launches);
 
 // Fused featurize + score + top-k. `p_by_value` non-null selects the single-problem form.
 // d_partial: workspace for the per-block partial lists and per-call tables, at least

@@ -1,5 +1,5 @@
 // Generic kernels of libks: the standalone feature map, the standalone scorers, the generic
-// fused featurize + score + top-k kernel (any tree shape, any MLP the ABI accepts) and the
+// fused featurize + score + top-k kernel (any tree shape), the linear scorer and the
 // per-problem merge of partial top-k lists. The quantised fast path for complete trees lives
 // in ks_gbdt_fast.cu.
 #include <cuda_bf16.h>
@@ -229,98 +229,46 @@ score_gbdt_kernel(const DevNode* __restrict__ nodes, const int* __restrict__ roo
 }
 
 // ------------------------------------------------------------------------------------------
-// generic MLP on a tile of kBlock rows held as [column][thread] fp32 in shared memory.
-// Rows are processed 32 at a time; thread (r = tid % 32, g = tid / 32) computes the outputs
-// o = g, g + 8, ... of row r. Activations are bf16 in shared memory, [unit][32].
+// ks_score with the linear scorer (one weight layer): one thread per row
 // ------------------------------------------------------------------------------------------
 
-__device__ __forceinline__ float bf16_bits_to_float(uint32_t b) { return __uint_as_float(b << 16); }
+// The model's input positions in order: weight (bf16), mean, deviation, by value.
+struct LinearRow {
+  float w[KS_F_ONEHOT], mu[KS_F_ONEHOT], sigma[KS_F_ONEHOT];
+  float bias;
+};
 
-__device__ void mlp_tile(const MlpView& m, int max_width, const float* s_cols /* [64][kBlock] */,
-                         __nv_bfloat16* s_act /* [2][max_width][32] */, float* s_scores /* [kBlock] */) {
-  const int r = threadIdx.x & 31, g = threadIdx.x >> 5;
-  constexpr int kGroups = kBlock / 32;
-  for (int grp = 0; grp < kGroups; ++grp) {
-    __nv_bfloat16* cur = s_act;
-    __nv_bfloat16* nxt = s_act + max_width * 32;
-    const bool onehot = m.widths[0] == KS_F_ONEHOT;
-    for (int pos = g; pos < m.widths[0]; pos += kGroups) {
-      float v = 0.0f;
-      bool live;
-      if (!onehot) {
-        live = pos < KS_F;
-        if (live) v = s_cols[pos * kBlock + grp * 32 + r];
-      } else {
-        // one-hot form: the columns other than 5, 9, 17, 18 in order, then the level indicators
-        live = pos < 73;
-        if (pos < 59) {
-          const int col = pos + (pos >= 5) + (pos >= 8) + 2 * (pos >= 15);
-          v = s_cols[col * kBlock + grp * 32 + r];
-        } else if (live) {
-          const int q = pos - 59;  // operand type 0..3, activation 4..6, kernel sched 7..10, epilogue sched 11..13
-          const int col = q < 4 ? 5 : (q < 7 ? 9 : (q < 11 ? 17 : 18));
-          const int level = q < 4 ? q : (q < 7 ? q - 4 : (q < 11 ? q - 7 : q - 11));
-          v = __float2int_rz(s_cols[col * kBlock + grp * 32 + r]) == level ? 1.0f : 0.0f;
-        }
-      }
-      if (live) {
-        if (!isfinite(v)) v = 0.0f;
-        v = __fdiv_rn(__fsub_rn(v, m.mu[pos]), m.sigma[pos]);
-      }
-      cur[pos * 32 + r] = __float2bfloat16_rn(v);
-    }
-    __syncthreads();
-    for (int l = 0; l < m.n_layers; ++l) {
-      const int wi = m.widths[l], wo = m.widths[l + 1];
-      const bool last = (l == m.n_layers - 1);
-      for (int o = g; o < wo; o += kGroups) {
-        const uint4* wrow = reinterpret_cast<const uint4*>(m.w[l] + static_cast<size_t>(o) * wi);
-        float acc = 0.0f;
-        for (int i8 = 0; i8 < wi / 8; ++i8) {
-          const uint4 wv = __ldg(wrow + i8);
-          const uint32_t ww[4] = {wv.x, wv.y, wv.z, wv.w};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int i = i8 * 8 + 2 * q;
-            acc = fmaf(bf16_bits_to_float(ww[q] & 0xFFFFu), __bfloat162float(cur[i * 32 + r]), acc);
-            acc = fmaf(bf16_bits_to_float(ww[q] >> 16), __bfloat162float(cur[(i + 1) * 32 + r]), acc);
-          }
-        }
-        float v = acc + m.b[l][o];
-        if (last) {
-          if (o == 0) s_scores[grp * 32 + r] = v;
-        } else {
-          nxt[o * 32 + r] = __float2bfloat16_rn(fmaxf(v, 0.0f));
-        }
-      }
-      __syncthreads();
-      __nv_bfloat16* tmp = cur;
-      cur = nxt;
-      nxt = tmp;
-    }
-  }
-}
-
+template <bool kOneHot>
 __global__ void __launch_bounds__(kBlock)
-score_mlp_kernel(MlpView m, int max_width, const float* __restrict__ feat, int64_t rows,
-                 float* __restrict__ scores) {
-  extern __shared__ __align__(16) unsigned char s_raw[];
-  float* s_cols = reinterpret_cast<float*>(s_raw);                       // [64][kBlock]
-  float* s_scores = s_cols + kRow * kBlock;                              // [kBlock]
-  __nv_bfloat16* s_act = reinterpret_cast<__nv_bfloat16*>(s_scores + kBlock);
+score_linear_kernel(const __grid_constant__ LinearRow m, const float* __restrict__ feat, int64_t rows,
+                    float* __restrict__ scores) {
   const int64_t r = static_cast<int64_t>(blockIdx.x) * kBlock + threadIdx.x;
-  const float4* src = reinterpret_cast<const float4*>(feat + min(r, rows - 1) * kRow);
-#pragma unroll 4
+  if (r >= rows) return;
+  const float4* src = reinterpret_cast<const float4*>(feat + r * kRow);
+  float x[kRow];
+#pragma unroll
   for (int q = 0; q < kRow / 4; ++q) {
     const float4 v = __ldg(src + q);
-    s_cols[(4 * q + 0) * kBlock + threadIdx.x] = v.x;
-    s_cols[(4 * q + 1) * kBlock + threadIdx.x] = v.y;
-    s_cols[(4 * q + 2) * kBlock + threadIdx.x] = v.z;
-    s_cols[(4 * q + 3) * kBlock + threadIdx.x] = v.w;
+    x[4 * q] = v.x; x[4 * q + 1] = v.y; x[4 * q + 2] = v.z; x[4 * q + 3] = v.w;
   }
-  __syncthreads();
-  mlp_tile(m, max_width, s_cols, s_act, s_scores);
-  if (r < rows) scores[r] = s_scores[threadIdx.x] + 0.0f;
+  float acc = 0.0f;
+#pragma unroll
+  for (int pos = 0; pos < (kOneHot ? 73 : KS_F); ++pos) {
+    float v;
+    if (!kOneHot) {
+      v = x[pos];
+    } else if (pos < 59) {  // the columns other than 5, 9, 17, 18 in order, then the level indicators
+      v = x[pos + (pos >= 5) + (pos >= 8) + 2 * (pos >= 15)];
+    } else {
+      const int q = pos - 59;  // operand type 0..3, activation 4..6, kernel sched 7..10, epilogue sched 11..13
+      const int col = q < 4 ? 5 : (q < 7 ? 9 : (q < 11 ? 17 : 18));
+      const int level = q < 4 ? q : (q < 7 ? q - 4 : (q < 11 ? q - 7 : q - 11));
+      v = __float2int_rz(x[col]) == level ? 1.0f : 0.0f;
+    }
+    if (!isfinite(v)) v = 0.0f;
+    acc = fmaf(m.w[pos], __bfloat162float(__float2bfloat16_rn(__fdiv_rn(__fsub_rn(v, m.mu[pos]), m.sigma[pos]))), acc);
+  }
+  scores[r] = (acc + m.bias) + 0.0f;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -328,17 +276,14 @@ score_mlp_kernel(MlpView m, int max_width, const float* __restrict__ feat, int64
 // keep one key per thread per sub-tile, rank the block's keys, write a partial top-k list.
 // ------------------------------------------------------------------------------------------
 
-template <int kModel>  // 0 = tree ensemble, 1 = MLP, 2 = static sampling score (no feature tile)
+template <bool kStatic>  // tree ensemble, or the static sampling score (no feature tile)
 __global__ void __launch_bounds__(kBlock)
 select_generic_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value,
                       int use_value, const ks_candidate* __restrict__ c, PairMap map, int sub_tiles,
                       const DevNode* __restrict__ nodes, const int* __restrict__ roots, int n_trees,
-                      float base, MlpView mlp, int max_width, int k,
-                      unsigned long long* __restrict__ partial /* [P][nblk][k] */) {
+                      float base, int k, unsigned long long* __restrict__ partial /* [P][nblk][k] */) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   float* s_cols = reinterpret_cast<float*>(s_raw);  // [64][kBlock]
-  float* s_scores = s_cols + kRow * kBlock;         // [kBlock] (MLP only)
-  __nv_bfloat16* s_act = reinterpret_cast<__nv_bfloat16*>(s_scores + kBlock);
   __shared__ ProblemTerms s_pt;
   __shared__ unsigned long long s_warp[kBlock / 32 * KS_MAX_K];
   __shared__ unsigned long long s_list[KS_MAX_K];
@@ -364,28 +309,17 @@ select_generic_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_pro
       const bool live = r < len;
       int idx = 0;
       __syncthreads();  // previous sub-tile's readers are done with s_cols
-      float direct = 0.0f;
+      float score = 0.0f;
       if (live) {
         idx = pool_index(map, lo, r);
         const ks_candidate cand = c[idx];
-        if (kModel == 2) {
-          direct = static_score(s_pt, cand, desc);
+        if (kStatic) {
+          score = static_score(s_pt, cand, desc);
         } else {
           float* col0 = s_cols + threadIdx.x;
           featurize_pair(s_pt, cand, desc, [&](int col, float v) { col0[col * kBlock] = v; });
+          score = walk_ensemble(nodes, roots, n_trees, base, s_cols + threadIdx.x, nullptr);
         }
-      } else if (kModel == 1) {
-        for (int col = 0; col < kRow; ++col) s_cols[col * kBlock + threadIdx.x] = 0.0f;
-      }
-      float score;
-      if (kModel == 2) {
-        score = direct;
-      } else if (kModel == 0) {
-        score = live ? walk_ensemble(nodes, roots, n_trees, base, s_cols + threadIdx.x, nullptr) : 0.0f;
-      } else {
-        __syncthreads();
-        mlp_tile(mlp, max_width, s_cols, s_act, s_scores);
-        score = s_scores[threadIdx.x];
       }
       const unsigned long long key = live ? make_key(score + 0.0f, idx) : 0ull;
 #pragma unroll
@@ -661,35 +595,6 @@ cudaError_t launch_score_gbdt(const GbdtModel& m, const float* d_feat, int64_t r
   return cudaGetLastError();
 }
 
-static MlpView make_view(const MlpModel& m) {
-  MlpView v{};
-  v.n_layers = m.n_layers;
-  for (int l = 0; l <= m.n_layers; ++l) v.widths[l] = m.widths[l];
-  for (int l = 0; l < m.n_layers; ++l) {
-    v.w[l] = m.d_w[l];
-    v.b[l] = m.d_b[l];
-  }
-  v.mu = m.d_mu;
-  v.sigma = m.d_sigma;
-  return v;
-}
-
-static size_t mlp_smem_bytes(int max_width) {
-  return sizeof(float) * (kRow * kBlock + kBlock) + sizeof(__nv_bfloat16) * 2 * max_width * 32;
-}
-
-cudaError_t launch_score_mlp(const MlpModel& m, const float* d_feat, int64_t rows, float* d_scores,
-                             cudaStream_t stream, int64_t* launches) {
-  if (rows == 0) return cudaSuccess;
-  const size_t smem = mlp_smem_bytes(m.max_width);
-  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(&score_mlp_kernel), smem);
-  if (e != cudaSuccess) return e;
-  score_mlp_kernel<<<static_cast<unsigned>((rows + kBlock - 1) / kBlock), kBlock, smem, stream>>>(
-      make_view(m), m.max_width, d_feat, rows, d_scores);
-  ++*launches;
-  return cudaGetLastError();
-}
-
 static float bf16_bits_host(uint16_t b) {
   const uint32_t u = static_cast<uint32_t>(b) << 16;
   float f;
@@ -744,12 +649,33 @@ cudaError_t build_ridge(MlpModel& m, const uint16_t* h_w, const float* h_b, cons
     }
   }
   m.h_ridge = r;
+  LinearRow* q = new (std::nothrow) LinearRow();
+  if (!q) return cudaErrorMemoryAllocation;
+  m.h_linear = q;
+  for (int j = 0; j < m.widths[0]; ++j) {
+    q->w[j] = bf16_bits_host(h_w[j]);
+    q->mu[j] = h_mu[j];
+    q->sigma[j] = h_sigma[j];
+  }
+  q->bias = h_b[0];
   return cudaSuccess;
 }
 
 void free_ridge(MlpModel& m) {
   delete m.h_ridge;
   m.h_ridge = nullptr;
+  delete m.h_linear;
+  m.h_linear = nullptr;
+}
+
+cudaError_t launch_score_linear(const MlpModel& m, const float* d_feat, int64_t rows, float* d_scores,
+                                cudaStream_t stream, int64_t* launches) {
+  if (rows == 0) return cudaSuccess;
+  const unsigned grid = static_cast<unsigned>((rows + kBlock - 1) / kBlock);
+  if (m.widths[0] == KS_F_ONEHOT) score_linear_kernel<true><<<grid, kBlock, 0, stream>>>(*m.h_linear, d_feat, rows, d_scores);
+  else score_linear_kernel<false><<<grid, kBlock, 0, stream>>>(*m.h_linear, d_feat, rows, d_scores);
+  ++*launches;
+  return cudaGetLastError();
 }
 
 size_t ridge_scratch_bytes(int C) { return (256 + sizeof(float2) * 16 * static_cast<size_t>(C) + 255) / 256 * 256; }
@@ -788,6 +714,10 @@ size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, 
     const int nblk = mlp_tc_blocks_per_problem(P, per);
     const size_t part = (static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
     return part + mlp_tc_scratch_bytes(C);
+  }
+  if (model.kind == 1 && model.mlp.wide) {
+    const size_t part = static_cast<size_t>(P) * wide_rank_blocks(per) * k * sizeof(unsigned long long);
+    return (part + 255) / 256 * 256 + wide_scratch_bytes(model.mlp, P, pairs);
   }
   const int st = pick_sub_tiles(P, per);
   int64_t nblk = (per + static_cast<int64_t>(st) * kBlock - 1) / (static_cast<int64_t>(st) * kBlock);
@@ -860,6 +790,20 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     ++*launches;
     return cudaGetLastError();
   }
+  if (model.kind == 1 && model.mlp.wide) {
+    const int nblk = wide_rank_blocks(per);
+    unsigned long long* part = static_cast<unsigned long long*>(d_partial);
+    const size_t part_bytes = (static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
+    cudaError_t e = launch_select_wide(desc, model.mlp, d_p, p_by_value, P, d_c, C, nblk, d_seg_off, d_seg_idx, pairs, k,
+                                       part, static_cast<char*>(d_partial) + part_bytes, d_status, stream, launches,
+                                       ev_begin, wait);
+    if (e != cudaSuccess) return e;
+    if (ev_end) cudaEventRecord(ev_end, stream);
+    topk_merge_kernel<<<(P * 32 + kBlock - 1) / kBlock, kBlock, 0, stream>>>(part, P, nblk * k, k, d_topk_idx,
+                                                                            d_topk_score);
+    ++*launches;
+    return cudaGetLastError();
+  }
   const int st = pick_sub_tiles(P, per);
   const PairMap map = make_map(P, C, pairs, d_seg_off, d_seg_idx, st * kBlock);
   unsigned long long* partial = static_cast<unsigned long long*>(d_partial);
@@ -915,23 +859,15 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
   }
   if (ev_begin) cudaEventRecord(ev_begin, stream);
   if (model.kind == 2) {
-    select_generic_kernel<2><<<grid, kBlock, 0, stream>>>(desc, d_p, pv, p_by_value != nullptr, d_c, map, st, nullptr,
-                                                          nullptr, 0, 0.0f, MlpView{}, 0, k, partial);
-  } else if (model.kind == 0) {
+    select_generic_kernel<true><<<grid, kBlock, 0, stream>>>(desc, d_p, pv, p_by_value != nullptr, d_c, map, st, nullptr,
+                                                             nullptr, 0, 0.0f, k, partial);
+  } else {
     const GbdtModel& g = model.gbdt;
     const size_t smem = sizeof(float) * kRow * kBlock;
-    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&select_generic_kernel<0>), smem);
+    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&select_generic_kernel<false>), smem);
     if (e != cudaSuccess) return e;
-    select_generic_kernel<0><<<grid, kBlock, smem, stream>>>(
-        desc, d_p, pv, p_by_value != nullptr, d_c, map, st, g.d_nodes, g.d_roots, g.n_trees, g.base,
-        MlpView{}, 0, k, partial);
-  } else {
-    const size_t smem = mlp_smem_bytes(model.mlp.max_width);
-    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&select_generic_kernel<1>), smem);
-    if (e != cudaSuccess) return e;
-    select_generic_kernel<1><<<grid, kBlock, smem, stream>>>(
-        desc, d_p, pv, p_by_value != nullptr, d_c, map, st, nullptr, nullptr, 0, 0.0f,
-        make_view(model.mlp), model.mlp.max_width, k, partial);
+    select_generic_kernel<false><<<grid, kBlock, smem, stream>>>(desc, d_p, pv, p_by_value != nullptr, d_c, map, st,
+                                                                 g.d_nodes, g.d_roots, g.n_trees, g.base, k, partial);
   }
   ++*launches;
   e = cudaGetLastError();
@@ -958,10 +894,10 @@ cudaError_t launch_select_generic_trees(const ks_gpu_desc& desc, const DevNode* 
   const int st = pick_sub_tiles(P, C);
   const PairMap map = make_map(P, C, static_cast<int64_t>(P) * C, nullptr, nullptr, st * kBlock);
   const size_t smem = sizeof(float) * kRow * kBlock;
-  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(&select_generic_kernel<0>), smem);
+  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(&select_generic_kernel<false>), smem);
   if (e != cudaSuccess) return e;
-  select_generic_kernel<0><<<static_cast<unsigned>(static_cast<int64_t>(P) * map.nblk), kBlock, smem, stream>>>(
-      desc, d_p, ks_problem{}, 0, d_c, map, st, d_nodes, d_roots, n_trees, base, MlpView{}, 0, k, partial);
+  select_generic_kernel<false><<<static_cast<unsigned>(static_cast<int64_t>(P) * map.nblk), kBlock, smem, stream>>>(
+      desc, d_p, ks_problem{}, 0, d_c, map, st, d_nodes, d_roots, n_trees, base, k, partial);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   topk_merge_kernel<<<(P * 32 + kBlock - 1) / kBlock, kBlock, 0, stream>>>(partial, P, map.nblk * k, k,
