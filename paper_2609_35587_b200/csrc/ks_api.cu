@@ -50,7 +50,7 @@ ks_status ensure_workspace(ks_ctx* ctx, size_t bytes) {
     ctx->ws_bytes = 0;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFree(workspace)");
   }
-  const size_t want = bytes + bytes / 2 + (1u << 20);
+  const size_t want = bytes + (bytes < (size_t(128) << 20) ? bytes / 2 : size_t(64) << 20) + (1u << 20);
   cudaError_t e = cudaMalloc(&ctx->ws, want);
   if (e != cudaSuccess) {
     ctx->ws = nullptr;

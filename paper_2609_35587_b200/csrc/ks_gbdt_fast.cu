@@ -55,6 +55,7 @@
 #include <vector>
 
 #include "ks_features.cuh"
+#include "ks_gbdt_quant.cuh"
 #include "ks_internal.h"
 #include "ks_memo.cuh"
 #include "ks_topk.cuh"
@@ -64,8 +65,6 @@ namespace ks {
 namespace {
 
 constexpr int kBufBytes = 16 * 1024;   // one tree-chunk buffer (twice that where the shared memory allows)
-constexpr int kSlice = 127;            // thresholds per row: a byte is 0x80 | (0..127)
-constexpr unsigned kSleepNs = 1200;    // asked-for sleep between two probes of a chunk barrier (400 to 2500 measured alike)
 constexpr int kCombos = 16;            // dtype_ab x dtype_d
 
 constexpr int kSmCount = 148;           // SMs of the one device this library is built for (sm_100a)
@@ -79,150 +78,9 @@ constexpr int kNBuf = 2;                // buffers of a ring (four of 8 KB and t
 // shared memory map (byte offsets from the dynamic shared base): the rings' chunk buffers, then the tile
 constexpr int kOffBuf0 = 0;
 
-#ifdef KS_DEBUG_BOUNDS
-// Checked build: every index formed from data (tile byte, node, chunk, record, partial list) is
-// compared with its range; a violation records its source line in this word and uses element 0.
-__device__ int g_bounds_line;
-__device__ __forceinline__ long long checked_index(long long i, long long n, int line) {
-  if (i < 0 || i >= n) {
-    atomicCAS(&g_bounds_line, 0, line);
-    return 0;
-  }
-  return i;
-}
-#define KS_IDX(i, n) checked_index(static_cast<long long>(i), static_cast<long long>(n), __LINE__)
-#else
-#define KS_IDX(i, n) (i)
-#endif
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait: one probe, then sleep-and-probe (measured faster than the blocking try_wait with
-// or without a time hint); gives up after `limit` probes, or as soon as another warp of the CTA
-// has given up (`fail`), and reports false.
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, int limit, volatile int* fail) {
-  if (mbar_test_wait(bar, parity)) return true;
-  for (int i = 0; i < limit; ++i) {
-    __nanosleep(kSleepNs);
-    if (mbar_test_wait(bar, parity)) return true;
-    if ((i & 63) == 63 && *fail) return false;
-  }
-  return false;
-}
-__device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ float lds_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
-  return v;
-}
-
 // Raised by a CTA whose bounded wait ran out, so that the CTAs after it leave at once; cleared by
 // the per-call table kernel that precedes every launch of the select kernel.
 __device__ int g_fast_abort;
-
-// #{j < n : T[j] <= v} over n sorted thresholds.
-__device__ __forceinline__ int count_le(const float* T, int n, float v) {
-  int pos = 0;
-  for (int s = n > 0 ? 1 << (31 - __clz(n)) : 0; s >= 1; s >>= 1) {
-    const int np = pos + s;
-    if (np <= n && T[np - 1] <= v) pos = np;
-  }
-  return pos;
-}
-
-// Tile bytes of one feature value: slice s of the feature's thresholds gets the number of its
-// thresholds that are <= v, i.e. the overall count less 127 s clamped to 0..127; a rank row gets
-// the rank of the level code v. `T` is the feature's own sorted threshold array. With
-// `nan_right` a NaN takes the last bin of every slice (x < t is false: it goes right).
-// `pos` is the count of the feature's thresholds that are <= v (unused for a feature without slices).
-template <typename Put>
-__device__ __forceinline__ void emit_rows(const FeatQ& q, int pos, float v, Put put) {
-  if (q.nslice) {
-    for (int s = 0; s < q.nslice; ++s) {
-      int b = pos - kSlice * s;
-      b = b < 0 ? 0 : (b > kSlice ? kSlice : b);
-      put(q.row0 + s, static_cast<uint8_t>(0x80 | b));
-    }
-  }
-  if (q.nrank) {
-    const int code = __float2int_rz(v);
-    for (int r = 0; r < q.nrank; ++r)
-      put(q.row0 + q.nslice + r, static_cast<uint8_t>(0x80 | ((code >= 0 && code < 4) ? q.rank[r][code] : 0)));
-  }
-}
-template <typename Put>
-__device__ __forceinline__ void quantise(const FeatQ& q, const float* T, float v, bool nan_right, Put put) {
-  const int pos = q.nslice ? ((nan_right && v != v) ? q.nthr : count_le(T, q.nthr, v)) : 0;
-  emit_rows(q, pos, v, put);
-}
-
-// The per-pair columns (class 2 of feat_class) in ascending order, and a column's place among them.
-constexpr int kPairCols = 21;
-__host__ __device__ constexpr int pair_slot(int col) {
-  return col <= 36 ? col - 23 : (col == 39 ? 14 : (col <= 44 ? col - 26 : col - 41));
-}
-__host__ __device__ constexpr int pair_col(int slot) {
-  return slot <= 13 ? slot + 23 : (slot == 14 ? 39 : (slot <= 18 ? slot + 26 : slot + 41));
-}
-constexpr bool pair_slots_match_classes() {
-  int n = 0;
-  for (int c = 0; c < KS_F; ++c)
-    if (feat_class(c) == 2) {
-      if (pair_slot(c) != n || pair_col(n) != c) return false;
-      ++n;
-    }
-  return n == kPairCols;
-}
-static_assert(pair_slots_match_classes(), "per-pair columns");
-
-// All per-pair columns of one pair at once: the binary searches advance in step (one probe of
-// every column per round), so that a thread has 21 independent loads in flight instead of one
-// dependent chain after the other. `T` is the staged (or global) array of per-pair thresholds.
-template <typename Put>
-__device__ __forceinline__ void quantise_pair_columns(const FeatQ* s_fq, const float* T, const float (&v)[kPairCols],
-                                                      int max_thr, Put put) {
-  int pos[kPairCols];
-#pragma unroll
-  for (int i = 0; i < kPairCols; ++i) pos[i] = 0;
-  for (int s = max_thr > 0 ? 1 << (31 - __clz(max_thr)) : 0; s >= 1; s >>= 1) {
-#pragma unroll
-    for (int i = 0; i < kPairCols; ++i) {
-      const FeatQ& q = s_fq[pair_col(i)];
-      const int np = pos[i] + s;
-      if (np <= q.nthr && T[q.thr0 + np - 1] <= v[i]) pos[i] = np;
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < kPairCols; ++i) emit_rows(s_fq[pair_col(i)], pos[i], v[i], put);
-}
 
 // Byte of row i (0 .. 4 W - 1) of a block within one tile row of W words: the four rows of a
 // word are consecutive, so that in a catalogue ranked in similarity order a thread's four
@@ -247,23 +105,6 @@ struct SliceArgs {
   int repeat;              // floor measurement only: passes over the resident chunks
 };
 
-struct FastView {
-  int n_rows, n_pair_rows, n_cand_rows, n_prob_rows;  // rows are ordered pair, candidate, problem
-  int depth, n_chunks, chunk_bytes, tpc;
-  int n_thr, thr_cand0, thr_prob0;  // thresholds in all, and where the candidate-only / problem-only features' begin
-  int cand_rec, pair_rec;           // bytes per record of the per-call tables (multiples of 16)
-  int wait_limit, starve;           // probes a chunk wait may take; test hook: arm the barrier for bytes that never come
-  int buf_bytes;                    // size of one chunk buffer in shared memory
-  float base;
-  const uint32_t* chunks;      // [n_chunks][chunk_bytes / 4]
-  const float* thr;            // [n_thr] sorted thresholds, feature after feature (per-pair features first)
-  const FeatQ* feat;           // [64] rows and thresholds of each feature column
-  const uint8_t* cand_rows;    // [kCombos][C][cand_rec] quantised candidate-only rows
-  const unsigned* pair_class;  // [kCombos][C] class of every candidate, or null (no memo)
-  const uint8_t* pair_tab;     // [P][kMemoCap][pair_rec] per-pair tile bytes of every (problem, class)
-  const uint8_t* prob_tab;     // [P][kProbRec] tile bytes of the problem-only rows and the problem's terms, or null
-};
-
 // ------------------------------------------------------------------------------------------
 // candidate-only rows, once per call
 // ------------------------------------------------------------------------------------------
@@ -276,18 +117,6 @@ __global__ void combo_mask_kernel(const ks_problem* __restrict__ p, int P, unsig
   }
   m = __reduce_or_sync(0xFFFFFFFFu, m);
   if ((threadIdx.x & 31) == 0 && m) atomicOr(mask, m);
-}
-
-// Thresholds of a range of features into shared memory when they fit `cap` floats, else the
-// global array is searched in place. Returns the pointer that stands for fv.thr + first.
-__device__ __forceinline__ const float* stage_thresholds(const FastView& fv, int first, int count, float* s_thr,
-                                                         int cap) {
-  if (count > cap) return fv.thr + first;
-  const int vec = (first & 3) == 0 ? count / 4 : 0;  // whole 16-byte words when the source is aligned like s_thr
-  for (int i = threadIdx.x; i < vec; i += blockDim.x)
-    reinterpret_cast<float4*>(s_thr)[i] = __ldg(reinterpret_cast<const float4*>(fv.thr + first) + i);
-  for (int i = 4 * vec + threadIdx.x; i < count; i += blockDim.x) s_thr[i] = __ldg(fv.thr + first + i);
-  return s_thr;
 }
 
 __global__ void __launch_bounds__(256)
@@ -348,7 +177,7 @@ static_assert(sizeof(ProblemTerms) <= 128, "problem record");
 
 __global__ void __launch_bounds__(256)
 pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int n_prob,
-                  const ks_candidate* __restrict__ c, FastView fv, MemoView memo, int thr_cap) {
+                  const ks_candidate* __restrict__ c, FastView fv, MemoView memo, int thr_cap, const int* path) {
   extern __shared__ __align__(16) float s_pthr[];  // thresholds of the per-pair features, then the records
   __shared__ ProblemTerms s_pt;
   __shared__ FeatQ s_fq[64];
@@ -357,7 +186,11 @@ pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem
   // the select kernel that follows may start its own set-up now (it waits for this grid to finish
   // before it reads the tables)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (blockIdx.x == 0 && tid == 0) g_fast_abort = 0;  // (also) precedes the select kernel
+  // (also) precedes the select kernel, whose CTAs leave at once when the class walk
+  // (ks_gbdt_classes.cu) serves the call; that one then writes the partial lists
+  const bool skip = path && *path == 1;
+  if (blockIdx.x == 0 && tid == 0) g_fast_abort = skip;
+  if (skip) return;
   int most = 0;
   for (int q = 0; q < kMemoCombos; ++q) most = max(most, memo.count[q]);
   // An item is (block of 256 classes, problem); the blocks of the grid deal the items among
@@ -1385,6 +1218,8 @@ cudaError_t build_fast_gbdt(GbdtModel& m, int n_trees, const int64_t* off, const
     delete top;
     return e;
   }
+  m.fixed_shift = fixed_point_shift(n_trees, off, nodes);
+  m.class_words = class_tree_words(n_trees, off, nodes);
   m.h_top = top;
   m.top_levels = L;
   m.top_compact = compact;
@@ -1426,9 +1261,6 @@ void fast_tiling(const GbdtModel& g, int P, int64_t per_problem, int* nblk, int*
   *nblk = static_cast<int>(n);
   *rows_per_cta = g.block_cands;
 }
-
-static int cand_rec_bytes(const GbdtModel& g) { return g.n_cand_rows > 0 ? (g.n_cand_rows + 15) / 16 * 16 : 16; }
-static int pair_rec_bytes(const GbdtModel& g) { return (g.n_pair_rows + 15) / 16 * 16; }
 
 size_t fast_scratch_bytes(const GbdtModel& g, int C) {
   return 256 + static_cast<size_t>(kCombos) * C * cand_rec_bytes(g);
@@ -1594,31 +1426,6 @@ cudaError_t launch_walk(const GbdtModel& g, const WalkArgs& a) {
   return launch_walk_geom<256, 1024>(g, a);
 }
 
-FastView make_view(const GbdtModel& g, const FastWait* wait) {
-  FastView fv{};
-  fv.n_rows = g.n_qrows;
-  fv.n_pair_rows = g.n_pair_rows;
-  fv.n_cand_rows = g.n_cand_rows;
-  fv.n_prob_rows = g.n_prob_rows;
-  fv.depth = g.fast_depth;
-  fv.n_chunks = g.n_chunks;
-  fv.chunk_bytes = g.chunk_bytes;
-  fv.tpc = g.tpc;
-  fv.n_thr = g.n_qthr;
-  fv.thr_cand0 = g.thr_cand0;
-  fv.thr_prob0 = g.thr_prob0;
-  fv.cand_rec = cand_rec_bytes(g);
-  fv.pair_rec = pair_rec_bytes(g);
-  fv.wait_limit = wait && wait->limit > 0 ? wait->limit : kFastWaitLimit;
-  fv.starve = wait ? wait->starve : 0;
-  fv.buf_bytes = g.buf_bytes;
-  fv.base = g.base;
-  fv.chunks = g.d_qnodes;
-  fv.thr = g.d_qthr;
-  fv.feat = g.d_qfeat;
-  return fv;
-}
-
 // Dynamic shared memory for `count` staged thresholds: all of them when they fit, else none (the
 // kernel then searches the global array). Returns the capacity in floats to pass to the kernel.
 int staged_floats(int count, size_t* bytes) {
@@ -1687,7 +1494,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
                                int k, unsigned long long* partial, void* scratch, int* status,
                                cudaStream_t stream, int64_t* launches, cudaEvent_t ev_begin,
                                const FastSlice* slice, void* memo_mem, const FastWait* wait,
-                               const FastPrepared* prep, const int32_t* perm) {
+                               const FastPrepared* prep, const int32_t* perm, const ClassCall* classes) {
   WalkArgs a{};
   a.desc = desc;
   if (p_by_value) a.pv = *p_by_value;
@@ -1787,6 +1594,11 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (ev_begin) cudaEventRecord(ev_begin, stream);
+  const int* path = nullptr;  // device word: whether the class walk serves the call
+  if (classes) {
+    e = prepare_classes(desc, g, d_p, P, d_c, C, *classes, stream, launches, &path);
+    if (e != cudaSuccess) return e;
+  }
 
   a.sl.n_slices = 1;
   if (slice && slice->n_slices > 1) {
@@ -1811,7 +1623,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
       const int64_t table_slots = static_cast<int64_t>(kSmCount) * (2 * (pthr_bytes + 4096) <= 227 * 1024 ? 2 : 1);
       pair_table_kernel<<<static_cast<unsigned>(table_items < table_slots ? table_items : table_slots), 256, pthr_bytes,
                           stream>>>(
-          desc, d_p ? d_p + first : nullptr, a.pv, a.uv, n, d_c, fv, memo, pthr_cap);
+          desc, d_p ? d_p + first : nullptr, a.pv, a.uv, n, d_c, fv, memo, pthr_cap, path);
       ++*launches;
     }
     a.dependent = memo.keys != nullptr;
@@ -1823,6 +1635,9 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     ++*launches;
     if (e != cudaSuccess) return e;
   }
+  if (classes)
+    return launch_classes(desc, g, P, d_c, C, d_rows, seg_off, seg_idx, nblk, rows_per_cta, k, partial, *classes, status,
+                          stream, launches, wait);
   return cudaSuccess;
 }
 
@@ -1876,11 +1691,12 @@ cudaError_t launch_score_fast(const ks_gpu_desc& desc, const GbdtModel& g, const
 int fast_bounds_line() {
   int v = 0;
   cudaMemcpyFromSymbol(&v, g_bounds_line, sizeof(int));
-  return v;
+  return v ? v : class_bounds_line();
 }
 void fast_bounds_clear() {
   const int z = 0;
   cudaMemcpyToSymbol(g_bounds_line, &z, sizeof(int));
+  class_bounds_clear();
 }
 #else
 int fast_bounds_line() { return -1; }

@@ -66,6 +66,8 @@ struct FastWait {
   int starve;
 };
 
+constexpr int kNoFixed = INT32_MIN;
+
 struct GbdtModel {
   int n_trees = 0;
   int max_depth = 0;
@@ -88,6 +90,8 @@ struct GbdtModel {
   FastTopParams* h_top = nullptr;  // host copy, passed by value at every launch
   int tpc = 0;                 // trees per chunk
   int n_chunks = 0;
+  int fixed_shift = kNoFixed;  // leaf values as integers, and the words of the largest tree compiled for
+  int class_words = 0;         // one candidate (ks_gbdt_classes.cu)
   int chunk_bytes = 0;
   uint32_t* d_qnodes = nullptr;  // [n_chunks][chunk_bytes / 4]
   float* d_qthr = nullptr;       // [n_qthr] sorted thresholds, feature after feature
@@ -191,6 +195,13 @@ bool valid_desc(const ks_gpu_desc& d);
 cudaError_t build_fast_gbdt(GbdtModel& m, int n_trees, const int64_t* h_tree_offsets,
                             const ks_node_host* h_nodes);
 
+// Walk of a whole class of candidates at once, for large batches (ks_gbdt_classes.cu).
+struct ClassCall {
+  int64_t pairs;
+  const int* order;  // the catalogue in similarity order
+  void* scratch;     // classes_scratch_bytes
+};
+
 // Slice mode of the quantised tree kernel (single-problem latency call).
 struct FastSlice {
   int n_slices;
@@ -217,6 +228,23 @@ size_t order_scratch_bytes(int C);
 cudaError_t launch_catalogue_order(const ks_candidate* d_c, int C, void* scratch, cudaStream_t stream,
                                    int64_t* launches);
 
+int class_tree_words(int n_trees, const int64_t* h_tree_offsets, const ks_node_host* h_nodes);
+int fixed_point_shift(int n_trees, const int64_t* h_tree_offsets, const ks_node_host* h_nodes);
+bool classes_apply(const GbdtModel& g, int P, int C, int64_t pairs);
+size_t classes_scratch_bytes(const GbdtModel& g, int P, int C);
+// units, sorted problems, and the choice: *path becomes a device word that is 1 when the class walk
+// serves the call
+cudaError_t prepare_classes(const ks_gpu_desc& desc, const GbdtModel& g, const ks_problem* d_p, int P,
+                            const ks_candidate* d_c, int C, const ClassCall& call, cudaStream_t stream,
+                            int64_t* launches, const int** path);
+// the walk and the ranking, which do nothing when the other path serves the call
+cudaError_t launch_classes(const ks_gpu_desc& desc, const GbdtModel& g, int P, const ks_candidate* d_c, int C,
+                           const uint8_t* cand_rows, const int64_t* seg_off, const int32_t* seg_idx, int nblk,
+                           int rows_per_block, int k, unsigned long long* partial, const ClassCall& call, int* status,
+                           cudaStream_t stream, int64_t* launches, const FastWait* wait);
+int class_bounds_line();  // checked build, as fast_bounds_line
+void class_bounds_clear();
+
 // Search-space enumeration and validity filtering (ks_catalogue.cu).
 cudaError_t launch_enumerate(long long first, long long count, ks_candidate* d_out, cudaStream_t stream,
                              int64_t* launches);
@@ -240,7 +268,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
                                cudaStream_t stream, int64_t* launches, cudaEvent_t ev_begin,
                                const FastSlice* slice = nullptr, void* memo_mem = nullptr,
                                const FastWait* wait = nullptr, const FastPrepared* prep = nullptr,
-                               const int32_t* perm = nullptr);
+                               const int32_t* perm = nullptr, const ClassCall* classes = nullptr);
 // Prepared catalogue (single-problem calls against a fixed catalogue and model).
 size_t fast_prepared_rows_bytes(const GbdtModel& g, int C);
 size_t fast_prepared_memo_bytes(const GbdtModel& g, int C);  // 0: the model's per-pair rows do not fit a record
