@@ -119,40 +119,64 @@ __global__ void combo_mask_kernel(const ks_problem* __restrict__ p, int P, unsig
   if ((threadIdx.x & 31) == 0 && m) atomicOr(mask, m);
 }
 
-__global__ void __launch_bounds__(256)
-cand_rows_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, const unsigned* mask_ptr,
-                 unsigned mask_value, FastView fv, uint8_t* __restrict__ out, MemoView memo, int thr_cap) {
-  extern __shared__ float s_cthr[];  // thresholds of the candidate-only features
+// A block of 256 threads stages the thresholds once and takes kBlock candidates of one type combination
+// after the other: kBlock threads evaluate the candidate-only columns, all search (256 / kBlock threads
+// a candidate, a column after the other), and the records, put together in shared memory, leave as whole
+// lines. What bounds it is latency: of the searches, and of fetching the instructions, so the columns
+// are a loop and not 29 copies of the search. kBlock = 64 where C leaves the machine idle (2,048
+// candidates: 30 us with one thread a candidate and byte stores, 11 us), else 256, which evaluates with
+// every thread. combo0: the only combination (grid y = 1), or -1: blockIdx.y.
+constexpr int kCandThreads = 256;
+template <int kBlockCands>
+__global__ void __launch_bounds__(kCandThreads)
+cand_rows_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, const unsigned* mask_ptr, int combo0,
+                 FastView fv, uint8_t* __restrict__ out, MemoView memo, int thr_cap) {
+  extern __shared__ __align__(16) float s_cthr[];  // thresholds of the candidate-only features, values, records
   __shared__ FeatQ s_fq[64];
-  const int combo = blockIdx.y;
-  if (blockIdx.x == 0 && combo == 0 && threadIdx.x == 0) g_fast_abort = 0;
-  const unsigned mask = mask_ptr ? *mask_ptr : mask_value;
-  if (!((mask >> combo) & 1u)) return;
+  const int combo = combo0 >= 0 ? combo0 : blockIdx.y, tid = threadIdx.x;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) g_fast_abort = 0;
+  if (mask_ptr && !((*mask_ptr >> combo) & 1u)) return;
   const float* T = stage_thresholds(fv, fv.thr_cand0, fv.thr_prob0 - fv.thr_cand0, s_cthr, thr_cap) - fv.thr_cand0;
-  if (threadIdx.x < 64) s_fq[threadIdx.x] = fv.feat[threadIdx.x];
-  __syncthreads();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= C) return;
+  if (tid < 64) s_fq[tid] = fv.feat[tid];
+  float* s_val = s_cthr + (thr_cap > 0 ? (thr_cap + 3) / 4 * 4 : 0);  // [column][candidate]
+  // records an odd number of words apart: no two threads of a warp on one bank
+  const int words = fv.cand_rec / 4, stride = words | 1, me = tid % kBlockCands;
+  uint32_t* recs = reinterpret_cast<uint32_t*>(s_val + kCandCols * kBlockCands);
+  uint8_t* rec = reinterpret_cast<uint8_t*>(recs + me * stride);
   ks_problem fake{};
   fake.m = fake.n = fake.k = 1;
   fake.dtype_ab = static_cast<uint8_t>(combo >> 2);
   fake.dtype_d = static_cast<uint8_t>(combo & 3);
-  ProblemTerms t;
-  problem_terms(fake, desc, t);
-  const ks_candidate cand = load_candidate(c + i);
-  uint8_t* rec = out + (static_cast<size_t>(combo) * C + i) * fv.cand_rec;
-  const int first = fv.n_pair_rows;
-  featurize_pair(t, cand, desc, [&](int col, float v) {
-    if (feat_class(col) != 1) return;
-    const FeatQ& q = s_fq[col];
-    quantise(q, T + q.thr0, v, false, [&](int row, uint8_t b) { rec[KS_IDX(row - first, fv.cand_rec)] = b; });
-  });
-  if (memo.keys)
-    memo.cls[static_cast<size_t>(combo) * C + i] = memo_assign(memo, combo, i, cand, resources(t, cand, desc).b_eff);
+  for (int base = blockIdx.x * kBlockCands; base < C; base += gridDim.x * kBlockCands) {
+    if (tid < kBlockCands) {
+      const int i = base + tid < C ? base + tid : C - 1;
+      ProblemTerms t;
+      problem_terms(fake, desc, t);
+      const ks_candidate cand = load_candidate(c + i);
+      featurize_pair(t, cand, desc, [&](int col, float v) {
+        if (feat_class(col) == 1) s_val[cand_slot(col) * kBlockCands + tid] = v;
+      });
+      if (memo.keys && base + tid < C)
+        memo.cls[static_cast<size_t>(combo) * C + i] = memo_assign(memo, combo, i, cand, resources(t, cand, desc).b_eff);
+    }
+    __syncthreads();
+    const int first = fv.n_pair_rows;
+#pragma unroll 1
+    for (int q = tid / kBlockCands; q < kCandCols; q += kCandThreads / kBlockCands) {
+      const FeatQ& f = s_fq[cand_col(q)];
+      quantise(f, T + f.thr0, s_val[q * kBlockCands + me], false,
+               [&](int row, uint8_t b) { rec[KS_IDX(row - first, fv.cand_rec)] = b; });
+    }
+    __syncthreads();
+    const int n = min(kBlockCands, C - base);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(out + (static_cast<size_t>(combo) * C + base) * fv.cand_rec);
+    for (int w = tid; w < n * words; w += kCandThreads) dst[w] = recs[w / words * stride + w % words];
+    __syncthreads();
+  }
 }
 
 // Packs the occupied slots of every type combination's table (one block per combination), so
-// that the per-problem kernel runs full warps over classes only.
+// that the per-problem kernel runs full warps over classes only. `keys` then holds a slot's place.
 __global__ void __launch_bounds__(1024)
 memo_compact_kernel(MemoView memo) {
   __shared__ int s_n;
@@ -160,8 +184,11 @@ memo_compact_kernel(MemoView memo) {
   if (threadIdx.x == 0) s_n = 0;
   __syncthreads();
   for (int slot = threadIdx.x; slot < kMemoCap; slot += 1024)
-    if (memo.keys[static_cast<size_t>(combo) * kMemoCap + slot] != 0ull)
-      memo.dense[static_cast<size_t>(combo) * kMemoCap + atomicAdd(&s_n, 1)] = slot;
+    if (memo.keys[static_cast<size_t>(combo) * kMemoCap + slot] != 0ull) {
+      const int j = atomicAdd(&s_n, 1);
+      memo.dense[static_cast<size_t>(combo) * kMemoCap + j] = slot;
+      memo.keys[static_cast<size_t>(combo) * kMemoCap + slot] = j;  // (the key is not needed any more)
+    }
   __syncthreads();
   if (threadIdx.x == 0) memo.count[combo] = s_n;
 }
@@ -1437,6 +1464,25 @@ int staged_floats(int count, size_t* bytes) {
 
 }  // namespace
 
+// combo >= 0: only that type combination; else those of the mask, or all (null).
+static cudaError_t launch_cand_rows(const ks_gpu_desc& desc, const GbdtModel& g, const ks_candidate* d_c, int C,
+                                    const unsigned* d_mask, int combo, const FastView& fv, uint8_t* d_rows,
+                                    const MemoView& memo, cudaStream_t stream, int64_t* launches) {
+  const int count = g.thr_prob0 - g.thr_cand0, block = C < 8192 ? 64 : 256;
+  const size_t own = static_cast<size_t>(block) * (cand_rec_bytes(g) + 4 + 4 * kCandCols);
+  size_t thr = (static_cast<size_t>(count) + 3) / 4 * 16;
+  int cap = count > 0 ? count : 1;
+  if (thr + own > 200 * 1024) cap = 0, thr = 0;  // (the global array is searched in place)
+  const size_t smem = std::max<size_t>(thr, 16) + own;
+  auto kernel = block == 64 ? &cand_rows_kernel<64> : &cand_rows_kernel<256>;
+  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<dim3(std::min((C + block - 1) / block, 2 * kSmCount), combo >= 0 ? 1 : kCombos), kCandThreads, smem, stream>>>(
+      desc, d_c, C, d_mask, combo, fv, d_rows, memo, cap);
+  ++*launches;
+  return cudaGetLastError();
+}
+
 // Prepared catalogue: the candidate-only rows of every candidate under every element-type
 // combination, and the candidates' classes, computed once for a (catalogue, model) pair.
 cudaError_t fast_prepare(const ks_gpu_desc& desc, const GbdtModel& g, const ks_candidate* d_c, int C, void* d_rows,
@@ -1444,17 +1490,13 @@ cudaError_t fast_prepare(const ks_gpu_desc& desc, const GbdtModel& g, const ks_c
   FastView fv = make_view(g, nullptr);
   MemoView memo{};
   if (memo_mem) memo = memo_view(memo_mem, C);
-  size_t cthr = 0;
-  const int cap = staged_floats(g.thr_prob0 - g.thr_cand0, &cthr);
-  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(&cand_rows_kernel), cthr);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   if (memo.keys) {
     e = memo_clear(memo, stream);
     if (e != cudaSuccess) return e;
   }
-  cand_rows_kernel<<<dim3((C + 255) / 256, kCombos), 256, cthr, stream>>>(desc, d_c, C, nullptr, 0xFFFFu, fv,
-                                                                          static_cast<uint8_t*>(d_rows), memo, cap);
-  ++*launches;
+  e = launch_cand_rows(desc, g, d_c, C, nullptr, -1, fv, static_cast<uint8_t*>(d_rows), memo, stream, launches);
+  if (e != cudaSuccess) return e;
   if (memo.keys) {
     e = memo_compact(memo, stream);
     if (e != cudaSuccess) return e;
@@ -1527,12 +1569,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
 
   // candidate-only rows for the type combinations in use
   cudaError_t e = cudaSuccess;
-  unsigned mask_value = 0;
-  if (prep) {
-    // nothing to do per call
-  } else if (a.uv) {
-    mask_value = 1u << ((a.pv.dtype_ab & 3) * 4 + (a.pv.dtype_d & 3));
-  } else {
+  if (!prep && !a.uv) {
     e = cudaMemsetAsync(d_mask, 0, sizeof(unsigned), stream);
     if (e != cudaSuccess) return e;
     combo_mask_kernel<<<P >= 4096 ? 16 : 1, 256, 0, stream>>>(d_p, P, d_mask);
@@ -1569,17 +1606,13 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
                                                                                    g.block_cands, slice->tiles, cap);
     ++*launches;
   } else if (C > 0) {
-    size_t cthr = 0;
-    const int cap = staged_floats(g.thr_prob0 - g.thr_cand0, &cthr);
-    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&cand_rows_kernel), cthr);
-    if (e != cudaSuccess) return e;
     if (memo.keys) {
       e = memo_clear(memo, stream);
       if (e != cudaSuccess) return e;
     }
-    cand_rows_kernel<<<dim3((C + 255) / 256, kCombos), 256, cthr, stream>>>(desc, d_c, C, a.uv ? nullptr : d_mask,
-                                                                            mask_value, fv, d_rows, memo, cap);
-    ++*launches;
+    e = launch_cand_rows(desc, g, d_c, C, a.uv ? nullptr : d_mask,
+                         a.uv ? (a.pv.dtype_ab & 3) * 4 + (a.pv.dtype_d & 3) : -1, fv, d_rows, memo, stream, launches);
+    if (e != cudaSuccess) return e;
     if (memo.keys) {
       e = ensure_dynamic_smem(reinterpret_cast<const void*>(&pair_table_kernel), pthr_bytes);
       if (e != cudaSuccess) return e;

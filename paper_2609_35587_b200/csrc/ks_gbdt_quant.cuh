@@ -116,25 +116,6 @@ __device__ __forceinline__ void quantise(const FeatQ& q, const float* T, float v
   emit_rows(q, pos, v, put);
 }
 
-// The per-pair columns (class 2 of feat_class) in ascending order, and a column's place among them.
-constexpr int kPairCols = 21;
-__host__ __device__ constexpr int pair_slot(int col) {
-  return col <= 36 ? col - 23 : (col == 39 ? 14 : (col <= 44 ? col - 26 : col - 41));
-}
-__host__ __device__ constexpr int pair_col(int slot) {
-  return slot <= 13 ? slot + 23 : (slot == 14 ? 39 : (slot <= 18 ? slot + 26 : slot + 41));
-}
-constexpr bool pair_slots_match_classes() {
-  int n = 0;
-  for (int c = 0; c < KS_F; ++c)
-    if (feat_class(c) == 2) {
-      if (pair_slot(c) != n || pair_col(n) != c) return false;
-      ++n;
-    }
-  return n == kPairCols;
-}
-static_assert(pair_slots_match_classes(), "per-pair columns");
-
 // All per-pair columns of one pair at once: the binary searches advance in step (one probe of
 // every column per round), so that a thread has 21 independent loads in flight instead of one
 // dependent chain after the other. `T` is the staged (or global) array of per-pair thresholds.

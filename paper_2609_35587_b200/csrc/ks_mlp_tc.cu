@@ -57,12 +57,8 @@ constexpr int kNC = 29, kNPair = 21;                  // candidate-only and per-
 // position of feature column `col` along K: candidate-only columns first, then per-pair, then
 // problem-only, each class in ascending column order; position 63 is the zero pad
 __host__ __device__ constexpr int kpos(int col) {
-  int pos = 0;
   const int cls = feat_class(col);
-  const int base = cls == 1 ? 0 : (cls == 2 ? kNC : kNC + kNPair);
-  for (int c = 0; c < col; ++c)
-    if (feat_class(c) == cls) ++pos;
-  return base + pos;
+  return cls == 1 ? cand_slot(col) : (cls == 2 ? kNC + pair_slot(col) : kNC + kNPair + prob_slot(col));
 }
 
 // One-hot input form: the candidate-only columns other than kernel / epilogue schedule at 0..26,
@@ -72,21 +68,14 @@ __host__ __device__ constexpr int kpos(int col) {
 __host__ __device__ constexpr int kpos_oh(int col) {
   const int cls = feat_class(col);
   if (cls == 0 || col == 17 || col == 18) return -1;
-  if (cls == 2) return kpos(col);
-  int pos = 0;
-  for (int c = 0; c < col; ++c)
-    if (feat_class(c) == 1 && c != 17 && c != 18) ++pos;
-  return pos;
+  return cls == 2 ? kpos(col) : cand_slot(col) - (col > 18 ? 2 : 0);
 }
 constexpr int kIndPos = 50;  // K position of the first level indicator
 // the folded inputs in order: problem-only columns other than operand type (5) and activation (9),
 // then the four operand-type indicators, then the three activation indicators
 __host__ __device__ constexpr int kfold(int col) {
   if (feat_class(col) != 0 || col == 5 || col == 9) return -1;
-  int pos = 0;
-  for (int c = 0; c < col; ++c)
-    if (feat_class(c) == 0 && c != 5 && c != 9) ++pos;
-  return pos;
+  return prob_slot(col) - (col > 5 ? 1 : 0) - (col > 9 ? 1 : 0);
 }
 constexpr int kFoldCols = 11, kFold = 18;
 
@@ -173,13 +162,15 @@ __global__ void mlp_combo_mask_kernel(const ks_problem* __restrict__ p, int P, u
   if ((threadIdx.x & 31) == 0 && m) atomicOr(mask, m);
 }
 
-__global__ void __launch_bounds__(256)
+// combo0: the only combination (grid y = 1), or -1: those of the mask, one per grid row. (Blocks of 128
+// threads spread 60,000 candidates evenly over the SMs; of 256, some SMs had twice the work of others.)
+constexpr int kCandThreads = 128;
+__global__ void __launch_bounds__(kCandThreads)
 mlp_cand_cols_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, const unsigned* mask_ptr,
-                     unsigned mask_value, const __grid_constant__ MlpTcParams prm, uint8_t* __restrict__ out) {
-  const int combo = blockIdx.y;
-  if (blockIdx.x == 0 && combo == 0 && threadIdx.x == 0) g_mlp_abort = 0;
-  const unsigned mask = mask_ptr ? *mask_ptr : mask_value;
-  if (!((mask >> combo) & 1u)) return;
+                     int combo0, const __grid_constant__ MlpTcParams prm, uint8_t* __restrict__ out) {
+  const int combo = combo0 >= 0 ? combo0 : blockIdx.y;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) g_mlp_abort = 0;
+  if (mask_ptr && !((*mask_ptr >> combo) & 1u)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= C) return;
   ks_problem fake{};
@@ -841,19 +832,16 @@ cudaError_t launch_select_mlp_tc(const ks_gpu_desc& desc, const MlpModel& m, con
   const int uv = p_by_value != nullptr;
   unsigned* d_mask = static_cast<unsigned*>(scratch);
   uint8_t* d_cols = static_cast<uint8_t*>(scratch) + 256;
-  unsigned mask_value = 0;
   cudaError_t e;
-  if (uv) {
-    mask_value = 1u << ((pv.dtype_ab & 3) * 4 + (pv.dtype_d & 3));
-  } else {
+  if (!uv) {
     e = cudaMemsetAsync(d_mask, 0, sizeof(unsigned), stream);
     if (e != cudaSuccess) return e;
     mlp_combo_mask_kernel<<<P >= 4096 ? 16 : 1, 256, 0, stream>>>(d_p, P, d_mask);
     ++*launches;
   }
   if (C > 0) {
-    mlp_cand_cols_kernel<<<dim3((C + 255) / 256, kCombos), 256, 0, stream>>>(desc, d_c, C, uv ? nullptr : d_mask,
-                                                                             mask_value, *m.h_tc_params, d_cols);
+    mlp_cand_cols_kernel<<<dim3((C + kCandThreads - 1) / kCandThreads, uv ? 1 : kCombos), kCandThreads, 0, stream>>>(
+        desc, d_c, C, uv ? nullptr : d_mask, uv ? (pv.dtype_ab & 3) * 4 + (pv.dtype_d & 3) : -1, *m.h_tc_params, d_cols);
     ++*launches;
   }
   e = cudaGetLastError();
