@@ -293,7 +293,6 @@ void free_fast_mlp(MlpModel& m);
 cudaError_t build_ridge(MlpModel& m, const uint16_t* h_w, const float* h_b, const float* h_mu,
                         const float* h_sigma);
 void free_ridge(MlpModel& m);
-size_t ridge_scratch_bytes(int C);
 int mlp_tc_blocks_per_problem(int P, int64_t per_problem);
 size_t mlp_tc_scratch_bytes(int C);
 // ks_score on the tensor-core kernel (ordinal input form only): the given rows are the input.

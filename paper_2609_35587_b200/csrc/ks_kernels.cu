@@ -4,6 +4,8 @@
 // in ks_gbdt_fast.cu.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -88,13 +90,6 @@ struct ProblemEntry {
   float pc[16];  // the problem-only columns, in column order
 };
 
-__host__ __device__ constexpr int class_slot(int col) {
-  int n = 0;
-  for (int q = 0; q < col; ++q)
-    if (feat_class(q) == feat_class(col)) ++n;
-  return n;
-}
-
 __global__ void __launch_bounds__(128)
 problem_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, int P, ProblemEntry* __restrict__ tab) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -107,7 +102,7 @@ problem_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, int P, 
 #pragma unroll
   for (int q = 0; q < 16; ++q) e.pc[q] = 0.0f;
   featurize_pair(e.t, dummy, desc, [&](int col, float v) {
-    if (feat_class(col) == 0) e.pc[class_slot(col)] = v;
+    if (feat_class(col) == 0) e.pc[prob_slot(col)] = v;
   });
   tab[i] = e;
 }
@@ -146,13 +141,13 @@ featurize_dense_kernel(ks_gpu_desc desc, const ProblemEntry* __restrict__ tab, c
       combo_prev = combo;
       b_eff = resources(t, cand, desc).b_eff;
       featurize_pair(t, cand, desc, [&](int col, float v) {
-        if (feat_class(col) == 1) cc[class_slot(col)] = v;
+        if (feat_class(col) == 1) cc[cand_slot(col)] = v;
       });
     }
 #pragma unroll
     for (int col = 0; col < KS_F; ++col) {
-      if (feat_class(col) == 1) row[col] = cc[class_slot(col)];
-      if (feat_class(col) == 0) row[col] = __ldg(&e.pc[class_slot(col)]);
+      if (feat_class(col) == 1) row[col] = cc[cand_slot(col)];
+      if (feat_class(col) == 0) row[col] = __ldg(&e.pc[prob_slot(col)]);
     }
     row[KS_F] = 0.0f;
     pair_columns<true>(t, cand, desc, b_eff, [&](int col, float v) { row[col] = v; });
@@ -352,11 +347,9 @@ __device__ __forceinline__ float ridge_level(const float (&lut)[4], float v) {
 // per (type combination, candidate): (candidate-only part of the sum, resident-block count)
 __global__ void __launch_bounds__(256)
 ridge_cand_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, const unsigned* mask_ptr,
-                  unsigned mask_value, const __grid_constant__ RidgeParams prm, float2* __restrict__ out,
-                  MemoView memo) {
+                  const __grid_constant__ RidgeParams prm, float2* __restrict__ out, MemoView memo) {
   const int combo = blockIdx.y;
-  const unsigned mask = mask_ptr ? *mask_ptr : mask_value;
-  if (!((mask >> combo) & 1u)) return;
+  if (!((*mask_ptr >> combo) & 1u)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= C) return;
   ks_problem fake{};
@@ -378,130 +371,237 @@ ridge_cand_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, c
   if (memo.keys) memo.cls[static_cast<size_t>(combo) * C + i] = memo_assign(memo, combo, i, cand, b_eff);
 }
 
-// Per (problem, class): the per-pair part of the sum, from the class's member (classes:
-// ks_memo.cuh). grid (kMemoCap / 256, P); blocks past the number of classes leave at once.
+// What a problem brings: its terms, and the bias + problem-only part of the sum; and the combinations
+// in use.
+struct RidgeProblem {
+  ProblemTerms t;
+  float sum;
+  int combo;
+};
+__global__ void __launch_bounds__(128)
+ridge_problem_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int P,
+                     const __grid_constant__ RidgeParams prm, RidgeProblem* __restrict__ out, unsigned* __restrict__ mask) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= P) return;
+  RidgeProblem e;
+  problem_terms(use_value ? p_value : p[i], desc, e.t);
+  e.combo = e.t.dtype_ab * 4 + e.t.dtype_d;
+  float s = prm.bias;
+  problem_columns(e.t, [&](int col, float v) {
+    s += ridge_term(prm, col, v);
+    if (col == 5) s += ridge_level(prm.lut5, v);
+    if (col == 9) s += ridge_level(prm.lut9, v);
+  });
+  e.sum = s;
+  out[i] = e;
+  const unsigned m = __reduce_or_sync(__activemask(), 1u << e.combo);
+  if ((threadIdx.x & 31) == 0) atomicOr(mask, m);
+}
+
+// With classes: a candidate's second word, so far its resident-block count b, becomes the number of
+// its class among the classes in use, or -b when it has none (memo_compact left the numbers in `keys`).
 __global__ void __launch_bounds__(256)
-ridge_pair_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, const ks_candidate* __restrict__ c,
-                  const float2* __restrict__ cand_tab, int C, const __grid_constant__ RidgeParams prm, MemoView memo) {
+ridge_pack_kernel(int C, const unsigned* __restrict__ mask, MemoView memo, float2* __restrict__ tab) {
+  const int combo = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (!((*mask >> combo) & 1u) || i >= C) return;
+  const unsigned slot = memo.cls[static_cast<size_t>(combo) * C + i];
+  float& y = tab[static_cast<size_t>(combo) * C + i].y;
+  const int v = slot == kNoClass ? -static_cast<int>(y) : static_cast<int>(memo.keys[static_cast<size_t>(combo) * kMemoCap + slot]);
+  y = __int_as_float(v);
+}
+
+// Per (problem, class): the per-pair part of the sum, from the class's member (classes: ks_memo.cuh).
+// grid (a few, P); record j of a problem is its j-th class.
+__global__ void __launch_bounds__(256)
+ridge_pair_kernel(ks_gpu_desc desc, const RidgeProblem* __restrict__ problems, const ks_candidate* __restrict__ c,
+                  const __grid_constant__ RidgeParams prm, MemoView memo) {
   __shared__ ProblemTerms s_pt;
-  const int prob = blockIdx.y, j = blockIdx.x * 256 + threadIdx.x;
-  const ks_problem pr = p[prob];
-  const int combo = (pr.dtype_ab & 3) * 4 + (pr.dtype_d & 3);
+  const int prob = blockIdx.y, combo = problems[prob].combo;
   const int n_classes = memo.count[combo];
-  if (blockIdx.x * 256 >= n_classes) return;
-  if (threadIdx.x == 0) problem_terms(pr, desc, s_pt);
+  if (threadIdx.x < sizeof(ProblemTerms) / 4)
+    reinterpret_cast<uint32_t*>(&s_pt)[threadIdx.x] = reinterpret_cast<const uint32_t*>(&problems[prob].t)[threadIdx.x];
   __syncthreads();
-  if (j >= n_classes) return;
-  const int slot = memo.dense[static_cast<size_t>(combo) * kMemoCap + j];
-  const int rep = memo.reps[static_cast<size_t>(combo) * kMemoCap + slot];
-  const ks_candidate cand = c[rep];
-  const float2 t = __ldg(cand_tab + static_cast<size_t>(combo) * C + rep);
+  for (int j = blockIdx.x * 256 + threadIdx.x; j < n_classes; j += gridDim.x * 256) {
+    const int slot = memo.dense[static_cast<size_t>(combo) * kMemoCap + j];
+    const ks_candidate cand = load_candidate(c + memo.reps[static_cast<size_t>(combo) * kMemoCap + slot]);
+    float pair = 0.0f;
+    pair_columns<true>(s_pt, cand, desc, resources(s_pt, cand, desc).b_eff,
+                       [&](int col, float v) { pair += ridge_term(prm, col, v); });
+    static_cast<float*>(memo.tab)[static_cast<size_t>(prob) * kMemoCap + j] = pair;
+  }
+}
+
+// the per-pair part in place, for a candidate without a class (out of line: it would cost the kernel
+// half its resident warps)
+__device__ __noinline__ float ridge_pair_in_place(const ks_gpu_desc& desc, const ProblemTerms& t, const ks_candidate* c,
+                                                  long long b_eff, const RidgeParams& prm) {
   float pair = 0.0f;
-  pair_columns<true>(s_pt, cand, desc, static_cast<long long>(t.y),
-                     [&](int col, float v) { pair += ridge_term(prm, col, v); });
-  static_cast<float*>(memo.tab)[static_cast<size_t>(prob) * kMemoCap + slot] = pair;
+  pair_columns<true>(t, load_candidate(c), desc, b_eff, [&](int col, float v) { pair += ridge_term(prm, col, v); });
+  return pair;
 }
 
-__global__ void ridge_combo_mask_kernel(const ks_problem* __restrict__ p, int P, unsigned* __restrict__ mask) {
-  unsigned m = 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P; i += gridDim.x * blockDim.x)
-    m |= 1u << ((p[i].dtype_ab & 3) * 4 + (p[i].dtype_d & 3));
-  m = __reduce_or_sync(0xFFFFFFFFu, m);
-  if ((threadIdx.x & 31) == 0 && m) atomicOr(mask, m);
-}
-
-__global__ void __launch_bounds__(kBlock)
-select_ridge_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value,
-                    const ks_candidate* __restrict__ c, PairMap map, int sub_tiles,
-                    const float2* __restrict__ cand_tab, const __grid_constant__ RidgeParams prm, int k,
+// A block ranks kQ problems against its share of the candidates. What bounds it is the instructions a
+// pair takes, so a candidate is fetched once for the kQ problems, the class sums are gathered from
+// shared memory, and a warp keeps a running top-k list (one key a lane): a score that does not reach
+// the best k-th score any of the block's warps has seen costs no more than the comparison. (Ranking
+// eight keys a thread from scratch, with sums from L2, took 852 us for 1,024 x 60,000 pairs.)
+constexpr int kRidgeThreads = 512, kRidgeProblems = 4;
+constexpr int kRidgeClasses = 2048;  // classes whose sums are staged; the others are fetched from L2
+// kClasses: with the class tables; without them (few problems) every pair is evaluated in place.
+template <int kQ, bool kClasses>
+__global__ void __launch_bounds__(kRidgeThreads, kClasses ? 2 : 1)
+select_ridge_kernel(const __grid_constant__ ks_gpu_desc desc, const RidgeProblem* __restrict__ problems, const ks_candidate* __restrict__ c,
+                    PairMap map, const float2* __restrict__ cand_tab, const __grid_constant__ RidgeParams prm, int k,
                     unsigned long long* __restrict__ partial /* [P][nblk][k] */, MemoView memo) {
-  __shared__ ProblemTerms s_pt;
-  __shared__ float s_prob;  // bias + problem-only part of the sum
-  __shared__ unsigned long long s_warp[kBlock / 32 * KS_MAX_K];
-  __shared__ unsigned long long s_list[KS_MAX_K];
-  const int prob = blockIdx.x / map.nblk, chunk = blockIdx.x % map.nblk;
-  int64_t lo, len;
-  segment_of(map, prob, lo, len);
-  if (threadIdx.x == 0) {
-    problem_terms(use_value ? p_value : p[prob], desc, s_pt);
-    ks_candidate dummy{};
-    dummy.tile_m = dummy.tile_n = dummy.tile_k = 64;
-    dummy.stages = dummy.cluster_m = dummy.cluster_n = 1;
-    float s = prm.bias;
-    featurize_pair(s_pt, dummy, desc, [&](int col, float v) {
-      if (feat_class(col) != 0) return;
-      s += ridge_term(prm, col, v);
-      if (col == 5) s += ridge_level(prm.lut5, v);
-      if (col == 9) s += ridge_level(prm.lut9, v);
-    });
-    s_prob = s;
-  }
-  if (threadIdx.x < KS_MAX_K) s_list[threadIdx.x] = 0ull;
-  __syncthreads();
-  const float2* tab = cand_tab + static_cast<size_t>(s_pt.dtype_ab * 4 + s_pt.dtype_d) * map.C;
-  // with classes: the per-pair part is one float per (problem, class)
-  const unsigned* cls = memo.keys ? memo.cls + static_cast<size_t>(s_pt.dtype_ab * 4 + s_pt.dtype_d) * map.C : nullptr;
-  const float* pair_tab = memo.keys ? static_cast<const float*>(memo.tab) + static_cast<size_t>(prob) * kMemoCap : nullptr;
-
-  const int64_t pass_rows = static_cast<int64_t>(sub_tiles) * kBlock;
-  for (int64_t start = static_cast<int64_t>(chunk) * pass_rows; start < len;
-       start += static_cast<int64_t>(map.nblk) * pass_rows) {
-    unsigned long long keys[kSubTilesMax + 1];
+  __shared__ float s_tab[kQ][kClasses ? kRidgeClasses : 1];
+  __shared__ ProblemTerms s_pt;  // (without classes, where kQ = 1)
+  __shared__ unsigned s_bar[kQ];  // upper word of a key below which nothing can make the list
+  __shared__ unsigned s_best[kQ][2 * kRidgeThreads / 32];  // the warps' best keys (one each, two for k > 16)
+  __shared__ unsigned long long s_list[kRidgeThreads / 32][32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int group = blockIdx.x / map.nblk, chunk = blockIdx.x % map.nblk;
+  __shared__ int s_combo[kQ];
+  __shared__ float s_sum[kQ];
+  auto prob = [&](int q) { return min(group * kQ + q, map.P - 1); };
+  unsigned long long top[kQ];
 #pragma unroll
-    for (int s = 0; s <= kSubTilesMax; ++s) keys[s] = 0ull;
-    if (threadIdx.x < k) keys[kSubTilesMax] = s_list[threadIdx.x];
-#pragma unroll 1
-    for (int s = 0; s < sub_tiles; ++s) {
-      const int64_t r = start + static_cast<int64_t>(s) * kBlock + threadIdx.x;
-      unsigned long long key = 0ull;
-      if (r < len) {
-        const int idx = pool_index(map, lo, r);
-        const float2 t = __ldg(tab + idx);
-        const unsigned cid = cls ? __ldg(cls + idx) : kNoClass;
-        float pair = 0.0f;
-        if (cid != kNoClass) {
-          pair = __ldg(pair_tab + cid);
-        } else {
-          const ks_candidate cand = c[idx];
-          pair_columns<true>(s_pt, cand, desc, static_cast<long long>(t.y),
-                             [&](int col, float v) { pair += ridge_term(prm, col, v); });
-        }
-        key = make_key(((s_prob + t.x) + pair) + 0.0f, idx);
-      }
-#pragma unroll
-      for (int q = 0; q < kSubTilesMax; ++q)
-        if (q == s) keys[q] = key;
+  for (int q = 0; q < kQ; ++q) {
+    const int combo = problems[prob(q)].combo;
+    if (tid == 0) {
+      s_combo[q] = combo;
+      s_sum[q] = problems[prob(q)].sum;
     }
-    block_topk<kSubTilesMax + 1>(keys, k, s_warp, s_list);
+    top[q] = 0ull;
+    if (kClasses) {
+      const int n = min(memo.count[combo], kRidgeClasses);
+      const float* src = static_cast<const float*>(memo.tab) + static_cast<size_t>(prob(q)) * kMemoCap;
+      for (int j = tid; j < n; j += kRidgeThreads) s_tab[q][j] = __ldg(src + j);
+    }
   }
-  if (threadIdx.x < k)
-    partial[(static_cast<size_t>(prob) * map.nblk + chunk) * k + threadIdx.x] = s_list[threadIdx.x];
+  if (!kClasses && tid < static_cast<int>(sizeof(ProblemTerms) / 4))
+    reinterpret_cast<uint32_t*>(&s_pt)[tid] = reinterpret_cast<const uint32_t*>(&problems[prob(0)].t)[tid];
+  if (tid < kQ) s_bar[tid] = 0u;
+  if (tid < kQ * 2 * kRidgeThreads / 32) (&s_best[0][0])[tid] = 0u;
+  __syncthreads();
+  int64_t lo, len;  // (per-problem segments: kQ = 1)
+  segment_of(map, prob(0), lo, len);
+  const int64_t share = (len + map.nblk - 1) / map.nblk, stop = min(len, share * (chunk + 1));
+  bool mixed = false;  // element types differ among the block's problems
+#pragma unroll
+  for (int q = 1; q < kQ; ++q) mixed |= s_combo[q] != s_combo[0];
+  const float2* tab0 = cand_tab + static_cast<size_t>(s_combo[0]) * map.C;
+  // a candidate's record is fetched one round ahead
+  auto row_index = [&](int64_t r) { return r < stop ? pool_index(map, lo, r) : 0; };
+  const int64_t r_first = share * chunk + warp * 32 + lane;
+  int next_idx = row_index(r_first);
+  float2 next = __ldg(tab0 + next_idx);
+  for (int64_t r = r_first; r - lane < stop; r += kRidgeThreads) {
+    const bool live = r < stop;
+    const int idx = next_idx;
+    float2 t = next;
+    next_idx = row_index(r + kRidgeThreads);
+    next = __ldg(tab0 + next_idx);
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) {
+      if (q > 0 && mixed) t = __ldg(cand_tab + static_cast<size_t>(s_combo[q]) * map.C + idx);
+      const int cls = __float_as_int(t.y);
+      float pair = 0.0f;
+      if (kClasses && cls >= 0) {
+        pair = cls < kRidgeClasses ? s_tab[q][cls]
+                                   : __ldg(static_cast<const float*>(memo.tab) + static_cast<size_t>(prob(q)) * kMemoCap + cls);
+      } else if (kClasses) {
+        pair = ridge_pair_in_place(desc, problems[prob(q)].t, c + idx, -static_cast<long long>(cls), prm);
+      } else {
+        pair_columns<true>(s_pt, load_candidate(c + idx), desc, static_cast<long long>(t.y),
+                           [&](int col, float v) { pair += ridge_term(prm, col, v); });
+      }
+      const float score = ((s_sum[q] + t.x) + pair) + 0.0f;
+      if (__any_sync(0xFFFFFFFFu, live && sortable(score) >= *const_cast<volatile unsigned*>(&s_bar[q]))) {
+        warp_topk_insert(top[q], live ? make_key(score, idx) : 0ull, k);
+        // The k-th largest of the warps' best keys bounds the k-th best score from below (each is a
+        // candidate of its own), far better than any one warp's k-th.
+        constexpr int kWarps = kRidgeThreads / 32;
+        unsigned* best = s_best[q];
+        const int each = k > kWarps ? 2 : 1;
+        if (lane < each) best[warp * 2 + lane] = static_cast<unsigned>(top[q] >> 32);
+        __syncwarp();
+        const unsigned v = (lane & 1) < each ? *const_cast<volatile unsigned*>(&best[lane]) : 0u;
+        int ahead = 0;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) ahead += __shfl_sync(0xFFFFFFFFu, v, i) >= v;
+        const unsigned bar = __reduce_max_sync(0xFFFFFFFFu, ahead >= k ? v : 0u);
+        if (lane == 0) atomicMax(&s_bar[q], bar);
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < kQ; ++q) {
+    __syncthreads();
+    s_list[warp][lane] = top[q];
+    __syncthreads();
+    if (warp == 0 && group * kQ + q < map.P) {
+      unsigned long long mine = top[q];
+      for (int w = 1; w < kRidgeThreads / 32; ++w) warp_topk_insert(mine, s_list[w][lane], k);
+      if (lane < k) partial[(static_cast<size_t>(prob(q)) * map.nblk + chunk) * k + lane] = mine;
+    }
+  }
+}
+
+// Problems a block ranks, and blocks per group of problems: as many as fill the machine once (two blocks
+// of 512 threads an SM), with about 512 candidates each at least.
+static int ridge_group(bool segmented, int P) { return segmented || P < kMemoMinProblems ? 1 : kRidgeProblems; }
+static int ridge_blocks(int P, int64_t per_problem, bool segmented) {
+  const int g = ridge_group(segmented, P);
+  const int64_t groups = (P + g - 1) / g, most = std::max<int64_t>(1, (per_problem + 511) / 512);
+  return static_cast<int>(std::min(most, std::max<int64_t>(1, 2 * 148 / groups)));
 }
 
 // ------------------------------------------------------------------------------------------
-// merge: one warp per problem ranks the nblk * k partial keys
+// merge: ranks the nblk * k partial keys of a problem
 // ------------------------------------------------------------------------------------------
 
+// A warp (kWarps = 1, eight problems a block) or a block of eight warps ranks a problem's keys, each
+// read once into the warp's running list; a block's lists are merged by its first warp. (One warp that
+// read the keys again for each of the k ranks took 19 us for the 1,480 keys of a single problem.)
+template <int kWarps>
 __global__ void __launch_bounds__(kBlock)
 topk_merge_kernel(const unsigned long long* __restrict__ partial, int P, int n_keys, int k,
                   int32_t* __restrict__ out_idx, float* __restrict__ out_score) {
-  const int warp = (blockIdx.x * kBlock + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= P) return;
-  const unsigned long long* keys = partial + static_cast<size_t>(warp) * n_keys;
-  unsigned long long prev = ~0ull;
-  for (int j = 0; j < k; ++j) {
-    unsigned long long best = 0ull;
-    for (int i = lane; i < n_keys; i += 32) {
-      const unsigned long long v = keys[i];
-      if (v < prev && v > best) best = v;
-    }
-    best = warp_max_u64(best);
-    if (lane == 0) {
-      out_idx[static_cast<size_t>(warp) * k + j] = key_index(best);
-      out_score[static_cast<size_t>(warp) * k + j] = key_score(best);
-    }
-    prev = best == 0ull ? 0ull : best;
+  __shared__ unsigned long long s_list[kWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int prob = kWarps == 1 ? blockIdx.x * (kBlock / 32) + warp : blockIdx.x, part = kWarps == 1 ? 0 : warp;
+  if (prob >= P) return;
+  const unsigned long long* keys = partial + static_cast<size_t>(prob) * n_keys;
+  unsigned long long mine = 0ull;
+  for (int i0 = part * 128; i0 < n_keys; i0 += kWarps * 128) {
+    unsigned long long v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = i0 + 32 * q + lane < n_keys ? keys[i0 + 32 * q + lane] : 0ull;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) warp_topk_insert(mine, v[q], k);
   }
+  if (kWarps > 1) {
+    s_list[part][lane] = mine;
+    __syncthreads();
+    if (warp != 0) return;
+    for (int w = 1; w < kWarps; ++w) warp_topk_insert(mine, s_list[w][lane], k);
+  }
+  if (lane < k) {
+    out_idx[static_cast<size_t>(prob) * k + lane] = key_index(mine);
+    out_score[static_cast<size_t>(prob) * k + lane] = key_score(mine);
+  }
+}
+
+// A block per problem while that leaves the machine room, else a warp.
+static cudaError_t launch_merge(const unsigned long long* partial, int P, int n_keys, int k, int32_t* d_topk_idx,
+                                float* d_topk_score, cudaStream_t stream, int64_t* launches) {
+  constexpr int kPer = kBlock / 32;
+  if (P <= 8 * 148 && n_keys > 128)
+    topk_merge_kernel<kPer><<<P, kBlock, 0, stream>>>(partial, P, n_keys, k, d_topk_idx, d_topk_score);
+  else
+    topk_merge_kernel<1><<<(P + kPer - 1) / kPer, kBlock, 0, stream>>>(partial, P, n_keys, k, d_topk_idx, d_topk_score);
+  if (launches) ++*launches;
+  return cudaGetLastError();
 }
 
 // Merge of ranked lists (the exchange step of a candidate-split selection): per problem, n
@@ -678,7 +778,9 @@ cudaError_t launch_score_linear(const MlpModel& m, const float* d_feat, int64_t 
   return cudaGetLastError();
 }
 
-size_t ridge_scratch_bytes(int C) { return (256 + sizeof(float2) * 16 * static_cast<size_t>(C) + 255) / 256 * 256; }
+size_t ridge_scratch_bytes(int P, int C) {
+  return 256 + (sizeof(float2) * 16 * static_cast<size_t>(C) + 255) / 256 * 256 + (sizeof(RidgeProblem) * static_cast<size_t>(P) + 255) / 256 * 256;
+}
 // classes and the per-(problem, class) sums of the linear scorer (0: not used)
 size_t ridge_memo_bytes(int P, int C) {
   if (P < kMemoMinProblems || P > kMemoMaxProblems || C < 1) return 0;
@@ -722,13 +824,14 @@ size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, 
     const size_t part = static_cast<size_t>(P) * wide_rank_blocks(per) * k * sizeof(unsigned long long);
     return (part + 255) / 256 * 256 + wide_scratch_bytes(model.mlp, P, pairs);
   }
+  if (model.kind == 1 && model.mlp.h_ridge) {
+    const size_t part = static_cast<size_t>(P) * ridge_blocks(P, per, segmented) * k * sizeof(unsigned long long);
+    return (part + 255) / 256 * 256 + ridge_scratch_bytes(P, C) + ridge_memo_bytes(P, C);
+  }
   const int st = pick_sub_tiles(P, per);
   int64_t nblk = (per + static_cast<int64_t>(st) * kBlock - 1) / (static_cast<int64_t>(st) * kBlock);
   if (nblk < 1) nblk = 1;
-  const size_t part = static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long);
-  if (model.kind == 1 && model.mlp.h_ridge)
-    return (part + 255) / 256 * 256 + ridge_scratch_bytes(C) + ridge_memo_bytes(P, C);
-  return part;
+  return static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long);
 }
 
 cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const ks_problem* d_p,
@@ -778,10 +881,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                                        nullptr, perm, use_classes ? &classes : nullptr);
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    topk_merge_kernel<<<(P * 32 + kBlock - 1) / kBlock, kBlock, 0, stream>>>(part, P, nblk * k, k, d_topk_idx,
-                                                                            d_topk_score);
-    ++*launches;
-    return cudaGetLastError();
+    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
   }
   if (model.kind == 1 && model.mlp.tc) {
     const int nblk = mlp_tc_blocks_per_problem(P, per);
@@ -792,10 +892,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                                          launches, ev_begin, wait);
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    topk_merge_kernel<<<(P * 32 + kBlock - 1) / kBlock, kBlock, 0, stream>>>(part, P, nblk * k, k, d_topk_idx,
-                                                                            d_topk_score);
-    ++*launches;
-    return cudaGetLastError();
+    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
   }
   if (model.kind == 1 && model.mlp.wide) {
     const int nblk = wide_rank_blocks(per);
@@ -806,10 +903,56 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                                        ev_begin, wait);
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    topk_merge_kernel<<<(P * 32 + kBlock - 1) / kBlock, kBlock, 0, stream>>>(part, P, nblk * k, k, d_topk_idx,
-                                                                            d_topk_score);
+    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
+  }
+  if (model.kind == 1 && model.mlp.h_ridge) {
+    // linear scorer: per-call tables of what a problem, a candidate and a class bring, then the kernel
+    // that adds and ranks
+    PairMap map = make_map(P, C, pairs, d_seg_off, d_seg_idx, kBlock);
+    map.nblk = ridge_blocks(P, per, d_seg_off != nullptr);
+    unsigned long long* partial = static_cast<unsigned long long*>(d_partial);
+    const size_t part_bytes = (static_cast<size_t>(P) * map.nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
+    char* mem = static_cast<char*>(d_partial) + part_bytes;
+    unsigned* d_mask = reinterpret_cast<unsigned*>(mem);
+    float2* d_tab = reinterpret_cast<float2*>(mem + 256);
+    RidgeProblem* d_prob =
+        reinterpret_cast<RidgeProblem*>(mem + 256 + (sizeof(float2) * 16 * static_cast<size_t>(C) + 255) / 256 * 256);
+    const RidgeParams& prm = *model.mlp.h_ridge;
+    ks_problem pv{};
+    if (p_by_value) pv = *p_by_value;
+    cudaError_t e = cudaMemsetAsync(d_mask, 0, sizeof(unsigned), stream);
+    if (e != cudaSuccess) return e;
+    ridge_problem_kernel<<<(P + 127) / 128, 128, 0, stream>>>(desc, d_p, pv, p_by_value != nullptr, P, prm, d_prob, d_mask);
     ++*launches;
-    return cudaGetLastError();
+    MemoView memo{};
+    if (!p_by_value && C > 0 && ridge_memo_bytes(P, C) != 0) {
+      memo = memo_view(mem + ridge_scratch_bytes(P, C), C);
+      e = memo_clear(memo, stream);
+      if (e != cudaSuccess) return e;
+    }
+    if (C > 0) {
+      ridge_cand_kernel<<<dim3((C + 255) / 256, 16), 256, 0, stream>>>(desc, d_c, C, d_mask, prm, d_tab, memo);
+      ++*launches;
+      if (memo.keys) {
+        e = memo_compact(memo, stream);
+        if (e != cudaSuccess) return e;
+        ridge_pack_kernel<<<dim3((C + 255) / 256, 16), 256, 0, stream>>>(C, d_mask, memo, d_tab);
+        // enough blocks for 2,048 classes a problem; they loop over more
+        ridge_pair_kernel<<<dim3(P < 512 ? 8 : 2, P), 256, 0, stream>>>(desc, d_prob, d_c, prm, memo);
+        *launches += 3;
+      }
+    }
+    if (ev_begin) cudaEventRecord(ev_begin, stream);
+    const int group = ridge_group(d_seg_off != nullptr, P);
+    const unsigned blocks = static_cast<unsigned>(static_cast<int64_t>((P + group - 1) / group) * map.nblk);
+    auto kernel = !memo.keys ? &select_ridge_kernel<1, false>
+                  : group == 1 ? &select_ridge_kernel<1, true> : &select_ridge_kernel<kRidgeProblems, true>;
+    kernel<<<blocks, kRidgeThreads, 0, stream>>>(desc, d_prob, d_c, map, d_tab, prm, k, partial, memo);
+    ++*launches;
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (ev_end) cudaEventRecord(ev_end, stream);
+    return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
   }
   const int st = pick_sub_tiles(P, per);
   const PairMap map = make_map(P, C, pairs, d_seg_off, d_seg_idx, st * kBlock);
@@ -818,52 +961,6 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
   ks_problem pv{};
   if (p_by_value) pv = *p_by_value;
   cudaError_t e;
-  if (model.kind == 1 && model.mlp.h_ridge) {
-    // linear scorer: per-call table of candidate-only sums, then the fused kernel
-    const size_t part_bytes = (static_cast<size_t>(P) * map.nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
-    unsigned* d_mask = reinterpret_cast<unsigned*>(static_cast<char*>(d_partial) + part_bytes);
-    float2* d_tab = reinterpret_cast<float2*>(static_cast<char*>(d_partial) + part_bytes + 256);
-    unsigned mask_value = 0;
-    if (p_by_value) {
-      mask_value = 1u << ((pv.dtype_ab & 3) * 4 + (pv.dtype_d & 3));
-    } else {
-      e = cudaMemsetAsync(d_mask, 0, sizeof(unsigned), stream);
-      if (e != cudaSuccess) return e;
-      ridge_combo_mask_kernel<<<P >= 4096 ? 16 : 1, 256, 0, stream>>>(d_p, P, d_mask);
-      ++*launches;
-    }
-    MemoView memo{};
-    if (!p_by_value && ridge_memo_bytes(P, C) != 0)
-      memo = memo_view(static_cast<char*>(d_partial) + part_bytes + ridge_scratch_bytes(C), C);
-    if (C > 0) {
-      if (memo.keys) {
-        e = memo_clear(memo, stream);
-        if (e != cudaSuccess) return e;
-      }
-      ridge_cand_kernel<<<dim3((C + 255) / 256, 16), 256, 0, stream>>>(desc, d_c, C, p_by_value ? nullptr : d_mask,
-                                                                      mask_value, *model.mlp.h_ridge, d_tab, memo);
-      ++*launches;
-      if (memo.keys) {
-        e = memo_compact(memo, stream);
-        if (e != cudaSuccess) return e;
-        ridge_pair_kernel<<<dim3(kMemoCap / 256, P), 256, 0, stream>>>(desc, d_p, d_c, d_tab, C, *model.mlp.h_ridge, memo);
-        *launches += 2;
-      }
-    } else {
-      memo = MemoView{};
-    }
-    if (ev_begin) cudaEventRecord(ev_begin, stream);
-    select_ridge_kernel<<<grid, kBlock, 0, stream>>>(desc, d_p, pv, p_by_value != nullptr, d_c, map, st, d_tab,
-                                                     *model.mlp.h_ridge, k, partial, memo);
-    ++*launches;
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (ev_end) cudaEventRecord(ev_end, stream);
-    topk_merge_kernel<<<(P * 32 + kBlock - 1) / kBlock, kBlock, 0, stream>>>(partial, P, map.nblk * k, k,
-                                                                            d_topk_idx, d_topk_score);
-    ++*launches;
-    return cudaGetLastError();
-  }
   if (ev_begin) cudaEventRecord(ev_begin, stream);
   if (model.kind == 2) {
     select_generic_kernel<true><<<grid, kBlock, 0, stream>>>(desc, d_p, pv, p_by_value != nullptr, d_c, map, st, nullptr,
@@ -880,10 +977,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (ev_end) cudaEventRecord(ev_end, stream);
-  topk_merge_kernel<<<(P * 32 + kBlock - 1) / kBlock, kBlock, 0, stream>>>(partial, P, map.nblk * k, k,
-                                                                          d_topk_idx, d_topk_score);
-  ++*launches;
-  return cudaGetLastError();
+  return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
 }
 
 
@@ -907,9 +1001,7 @@ cudaError_t launch_select_generic_trees(const ks_gpu_desc& desc, const DevNode* 
       desc, d_p, ks_problem{}, 0, d_c, map, st, d_nodes, d_roots, n_trees, base, k, partial);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  topk_merge_kernel<<<(P * 32 + kBlock - 1) / kBlock, kBlock, 0, stream>>>(partial, P, map.nblk * k, k,
-                                                                          d_topk_idx, d_topk_score);
-  return cudaGetLastError();
+  return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, nullptr);
 }
 
 size_t featurize_scratch_bytes(int P) { return sizeof(ProblemEntry) * static_cast<size_t>(P > 0 ? P : 1); }

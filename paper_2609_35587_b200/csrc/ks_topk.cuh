@@ -10,10 +10,13 @@
 
 namespace ks {
 
+// a score's bits in the order of the scores
+__device__ __forceinline__ unsigned sortable(float score) {
+  const unsigned u = __float_as_uint(score);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
 __device__ __forceinline__ unsigned long long make_key(float score, int idx) {
-  unsigned u = __float_as_uint(score);
-  u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-  return (static_cast<unsigned long long>(u) << 32) | static_cast<unsigned>(~idx);
+  return (static_cast<unsigned long long>(sortable(score)) << 32) | static_cast<unsigned>(~idx);
 }
 
 __device__ __forceinline__ int key_index(unsigned long long key) {

@@ -1,0 +1,66 @@
+"""The linear scorer's kernels at the sizes where they can go wrong: with the class tables (32 problems or
+more, four of them a block) and without, a last group of fewer than four problems, element types that
+change within a group, more classes than are staged (2,048) and more than there are slots (8,192), small
+and ragged pools, k = 1, 10 and 32. The sums run in the same order as the oracle's problem, candidate and
+pair parts do not, so scores agree to 1e-4 as in the other tests of this scorer."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2609_35587_b200 import workloads as wl
+from tests.helpers import topk_accept
+
+pytestmark = pytest.mark.gpu
+DESC = wl.gpu_desc()
+
+
+@pytest.fixture(scope="module")
+def ks():
+    from paper_2609_35587_b200 import binding
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ctx(ks):
+    return ks.Context(DESC, 0)
+
+
+@pytest.mark.parametrize("P,C,k,valid,onehot", [(5, 1, 1, False, False), (31, 513, 32, False, True),
+                                                (32, 4097, 10, False, False), (37, 20000, 32, True, False),
+                                                (66, 61000, 10, True, True), (150, 3000, 1, False, False)])
+def test_select_linear(ks, ctx, P, C, k, valid, onehot):
+    dev = torch.device("cuda", 0)
+    st = wl.feature_stats("cfg2")
+    mu, sg = wl.onehot_stats(st["mu"], st["sigma"]) if onehot else (st["mu"], st["sigma"])
+    mlp = wl.mlp_xavier(P, [80 if onehot else 64, 1], mu, sg)
+    model = ctx.model_create_mlp(mlp)
+    prob = wl.problems_batch(P, P, cross_precision=True)
+    if valid:
+        rec, _, n = ctx.valid_catalogue(prob[:1], ks.KS_VALID_COUPLED)
+        d_c = rec[torch.arange(min(C, n), device=dev) * n // min(C, n)].contiguous()
+        cand = d_c.cpu().numpy().view(wl.CANDIDATE_DT).reshape(-1)
+    else:
+        cand = wl.candidates_full_grid(3, C)
+        d_c = ks.to_device(cand, dev)
+    idx, sc = ctx.select(ks.to_device(prob, dev), P, d_c, len(cand), model, k)
+    idx, sc = idx.cpu().numpy(), sc.cpu().numpy()
+    pool = np.arange(len(cand), dtype=np.int32)
+    for p in sorted({0, 1, 3, P // 2, P - 2, P - 1}):
+        _, _, ref = oracle.select(prob[p:p + 1], cand, DESC, k, mlp=mlp, want_scores=True)
+        ok, msg = topk_accept(idx[p], sc[p], ref, pool, k, 1e-4)
+        assert ok, (p, msg)
+
+
+@pytest.mark.parametrize("P,n", [(1, 1480), (3, 40), (1200, 90), (1184, 300), (2, 5000)])
+def test_merge_of_partial_lists(ks, ctx, P, n):
+    """A block or a warp per problem, numbers of keys around their steps: the static score, whose
+    ranking is exact, on pools that give n partial lists' worth of keys."""
+    C = min(60000, max(1, n // 10 * 1024))
+    model = ctx.model_create_static()
+    prob, cand, _, _ = wl.make_inputs(3, P=P, C=C)
+    dev = torch.device("cuda", 0)
+    idx, sc = ctx.select(ks.to_device(prob, dev), P, ks.to_device(cand, dev), C, model, 10)
+    some = sorted({0, P // 2, P - 1})
+    ridx, rsc = oracle.select(prob[some], cand, DESC, 10, static=True)
+    assert np.array_equal(idx.cpu().numpy()[some], ridx) and np.array_equal(sc.cpu().numpy()[some], rsc)
