@@ -1315,8 +1315,10 @@ size_t fast_scratch_bytes(const GbdtModel& g, int C) {
 }
 
 // Memo of the per-pair rows (see MemoView): worth its per-problem table only for a batch of
-// problems. The table is held for at most `fast_memo_batch` problems at a time (256 MiB of
-// records); a larger call is served batch by batch. 0 = not used.
+// problems, whether or not the walk splits the trees (64 problems x 2,048 candidates, 100 trees of depth 6 in
+// two slices: walk 105 -> 49 us, table 22 and numbering the classes 7; but 7 problems x 61,140 candidates:
+// 537 -> 693 us, of which 100 go to finding the classes). The table is held for at most `fast_memo_batch`
+// problems at a time (256 MiB of records); a larger call is served batch by batch. 0 = not used.
 size_t memo_fixed_bytes(int C) {
   return static_cast<size_t>(kMemoCombos) * kMemoCap * (sizeof(unsigned long long) + 2 * sizeof(int)) + 256 +
          (static_cast<size_t>(kMemoCombos) * C * sizeof(unsigned) + 255) / 256 * 256;
@@ -1349,9 +1351,9 @@ int fast_memo_batch(const GbdtModel& g, int P) {
   return static_cast<int>(batch < P ? batch : P);
 }
 
-size_t fast_memo_bytes(const GbdtModel& g, int P, int C) {
+size_t fast_memo_bytes(const GbdtModel& g, int P, int C, int slices) {
   const int batch = fast_memo_batch(g, P);
-  if (batch == 0 || C < 1) return 0;
+  if (batch == 0 || C < 1 || (slices > 1 && batch < P)) return 0;  // (slices number their scores within one launch)
   return memo_fixed_bytes(C) + static_cast<size_t>(batch) * (static_cast<size_t>(kMemoCap) * pair_rec_bytes(g) + kProbRec);
 }
 
@@ -1446,11 +1448,11 @@ cudaError_t launch_walk_geom(const GbdtModel& g, const WalkArgs& a) {
   }
   if (L == 3 && np == 5) return launch_ln<3, 5, false, THREADS, NC>(a);
   if (THREADS == 512 && NC == 1024) {  // the shapes met so far only in small ensembles
-    if (L == 3 && np == 3) return launch_ln<3, 3, false, 512, 1024>(a);
     if (L == 2 && np == 6) return launch_ln<2, 6, false, 512, 1024>(a);
     if (L == 2 && np == 5) return launch_ln<2, 5, false, 512, 1024>(a);  // the paper-sized ensemble: 916 trees of depth 7
   }
   if (L == 3 && np == 4) return launch_ln<3, 4, false, THREADS, NC>(a);
+  if (L == 3 && np == 3) return launch_ln<3, 3, false, THREADS, NC>(a);
   if (L == 3) return launch_ln<3, -1, false, THREADS, NC>(a);
   if (L == 2) return launch_ln<2, -1, false, THREADS, NC>(a);
   if (L == 1) return launch_ln<1, -1, false, THREADS, NC>(a);

@@ -259,7 +259,7 @@ cudaError_t launch_remap_indices(int32_t* d_idx, long long n, const int32_t* d_m
 // Quantised tree path: blocks per problem for `per_problem` rows, and the launch itself.
 void fast_tiling(const GbdtModel& g, int P, int64_t per_problem, int* nblk, int* rows_per_cta);
 size_t fast_scratch_bytes(const GbdtModel& g, int C);  // per-call table of candidate-only rows
-size_t fast_memo_bytes(const GbdtModel& g, int P, int C);  // memo of the per-pair rows (0: not used)
+size_t fast_memo_bytes(const GbdtModel& g, int P, int C, int slices);  // memo of the per-pair rows (0: not used)
 void free_fast_gbdt(GbdtModel& m);
 cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, const ks_problem* d_p,
                                const ks_problem* p_by_value, int P, const ks_candidate* d_c, int C,

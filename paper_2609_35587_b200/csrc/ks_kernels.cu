@@ -845,10 +845,10 @@ size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, 
     const size_t part = (static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
     const int S = segmented ? 1 : fast_slices(model.gbdt, static_cast<int64_t>(P) * nblk);
     const size_t planes = S > 1 ? (sizeof(float) * S * static_cast<size_t>(pairs) + 255) / 256 * 256 : 0;
-    const size_t memo = S > 1 ? 0 : (fast_memo_bytes(model.gbdt, P, C) + 255) / 256 * 256;
+    const size_t memo = (fast_memo_bytes(model.gbdt, P, C, S) + 255) / 256 * 256;
     // a dense batch is ranked in similarity order of the catalogue (ks_order.cu)
-    const bool classes = memo > 0 && classes_apply(model.gbdt, P, C, pairs);
-    const size_t order = (memo > 0 && P >= kOrderMinProblems && (!segmented || classes))
+    const bool classes = memo > 0 && S == 1 && classes_apply(model.gbdt, P, C, pairs);
+    const size_t order = (memo > 0 && S == 1 && P >= kOrderMinProblems && (!segmented || classes))
                              ? (order_scratch_bytes(C) + 255) / 256 * 256 : 0;
     return part + (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256 + planes + memo + order +
            (classes ? classes_scratch_bytes(model.gbdt, P, C) : 0);
@@ -895,18 +895,21 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                                            (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256);
       sl.counters = d_counters;
     }
-    // the memo of the per-pair rows sits behind the per-call table (batches of whole-ensemble CTAs only)
+    // the memo of the per-pair rows sits behind the per-call table and the slices' score planes
     const int sized_slices = d_seg_off ? 1 : fast_slices(model.gbdt, static_cast<int64_t>(P) * nblk);  // as sized
-    void* memo_mem = (sized_slices > 1 || p_by_value || fast_memo_bytes(model.gbdt, P, C) == 0)
+    const size_t planes = sized_slices > 1 ? (sizeof(float) * sized_slices * static_cast<size_t>(pairs) + 255) / 256 * 256 : 0;
+    const size_t memo_bytes = fast_memo_bytes(model.gbdt, P, C, sized_slices);
+    void* memo_mem = (p_by_value || memo_bytes == 0)
                          ? nullptr
-                         : static_cast<char*>(d_partial) + part_bytes + (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256;
+                         : static_cast<char*>(d_partial) + part_bytes +
+                               (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256 + planes;
     // a dense batch of problems: rank the catalogue in similarity order (neighbouring candidates
     // then take similar paths through the trees); the order sits behind the memo
     const int32_t* perm = nullptr;
     ClassCall classes{pairs, nullptr, nullptr};
-    const bool use_classes = memo_mem && classes_apply(model.gbdt, P, C, pairs);
-    if (memo_mem && P >= kOrderMinProblems && C > 0 && (!d_seg_off || use_classes)) {
-      char* order_mem = static_cast<char*>(memo_mem) + (fast_memo_bytes(model.gbdt, P, C) + 255) / 256 * 256;
+    const bool use_classes = memo_mem && sized_slices == 1 && classes_apply(model.gbdt, P, C, pairs);
+    if (memo_mem && sized_slices == 1 && P >= kOrderMinProblems && C > 0 && (!d_seg_off || use_classes)) {
+      char* order_mem = static_cast<char*>(memo_mem) + (memo_bytes + 255) / 256 * 256;
       cudaError_t eo = launch_catalogue_order(d_c, C, order_mem, stream, launches);
       if (eo != cudaSuccess) return eo;
       if (!d_seg_off) perm = reinterpret_cast<const int32_t*>(order_mem);
