@@ -28,7 +28,7 @@
 //
 // Other entries into the same walk
 //   single-problem call: the trees are split over several CTAs per candidate block (slices),
-//   the tiles are built once by tile_one_kernel; scoring call (ks_score): tiles are quantised
+//   the tiles are built once by tile_pairs_kernel; scoring call (ks_score): tiles are quantised
 //   from given feature rows by tile_rows_kernel and the scores are stored instead of ranked.
 //
 // Kernel (an item = one problem x up to NC candidates; a CTA of THREADS threads serves one item,
@@ -82,11 +82,6 @@ constexpr int kOffBuf0 = 0;
 // the per-call table kernel that precedes every launch of the select kernel.
 __device__ int g_fast_abort;
 
-// Byte of row i (0 .. 4 W - 1) of a block within one tile row of W words: the four rows of a
-// word are consecutive, so that in a catalogue ranked in similarity order a thread's four
-// candidates are near-duplicates.
-__device__ __forceinline__ int tile_byte(int i, int) { return i; }
-
 // Slice mode (single-problem latency call): the trees are split over n_slices CTAs per
 // candidate block. Every CTA stores its partial scores; the last CTA to arrive for a block
 // (atomic counter, nobody waits) adds the slices in a fixed order and ranks the block; the
@@ -98,7 +93,7 @@ struct SliceArgs {
   int* counters;           // [P * nblk + 1], zero on entry; every counter is reset by its last user
   int32_t* out_idx;        // single-problem form only: [k] final result (device-visible, may be
   float* out_score;        // mapped host memory); null when a merge kernel follows
-  const uint8_t* tiles;    // prepared tiles [blocks][rows][NC] (tile_one_kernel), or null
+  const uint8_t* tiles;    // prepared tiles [blocks][rows][NC] (tile_pairs_kernel), or null
   int* out_seq;            // single-problem form: receives `seq` once the k results are written
   int seq;
   float* score_out;        // scoring call (ks_score): the scores of the block's rows go here, no ranking
@@ -276,52 +271,117 @@ pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem
 }
 
 // ------------------------------------------------------------------------------------------
-// single-problem call: the whole tile of every candidate block, once per call
+// split walks: the whole tile of every (problem, candidate block), once per call
 // ------------------------------------------------------------------------------------------
 
-// One thread per tile slot writes all rows of its candidate's tile column, in the layout phase A
-// would produce, for the one problem of the call. The CTAs that share a candidate block in slice
-// mode then copy the block's tile instead of each rebuilding it. Slots past the catalogue get the
-// neutral byte. Also clears the abort flag (this kernel precedes the select kernel).
-template <bool kPairRows>  // true: the per-pair rows; false: the candidate-only and problem-only rows
-__device__ __forceinline__ void tile_one_rows(const ks_gpu_desc& desc, const ks_problem& p_value,
-                                              const ks_candidate* __restrict__ c, int C, const FastView& fv,
-                                              int NC, uint8_t* __restrict__ tiles, float* s_thr, int thr_cap) {
-  __shared__ ProblemTerms s_pt;
-  __shared__ FeatQ s_fq[64];
-  const int tid = threadIdx.x;
-  if (blockIdx.x == 0 && tid == 0) g_fast_abort = 0;
-  // rows and thresholds are ordered per-pair, candidate-only, problem-only
-  const int first = kPairRows ? 0 : fv.n_pair_rows;
-  const int count = kPairRows ? fv.n_pair_rows : fv.n_rows - fv.n_pair_rows;
-  const int t_first = kPairRows ? 0 : fv.thr_cand0;
-  const int t_count = kPairRows ? fv.thr_cand0 : fv.n_thr - fv.thr_cand0;
-  const float* T = stage_thresholds(fv, t_first, t_count, s_thr, thr_cap) - t_first;
-  if (tid < 64) s_fq[tid] = fv.feat[tid];
-  if (tid == 0) problem_terms(p_value, desc, s_pt);
-  __syncthreads();
-  const int slot = blockIdx.x * blockDim.x + tid;
-  const int blk = slot / NC, in = slot % NC;
-  uint8_t* my = tiles + static_cast<size_t>(blk) * fv.n_rows * NC + tile_byte(in, NC / 4);
-  if (slot >= C) {
-    for (int q = first; q < first + count; ++q) my[static_cast<size_t>(q) * NC] = 0x80;
-    return;
+// The rows of one column in 32 words of a tile: x holds the column's values for the lane's four
+// candidates. The four searches halve the same interval in step, four instructions a probe and no bound to
+// test; slices are cut from pairs of 16-bit counts (a model on this path has fewer than 48 K thresholds) and
+// a rank is one byte permutation. A NaN goes right at every numeric split (x < t is false), like +inf.
+__device__ __forceinline__ void tile_column(const FeatQ& q, float4 x, uint32_t thr, int n_rows, int W, uint32_t* out) {
+  const float v[4] = {x.x, x.y, x.z, x.w};
+  if (q.nslice) {
+    // the thresholds <= v end at an address in [at, at + 4 n]; !(T > v) holds for a NaN too
+    const uint32_t first = thr + 4 * q.thr0;
+    uint32_t at[4] = {first, first, first, first};
+    const auto probe = [&](uint32_t step) {
+      float t[4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) t[b] = lds_f32(at[b] + step - 4);
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if (!(t[b] > v[b])) at[b] += step;
+    };
+    int n = q.nthr;
+    for (; n > 1; n -= n >> 1) probe(4u * (n >> 1));
+    if (n == 1) probe(4);
+    uint32_t lo = (at[0] - first) / 4 | (at[1] - first) / 4 << 16, hi = (at[2] - first) / 4 | (at[3] - first) / 4 << 16;
+    for (int s = 0; s < q.nslice; ++s) {
+      const uint32_t a = __vminu2(lo, kSlice * 0x00010001u), b = __vminu2(hi, kSlice * 0x00010001u);
+      lo -= a;
+      hi -= b;
+      out[static_cast<size_t>(KS_IDX(q.row0 + s, n_rows)) * W] = 0x80808080u | __byte_perm(a, b, 0x6420);
+    }
   }
-  const ks_candidate cand = load_candidate(c + slot);
-  featurize_pair(s_pt, cand, desc, [&](int col, float v) {
-    if (col >= KS_F || (feat_class(col) == 2) != kPairRows) return;
-    const FeatQ& q = s_fq[col];
-    quantise(q, T + q.thr0, v, false, [&](int row, uint8_t b) { my[static_cast<size_t>(KS_IDX(row, fv.n_rows)) * NC] = b; });
-  });
+  if (q.nrank) {
+    // a selector per candidate: its level code picks a byte of the rank word, any other value a zero
+    uint32_t sel = 0;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) sel |= min(static_cast<unsigned>(__float2int_rz(v[b])), 4u) << (4 * b);
+    for (int k = 0; k < q.nrank; ++k)
+      out[static_cast<size_t>(KS_IDX(q.row0 + q.nslice + k, n_rows)) * W] =
+          0x80808080u | __byte_perm(*reinterpret_cast<const uint32_t*>(q.rank[k]), 0u, sel);
+  }
 }
 
-// blockIdx.y picks the role, so that both halves of the work are in flight together
-__global__ void __launch_bounds__(256)
-tile_one_kernel(ks_gpu_desc desc, ks_problem p_value, const ks_candidate* __restrict__ c, int C, FastView fv,
-                int NC, uint8_t* __restrict__ tiles, int thr_cap) {
-  extern __shared__ float s_thr[];  // thresholds of this role's features
-  if (blockIdx.y == 0) tile_one_rows<true>(desc, p_value, c, C, fv, NC, tiles, s_thr, thr_cap);
-  else tile_one_rows<false>(desc, p_value, c, C, fv, NC, tiles, s_thr, thr_cap);
+// An item is 128 candidates (32 words of a tile) of one problem; a block takes a run of items, so that the
+// thresholds are staged once and a problem's terms evaluated once or twice. Half of the threads
+// compute the per-pair columns of a candidate each, the other half the candidate-only ones; then a warp takes
+// every eighth column, four candidates a lane, and stores whole lines, in the layout phase A would produce.
+// Slots past the catalogue get the last candidate's bytes (they are not ranked). Also clears the abort flag
+// (this kernel precedes the select kernel). What bounds it is the latency of the columns' divisions and of
+// the searches. One problem x 61,140 candidates, 500 trees: 29 us, where a thread that wrote its candidate's
+// bytes one by one took 72. Every split walk of a dense batch takes its tiles from here: left to the slices,
+// each computed the per-pair columns again (10 problems x 934 candidates, 326 trees: 125 -> 48 us the whole call;
+// 64 x 2,048 candidates, 100 trees: 161 -> 124, with the memo in its place 143; four calls of one problem with
+// its 61,140 valid candidates: 900 -> 682).
+constexpr int kTileRows = 128, kTileCols = kPairCols + kCandCols;
+
+__global__ void __launch_bounds__(256, 3)
+tile_pairs_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int P,
+                  const ks_candidate* __restrict__ c, int C, FastView fv, int W, int groups,
+                  uint8_t* __restrict__ tiles) {
+  extern __shared__ __align__(16) float s_x[];  // [kTileCols][kTileRows], then the thresholds of every feature
+  __shared__ ProblemTerms s_pt;
+  __shared__ FeatQ s_fq[64];
+  __shared__ float s_pf[64];
+  float* s_thr = s_x + kTileCols * kTileRows;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (blockIdx.x == 0 && tid == 0) g_fast_abort = 0;
+  stage_thresholds(fv, 0, fv.n_thr, s_thr, fv.n_thr);
+  if (tid < 64) s_fq[tid] = fv.feat[tid];
+  const uint32_t thr = smem_u32(s_thr);
+  const int n_items = P * groups, per_block = (n_items + gridDim.x - 1) / gridDim.x;
+  const int begin = blockIdx.x * per_block, end = min(begin + per_block, n_items);
+  int held = -1;
+  for (int item = begin; item < end; ++item) {
+    const int prob = item / groups, g = item - prob * groups;
+    __syncthreads();  // the columns of the item before have been read
+    if (prob != held) {
+      if (tid == 0) {
+        problem_terms(use_value ? p_value : load_problem(p + prob), desc, s_pt);
+        problem_columns(s_pt, [&](int col, float v) { s_pf[col] = v; });
+      }
+      held = prob;
+      __syncthreads();
+    }
+    const int row = tid % kTileRows;
+    const ks_candidate cand = load_candidate(c + min(g * kTileRows + row, C - 1));
+    if (tid < kTileRows) {
+      const long long b_eff = resources(s_pt, cand, desc).b_eff;
+      pair_columns<true>(s_pt, cand, desc, b_eff, [&](int col, float v) { s_x[pair_slot(col) * kTileRows + row] = v; });
+    } else {
+      featurize_pair(s_pt, cand, desc, [&](int col, float v) {
+        if (col < KS_F && feat_class(col) == 1) s_x[(kPairCols + cand_slot(col)) * kTileRows + row] = v;
+      });
+    }
+    __syncthreads();
+    const int in_block = g * 32 / W;
+    uint32_t* out = reinterpret_cast<uint32_t*>(tiles) +
+                    (static_cast<size_t>(prob) * (groups * 32 / W) + in_block) * fv.n_rows * W + (g * 32 - in_block * W) + lane;
+#pragma unroll 1
+    for (int col = warp; col < KS_F; col += 8) {
+      const int cls = feat_class(col);
+      float4 x;
+      if (cls == 0) {
+        x.x = x.y = x.z = x.w = s_pf[col];
+      } else {
+        const int slot = cls == 2 ? pair_slot(col) : kPairCols + cand_slot(col);
+        x = *reinterpret_cast<const float4*>(s_x + slot * kTileRows + 4 * lane);
+      }
+      tile_column(s_fq[col], x, thr, fv.n_rows, W, out);
+    }
+  }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -331,16 +391,12 @@ tile_one_kernel(ks_gpu_desc desc, ks_problem p_value, const ks_candidate* __rest
 // ks_score with a qualifying ensemble: quantise feature rows into the tile layout of phase A. A block
 // brings 128 rows (32 words of a tile) into shared memory by whole sectors and column by column, the next
 // ones on their way in registers meanwhile; a warp then takes every 16th column, four rows a lane, and
-// stores whole lines. The walk kernel copies the tiles as in the single-problem call and writes the scores
-// instead of ranking. A NaN goes right at every numeric split (x < t is false), like +inf: the last bin.
-// Slots past the last row get the last row's bytes (their scores are not stored). Also clears the abort flag.
+// stores whole lines. The walk kernel copies the tiles as in a split walk and writes the scores instead of
+// ranking. Slots past the last row get the last row's bytes (their scores are not stored). Also clears the abort flag.
 //
-// What bounds it is the searches' chains of shared-memory loads and their issue: the four rows of a lane
-// halve the same interval in step, four instructions a probe and no bound to test, columns no tree reads
-// are left out, slices are cut from pairs of 16-bit counts and a rank is one byte permutation for all four
-// rows. A million rows, 500 trees of depth 8: 166 us (260 MB of rows and 180 MB of tiles: 68 us); a thread
+// What bounds it is the searches' chains of shared-memory loads and their issue. A million rows, 500 trees of depth 8: 166 us (260 MB of rows and 180 MB of tiles: 68 us); a thread
 // reading 16 bytes of its four rows at a time and searching row by row took 405 us.
-constexpr int kTileWarps = 16, kTileRows = 128;
+constexpr int kTileWarps = 16;
 
 __global__ void __launch_bounds__(kTileWarps * 32, 2)
 tile_rows_kernel(const float* __restrict__ feat, int64_t rows, FastView fv, uint8_t* __restrict__ tiles, int W,
@@ -378,42 +434,8 @@ tile_rows_kernel(const float* __restrict__ feat, int64_t rows, FastView fv, uint
     uint32_t* out = reinterpret_cast<uint32_t*>(tiles) + static_cast<size_t>(block) * fv.n_rows * W + word;
 #pragma unroll 1
     for (int col = warp; col < KS_F; col += kTileWarps) {
-      const FeatQ& q = s_fq[col];
       const float4 x = *reinterpret_cast<const float4*>(s_x + col * kTileRows + (4 * lane ^ 8 * (col / 4 & 3)));
-      const float v[4] = {x.x, x.y, x.z, x.w};
-      if (q.nslice) {
-        // the thresholds <= v end at an address in [at, at + 4 n]; !(T > v) holds for a NaN too
-        const uint32_t first = thr + 4 * q.thr0;
-        uint32_t at[4] = {first, first, first, first};
-        const auto probe = [&](uint32_t step) {
-          float t[4];
-#pragma unroll
-          for (int b = 0; b < 4; ++b) t[b] = lds_f32(at[b] + step - 4);
-#pragma unroll
-          for (int b = 0; b < 4; ++b)
-            if (!(t[b] > v[b])) at[b] += step;
-        };
-        int n = q.nthr;
-        for (; n > 1; n -= n >> 1) probe(4u * (n >> 1));
-        if (n == 1) probe(4);
-        // counts as pairs of 16 bits (a model has fewer than 48 K thresholds); a slice takes up to 127 of each
-        uint32_t lo = (at[0] - first) / 4 | (at[1] - first) / 4 << 16, hi = (at[2] - first) / 4 | (at[3] - first) / 4 << 16;
-        for (int s = 0; s < q.nslice; ++s) {
-          const uint32_t a = __vminu2(lo, kSlice * 0x00010001u), b = __vminu2(hi, kSlice * 0x00010001u);
-          lo -= a;
-          hi -= b;
-          out[static_cast<size_t>(KS_IDX(q.row0 + s, fv.n_rows)) * W] = 0x80808080u | __byte_perm(a, b, 0x6420);
-        }
-      }
-      if (q.nrank) {
-        // a selector per row: its level code picks a byte of the rank word, any other value a zero
-        uint32_t sel = 0;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) sel |= min(static_cast<unsigned>(__float2int_rz(v[b])), 4u) << (4 * b);
-        for (int k = 0; k < q.nrank; ++k)
-          out[static_cast<size_t>(KS_IDX(q.row0 + q.nslice + k, fv.n_rows)) * W] =
-              0x80808080u | __byte_perm(*reinterpret_cast<const uint32_t*>(q.rank[k]), 0u, sel);
-      }
+      tile_column(s_fq[col], x, thr, fv.n_rows, W, out);
     }
   }
 }
@@ -716,8 +738,9 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     // ---- phase A ---------------------------------------------------------------------------------
     __syncthreads();
     if (sl.tiles) {
-      // single-problem call: the block's tile was built once for all the CTAs that share it
-      const uint4* src = reinterpret_cast<const uint4*>(sl.tiles + static_cast<size_t>(chunk) * fv.n_rows * NC);
+      // the block's tile was built once for all the CTAs that share it
+      const uint4* src =
+          reinterpret_cast<const uint4*>(sl.tiles + (static_cast<size_t>(prob) * nblk + chunk) * fv.n_rows * NC);
       uint4* dst = reinterpret_cast<uint4*>(smem + kOffTile);
       for (int i = tid; i < fv.n_rows * (NC / 16); i += THREADS) dst[i] = __ldcg(src + i);
     } else {
@@ -1310,15 +1333,19 @@ void fast_tiling(const GbdtModel& g, int P, int64_t per_problem, int* nblk, int*
   *rows_per_cta = g.block_cands;
 }
 
+size_t fast_tiles_bytes(const GbdtModel& g, int64_t blocks) {
+  return static_cast<size_t>(blocks) * g.n_qrows * g.block_cands;
+}
+
 size_t fast_scratch_bytes(const GbdtModel& g, int C) {
   return 256 + static_cast<size_t>(kCombos) * C * cand_rec_bytes(g);
 }
 
 // Memo of the per-pair rows (see MemoView): worth its per-problem table only for a batch of
-// problems, whether or not the walk splits the trees (64 problems x 2,048 candidates, 100 trees of depth 6 in
-// two slices: walk 105 -> 49 us, table 22 and numbering the classes 7; but 7 problems x 61,140 candidates:
-// 537 -> 693 us, of which 100 go to finding the classes). The table is held for at most `fast_memo_batch`
-// problems at a time (256 MiB of records); a larger call is served batch by batch. 0 = not used.
+// problems (7 problems x 61,140 candidates with it: 537 -> 693 us, of which 100 go to finding the classes)
+// and only where the walk is not split, since a split walk takes whole tiles (see tile_pairs_kernel). The
+// table is held for at most `fast_memo_batch` problems at a time (256 MiB of
+// records); a larger call is served batch by batch. 0 = not used.
 size_t memo_fixed_bytes(int C) {
   return static_cast<size_t>(kMemoCombos) * kMemoCap * (sizeof(unsigned long long) + 2 * sizeof(int)) + 256 +
          (static_cast<size_t>(kMemoCombos) * C * sizeof(unsigned) + 255) / 256 * 256;
@@ -1351,9 +1378,9 @@ int fast_memo_batch(const GbdtModel& g, int P) {
   return static_cast<int>(batch < P ? batch : P);
 }
 
-size_t fast_memo_bytes(const GbdtModel& g, int P, int C, int slices) {
+size_t fast_memo_bytes(const GbdtModel& g, int P, int C) {
   const int batch = fast_memo_batch(g, P);
-  if (batch == 0 || C < 1 || (slices > 1 && batch < P)) return 0;  // (slices number their scores within one launch)
+  if (batch == 0 || C < 1) return 0;
   return memo_fixed_bytes(C) + static_cast<size_t>(batch) * (static_cast<size_t>(kMemoCap) * pair_rec_bytes(g) + kProbRec);
 }
 
@@ -1592,13 +1619,13 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
 
   // candidate-only rows for the type combinations in use
   cudaError_t e = cudaSuccess;
-  if (!prep && !a.uv) {
+  const bool tiles_mode = !prep && slice && slice->n_slices > 1 && slice->tiles && !seg_off;
+  if (!prep && !a.uv && !tiles_mode) {
     e = cudaMemsetAsync(d_mask, 0, sizeof(unsigned), stream);
     if (e != cudaSuccess) return e;
     combo_mask_kernel<<<P >= 4096 ? 16 : 1, 256, 0, stream>>>(d_p, P, d_mask);
     ++*launches;
   }
-  const bool tiles_mode = a.uv && slice && slice->n_slices > 1 && slice->tiles && P == 1 && !seg_off;
   // shared memory of the table kernel: the per-pair thresholds when they fit beside its 256 records
   size_t pthr_bytes = 0;
   int pthr_cap = staged_floats(g.thr_cand0, &pthr_bytes);
@@ -1620,13 +1647,17 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
       fv.prob_tab = fv.pair_tab + static_cast<size_t>(kMemoCap) * pair_rec_bytes(g);
     }
   } else if (tiles_mode) {
-    // one launch, two roles (blockIdx.y): the per-pair rows, and the candidate- / problem-only rows
-    size_t tthr = 0;
-    const int cap = staged_floats(std::max(g.thr_cand0, g.n_qthr - g.thr_cand0), &tthr);
-    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&tile_one_kernel), tthr);
+    const size_t smem = sizeof(float) * (kTileCols * kTileRows + g.n_qthr);
+    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&tile_pairs_kernel), smem);
     if (e != cudaSuccess) return e;
-    tile_one_kernel<<<dim3(nblk * (g.block_cands / 256), 2), 256, tthr, stream>>>(desc, a.pv, d_c, C, fv,
-                                                                                   g.block_cands, slice->tiles, cap);
+    const int W = g.block_cands / 4, groups = nblk * (W / 32);
+    const int resident = std::max<int>(1, std::min<int>(3, 226 * 1024 / (smem + 4096)));
+    if (C > 0)
+      tile_pairs_kernel<<<std::min(P * groups, resident * kSmCount), 256, smem, stream>>>(
+          desc, d_p, a.pv, a.uv, P, d_c, C, fv, W, groups, slice->tiles);
+    else
+      e = cudaMemsetAsync(slice->tiles, 0x80, fast_tiles_bytes(g, static_cast<int64_t>(P) * nblk), stream);
+    if (e != cudaSuccess) return e;
     ++*launches;
   } else if (C > 0) {
     if (memo.keys) {

@@ -202,7 +202,7 @@ struct ClassCall {
   void* scratch;     // classes_scratch_bytes
 };
 
-// Slice mode of the quantised tree kernel (single-problem latency call).
+// Slice mode of the quantised tree kernel (few candidate blocks: the trees are split over several CTAs).
 struct FastSlice {
   int n_slices;
   long long pairs;   // rows of one partial-score plane
@@ -210,7 +210,7 @@ struct FastSlice {
   int* counters;     // [blocks + 1], zero between calls
   int32_t* out_idx;  // single-problem form: [k], device-visible; else null (a merge kernel follows)
   float* out_score;
-  uint8_t* tiles;    // single-problem form: scratch for the prepared tiles [blocks][rows][block_cands], or null
+  uint8_t* tiles;    // scratch for the tiles [problems * blocks][rows][block_cands], or null
   int* out_seq;      // single-problem form: device-visible word that receives `seq` after the results
   int seq;
 };
@@ -259,7 +259,8 @@ cudaError_t launch_remap_indices(int32_t* d_idx, long long n, const int32_t* d_m
 // Quantised tree path: blocks per problem for `per_problem` rows, and the launch itself.
 void fast_tiling(const GbdtModel& g, int P, int64_t per_problem, int* nblk, int* rows_per_cta);
 size_t fast_scratch_bytes(const GbdtModel& g, int C);  // per-call table of candidate-only rows
-size_t fast_memo_bytes(const GbdtModel& g, int P, int C, int slices);  // memo of the per-pair rows (0: not used)
+size_t fast_tiles_bytes(const GbdtModel& g, int64_t blocks);  // the tiles of that many (problem, candidate block) pairs
+size_t fast_memo_bytes(const GbdtModel& g, int P, int C);  // memo of the per-pair rows (0: not used)
 void free_fast_gbdt(GbdtModel& m);
 cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, const ks_problem* d_p,
                                const ks_problem* p_by_value, int P, const ks_candidate* d_c, int C,

@@ -844,13 +844,17 @@ size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, 
     fast_tiling(model.gbdt, P, per, &nblk, &rows);
     const size_t part = (static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
     const int S = segmented ? 1 : fast_slices(model.gbdt, static_cast<int64_t>(P) * nblk);
-    const size_t planes = S > 1 ? (sizeof(float) * S * static_cast<size_t>(pairs) + 255) / 256 * 256 : 0;
-    const size_t memo = (fast_memo_bytes(model.gbdt, P, C, S) + 255) / 256 * 256;
+    if (S > 1) {
+      const size_t planes = (sizeof(float) * S * static_cast<size_t>(pairs) + 255) / 256 * 256;
+      return part + planes + 256 +
+             std::max(fast_scratch_bytes(model.gbdt, C), fast_tiles_bytes(model.gbdt, static_cast<int64_t>(P) * nblk));
+    }
+    const size_t memo = (fast_memo_bytes(model.gbdt, P, C) + 255) / 256 * 256;
     // a dense batch is ranked in similarity order of the catalogue (ks_order.cu)
-    const bool classes = memo > 0 && S == 1 && classes_apply(model.gbdt, P, C, pairs);
-    const size_t order = (memo > 0 && S == 1 && P >= kOrderMinProblems && (!segmented || classes))
+    const bool classes = memo > 0 && classes_apply(model.gbdt, P, C, pairs);
+    const size_t order = (memo > 0 && P >= kOrderMinProblems && (!segmented || classes))
                              ? (order_scratch_bytes(C) + 255) / 256 * 256 : 0;
-    return part + (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256 + planes + memo + order +
+    return part + (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256 + memo + order +
            (classes ? classes_scratch_bytes(model.gbdt, P, C) : 0);
   }
   if (model.kind == 1 && model.mlp.tc) {
@@ -887,29 +891,28 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     const size_t part_bytes = (static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
     // an under-filled machine: split the trees over several CTAs per block (dense form only,
     // where a block covers its rows in one pass)
+    const int sized_slices = d_seg_off ? 1 : fast_slices(model.gbdt, static_cast<int64_t>(P) * nblk);  // as sized
+    char* mem = static_cast<char*>(d_partial) + part_bytes;
     FastSlice sl{};
-    sl.n_slices = (d_seg_off || !d_counters) ? 1 : fast_slices(model.gbdt, static_cast<int64_t>(P) * nblk);
+    sl.n_slices = d_counters ? sized_slices : 1;
     if (sl.n_slices > 1) {
+      // the slices of a block share a tile that is built in front of them; behind the tiles, their score planes
       sl.pairs = pairs;
-      sl.scores = reinterpret_cast<float*>(static_cast<char*>(d_partial) + part_bytes +
-                                           (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256);
+      sl.tiles = reinterpret_cast<uint8_t*>(mem);
+      sl.scores = reinterpret_cast<float*>(mem + (fast_tiles_bytes(model.gbdt, static_cast<int64_t>(P) * nblk) + 255) / 256 * 256);
       sl.counters = d_counters;
     }
-    // the memo of the per-pair rows sits behind the per-call table and the slices' score planes
-    const int sized_slices = d_seg_off ? 1 : fast_slices(model.gbdt, static_cast<int64_t>(P) * nblk);  // as sized
-    const size_t planes = sized_slices > 1 ? (sizeof(float) * sized_slices * static_cast<size_t>(pairs) + 255) / 256 * 256 : 0;
-    const size_t memo_bytes = fast_memo_bytes(model.gbdt, P, C, sized_slices);
-    void* memo_mem = (p_by_value || memo_bytes == 0)
+    // the memo of the per-pair rows sits behind the per-call table (batches of whole-ensemble CTAs only)
+    void* memo_mem = (sized_slices > 1 || p_by_value || fast_memo_bytes(model.gbdt, P, C) == 0)
                          ? nullptr
-                         : static_cast<char*>(d_partial) + part_bytes +
-                               (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256 + planes;
+                         : mem + (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256;
     // a dense batch of problems: rank the catalogue in similarity order (neighbouring candidates
     // then take similar paths through the trees); the order sits behind the memo
     const int32_t* perm = nullptr;
     ClassCall classes{pairs, nullptr, nullptr};
-    const bool use_classes = memo_mem && sized_slices == 1 && classes_apply(model.gbdt, P, C, pairs);
-    if (memo_mem && sized_slices == 1 && P >= kOrderMinProblems && C > 0 && (!d_seg_off || use_classes)) {
-      char* order_mem = static_cast<char*>(memo_mem) + (memo_bytes + 255) / 256 * 256;
+    const bool use_classes = memo_mem && classes_apply(model.gbdt, P, C, pairs);
+    if (memo_mem && P >= kOrderMinProblems && C > 0 && (!d_seg_off || use_classes)) {
+      char* order_mem = static_cast<char*>(memo_mem) + (fast_memo_bytes(model.gbdt, P, C) + 255) / 256 * 256;
       cudaError_t eo = launch_catalogue_order(d_c, C, order_mem, stream, launches);
       if (eo != cudaSuccess) return eo;
       if (!d_seg_off) perm = reinterpret_cast<const int32_t*>(order_mem);
@@ -917,7 +920,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
       classes.scratch = order_mem + (order_scratch_bytes(C) + 255) / 256 * 256;
     }
     cudaError_t e = launch_select_fast(desc, model.gbdt, d_p, p_by_value, P, d_c, C, nblk, rows, d_seg_off,
-                                       d_seg_idx, k, part, static_cast<char*>(d_partial) + part_bytes, d_status,
+                                       d_seg_idx, k, part, mem, d_status,
                                        stream, launches, ev_begin, sl.n_slices > 1 ? &sl : nullptr, memo_mem, wait,
                                        nullptr, perm, use_classes ? &classes : nullptr);
     if (e != cudaSuccess) return e;

@@ -1,6 +1,6 @@
-"""Tree ensembles on batches too small to fill the machine, where the table of the per-pair columns serves
-CTAs that split the trees: both sides of the rule that takes the table (32 problems) and of the one that
-splits the trees, ragged pools, mixed element types, segments of unequal length, depth 6. Scores agree to the tolerance of the other tests of tree ensembles."""
+"""Tree ensembles on batches too small to fill the machine, whose tiles are built in front of a walk that
+splits the trees: both sides of the rule that splits them, one problem and many, ragged pools, mixed element
+types, segments of unequal length (never split), depth 6. Scores agree to the tolerance of the other tests of tree ensembles."""
 import numpy as np
 import pytest
 import torch
@@ -15,7 +15,8 @@ TOL = 1e-5
 
 
 @pytest.mark.parametrize("P,C,trees,depth,k,segmented", [
-    (7, 5011, 60, 6, 10, False), (31, 517, 400, 6, 32, False), (32, 517, 400, 5, 10, False), (64, 2048, 100, 6, 5, False),
+    (1, 30011, 60, 8, 10, False), (2, 1025, 33, 7, 10, False), (7, 5011, 60, 6, 10, False), (31, 517, 400, 6, 32, False),
+    (32, 517, 400, 5, 10, False), (64, 2048, 100, 6, 5, False),
     (40, 1024, 90, 6, 32, False), (300, 1000, 30, 6, 1, False), (40, 700, 30, 6, 10, True)])
 def test_select(P, C, trees, depth, k, segmented):
     from paper_2609_35587_b200 import binding as ks
@@ -37,7 +38,7 @@ def test_select(P, C, trees, depth, k, segmented):
         idx, sc = ctx.select(d_p, P, d_c, len(cand), model, k, *args)
         torch.cuda.synchronize()
     idx, sc = idx.cpu().numpy(), sc.cpu().numpy()
-    for p in {0, 1, P // 2, P - 1}:
+    for p in {0, P // 3, P // 2, P - 1}:
         seg = np.arange(len(cand), dtype=np.int32) if so is None else si[so[p]:so[p + 1]]
         _, _, ref = oracle.select(prob[p:p + 1], cand, DESC, k, gbdt=(off, nodes, 0.1), want_scores=True,
                                   seg_off=np.array([0, len(seg)], np.int64), seg_idx=seg)
