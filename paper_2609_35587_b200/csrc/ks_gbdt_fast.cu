@@ -341,8 +341,9 @@ tile_pairs_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem
   stage_thresholds(fv, 0, fv.n_thr, s_thr, fv.n_thr);
   if (tid < 64) s_fq[tid] = fv.feat[tid];
   const uint32_t thr = smem_u32(s_thr);
-  const int n_items = P * groups, per_block = (n_items + gridDim.x - 1) / gridDim.x;
-  const int begin = blockIdx.x * per_block, end = min(begin + per_block, n_items);
+  const long long n_items = static_cast<long long>(P) * groups;
+  const int begin = static_cast<int>(n_items * blockIdx.x / gridDim.x);
+  const int end = static_cast<int>(n_items * (blockIdx.x + 1) / gridDim.x);
   int held = -1;
   for (int item = begin; item < end; ++item) {
     const int prob = item / groups, g = item - prob * groups;
