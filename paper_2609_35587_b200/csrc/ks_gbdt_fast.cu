@@ -323,8 +323,8 @@ __device__ __forceinline__ void tile_column(const FeatQ& q, float4 x, uint32_t t
 // the searches. One problem x 61,140 candidates, 500 trees: 29 us, where a thread that wrote its candidate's
 // bytes one by one took 72. Every split walk of a dense batch takes its tiles from here: left to the slices,
 // each computed the per-pair columns again (10 problems x 934 candidates, 326 trees: 125 -> 48 us the whole call;
-// 64 x 2,048 candidates, 100 trees: 161 -> 124, with the memo in its place 143; four calls of one problem with
-// its 61,140 valid candidates: 900 -> 682).
+// 64 x 2,048 candidates, 100 trees: 161 -> 120, with the memo in its place 143; four calls of one problem with
+// its 61,140 valid candidates: 900 -> 677).
 constexpr int kTileRows = 128, kTileCols = kPairCols + kCandCols;
 
 __global__ void __launch_bounds__(256, 3)
@@ -338,21 +338,23 @@ tile_pairs_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem
   float* s_thr = s_x + kTileCols * kTileRows;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (blockIdx.x == 0 && tid == 0) g_fast_abort = 0;
-  stage_thresholds(fv, 0, fv.n_thr, s_thr, fv.n_thr);
-  if (tid < 64) s_fq[tid] = fv.feat[tid];
-  const uint32_t thr = smem_u32(s_thr);
   const long long n_items = static_cast<long long>(P) * groups;
   const int begin = static_cast<int>(n_items * blockIdx.x / gridDim.x);
   const int end = static_cast<int>(n_items * (blockIdx.x + 1) / gridDim.x);
-  int held = -1;
+  const auto evaluate = [&](int prob) {
+    problem_terms(use_value ? p_value : load_problem(p + prob), desc, s_pt);
+    problem_columns(s_pt, [&](int col, float v) { s_pf[col] = v; });
+  };
+  int held = begin / groups;
+  if (tid == 0 && begin < end) evaluate(held);  // while the other warps stage
+  stage_thresholds(fv, 0, fv.n_thr, s_thr, fv.n_thr);
+  if (tid < 64) s_fq[tid] = fv.feat[tid];
+  const uint32_t thr = smem_u32(s_thr);
   for (int item = begin; item < end; ++item) {
     const int prob = item / groups, g = item - prob * groups;
     __syncthreads();  // the columns of the item before have been read
     if (prob != held) {
-      if (tid == 0) {
-        problem_terms(use_value ? p_value : load_problem(p + prob), desc, s_pt);
-        problem_columns(s_pt, [&](int col, float v) { s_pf[col] = v; });
-      }
+      if (tid == 0) evaluate(prob);
       held = prob;
       __syncthreads();
     }
