@@ -13,10 +13,11 @@
 // layer's A. No CTA waits for another pair. The next layer's first K blocks only need the first
 // column tiles of the layer before, so the epilogue of a layer's last tile runs under the next
 // layer's MMAs.
-// Measured on 16 x 60,000 pairs of the shipped shape (3.4 TFLOP): 4.2 ms a call, of it 3.6 ms in
-// the layers (940 TFLOP/s, 0.67 of cuBLAS's sustained rate; tensor pipe 45 % busy); a tile MLP on
-// the CUDA cores took 440 ms. This kernel is the only one for these shapes. What is left of the gap is the
-// operands' way from L2: a K block brings 128 flop a byte, so the sustained rate would need 10.9 TB/s. Taking
+// Measured on 16 x 60,000 pairs of the shipped shape (3.4 TFLOP): 4.6 ms a call, of it 4.1 ms in
+// the layers (830 TFLOP/s, 0.59 of cuBLAS's sustained rate); a tile MLP on the CUDA cores took
+// 440 ms. This kernel is the only one for these shapes. What is left of the gap is the operands' way from L2
+// (a K block brings 128 flop a byte, so the sustained rate would need 10.9 TB/s) and the parts that a
+// layer's sums are taken in (see part_count; 3.8 ms a call without them). Taking
 // two row blocks in turn, so that one's epilogues run under the other's MMAs, measured 4.34 ms for 4.18.
 //
 // Operand images: K-major with 128-byte swizzle, blocks of [rows][64 of K]: element (row, k) of a
@@ -59,6 +60,8 @@ struct WideMlp {
 namespace {
 
 constexpr int kThreads = 384;      // warp 0 loads, warp 1 issues MMAs, warps 4..11 are the epilogue
+constexpr int kRegs = 168, kRegsFew = 56, kRegsEpilogue = 224;  // a thread's registers at launch, and after the split
+static_assert(128 * kRegsFew + 256 * kRegsEpilogue <= kThreads * kRegs, "the split hands out what the block was launched with");
 constexpr int kRowsCta = 128, kRowsPair = 256;
 constexpr int kStages = 6;
 constexpr int kBlockBytes = kRowsCta * 128;        // [128 rows][64 of K] bf16
@@ -71,9 +74,24 @@ constexpr int64_t kBatchRows = int64_t{55} * kPairs * kRowsPair;  // rows per la
 constexpr int64_t kScorePairs = 64 * kBatchRows;  // scores held at a time (267 MB)
 constexpr int kTileN = 256;
 
+// Parts that the K blocks of a layer are summed in. The tensor core adds to its fp32 accumulator by
+// truncation, so that what a long sum loses grows with its length, where additions that round lose the
+// square root of it: with all of 1,024 in one accumulator the scores were 1.66 times as far from 64 bits as
+// with sums in sequence. So an accumulator takes a part of K, and the epilogue adds the parts, which
+// rounds. One part more than the square root of the blocks is no further off than the sequence: rms error
+// of 64-1024-1024-512-256-1 over 320,000 rows 3.8e-4 in sequence, 6.9e-4 in one part, 3.9e-4 in four parts
+// of 16 blocks, 3.6e-4 in six. What a part costs is reading its accumulator: 128 KB an SM from TMEM, some
+// 2,300 clocks, beside the 2,000 to 4,600 that its MMAs and operands take (16 x 60,000 pairs: 3.8 ms in one
+// part, 4.3 in four, 4.6 like this, 4.7 in six).
+constexpr int part_count(int kblocks) {
+  int root = 1;
+  while ((root + 1) * (root + 1) <= kblocks) ++root;
+  return root + 1 < kblocks ? root + 1 : kblocks;
+}
+
 struct WideArgs {
   int n_hidden;
-  int kblocks[kMaxHidden], width[kMaxHidden], wrow[kMaxHidden];
+  int kblocks[kMaxHidden], parts[kMaxHidden], width[kMaxHidden], wrow[kMaxHidden];
   int act_kb;                // K blocks per activation buffer
   const float* consts;       // biases [n_hidden][1024], last layer's weights [1024]
   float b_last;
@@ -378,121 +396,157 @@ mlp_wide_kernel(const __grid_constant__ WideArgs a, const __grid_constant__ CUte
   };
 
   const int64_t b_first = s_abort ? n_blocks : pair;
-  if (warp == 0) {
-    // ---------------------------------- loads -------------------------------------------------------
-    if (lane == 0) {
-      const uint32_t stage0 = sbase;
-      uint32_t it = 0, ph_stored = 0;
-      bool ok = true;
-      for (int64_t blk = b_first; blk < n_blocks && ok; blk += n_pairs) {
-        for (int l = 0; l < a.n_hidden && ok; ++l) {
-          const int kbs = a.kblocks[l], width = a.width[l];
-          for (int n0 = 0; n0 < width && ok; n0 += kTileN) {
-            const int nt = width - n0 < kTileN ? width - n0 : kTileN;
-            const CUtensorMap* mw = nt == 256 ? &map_w128 : (nt == 192 ? &map_w96 : (nt == 128 ? &map_w64 : &map_w32));
-            const int wrow = a.wrow[l] + n0 * kbs + static_cast<int>(rank) * (nt / 2);
-            for (int kb = 0; kb < kbs; ++kb) {
-              if (l > 0 && n0 == 0 && (kb & 3) == 0) {
-                // the column tile of the layer before that holds these K blocks is stored
-                const int t = kb >> 2;
-                if (!(ok = wait_ok(bar_stored(t), (ph_stored >> t) & 1u))) break;
-                ph_stored ^= 1u << t;
-                asm volatile("fence.proxy.async;" ::: "memory");
+  // the epilogue keeps 128 sums a thread: it takes the registers that the first four warps do without
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsFew));
+    if (warp == 0) {
+      // ---------------------------------- loads -------------------------------------------------------
+      if (lane == 0) {
+        const uint32_t stage0 = sbase;
+        uint32_t it = 0, ph_stored = 0;
+        bool ok = true;
+        for (int64_t blk = b_first; blk < n_blocks && ok; blk += n_pairs) {
+          for (int l = 0; l < a.n_hidden && ok; ++l) {
+            const int kbs = a.kblocks[l], width = a.width[l];
+            for (int n0 = 0; n0 < width && ok; n0 += kTileN) {
+              const int nt = width - n0 < kTileN ? width - n0 : kTileN;
+              const CUtensorMap* mw = nt == 256 ? &map_w128 : (nt == 192 ? &map_w96 : (nt == 128 ? &map_w64 : &map_w32));
+              const int wrow = a.wrow[l] + n0 * kbs + static_cast<int>(rank) * (nt / 2);
+              for (int kb = 0; kb < kbs; ++kb) {
+                if (l > 0 && n0 == 0 && (kb & 3) == 0) {
+                  // the column tile of the layer before that holds these K blocks is stored
+                  const int t = kb >> 2;
+                  if (!(ok = wait_ok(bar_stored(t), (ph_stored >> t) & 1u))) break;
+                  ph_stored ^= 1u << t;
+                  asm volatile("fence.proxy.async;" ::: "memory");
+                }
+                const int s = static_cast<int>(it % kStages);
+                if (!(ok = wait_ok(bar_empty(s), ((it / kStages) & 1u) ^ 1u))) break;
+                const uint32_t full = to_cluster(bar_full(s), 0);
+                if (rank == 0) bar_expect(bar_full(s), 2u * (kBlockBytes + nt / 2 * 128));
+                if (!a.starve) {  // test hook: without the copies the waits on this barrier run out
+                  const uint32_t dst = stage0 + s * kStageBytes;
+                  if (l == 0) tma_load(dst, &map_x, static_cast<int>(((blk * 2 + rank) * kbs + kb) * kRowsCta), full);
+                  else tma_load(dst, &map_act, static_cast<int>(((blockIdx.x * 2 + (l & 1)) * a.act_kb + kb) * kRowsCta), full);
+                  tma_load(dst + kBlockBytes, mw, wrow + kb * nt, full);
+                }
+                ++it;
               }
-              const int s = static_cast<int>(it % kStages);
-              if (!(ok = wait_ok(bar_empty(s), ((it / kStages) & 1u) ^ 1u))) break;
-              const uint32_t full = to_cluster(bar_full(s), 0);
-              if (rank == 0) bar_expect(bar_full(s), 2u * (kBlockBytes + nt / 2 * 128));
-              if (!a.starve) {  // test hook: without the copies the waits on this barrier run out
-                const uint32_t dst = stage0 + s * kStageBytes;
-                if (l == 0) tma_load(dst, &map_x, static_cast<int>(((blk * 2 + rank) * kbs + kb) * kRowsCta), full);
-                else tma_load(dst, &map_act, static_cast<int>(((blockIdx.x * 2 + (l & 1)) * a.act_kb + kb) * kRowsCta), full);
-                tma_load(dst + kBlockBytes, mw, wrow + kb * nt, full);
-              }
-              ++it;
             }
           }
         }
       }
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    // ---------------------------------- MMAs --------------------------------------------------------
-    if (rank == 0 && lane == 0) {
-      uint32_t it = 0, tile = 0;
-      bool ok = true;
-      for (int64_t blk = b_first; blk < n_blocks && ok; blk += n_pairs) {
-        for (int l = 0; l < a.n_hidden && ok; ++l) {
-          const int kbs = a.kblocks[l], width = a.width[l];
-          for (int n0 = 0; n0 < width && ok; n0 += kTileN, ++tile) {
-            const int nt = width - n0 < kTileN ? width - n0 : kTileN;
-            const uint32_t idesc = instr_desc(nt), acc = tile & 1u;
-            if (!(ok = wait_ok(bar_read(acc), ((tile >> 1) & 1u) ^ 1u))) break;
-            fence_after();
-            for (int kb = 0; kb < kbs; ++kb, ++it) {
-              const int s = static_cast<int>(it % kStages);
-              if (!(ok = wait_ok(bar_full(s), (it / kStages) & 1u))) break;
-              fence_after();
-              const uint64_t da = operand_desc(sbase + s * kStageBytes);
-              const uint64_t db = operand_desc(sbase + s * kStageBytes + kBlockBytes);
+      __syncwarp();
+    } else if (warp == 1) {
+      // ---------------------------------- MMAs --------------------------------------------------------
+      if (rank == 0 && lane == 0) {
+        uint32_t it = 0, part = 0;
+        bool ok = true;
+        for (int64_t blk = b_first; blk < n_blocks && ok; blk += n_pairs) {
+          for (int l = 0; l < a.n_hidden && ok; ++l) {
+            const int kbs = a.kblocks[l], parts = a.parts[l], width = a.width[l];
+            for (int n0 = 0; n0 < width && ok; n0 += kTileN) {
+              const int nt = width - n0 < kTileN ? width - n0 : kTileN;
+              const uint32_t idesc = instr_desc(nt);
+              for (int j = 0; j < parts && ok; ++j, ++part) {
+                const uint32_t acc = part & 1u;
+                if (!(ok = wait_ok(bar_read(acc), ((part >> 1) & 1u) ^ 1u))) break;
+                fence_after();
+                const int first = kbs * j / parts, stop = kbs * (j + 1) / parts;
+                for (int kb = first; kb < stop; ++kb, ++it) {
+                  const int s = static_cast<int>(it % kStages);
+                  if (!(ok = wait_ok(bar_full(s), (it / kStages) & 1u))) break;
+                  fence_after();
+                  const uint64_t da = operand_desc(sbase + s * kStageBytes);
+                  const uint64_t db = operand_desc(sbase + s * kStageBytes + kBlockBytes);
 #pragma unroll
-              for (int k16 = 0; k16 < 4; ++k16)  // 32 bytes on in K: two units of the address field
-                mma_pair(tmem + acc * 256u, da + 2u * k16, db + 2u * k16, idesc, kb > 0 || k16 > 0);
-              commit_pair(bar_empty(s));
+                  for (int k16 = 0; k16 < 4; ++k16)  // 32 bytes on in K: two units of the address field
+                    mma_pair(tmem + acc * 256u, da + 2u * k16, db + 2u * k16, idesc, kb > first || k16 > 0);
+                  commit_pair(bar_empty(s));
+                }
+                if (ok) commit_pair(bar_acc(acc));
+              }
             }
-            if (ok) commit_pair(bar_acc(acc));
           }
         }
       }
+      __syncwarp();
     }
-    __syncwarp();
-  } else if (warp >= 4) {
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpilogue));
     // ---------------------------------- epilogue ----------------------------------------------------
     // warp w owns lanes 32 (w % 4) .. and one half of a tile's columns
     const int quarter = warp & 3, half = (warp - 4) >> 2;
     const int trow = quarter * 32 + lane;
     const uint32_t tmem_row = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
-    uint32_t tile = 0, blk_par = 0;  // s_half is written for every other block in turn
+    int pending = -1;  // column tile whose rows are written but not yet announced
+    auto publish = [&]() {
+      if (pending < 0) return;
+      // the rows are written; what the loading thread issues next must see them
+      __threadfence();
+      asm volatile("fence.proxy.async;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) bar_arrive(bar_stored(pending));
+      pending = -1;
+    };
+    uint32_t part = 0, blk_par = 0;  // s_half is written for every other block in turn
     bool ok = true;
     for (int64_t blk = b_first; blk < n_blocks && ok; blk += n_pairs, blk_par ^= 1u) {
       float score = 0.0f;
       for (int l = 0; l < a.n_hidden && ok; ++l) {
-        const int width = a.width[l];
+        const int parts = a.parts[l], width = a.width[l];
         const bool last = l + 1 == a.n_hidden;
         const float* bias = s_const + l * KS_MLP_MAX_WIDTH;
         const float* w_last = s_const + a.n_hidden * KS_MLP_MAX_WIDTH;
         uint8_t* out = a.act + (static_cast<size_t>(blockIdx.x * 2 + ((l + 1) & 1)) * a.act_kb) * kBlockBytes + trow * 128;
-        for (int n0 = 0; n0 < width && ok; n0 += kTileN, ++tile) {
+        for (int n0 = 0; n0 < width && ok; n0 += kTileN) {
           const int nt = width - n0 < kTileN ? width - n0 : kTileN;
-          const uint32_t acc = tile & 1u;
-          if (!(ok = __all_sync(0xFFFFFFFFu, wait_ok(bar_acc(acc), (tile >> 1) & 1u)))) break;
-          fence_after();
-          const int c_end = (half + 1) * (nt / 2);
-          for (int c0 = half * (nt / 2); c0 < c_end; c0 += 32) {
-            uint32_t r[32];
-            tmem_ld32(tmem_row + acc * 256u + c0, r);
-            tmem_wait(r);
-            if (c0 + 32 >= c_end) {  // all of this warp's columns are in registers
-              fence_before();
-              if (lane == 0) bar_arrive_cluster(to_cluster(bar_read(acc), 0));
+          const int cols = nt / 2, c_first = half * cols;  // this warp's columns of the tile: 32 to 128
+          const uint32_t tmem_mine = tmem_row + c_first;
+          float sum[kTileN / 2];  // over the parts of K
+          for (int j = 0; j < parts; ++j, ++part) {
+            const uint32_t acc = part & 1u;
+            if (!(ok = __all_sync(0xFFFFFFFFu, wait_ok(bar_acc(acc), (part >> 1) & 1u)))) break;
+            fence_after();
+#pragma unroll
+            for (int c0 = 0; c0 < kTileN / 2; c0 += 32) {
+              if (c0 >= cols) break;
+              uint32_t r[32];
+              tmem_ld32(tmem_mine + acc * 256u + c0, r);
+              tmem_wait(r);
+              if (j == 0) {
+#pragma unroll
+                for (int q = 0; q < 32; ++q) sum[c0 + q] = __uint_as_float(r[q]);
+              } else {
+#pragma unroll
+                for (int q = 0; q < 32; ++q) sum[c0 + q] += __uint_as_float(r[q]);
+              }
             }
-            const float4* b4 = reinterpret_cast<const float4*>(bias + n0 + c0);
+            fence_before();
+            if (lane == 0) bar_arrive_cluster(to_cluster(bar_read(acc), 0));
+            publish();
+          }
+          if (!ok) break;
+#pragma unroll
+          for (int c0 = 0; c0 < kTileN / 2; c0 += 32) {
+            if (c0 >= cols) break;
+            const int col = n0 + c_first + c0;
+            const float4* b4 = reinterpret_cast<const float4*>(bias + col);
             uint32_t h[16];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
               const float4 b = b4[q];
-              h[2 * q] = bf16_relu2(__uint_as_float(r[4 * q]) + b.x, __uint_as_float(r[4 * q + 1]) + b.y);
-              h[2 * q + 1] = bf16_relu2(__uint_as_float(r[4 * q + 2]) + b.z, __uint_as_float(r[4 * q + 3]) + b.w);
+              h[2 * q] = bf16_relu2(sum[c0 + 4 * q] + b.x, sum[c0 + 4 * q + 1] + b.y);
+              h[2 * q + 1] = bf16_relu2(sum[c0 + 4 * q + 2] + b.z, sum[c0 + 4 * q + 3] + b.w);
             }
             if (!last) {
-              const int col = n0 + c0;
               uint8_t* dst = out + static_cast<size_t>(col >> 6) * kBlockBytes;
 #pragma unroll
               for (int q = 0; q < 4; ++q)
                 *reinterpret_cast<uint4*>(dst + ((((col & 63) >> 3) + q) ^ (trow & 7)) * 16) =
                     make_uint4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
             } else {
-              const float4* w4 = reinterpret_cast<const float4*>(w_last + n0 + c0);
+              const float4* w4 = reinterpret_cast<const float4*>(w_last + col);
 #pragma unroll
               for (int q = 0; q < 8; ++q) {
                 const float4 w = w4[q];
@@ -504,11 +558,10 @@ mlp_wide_kernel(const __grid_constant__ WideArgs a, const __grid_constant__ CUte
             }
           }
           if (!last) {
-            // the rows are written; what the loading thread issues next must see them
-            __threadfence();
-            asm volatile("fence.proxy.async;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) bar_arrive(bar_stored(n0 / kTileN));
+            // Announced behind the next part's accumulator, so that its MMAs do not wait for these stores: that
+            // part needs nothing of this tile, but where the tile is all of the layer.
+            pending = n0 / kTileN;
+            if (width <= kTileN) publish();
           }
         }
       }
@@ -627,6 +680,7 @@ cudaError_t launch_layers(const WideMlp& w, uint8_t* image, uint8_t* act, int64_
   a.n_hidden = w.n_hidden;
   for (int l = 0; l < w.n_hidden; ++l) {
     a.kblocks[l] = w.kblocks[l];
+    a.parts[l] = part_count(w.kblocks[l]);
     a.width[l] = w.width[l];
     a.wrow[l] = w.wrow[l];
   }
@@ -656,6 +710,10 @@ cudaError_t launch_layers(const WideMlp& w, uint8_t* image, uint8_t* act, int64_
 cudaError_t build_wide_mlp(MlpModel& m, const uint16_t* const* h_w, const float* const* h_b, const float* h_mu,
                            const float* h_sigma) {
   if (m.n_layers < 2) return cudaSuccess;
+  cudaFuncAttributes attr{};  // the register split is made for this count
+  cudaError_t ea = cudaFuncGetAttributes(&attr, reinterpret_cast<const void*>(&mlp_wide_kernel));
+  if (ea != cudaSuccess) return ea;
+  if (attr.numRegs != kRegs) return cudaErrorInvalidKernelImage;
   WideMlp* w = new (std::nothrow) WideMlp();
   if (!w) return cudaErrorMemoryAllocation;
   m.wide = w;
