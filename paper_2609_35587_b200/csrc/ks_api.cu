@@ -106,7 +106,7 @@ ks_status read_status(ks_ctx* ctx) {
   if (v != 0) {
     *ctx->h_status = 0;
     // a failed launch may have left arrival counters of the slice mode behind
-    if (ctx->d_counters) cudaMemset(ctx->d_counters, 0, sizeof(int) * (ks::kMaxSliceBlocks + 1));
+    if (ctx->d_words) cudaMemset(ctx->d_words, 0, sizeof(int) * ks::kContextWords);
     return static_cast<ks_status>(v);
   }
   return KS_OK;
@@ -235,14 +235,15 @@ ks_status ks_create(ks_ctx** out_ctx, int cuda_device, const ks_gpu_desc* desc) 
   std::memset(ctx->pinned, 0, ctx->pinned_bytes);
   ctx->d_pinned_idx = static_cast<int32_t*>(d_pin);
   ctx->d_pinned_score = reinterpret_cast<float*>(ctx->d_pinned_idx + KS_MAX_K);
-  if (cudaMalloc(reinterpret_cast<void**>(&ctx->d_counters), sizeof(int) * (ks::kMaxSliceBlocks + 1)) != cudaSuccess ||
-      cudaMemset(ctx->d_counters, 0, sizeof(int) * (ks::kMaxSliceBlocks + 1)) != cudaSuccess) {
+  if (cudaMalloc(reinterpret_cast<void**>(&ctx->d_words), sizeof(int) * ks::kContextWords) != cudaSuccess ||
+      cudaMemset(ctx->d_words, 0, sizeof(int) * ks::kContextWords) != cudaSuccess) {
     cudaGetLastError();
-    cudaFree(ctx->d_counters);
+    cudaFree(ctx->d_words);
     cudaFreeHost(ctx->pinned);
     delete ctx;
     return KS_ERR_OOM;
   }
+  ctx->wait.words = ctx->d_words;
   ks_status s = ensure_workspace(ctx, 1u << 20);
   // status word in mapped pinned host memory: kernels write it through d_status, the host
   // reads h_status after a synchronisation without issuing a copy
@@ -254,7 +255,7 @@ ks_status ks_create(ks_ctx** out_ctx, int cuda_device, const ks_gpu_desc* desc) 
   if (s == KS_OK) *ctx->h_status = 0;
   if (s != KS_OK) {
     cudaFree(ctx->ws);
-    cudaFree(ctx->d_counters);
+    cudaFree(ctx->d_words);
     if (ctx->h_status) cudaFreeHost(ctx->h_status);
     cudaFreeHost(ctx->pinned);
     delete ctx;
@@ -270,7 +271,7 @@ ks_status ks_destroy(ks_ctx* ctx) {
   if (ctx->ev_begin) cudaEventDestroy(ctx->ev_begin);
   if (ctx->ev_end) cudaEventDestroy(ctx->ev_end);
   cudaFree(ctx->ws);
-  cudaFree(ctx->d_counters);
+  cudaFree(ctx->d_words);
   cudaFreeHost(ctx->h_status);
   cudaFreeHost(ctx->pinned);
   delete ctx;
@@ -594,7 +595,7 @@ ks_status ks_select(ks_ctx* ctx, const ks_problem* d_p, int P, const ks_candidat
                                     d_seg_index, pairs, k, ctx->ws, d_topk_idx, d_topk_score,
                                     static_cast<cudaStream_t>(stream), &ctx->launches, ctx->d_status,
                                     ctx->profile ? ctx->ev_begin : nullptr,
-                                    ctx->profile ? ctx->ev_end : nullptr, ctx->d_counters, &ctx->wait);
+                                    ctx->profile ? ctx->ev_end : nullptr, &ctx->wait);
   ctx->profile_valid = ctx->profile && e == cudaSuccess;
   return e == cudaSuccess ? KS_OK : cuda_fail(ctx, e, "ks_select");
 }
@@ -629,7 +630,6 @@ ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int 
       sl.n_slices = S;
       sl.pairs = C;
       sl.scores = reinterpret_cast<float*>(base + b_part + b_scratch);
-      sl.counters = ctx->d_counters;
       sl.out_idx = ctx->d_pinned_idx;
       sl.out_score = ctx->d_pinned_score;
       sl.tiles = reinterpret_cast<uint8_t*>(base + b_part);
@@ -650,10 +650,7 @@ ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int 
       }
       if (e != cudaSuccess) return cuda_fail(ctx, e, "ks_select_one");
       s = read_status(ctx);
-      if (s != KS_OK) {
-        cudaMemset(ctx->d_counters, 0, sizeof(int) * (ks::kMaxSliceBlocks + 1));
-        return s;
-      }
+      if (s != KS_OK) return s;  // (with the slice mode's counters cleared)
       std::memcpy(h_topk_idx, pin_idx, k * sizeof(int32_t));
       std::memcpy(h_topk_score, pin_sc, k * sizeof(float));
       return KS_OK;
@@ -667,7 +664,7 @@ ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int 
   if (s != KS_OK) return s;
   cudaError_t e = ks::launch_select(ctx->desc, *model, nullptr, &p, 1, d_c, C, nullptr, nullptr, C, k,
                                     ctx->ws, ctx->d_pinned_idx, ctx->d_pinned_score, st, &ctx->launches,
-                                    ctx->d_status, nullptr, nullptr, nullptr, &ctx->wait);
+                                    ctx->d_status, nullptr, nullptr, &ctx->wait);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "ks_select_one");
   std::memcpy(h_topk_idx, pin_idx, k * sizeof(int32_t));
@@ -750,7 +747,6 @@ ks_status ks_select_one_prepared(ks_ctx* ctx, const ks_catalogue* cat, ks_proble
   sl.n_slices = cat->slices;
   sl.pairs = cat->C;
   sl.scores = reinterpret_cast<float*>(base + cat->off_scores);
-  sl.counters = ctx->d_counters;
   sl.out_idx = ctx->d_pinned_idx;
   sl.out_score = ctx->d_pinned_score;
   sl.tiles = nullptr;
@@ -808,7 +804,7 @@ ks_status ks_select_host(ks_ctx* ctx, const ks_problem* h_p, int P, const ks_can
   if (e == cudaSuccess && seg && pairs > 0) e = cudaMemcpyAsync(d_si, h_seg_index, sizeof(int32_t) * pairs, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = ks::launch_select(ctx->desc, *model, d_p, nullptr, P, d_c, C, d_so, d_si, pairs, k, ctx->ws, d_oi,
-                          d_os, st, &ctx->launches, ctx->d_status, nullptr, nullptr, ctx->d_counters, &ctx->wait);
+                          d_os, st, &ctx->launches, ctx->d_status, nullptr, nullptr, &ctx->wait);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h_topk_idx, d_oi, sizeof(int32_t) * P * k, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h_topk_score, d_os, sizeof(float) * P * k, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);

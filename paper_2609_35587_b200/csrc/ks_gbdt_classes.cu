@@ -76,7 +76,7 @@ struct ClassArgs {
   int C, P;
   const int* order;           // [C] catalogue positions in similarity order
   const int2* units;          // (first position in `order`, candidates)
-  int* counters;              // [0] units, [1] 1: this path serves the call, [2] work counter, [8..25) first problem of every combination
+  int* counters;              // [0] units, [1] 1: this path serves the call, [2] work counter, [3] 1: a wait ran out, [8..25) first problem of every combination
   const int* prob_order;      // [P] problems by combination and size
   const uint8_t* prob_tab;    // [P][kProbBytes], in that order
   uint8_t* programs;          // per CTA: [n_trees][32] uint4 (sets of the leaves), [n_trees * prog_words] words
@@ -85,8 +85,6 @@ struct ClassArgs {
   int pitch, first, count;    // problems first .. first + count - 1 of the order
   int* status;
 };
-
-__device__ int g_class_abort;  // as in ks_gbdt_fast.cu; cleared by the kernel that makes the units
 
 // ------------------------------------------------------------------------------------------
 // preparation of a call
@@ -102,7 +100,6 @@ __global__ void __launch_bounds__(256)
 units_kernel(const ks_candidate* __restrict__ c, int C, const int* __restrict__ order, int2* __restrict__ units,
              int* __restrict__ counters) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) g_class_abort = 0;
   if (i >= C) return;
   // a run also ends at every multiple of kRunCut, so that no thread walks a whole catalogue
   const ks_candidate me = load_candidate(c + order[i]);
@@ -952,12 +949,15 @@ class_walk_kernel(ks_gpu_desc desc, const __grid_constant__ ClassArgs a) {
     sh.fail = 0;
     sh.done[0] = sh.done[1] = 0;
     sh.pending[0] = sh.pending[1] = 0;
-    sh.abort = *reinterpret_cast<volatile int*>(&g_class_abort);
+    sh.abort = *reinterpret_cast<volatile int*>(a.counters + 3);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid < 64) sh.fq[tid] = fv.feat[tid];
   __syncthreads();
-  if (sh.abort) return;
+  if (sh.abort) {  // a wait ran out in an earlier CTA of this call, which fails
+    if (tid == 0 && a.status) atomicExch(a.status, KS_ERR_TIMEOUT);
+    return;
+  }
   if (buf0 - sbase + walk_smem(a.tile_rows, a.n_buckets) > dyn) {  // (the host's allowance for the alignment is too small)
     if (tid == 0 && a.status) atomicExch(a.status, KS_ERR_UNSUPPORTED);
     return;
@@ -1090,7 +1090,7 @@ class_walk_kernel(ks_gpu_desc desc, const __grid_constant__ ClassArgs a) {
           if (!__all_sync(0xFFFFFFFFu, here)) {  // the warp gives up together
             if (!*v_fail) {
               sh.fail = 1;
-              atomicExch(&g_class_abort, 1);
+              atomicExch(a.counters + 3, 1);
               if (a.status) atomicExch(a.status, KS_ERR_TIMEOUT);
             }
             break;

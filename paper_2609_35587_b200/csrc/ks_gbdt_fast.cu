@@ -78,10 +78,6 @@ constexpr int kNBuf = 2;                // buffers of a ring (four of 8 KB and t
 // shared memory map (byte offsets from the dynamic shared base): the rings' chunk buffers, then the tile
 constexpr int kOffBuf0 = 0;
 
-// Raised by a CTA whose bounded wait ran out, so that the CTAs after it leave at once; cleared by
-// the per-call table kernel that precedes every launch of the select kernel.
-__device__ int g_fast_abort;
-
 // Slice mode (single-problem latency call): the trees are split over n_slices CTAs per
 // candidate block. Every CTA stores its partial scores; the last CTA to arrive for a block
 // (atomic counter, nobody waits) adds the slices in a fixed order and ranks the block; the
@@ -90,7 +86,6 @@ struct SliceArgs {
   int n_slices;            // 1 = every CTA walks the whole ensemble
   long long pairs;         // rows of the partial-score planes
   float* scores;           // [n_slices][pairs] partial scores
-  int* counters;           // [P * nblk + 1], zero on entry; every counter is reset by its last user
   int32_t* out_idx;        // single-problem form only: [k] final result (device-visible, may be
   float* out_score;        // mapped host memory); null when a merge kernel follows
   const uint8_t* tiles;    // prepared tiles [blocks][rows][NC] (tile_pairs_kernel), or null
@@ -129,7 +124,7 @@ cand_rows_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, co
   extern __shared__ __align__(16) float s_cthr[];  // thresholds of the candidate-only features, values, records
   __shared__ FeatQ s_fq[64];
   const int combo = combo0 >= 0 ? combo0 : blockIdx.y, tid = threadIdx.x;
-  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) g_fast_abort = 0;
+  if (fv.words && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) fv.words[kWordWalk] = 0;
   if (mask_ptr && !((*mask_ptr >> combo) & 1u)) return;
   const float* T = stage_thresholds(fv, fv.thr_cand0, fv.thr_prob0 - fv.thr_cand0, s_cthr, thr_cap) - fv.thr_cand0;
   if (tid < 64) s_fq[tid] = fv.feat[tid];
@@ -211,7 +206,7 @@ pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem
   // (also) precedes the select kernel, whose CTAs leave at once when the class walk
   // (ks_gbdt_classes.cu) serves the call; that one then writes the partial lists
   const bool skip = path && *path == 1;
-  if (blockIdx.x == 0 && tid == 0) g_fast_abort = skip;
+  if (blockIdx.x == 0 && tid == 0) fv.words[kWordWalk] = skip ? kLeaveServed : 0;
   if (skip) return;
   int most = 0;
   for (int q = 0; q < kMemoCombos; ++q) most = max(most, memo.count[q]);
@@ -337,7 +332,7 @@ tile_pairs_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem
   __shared__ float s_pf[64];
   float* s_thr = s_x + kTileCols * kTileRows;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (blockIdx.x == 0 && tid == 0) g_fast_abort = 0;
+  if (blockIdx.x == 0 && tid == 0) fv.words[kWordWalk] = 0;
   const long long n_items = static_cast<long long>(P) * groups;
   const int begin = static_cast<int>(n_items * blockIdx.x / gridDim.x);
   const int end = static_cast<int>(n_items * (blockIdx.x + 1) / gridDim.x);
@@ -408,7 +403,7 @@ tile_rows_kernel(const float* __restrict__ feat, int64_t rows, FastView fv, uint
   __shared__ FeatQ s_fq[64];
   float* s_thr = s_x + 64 * kTileRows;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (blockIdx.x == 0 && threadIdx.x == 0) g_fast_abort = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) fv.words[kWordWalk] = 0;
   stage_thresholds(fv, 0, fv.n_thr, s_thr, fv.n_thr);
   if (threadIdx.x < 64) s_fq[threadIdx.x] = fv.feat[threadIdx.x];
   const uint32_t thr = smem_u32(s_thr);
@@ -714,7 +709,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
       problem_terms(use_value ? p_value : load_problem(p + prob), desc, s_pt);
       problem_columns(s_pt, [&](int col, float v) { s_pfeat[col] = v; });
     }
-    s_abort = *reinterpret_cast<volatile int*>(&g_fast_abort);
+    s_abort = *reinterpret_cast<volatile int*>(fv.words + kWordWalk);
   }
   if (tid < KS_MAX_K) s_list[tid] = 0ull;
   if (!tiles_given && fv.prob_tab) {
@@ -724,7 +719,8 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
       reinterpret_cast<uint32_t*>(&s_pt)[tid] = __ldcg(reinterpret_cast<const uint32_t*>(rec + kFastMaxProbRows) + tid);
   }
   __syncthreads();
-  if (s_abort) {  // a wait ran out in an earlier CTA of this launch: the call fails, leave at once
+  if (s_abort) {  // a wait ran out in an earlier CTA of this call, which fails, or the class walk serves the call: leave at once
+    if (s_abort == kLeaveFailed && tid == 0 && status) atomicExch(status, KS_ERR_TIMEOUT);
     if (tid < k && slice == 0 && partial) partial[(static_cast<size_t>(prob) * nblk + chunk) * k + tid] = 0ull;
     return;
   }
@@ -804,7 +800,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
         if (*v_fail || !mbar_wait_bounded(bar, par, fv.wait_limit, v_fail)) {
           if (!*v_fail) {
             s_fail = 1;
-            atomicExch(&g_fast_abort, 1);
+            atomicExch(fv.words + kWordWalk, kLeaveFailed);
             if (status) atomicExch(status, KS_ERR_TIMEOUT);
           }
           break;
@@ -952,7 +948,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
       __threadfence();
       __syncthreads();
       if (tid == 0) {
-        int* cnt = sl.counters + static_cast<size_t>(prob) * nblk + chunk;
+        int* cnt = fv.words + static_cast<size_t>(prob) * nblk + chunk;
         s_last = atomicAdd(cnt, 1) == S - 1;
         if (s_last) *cnt = 0;  // nobody else touches this counter again in this launch
       }
@@ -988,7 +984,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     // single-problem form: the last block to finish merges the per-block lists
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(sl.counters + nblk, 1) == nblk - 1;
+    if (tid == 0) s_last = atomicAdd(fv.words + nblk, 1) == nblk - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
@@ -1012,7 +1008,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     }
     __syncthreads();
     if (tid == 0) {
-      sl.counters[nblk] = 0;
+      fv.words[nblk] = 0;
       if (sl.out_seq) {  // the results are in place: tell the host, which polls this word
         __threadfence_system();
         *reinterpret_cast<volatile int*>(sl.out_seq) = sl.seq;
@@ -1681,6 +1677,10 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
       fv.prob_tab = fv.pair_tab + static_cast<size_t>(memo_batch) * kMemoCap * pair_rec_bytes(g);
     }
   }
+  if (C == 0) {  // no kernel in front of the walk: the word that a failed call may have left is cleared here
+    e = cudaMemsetAsync(fv.words + kWordWalk, 0, sizeof(int), stream);
+    if (e != cudaSuccess) return e;
+  }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (ev_begin) cudaEventRecord(ev_begin, stream);
@@ -1695,7 +1695,6 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     a.sl.n_slices = slice->n_slices;
     a.sl.pairs = slice->pairs;
     a.sl.scores = slice->scores;
-    a.sl.counters = slice->counters;
     a.sl.out_idx = slice->out_idx;
     a.sl.out_score = slice->out_score;
     a.sl.tiles = tiles_mode ? slice->tiles : nullptr;

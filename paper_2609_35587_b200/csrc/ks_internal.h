@@ -31,6 +31,7 @@ struct alignas(16) MlpTcParams {
   const float* w1_prob;                // device, [18][256]: first-layer weights of the folded inputs
   int wait_limit;                      // tries a barrier wait may take (set at every launch)
   int starve;                          // test hook: the weight image is never copied, so the first wait runs out
+  int* leave;                          // the context's word kWordMlp
 };
 
 // Linear scorer (one weight layer) in a form the fused ridge kernel consumes: per feature column
@@ -59,11 +60,14 @@ struct FeatQ {
   uint8_t rank[3][4];
 };
 
-// Probe budget of the quantised kernel's chunk waits (0: the default) and the test hook that
-// starves a wait (the barrier is armed for more bytes than its copy brings).
+// What a launch takes from its context: the probe budget of the kernels' bounded waits (0: the
+// default), the test hook that starves a wait (the barrier is armed for more bytes than its copy
+// brings), and the context's device words (kWord...). The words belong to the context and not to the
+// process: another context's kernels may run at the same time.
 struct FastWait {
   int limit;
   int starve;
+  int* words;
 };
 
 constexpr int kNoFixed = INT32_MIN;
@@ -125,14 +129,14 @@ struct ks_ctx {
   size_t ws_bytes = 0;
   void* pinned = nullptr;  // host staging for ks_select_one results
   size_t pinned_bytes = 0;
-  int* d_counters = nullptr;  // [kMaxSliceBlocks + 1] arrival counters of the slice mode, zero between calls
+  int* d_words = nullptr;  // [kContextWords], see there
   int32_t* d_pinned_idx = nullptr;  // device aliases of `pinned` (mapped host memory)
   float* d_pinned_score = nullptr;
   int* h_status = nullptr;  // status word (mapped pinned host memory) set by kernels whose
   int* d_status = nullptr;  // bounded waits give up; d_status is its device alias
   int64_t launches = 0;
   int select_one_seq = 0;  // sequence number of the last single-problem call
-  ks::FastWait wait{0, 0};  // probe budget of bounded device waits (0: default) and the starve hook (tests)
+  ks::FastWait wait{0, 0, nullptr};  // probe budget of bounded device waits (0: default), starve hook (tests), d_words
   char err[256] = {0};
   // optional timing of the dominant kernel of the last ks_select* call (ks_profile_enable)
   bool profile = false;
@@ -173,6 +177,12 @@ constexpr size_t kMemoTableBytes = size_t(256) << 20;  // per-(problem, class) r
 constexpr int kFastWaitLimit = 1 << 17;  // probes of a chunk wait (a sleep ends early, ~0.2 us measured): tens of ms
 constexpr int kMlpThreads = 512;        // threads per block of the tensor-core MLP kernel
 constexpr int kMaxSliceBlocks = 1024;  // candidate blocks the slice mode supports
+// A context's device words: the arrival counters of the slice mode (zero between calls), then a word per
+// kernel family that makes the CTAs which start after it was raised leave at once. It is cleared in front
+// of every launch of the family.
+constexpr int kWordWalk = kMaxSliceBlocks + 1, kWordMlp = kWordWalk + 1, kWordWide = kWordMlp + 1;
+constexpr int kContextWords = kWordWide + 1;
+constexpr int kLeaveFailed = 1, kLeaveServed = 2;  // a wait ran out; another kernel serves the call
 
 // Levels of the categorical field held by feature column `col` (0: not a level-code column):
 // layout flags, operand type, bias flag, activation, kernel / epilogue schedule, tile scheduler.
@@ -207,7 +217,6 @@ struct FastSlice {
   int n_slices;
   long long pairs;   // rows of one partial-score plane
   float* scores;     // [n_slices][pairs]
-  int* counters;     // [blocks + 1], zero between calls
   int32_t* out_idx;  // single-problem form: [k], device-visible; else null (a merge kernel follows)
   float* out_score;
   uint8_t* tiles;    // scratch for the tiles [problems * blocks][rows][block_cands], or null
@@ -267,9 +276,9 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
                                int nblk, int rows_per_cta, const int64_t* seg_off, const int32_t* seg_idx,
                                int k, unsigned long long* partial, void* scratch, int* status,
                                cudaStream_t stream, int64_t* launches, cudaEvent_t ev_begin,
-                               const FastSlice* slice = nullptr, void* memo_mem = nullptr,
-                               const FastWait* wait = nullptr, const FastPrepared* prep = nullptr,
-                               const int32_t* perm = nullptr, const ClassCall* classes = nullptr);
+                               const FastSlice* slice, void* memo_mem, const FastWait* wait,
+                               const FastPrepared* prep = nullptr, const int32_t* perm = nullptr,
+                               const ClassCall* classes = nullptr);
 // Prepared catalogue (single-problem calls against a fixed catalogue and model).
 size_t fast_prepared_rows_bytes(const GbdtModel& g, int C);
 size_t fast_prepared_memo_bytes(const GbdtModel& g, int C);  // 0: the model's per-pair rows do not fit a record
@@ -280,7 +289,7 @@ int fast_slices(const GbdtModel& g, int64_t blocks);
 size_t score_fast_scratch_bytes(const GbdtModel& g, int64_t rows);
 cudaError_t launch_score_fast(const ks_gpu_desc& desc, const GbdtModel& g, const float* d_feat, int64_t rows,
                               float* d_scores, void* scratch, int* status, cudaStream_t stream,
-                              int64_t* launches, const FastWait* wait = nullptr, int floor_repeat = 0);
+                              int64_t* launches, const FastWait* wait, int floor_repeat = 0);
 // checked build (KS_DEBUG_BOUNDS): source line of the first index found out of range (0: none;
 // -1: not a checked build), and its reset
 int fast_bounds_line();
@@ -300,13 +309,13 @@ size_t mlp_tc_scratch_bytes(int C);
 bool score_mlp_tc_ok(const MlpModel& m);
 cudaError_t launch_score_mlp_tc(const ks_gpu_desc& desc, const MlpModel& m, const float* d_feat, int64_t rows,
                                 float* d_scores, int* status, cudaStream_t stream, int64_t* launches,
-                                const FastWait* wait = nullptr);
+                                const FastWait* wait);
 constexpr int kMlpWaitLimit = 1 << 14;  // tries of a barrier wait of the tensor-core kernel (each blocks for up to a few microseconds): tens of ms
 cudaError_t launch_select_mlp_tc(const ks_gpu_desc& desc, const MlpModel& m, const ks_problem* d_p,
                                  const ks_problem* p_by_value, int P, const ks_candidate* d_c, int C, int nblk,
                                  const int64_t* seg_off, const int32_t* seg_idx, int k,
                                  unsigned long long* partial, void* scratch, int* status, cudaStream_t stream,
-                                 int64_t* launches, cudaEvent_t ev_begin, const FastWait* wait = nullptr);
+                                 int64_t* launches, cudaEvent_t ev_begin, const FastWait* wait);
 
 // Tensor-core path for rankers of any width (ks_mlp_wide.cu).
 cudaError_t build_wide_mlp(MlpModel& m, const uint16_t* const* h_w, const float* const* h_b, const float* h_mu,
@@ -349,7 +358,6 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                           const int64_t* d_seg_off, const int32_t* d_seg_idx, int64_t pairs, int k,
                           void* d_partial, int32_t* d_topk_idx, float* d_topk_score,
                           cudaStream_t stream, int64_t* launches, int* d_status,
-                          cudaEvent_t ev_begin = nullptr, cudaEvent_t ev_end = nullptr, int* d_counters = nullptr,
-                          const FastWait* wait = nullptr);
+                          cudaEvent_t ev_begin, cudaEvent_t ev_end, const FastWait* wait);
 
 }  // namespace ks

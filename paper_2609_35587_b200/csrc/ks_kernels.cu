@@ -881,7 +881,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                           const int64_t* d_seg_off, const int32_t* d_seg_idx, int64_t pairs, int k,
                           void* d_partial, int32_t* d_topk_idx, float* d_topk_score,
                           cudaStream_t stream, int64_t* launches, int* d_status, cudaEvent_t ev_begin,
-                          cudaEvent_t ev_end, int* d_counters, const FastWait* wait) {
+                          cudaEvent_t ev_end, const FastWait* wait) {
   if (P == 0) return cudaSuccess;
   const int64_t per = per_problem_rows(P, C, pairs, d_seg_off != nullptr);
   if (model.kind == 0 && model.gbdt.fast) {
@@ -894,13 +894,12 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     const int sized_slices = d_seg_off ? 1 : fast_slices(model.gbdt, static_cast<int64_t>(P) * nblk);  // as sized
     char* mem = static_cast<char*>(d_partial) + part_bytes;
     FastSlice sl{};
-    sl.n_slices = d_counters ? sized_slices : 1;
+    sl.n_slices = p_by_value ? 1 : sized_slices;  // (a single problem has a path of its own)
     if (sl.n_slices > 1) {
       // the slices of a block share a tile that is built in front of them; behind the tiles, their score planes
       sl.pairs = pairs;
       sl.tiles = reinterpret_cast<uint8_t*>(mem);
       sl.scores = reinterpret_cast<float*>(mem + (fast_tiles_bytes(model.gbdt, static_cast<int64_t>(P) * nblk) + 255) / 256 * 256);
-      sl.counters = d_counters;
     }
     // the memo of the per-pair rows sits behind the per-call table (batches of whole-ensemble CTAs only)
     void* memo_mem = (sized_slices > 1 || p_by_value || fast_memo_bytes(model.gbdt, P, C) == 0)

@@ -146,13 +146,12 @@ __device__ __forceinline__ uint32_t pack_bf16_relu(float lo, float hi) {
 // candidate-only columns, standardised and rounded to bf16, once per call
 // ------------------------------------------------------------------------------------------
 
-// Raised by a CTA whose bounded wait ran out, so that the CTAs after it leave at once; cleared by
-// the per-call table kernel that precedes every launch. (The status word itself lives in mapped
-// host memory: reading it from every CTA would cost a PCIe round trip each.)
-__device__ int g_mlp_abort;
+// The context's word kWordMlp is raised by a CTA whose bounded wait ran out, so that the CTAs after it
+// leave at once; the per-call table kernel that precedes every launch clears it. (The status word itself
+// lives in mapped host memory: reading it from every CTA would cost a PCIe round trip each.)
 
-// the scoring call has no per-call table kernel in front: this clears the abort flag instead
-__global__ void mlp_reset_abort_kernel() { g_mlp_abort = 0; }
+// the scoring call has no per-call table kernel in front: this clears the word instead
+__global__ void mlp_reset_leave_kernel(int* leave) { *leave = 0; }
 
 __global__ void mlp_combo_mask_kernel(const ks_problem* __restrict__ p, int P, unsigned* __restrict__ mask) {
   unsigned m = 0;
@@ -169,7 +168,7 @@ __global__ void __launch_bounds__(kCandThreads)
 mlp_cand_cols_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, const unsigned* mask_ptr,
                      int combo0, const __grid_constant__ MlpTcParams prm, uint8_t* __restrict__ out) {
   const int combo = combo0 >= 0 ? combo0 : blockIdx.y;
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) g_mlp_abort = 0;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *prm.leave = 0;
   if (mask_ptr && !((*mask_ptr >> combo) & 1u)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= C) return;
@@ -365,9 +364,10 @@ select_mlp_tc_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_prob
   __shared__ int s_fail, s_abort;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid == 0) s_abort = *reinterpret_cast<volatile int*>(&g_mlp_abort);
+  if (tid == 0) s_abort = *reinterpret_cast<volatile int*>(prm.leave);
   __syncthreads();
-  if (s_abort) {  // a wait ran out in an earlier CTA of this launch: the call fails, leave at once
+  if (s_abort) {  // a wait ran out in an earlier CTA of this call: it fails, leave at once
+    if (tid == 0 && status) atomicExch(status, KS_ERR_TIMEOUT);
     if (!kRows && tid < k) partial[static_cast<size_t>(blockIdx.x) * k + tid] = 0ull;
     return;
   }
@@ -465,7 +465,7 @@ select_mlp_tc_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_prob
       if ((i & 255) == 255 && *reinterpret_cast<volatile int*>(&s_fail)) break;
     }
     *reinterpret_cast<volatile int*>(&s_fail) = 1;
-    atomicExch(&g_mlp_abort, 1);
+    atomicExch(prm.leave, kLeaveFailed);
     return false;
   };
   if (!wait_ok(bar_w, 0)) failed = true;
@@ -825,8 +825,9 @@ cudaError_t launch_select_mlp_tc(const ks_gpu_desc& desc, const MlpModel& m, con
                                  const int64_t* seg_off, const int32_t* seg_idx, int k,
                                  unsigned long long* partial, void* scratch, int* status, cudaStream_t stream,
                                  int64_t* launches, cudaEvent_t ev_begin, const FastWait* wait) {
-  m.h_tc_params->wait_limit = wait && wait->limit > 0 ? wait->limit : kMlpWaitLimit;
-  m.h_tc_params->starve = wait ? wait->starve : 0;
+  m.h_tc_params->wait_limit = wait->limit > 0 ? wait->limit : kMlpWaitLimit;
+  m.h_tc_params->starve = wait->starve;
+  m.h_tc_params->leave = wait->words + kWordMlp;
   ks_problem pv{};
   if (p_by_value) pv = *p_by_value;
   const int uv = p_by_value != nullptr;
@@ -843,6 +844,9 @@ cudaError_t launch_select_mlp_tc(const ks_gpu_desc& desc, const MlpModel& m, con
     mlp_cand_cols_kernel<<<dim3((C + kCandThreads - 1) / kCandThreads, uv ? 1 : kCombos), kCandThreads, 0, stream>>>(
         desc, d_c, C, uv ? nullptr : d_mask, uv ? (pv.dtype_ab & 3) * 4 + (pv.dtype_d & 3) : -1, *m.h_tc_params, d_cols);
     ++*launches;
+  } else {
+    e = cudaMemsetAsync(m.h_tc_params->leave, 0, sizeof(int), stream);
+    if (e != cudaSuccess) return e;
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -873,14 +877,15 @@ bool score_mlp_tc_ok(const MlpModel& m) { return m.tc && m.h_tc_params && !m.h_t
 cudaError_t launch_score_mlp_tc(const ks_gpu_desc& desc, const MlpModel& m, const float* d_feat, int64_t rows,
                                 float* d_scores, int* status, cudaStream_t stream, int64_t* launches,
                                 const FastWait* wait) {
-  m.h_tc_params->wait_limit = wait && wait->limit > 0 ? wait->limit : kMlpWaitLimit;
-  m.h_tc_params->starve = wait ? wait->starve : 0;
+  m.h_tc_params->wait_limit = wait->limit > 0 ? wait->limit : kMlpWaitLimit;
+  m.h_tc_params->starve = wait->starve;
+  m.h_tc_params->leave = wait->words + kWordMlp;
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(&select_mlp_tc_kernel<2>), kSmemBytes);
   if (e != cudaSuccess) return e;
   const uint8_t* image = reinterpret_cast<const uint8_t*>(m.d_tc_image);
   const ks_problem pv{};
   constexpr int64_t kBatch = int64_t{1} << 30;
-  mlp_reset_abort_kernel<<<1, 1, 0, stream>>>();
+  mlp_reset_leave_kernel<<<1, 1, 0, stream>>>(m.h_tc_params->leave);
   ++*launches;
   for (int64_t first = 0; first < rows; first += kBatch) {
     const int64_t n = rows - first < kBatch ? rows - first : kBatch;

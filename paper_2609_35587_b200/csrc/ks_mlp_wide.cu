@@ -99,6 +99,7 @@ struct WideArgs {
   float* scores;
   int64_t rows;
   int wait_limit, starve;
+  int* leave;   // the context's word kWordWide: raised by a CTA whose wait ran out, cleared by the input kernel in front
   int* status;
 };
 
@@ -208,10 +209,6 @@ __device__ __forceinline__ bool epilogue_and(bool v) {
   return r != 0;
 }
 
-// Raised by a CTA whose bounded wait ran out, so that the CTAs after it leave at once; cleared by
-// the input kernel in front.
-__device__ int g_wide_abort;
-
 // ------------------------------------------------------------------------------------------
 // the input rows: features (or given rows), standardised, rounded to bf16, in operand form
 // ------------------------------------------------------------------------------------------
@@ -276,8 +273,8 @@ template <bool kOneHot>
 __global__ void __launch_bounds__(128)
 wide_pair_rows_kernel(ks_gpu_desc desc, const ProblemTerms* __restrict__ terms, int P, const ks_candidate* __restrict__ c,
                       int C, const int64_t* __restrict__ seg_off, const int32_t* __restrict__ seg_idx, int64_t first,
-                      int64_t n, int64_t n_padded, const __grid_constant__ WideInput in, uint8_t* __restrict__ image) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) g_wide_abort = 0;
+                      int64_t n, int64_t n_padded, const __grid_constant__ WideInput in, uint8_t* __restrict__ image, int* leave) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *leave = 0;
   const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (r >= n_padded) return;
   float x[KS_F_PAD];
@@ -309,8 +306,8 @@ wide_pair_rows_kernel(ks_gpu_desc desc, const ProblemTerms* __restrict__ terms, 
 template <bool kOneHot>
 __global__ void __launch_bounds__(128)
 wide_given_rows_kernel(const float* __restrict__ feat, int64_t n, int64_t n_padded,
-                       const __grid_constant__ WideInput in, uint8_t* __restrict__ image) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) g_wide_abort = 0;
+                       const __grid_constant__ WideInput in, uint8_t* __restrict__ image, int* leave) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *leave = 0;
   const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (r >= n_padded) return;
   float x[KS_F_PAD];
@@ -353,7 +350,8 @@ mlp_wide_kernel(const __grid_constant__ WideArgs a, const __grid_constant__ CUte
   auto bar_stored = [&](int i) { return bar0 + 8u * (2 * kStages + 4 + i); };
 
   if (tid == 0) {
-    s_abort = *reinterpret_cast<volatile int*>(&g_wide_abort);
+    s_abort = *reinterpret_cast<volatile int*>(a.leave);
+    if (s_abort && a.status) atomicExch(a.status, KS_ERR_TIMEOUT);
     s_fail = 0;
     for (int s = 0; s < kStages; ++s) {
       bar_init(bar_full(s), 1);
@@ -390,7 +388,7 @@ mlp_wide_kernel(const __grid_constant__ WideArgs a, const __grid_constant__ CUte
       if ((i & 63) == 63 && *v_fail) return false;
     }
     *v_fail = 1;
-    atomicExch(&g_wide_abort, 1);
+    atomicExch(a.leave, kLeaveFailed);
     if (a.status) atomicExch(a.status, KS_ERR_TIMEOUT);
     return false;
   };
@@ -690,8 +688,9 @@ cudaError_t launch_layers(const WideMlp& w, uint8_t* image, uint8_t* act, int64_
   a.act = act;
   a.scores = scores;
   a.rows = rows;
-  a.wait_limit = wait && wait->limit > 0 ? wait->limit : kMlpWaitLimit;
-  a.starve = wait ? wait->starve : 0;
+  a.wait_limit = wait->limit > 0 ? wait->limit : kMlpWaitLimit;
+  a.starve = wait->starve;
+  a.leave = wait->words + kWordWide;
   a.status = status;
   const int64_t n_blocks = (rows + kRowsPair - 1) / kRowsPair;
   CUtensorMap mx, ma, mw[4];
@@ -806,10 +805,10 @@ cudaError_t launch_select_wide(const ks_gpu_desc& desc, const MlpModel& m, const
       const unsigned grid = static_cast<unsigned>((padded + 127) / 128);
       if (w.input.onehot)
         wide_pair_rows_kernel<true><<<grid, 128, 0, stream>>>(desc, terms, P, d_c, C, seg_off, seg_idx, first, n, padded,
-                                                              w.input, image);
+                                                              w.input, image, wait->words + kWordWide);
       else
         wide_pair_rows_kernel<false><<<grid, 128, 0, stream>>>(desc, terms, P, d_c, C, seg_off, seg_idx, first, n,
-                                                               padded, w.input, image);
+                                                               padded, w.input, image, wait->words + kWordWide);
       cudaError_t e = cudaGetLastError();
       if (e == cudaSuccess) e = launch_layers(w, image, act, n, scores + (first - round0), status, wait, stream);
       if (e != cudaSuccess) return e;
@@ -836,8 +835,8 @@ cudaError_t launch_score_wide(const MlpModel& m, const float* d_feat, int64_t ro
     const int64_t n = std::min(rows - first, kBatchRows), padded = (n + kRowsPair - 1) / kRowsPair * kRowsPair;
     const unsigned grid = static_cast<unsigned>((padded + 127) / 128);
     const float* x = d_feat + first * KS_F_PAD;
-    if (w.input.onehot) wide_given_rows_kernel<true><<<grid, 128, 0, stream>>>(x, n, padded, w.input, image);
-    else wide_given_rows_kernel<false><<<grid, 128, 0, stream>>>(x, n, padded, w.input, image);
+    if (w.input.onehot) wide_given_rows_kernel<true><<<grid, 128, 0, stream>>>(x, n, padded, w.input, image, wait->words + kWordWide);
+    else wide_given_rows_kernel<false><<<grid, 128, 0, stream>>>(x, n, padded, w.input, image, wait->words + kWordWide);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_layers(w, image, act, n, d_scores + first, status, wait, stream);
     if (e != cudaSuccess) return e;
