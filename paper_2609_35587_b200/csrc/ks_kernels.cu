@@ -581,9 +581,11 @@ select_ridge_kernel(const __grid_constant__ ks_gpu_desc desc, const RidgeProblem
 
 // Problems a block ranks, and blocks per group of problems: as many as fill the machine once (two blocks
 // of 512 threads an SM), with about 512 candidates each at least.
-static int ridge_group(bool segmented, int P) { return segmented || P < kMemoMinProblems ? 1 : kRidgeProblems; }
-static int ridge_blocks(int P, int64_t per_problem, bool segmented) {
-  const int g = ridge_group(segmented, P);
+// Several problems share a block only where the class tables are used: without them the kernel ranks one.
+size_t ridge_memo_bytes(int P, int C);
+static int ridge_group(bool segmented, int P, int C) { return segmented || ridge_memo_bytes(P, C) == 0 ? 1 : kRidgeProblems; }
+static int ridge_blocks(int P, int C, int64_t per_problem, bool segmented) {
+  const int g = ridge_group(segmented, P, C);
   const int64_t groups = (P + g - 1) / g, most = std::max<int64_t>(1, (per_problem + 511) / 512);
   return static_cast<int>(std::min(most, std::max<int64_t>(1, 2 * 148 / groups)));
 }
@@ -867,7 +869,7 @@ size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, 
     return (part + 255) / 256 * 256 + wide_scratch_bytes(model.mlp, P, pairs);
   }
   if (model.kind == 1 && model.mlp.h_ridge) {
-    const size_t part = static_cast<size_t>(P) * ridge_blocks(P, per, segmented) * k * sizeof(unsigned long long);
+    const size_t part = static_cast<size_t>(P) * ridge_blocks(P, C, per, segmented) * k * sizeof(unsigned long long);
     return (part + 255) / 256 * 256 + ridge_scratch_bytes(P, C) + ridge_memo_bytes(P, C);
   }
   const int st = pick_sub_tiles(P, per);
@@ -952,7 +954,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     // linear scorer: per-call tables of what a problem, a candidate and a class bring, then the kernel
     // that adds and ranks
     PairMap map = make_map(P, C, pairs, d_seg_off, d_seg_idx, kBlock);
-    map.nblk = ridge_blocks(P, per, d_seg_off != nullptr);
+    map.nblk = ridge_blocks(P, C, per, d_seg_off != nullptr);
     unsigned long long* partial = static_cast<unsigned long long*>(d_partial);
     const size_t part_bytes = (static_cast<size_t>(P) * map.nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
     char* mem = static_cast<char*>(d_partial) + part_bytes;
@@ -968,7 +970,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     ridge_problem_kernel<<<(P + 127) / 128, 128, 0, stream>>>(desc, d_p, pv, p_by_value != nullptr, P, prm, d_prob, d_mask);
     ++*launches;
     MemoView memo{};
-    if (!p_by_value && C > 0 && ridge_memo_bytes(P, C) != 0) {
+    if (ridge_memo_bytes(P, C) != 0) {  // (never for a single problem)
       memo = memo_view(mem + ridge_scratch_bytes(P, C), C);
       e = memo_clear(memo, stream);
       if (e != cudaSuccess) return e;
@@ -986,7 +988,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
       }
     }
     if (ev_begin) cudaEventRecord(ev_begin, stream);
-    const int group = ridge_group(d_seg_off != nullptr, P);
+    const int group = ridge_group(d_seg_off != nullptr, P, C);
     const unsigned blocks = static_cast<unsigned>(static_cast<int64_t>((P + group - 1) / group) * map.nblk);
     auto kernel = !memo.keys ? &select_ridge_kernel<1, false>
                   : group == 1 ? &select_ridge_kernel<1, true> : &select_ridge_kernel<kRidgeProblems, true>;

@@ -64,3 +64,25 @@ def test_merge_of_partial_lists(ks, ctx, P, n):
     some = sorted({0, P // 2, P - 1})
     ridx, rsc = oracle.select(prob[some], cand, DESC, 10, static=True)
     assert np.array_equal(idx.cpu().numpy()[some], ridx) and np.array_equal(sc.cpu().numpy()[some], rsc)
+
+
+@pytest.mark.parametrize("P,C", [(8192, 300), (8193, 300), (8195, 70), (40, 0), (31, 0)])
+def test_problems_beyond_the_class_tables(ks, ctx, P, C):
+    """The class tables serve 32 to 8,192 problems and a pool that is not empty; four problems share a block
+    only with them. An empty pool gives empty lists."""
+    dev = torch.device("cuda", 0)
+    st = wl.feature_stats("cfg2")
+    mlp = wl.mlp_xavier(2, [64, 1], st["mu"], st["sigma"])
+    prob, cand = wl.problems_batch(P, P, cross_precision=True), wl.candidates_full_grid(3, 300)[:C]
+    idx = torch.full((P, 5), 7, dtype=torch.int32, device=dev)
+    sc = torch.full((P, 5), 7.0, device=dev)
+    ctx.select(ks.to_device(prob, dev), P, ks.to_device(cand, dev) if C else None, C, ctx.model_create_mlp(mlp), 5,
+               out_idx=idx, out_score=sc)
+    idx, sc = idx.cpu().numpy(), sc.cpu().numpy()
+    if C == 0:
+        assert (idx == -1).all() and np.isneginf(sc).all()
+        return
+    for p in (0, 1, P // 4, P // 4 + 1, P - 2, P - 1):
+        _, _, ref = oracle.select(prob[p:p + 1], cand, DESC, 5, mlp=mlp, want_scores=True)
+        ok, msg = topk_accept(idx[p], sc[p], ref, np.arange(C, dtype=np.int32), 5, 1e-4)
+        assert ok, (p, msg)
