@@ -414,20 +414,24 @@ __global__ void __launch_bounds__(128)
 ridge_problem_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int P,
                      const __grid_constant__ RidgeParams prm, RidgeProblem* __restrict__ out, unsigned* __restrict__ mask) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= P) return;
-  RidgeProblem e;
-  problem_terms(use_value ? p_value : p[i], desc, e.t);
-  e.combo = e.t.dtype_ab * 4 + e.t.dtype_d;
-  float s = prm.bias;
-  problem_columns(e.t, [&](int col, float v) {
-    s += ridge_term(prm, col, v);
-    if (col == 5) s += ridge_level(prm.lut5, v);
-    if (col == 9) s += ridge_level(prm.lut9, v);
-  });
-  e.sum = s;
-  out[i] = e;
-  const unsigned m = __reduce_or_sync(__activemask(), 1u << e.combo);
-  if ((threadIdx.x & 31) == 0) atomicOr(mask, m);
+  unsigned m = 0;
+  if (i < P) {
+    RidgeProblem e;
+    problem_terms(use_value ? p_value : p[i], desc, e.t);
+    e.combo = e.t.dtype_ab * 4 + e.t.dtype_d;
+    float s = prm.bias;
+    problem_columns(e.t, [&](int col, float v) {
+      s += ridge_term(prm, col, v);
+      if (col == 5) s += ridge_level(prm.lut5, v);
+      if (col == 9) s += ridge_level(prm.lut9, v);
+    });
+    e.sum = s;
+    out[i] = e;
+    m = 1u << e.combo;
+  }
+  // (the whole warp: which of its threads run together after the arithmetic above is not given)
+  m = __reduce_or_sync(0xFFFFFFFFu, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicOr(mask, m);
 }
 
 // With classes: a candidate's second word, so far its resident-block count b, becomes the number of
