@@ -492,7 +492,9 @@ select_ridge_kernel(const __grid_constant__ ks_gpu_desc desc, const RidgeProblem
   __shared__ float s_tab[kQ][kClasses ? kRidgeClasses : 1];
   __shared__ ProblemTerms s_pt;  // (without classes, where kQ = 1)
   __shared__ unsigned s_bar[kQ];  // upper word of a key below which nothing can make the list
-  __shared__ unsigned s_best[kQ][2 * kRidgeThreads / 32];  // the warps' best keys (one each, two for k > 16)
+  // The upper words of a warp's best key and (for k > 16) its second best, in one 64-bit word: another warp
+  // sees both from before or both from after an update, so no candidate counts twice in the bar.
+  __shared__ unsigned long long s_best[kQ][kRidgeThreads / 32];
   __shared__ unsigned long long s_list[kRidgeThreads / 32][32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int group = blockIdx.x / map.nblk, chunk = blockIdx.x % map.nblk;
@@ -517,7 +519,7 @@ select_ridge_kernel(const __grid_constant__ ks_gpu_desc desc, const RidgeProblem
   if (!kClasses && tid < static_cast<int>(sizeof(ProblemTerms) / 4))
     reinterpret_cast<uint32_t*>(&s_pt)[tid] = reinterpret_cast<const uint32_t*>(&problems[prob(0)].t)[tid];
   if (tid < kQ) s_bar[tid] = 0u;
-  if (tid < kQ * 2 * kRidgeThreads / 32) (&s_best[0][0])[tid] = 0u;
+  if (tid < kQ * kRidgeThreads / 32) (&s_best[0][0])[tid] = 0ull;
   __syncthreads();
   int64_t lo, len;  // (per-problem segments: kQ = 1)
   segment_of(map, prob(0), lo, len);
@@ -557,15 +559,26 @@ select_ridge_kernel(const __grid_constant__ ks_gpu_desc desc, const RidgeProblem
         // The k-th largest of the warps' best keys bounds the k-th best score from below (each is a
         // candidate of its own), far better than any one warp's k-th.
         constexpr int kWarps = kRidgeThreads / 32;
-        unsigned* best = s_best[q];
-        const int each = k > kWarps ? 2 : 1;
-        if (lane < each) best[warp * 2 + lane] = static_cast<unsigned>(top[q] >> 32);
+        volatile unsigned long long* best = s_best[q];
+        const unsigned mine = static_cast<unsigned>(top[q] >> 32), after = __shfl_sync(0xFFFFFFFFu, mine, 1);
+        if (lane == 0) best[warp] = static_cast<unsigned long long>(mine) << 32 | (k > kWarps ? after : 0u);
         __syncwarp();
-        const unsigned v = (lane & 1) < each ? *const_cast<volatile unsigned*>(&best[lane]) : 0u;
-        int ahead = 0;
+        const unsigned long long pair = lane < kWarps ? best[lane] : 0ull;
+        const unsigned first = static_cast<unsigned>(pair >> 32), second = static_cast<unsigned>(pair);
+        int ahead = 0, ahead2 = 0;  // of the two: keys that are at least as good
 #pragma unroll
-        for (int i = 0; i < 32; ++i) ahead += __shfl_sync(0xFFFFFFFFu, v, i) >= v;
-        const unsigned bar = __reduce_max_sync(0xFFFFFFFFu, ahead >= k ? v : 0u);
+        for (int i = 0; i < kWarps; ++i) ahead += __shfl_sync(0xFFFFFFFFu, first, i) >= first;
+        unsigned bar = ahead >= k ? first : 0u;
+        if (k > kWarps) {
+#pragma unroll
+          for (int i = 0; i < kWarps; ++i) {
+            const unsigned f = __shfl_sync(0xFFFFFFFFu, first, i), s = __shfl_sync(0xFFFFFFFFu, second, i);
+            ahead += s >= first;
+            ahead2 += (f >= second) + (s >= second);
+          }
+          bar = max(ahead >= k ? first : 0u, ahead2 >= k ? second : 0u);
+        }
+        bar = __reduce_max_sync(0xFFFFFFFFu, bar);
         if (lane == 0) atomicMax(&s_bar[q], bar);
       }
     }
