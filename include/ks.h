@@ -402,6 +402,9 @@ ks_status ks_model_describe(const ks_model* model, char* buf, int len);
  * runs out, the kernel sets the status word and returns, and the call reports KS_ERR_TIMEOUT
  * without any fault: the failure path can be tested on a healthy GPU. */
 ks_status ks_debug_set_wait(ks_ctx* ctx, int probe_limit, int starve);
+/* How many calls of this context the walk of whole classes of candidates has served so far (a tree
+ * ensemble on a large batch; the choice falls on the device). Waits for the device; -1 on failure. */
+int64_t ks_debug_class_walks(ks_ctx* ctx);
 /* Measurement aid, no counterpart in the paper: the tree walk of ks_score stripped of everything
  * but its gather and instruction stream, to measure the floor that stream sets for the tree
  * kernel. Tiles are built from the `rows` feature rows (device, [rows][64] floats) exactly as

@@ -106,7 +106,7 @@ ks_status read_status(ks_ctx* ctx) {
   if (v != 0) {
     *ctx->h_status = 0;
     // a failed launch may have left arrival counters of the slice mode behind
-    if (ctx->d_words) cudaMemset(ctx->d_words, 0, sizeof(int) * ks::kContextWords);
+    if (ctx->d_words) cudaMemset(ctx->d_words, 0, sizeof(int) * ks::kWordServed);
     return static_cast<ks_status>(v);
   }
   return KS_OK;
@@ -350,6 +350,16 @@ ks_status ks_debug_set_wait(ks_ctx* ctx, int probe_limit, int starve) {
   ctx->wait.limit = probe_limit;
   ctx->wait.starve = starve != 0;
   return KS_OK;
+}
+
+int64_t ks_debug_class_walks(ks_ctx* ctx) {
+  if (!ctx) return -1;
+  DeviceGuard g(ctx->device);
+  int n = -1;
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e == cudaSuccess) e = cudaMemcpy(&n, ctx->d_words + ks::kWordServed, sizeof(int), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) cuda_fail(ctx, e, "ks_debug_class_walks");
+  return e == cudaSuccess ? n : -1;
 }
 
 int ks_debug_bounds_line(void) {

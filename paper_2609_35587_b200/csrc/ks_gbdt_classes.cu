@@ -193,7 +193,7 @@ __host__ __device__ constexpr int rounds_of(int n, int s) { return (n * s + kSlo
 // 1,024 x 60,000 pairs and 500 trees); a class 900 for every round of problem slots and 3,600 to be
 // compiled (measured on the same batch: 1,712 classes, 1.3 a unit, 8 rounds, 17 ms). The line is put a
 // tenth to the safe side.
-__global__ void choose_path_kernel(int64_t pairs, int* counters) {
+__global__ void choose_path_kernel(int64_t pairs, int* counters, int* served) {
   const int64_t units = counters[0];
   int64_t cost = 0;
   for (int q = 0; q < 16; ++q) {
@@ -201,6 +201,7 @@ __global__ void choose_path_kernel(int64_t pairs, int* counters) {
     if (n > 0) cost += units * 13 / 10 * (static_cast<int64_t>(rounds_of(n, 1)) * 900 + 3600);
   }
   counters[1] = cost + cost / 10 < pairs ? 1 : 0;
+  *served += counters[1];
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1349,7 +1350,7 @@ ClassScratch class_scratch(const GbdtModel& g, int P, int C, void* mem) {
 
 cudaError_t prepare_classes(const ks_gpu_desc& desc, const GbdtModel& g, const ks_problem* d_p, int P,
                             const ks_candidate* d_c, int C, const ClassCall& call, cudaStream_t stream,
-                            int64_t* launches, const int** path) {
+                            int64_t* launches, const FastWait* wait, const int** path) {
   const ClassScratch s = class_scratch(g, P, C, call.scratch);
   *path = s.counters + 1;
   cudaError_t e = cudaMemsetAsync(s.counters, 0, 256, stream);
@@ -1365,7 +1366,7 @@ cudaError_t prepare_classes(const ks_gpu_desc& desc, const GbdtModel& g, const k
     if (e != cudaSuccess) return e;
   }
   problem_rows_kernel<<<P, 64, 0, stream>>>(desc, d_p, P, s.order, s.keys, make_view(g, nullptr), s.prob_tab, s.counters);
-  choose_path_kernel<<<1, 1, 0, stream>>>(call.pairs, s.counters);
+  choose_path_kernel<<<1, 1, 0, stream>>>(call.pairs, s.counters, wait->words + kWordServed);
   *launches += 4;
   return cudaGetLastError();
 }

@@ -1686,7 +1686,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
   if (ev_begin) cudaEventRecord(ev_begin, stream);
   const int* path = nullptr;  // device word: whether the class walk serves the call
   if (classes) {
-    e = prepare_classes(desc, g, d_p, P, d_c, C, *classes, stream, launches, &path);
+    e = prepare_classes(desc, g, d_p, P, d_c, C, *classes, stream, launches, wait, &path);
     if (e != cudaSuccess) return e;
   }
 

@@ -181,7 +181,8 @@ constexpr int kMaxSliceBlocks = 1024;  // candidate blocks the slice mode suppor
 // kernel family that makes the CTAs which start after it was raised leave at once. It is cleared in front
 // of every launch of the family.
 constexpr int kWordWalk = kMaxSliceBlocks + 1, kWordMlp = kWordWalk + 1, kWordWide = kWordMlp + 1;
-constexpr int kContextWords = kWordWide + 1;
+constexpr int kWordServed = kWordWide + 1;  // calls that the walk of whole classes has served (ks_debug_class_walks)
+constexpr int kContextWords = kWordServed + 1;
 constexpr int kLeaveFailed = 1, kLeaveServed = 2;  // a wait ran out; another kernel serves the call
 
 // Levels of the categorical field held by feature column `col` (0: not a level-code column):
@@ -245,7 +246,7 @@ size_t classes_scratch_bytes(const GbdtModel& g, int P, int C);
 // serves the call
 cudaError_t prepare_classes(const ks_gpu_desc& desc, const GbdtModel& g, const ks_problem* d_p, int P,
                             const ks_candidate* d_c, int C, const ClassCall& call, cudaStream_t stream,
-                            int64_t* launches, const int** path);
+                            int64_t* launches, const FastWait* wait, const int** path);
 // the walk and the ranking, which do nothing when the other path serves the call
 cudaError_t launch_classes(const ks_gpu_desc& desc, const GbdtModel& g, int P, const ks_candidate* d_c, int C,
                            const uint8_t* cand_rows, const int64_t* seg_off, const int32_t* seg_idx, int nblk,

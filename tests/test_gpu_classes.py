@@ -2,7 +2,7 @@
 catalogue with many near-duplicates: the depths it compiles (5 to 8), ragged numbers of problems (a round
 serves 128, 64 or 32 of them), one tree, odd tree counts, mixed element types, partition splits, per-problem
 segments (one empty, one of a single candidate), k from 1 to 32, units of more than 64 candidates, and
-duplicate candidates. The batches are ones its dispatch rule takes; a few problems of each are compared
+duplicate candidates. Each test asks which walk served its calls; a few problems of each batch are compared
 with the oracle, first and last among them."""
 import numpy as np
 import pytest
@@ -47,6 +47,13 @@ def check(prob, cand, gbdt, k, idx, sc, which, so=None, si=None):
         assert ok, (p, msg)
 
 
+def served(ctx, call):
+    """The call's answer, and whether the walk of whole classes gave it."""
+    before = ctx.debug_class_walks()
+    answer = call()
+    return answer, ctx.debug_class_walks() - before == 1
+
+
 @pytest.mark.parametrize("P,trees,depth,law,stats,k,partition", [
     (257, 37, 5, "pernode", "cfg1", 10, False), (320, 33, 6, "hist256", "cfg2", 32, True),
     (300, 1, 7, "slots128", "cfg1", 1, False), (513, 24, 8, "pernode", "cfg2", 10, True),
@@ -60,7 +67,8 @@ def test_dense_batches(ks, ctx, P, trees, depth, law, stats, k, partition):
     if partition:
         nodes = wl.with_partition_splits(3, nodes)
     model = ctx.model_create_gbdt(off, nodes, 0.5)
-    idx, sc = ctx.select(dev(ks, prob), P, dev(ks, cand), len(cand), model, k)
+    (idx, sc), classes = served(ctx, lambda: ctx.select(dev(ks, prob), P, dev(ks, cand), len(cand), model, k))
+    assert classes == (P != 96)  # (one round of problems does not pay for compiling units of 48)
     assert ctx.device_status() == ks.KS_OK
     check(prob, cand, (off, nodes, 0.5), k, idx.cpu().numpy(), sc.cpu().numpy(), [0, 1, 5, 39, P // 2, P - 1])
 
@@ -75,7 +83,9 @@ def test_segments(ks, ctx):
     prob = wl.problems_stream(6, P)
     off, nodes = wl.gbdt_complete(8, 20, 8, wl.feature_stats("cfg1"), 0.1)
     model = ctx.model_create_gbdt(off, nodes, 0.0)
-    idx, sc = ctx.select(dev(ks, prob), P, dev(ks, cand), len(cand), model, 10, dev(ks, so), dev(ks, si), int(so[-1]))
+    (idx, sc), classes = served(ctx, lambda: ctx.select(dev(ks, prob), P, dev(ks, cand), len(cand), model, 10,
+                                                        dev(ks, so), dev(ks, si), int(so[-1])))
+    assert classes
     check(prob, cand, (off, nodes, 0.0), 10, idx.cpu().numpy(), sc.cpu().numpy(), [0, 1, 2, 3, 200, P - 1], so, si)
 
 
@@ -97,9 +107,45 @@ def test_large_units_and_duplicates(ks, ctx):
     prob = wl.problems_batch(9, 300)
     off, nodes = wl.gbdt_complete(2, 40, 7, wl.feature_stats("cfg1"), 0.1, "hist256")
     model = ctx.model_create_gbdt(off, nodes, 0.0)
-    idx, sc = ctx.select(dev(ks, prob), 300, dev(ks, cand), len(cand), model, 32)
+    (idx, sc), classes = served(ctx, lambda: ctx.select(dev(ks, prob), 300, dev(ks, cand), len(cand), model, 32))
+    assert classes
     assert ctx.device_status() == ks.KS_OK
     check(prob, cand, (off, nodes, 0.0), 32, idx.cpu().numpy(), sc.cpu().numpy(), [0, 17, 299])
+
+
+def full_units(n):
+    """n groups that agree in the six knobs, of 64 candidates each."""
+    base = pool([64, 128, 192, 256])
+    knobs = ["tile_m", "tile_n", "tile_k", "stages", "cluster_m", "cluster_n"]
+    c = np.zeros((n, 64), wl.CANDIDATE_DT)
+    for name in knobs:
+        c[name] = np.unique(base[knobs])[:n][name][:, None]
+    i = np.arange(64)
+    c["kernel_sched"], c["epi_sched"], c["tile_sched"] = i % 4, i // 4 % 3, i % 2
+    c["instr_m"], c["instr_n"], c["instr_k"] = 64, c["tile_n"] // (1 + i % 2), 8 + i // 4
+    return np.ascontiguousarray(c.reshape(-1)[np.random.default_rng(n).permutation(64 * n)])
+
+
+def test_one_round_of_problems(ks, ctx):
+    """The fewest problems that are served: a single round of the slots."""
+    cand, prob = full_units(80), wl.problems_batch(2, 120, cross_precision=False)
+    off, nodes = wl.gbdt_complete(3, 30, 7, wl.feature_stats("cfg1"), 0.1)
+    model = ctx.model_create_gbdt(off, nodes, 0.0)
+    (idx, sc), classes = served(ctx, lambda: ctx.select(dev(ks, prob), 120, dev(ks, cand), len(cand), model, 10))
+    assert classes
+    check(prob, cand, (off, nodes, 0.0), 10, idx.cpu().numpy(), sc.cpu().numpy(), [0, 1, 31, 32, 64, 119])
+
+
+def test_several_planes_of_scores(ks, ctx):
+    """More problems than a gigabyte of scores holds (4,224 with this pool, then the rest), and than are
+    ordered by counting."""
+    cand, P = wl.candidates_full_grid(1, None), 4300
+    prob = wl.problems_batch(2, P, cross_precision=False)
+    off, nodes = wl.gbdt_complete(3, 6, 5, wl.feature_stats("cfg1"), 0.1)
+    model = ctx.model_create_gbdt(off, nodes, 0.0)
+    (idx, sc), classes = served(ctx, lambda: ctx.select(dev(ks, prob), P, dev(ks, cand), len(cand), model, 10))
+    assert classes
+    check(prob, cand, (off, nodes, 0.0), 10, idx.cpu().numpy(), sc.cpu().numpy(), [0, 4223, 4224, 4290, P - 1])
 
 
 def test_wait_runs_out(ks):
@@ -113,7 +159,7 @@ def test_wait_runs_out(ks):
     ctx.select(*args)
     assert ctx.device_status() == ks.KS_ERR_TIMEOUT
     ctx.debug_set_wait(0, False)
-    idx, sc = ctx.select(*args)
-    assert ctx.device_status() == ks.KS_OK
+    (idx, sc), classes = served(ctx, lambda: ctx.select(*args))
+    assert classes and ctx.device_status() == ks.KS_OK
     check(prob, cand, (off, nodes, 0.0), 10, idx.cpu().numpy(), sc.cpu().numpy(), [0, 319])
     ctx.close()

@@ -1,6 +1,6 @@
 """Batches of tree ensembles against small catalogues, which are ordered by counting (up to 8,192 candidates,
-with many equal keys), and the first size that is sorted; problems past and up to the number that is ordered by
-counting in the walk of whole classes. Scores agree to the tolerance of the other tests of tree ensembles."""
+with many equal keys), and the first size that is sorted, each ranked by the candidates' own walks (the orders as
+the walk of whole classes uses them: test_gpu_classes.py). Scores agree to the tolerance of the other tests of tree ensembles."""
 import numpy as np
 import pytest
 import torch
@@ -24,6 +24,7 @@ def test_small_catalogue(P, C):
     ctx = ks.Context(DESC, 0)
     model = ctx.model_create_gbdt(off, nodes, 0.5)
     idx, sc = ctx.select(ks.to_device(prob, dev), P, ks.to_device(cand, dev), C, model, 10)
+    assert ctx.debug_class_walks() == 0
     idx, sc = idx.cpu().numpy(), sc.cpu().numpy()
     pool = np.arange(C, dtype=np.int32)
     for p in (0, P // 2, P - 1):
