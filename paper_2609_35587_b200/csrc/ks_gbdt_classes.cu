@@ -1004,29 +1004,32 @@ class_walk_kernel(ks_gpu_desc desc, const __grid_constant__ ClassArgs a) {
     __syncthreads();
     unsigned long long todo = unit.y == 64 ? ~0ull : (1ull << unit.y) - 1ull;
     int cap = min(kMembers, (a.n_buckets - 2) * 3 / 4);  // single members take a bucket each when sets have to share
-    for (int seen = 0, lead = 0; lead < unit.y; ++lead) {
-      if (!((todo >> lead) & 1ull)) continue;
-      const int b_eff = sh.b_eff[lead];
-      // the members of this class: for this item, or passed over (a class taken in several pieces
-      // comes by several times and is counted when its last piece is done)
-      unsigned long long all = 0ull;
-      for (int i = lead; i < unit.y; ++i)
-        if (((todo >> i) & 1ull) && sh.b_eff[i] == b_eff) all |= 1ull << i;
-      if (seen != which && !(which == 3 && seen > 3)) {
+    unsigned long long rest = 0ull;  // members of the class at hand that are still to be done
+    for (int nth = 0;;) {
+      // the unit's classes one after the other, whole: this item's, or passed over
+      while (!rest && todo) {
+        const int first_b = sh.b_eff[__ffsll(static_cast<long long>(todo)) - 1];
+        unsigned long long all = 0ull;
+        for (int i = 0; i < unit.y; ++i)
+          if (((todo >> i) & 1ull) && sh.b_eff[i] == first_b) all |= 1ull << i;
         todo &= ~all;
-        ++seen;
-        continue;
+        if (nth == which || (which == 3 && nth > 3)) rest = all;
+        ++nth;
       }
+      if (!rest) break;
+      const int b_eff = sh.b_eff[__ffsll(static_cast<long long>(rest)) - 1];
+      // all of it, or a piece that can be compiled together
       unsigned long long cls = 0ull;
       int m = 0;
-      for (unsigned long long rest = all; rest && m < cap; rest &= rest - 1) {
-        cls |= rest & (0ull - rest);
+      for (unsigned long long left = rest; left && m < cap; left &= left - 1) {
+        cls |= left & (0ull - left);
         ++m;
       }
       __syncthreads();
       if (tid < kMembers && ((cls >> tid) & 1ull)) {
-        sh.member[__popcll(cls & ((1ull << tid) - 1ull))] = sh.cand[tid];
-        if (tid == lead) sh.rep = load_candidate(a.c + sh.cand[tid]);
+        const int at = __popcll(cls & ((1ull << tid) - 1ull));
+        sh.member[at] = sh.cand[tid];
+        if (at == 0) sh.rep = load_candidate(a.c + sh.cand[tid]);
       }
       __syncthreads();
       if (!compile_class(a, sh, build, m, combo, S, ids, prog, reinterpret_cast<uint32_t*>(tile - 2 * kBufBytes))) {
@@ -1036,11 +1039,9 @@ class_walk_kernel(ks_gpu_desc desc, const __grid_constant__ ClassArgs a) {
           return;
         }
         cap = max(1, min(cap, m) / 2);  // fewer members have fewer sets and fewer second sides
-        --lead;
         continue;
       }
-      todo &= ~cls;
-      if (cls == all) ++seen;
+      rest &= ~cls;
       const int n_chunks = sh.n_chunks;
 
       for (int p0 = p_begin; p0 < p_end; p0 += n_slots) {

@@ -136,6 +136,31 @@ def test_one_round_of_problems(ks, ctx):
     check(prob, cand, (off, nodes, 0.0), 10, idx.cpu().numpy(), sc.cpu().numpy(), [0, 1, 31, 32, 64, 119])
 
 
+def test_classes_in_pieces(ks, ctx):
+    """Units of two classes (schedules of another resident-block count) whose members alternate in the order
+    of the catalogue, the larger of them too large to be compiled at once: 62 of 64 candidates, where an
+    ensemble of so many tile rows leaves room for 59."""
+    base = pool([64, 128, 192, 256])
+    knobs = ["tile_m", "tile_n", "tile_k", "stages", "cluster_m", "cluster_n"]
+    groups = np.unique(base[knobs])
+    c = np.zeros((len(groups), 64), wl.CANDIDATE_DT)
+    for name in knobs:
+        c[name] = groups[name][:, None]
+    c["kernel_sched"], c["epi_sched"] = [0] * 31 + [1] * 2 + [3] * 31, 1
+    i = np.arange(64)
+    c["instr_m"], c["instr_n"], c["instr_k"] = 64, c["tile_n"] // (1 + i % 2), 8 + i // 2
+    prob = wl.problems_batch(4, 130)
+    x = oracle.featurize(prob[:1], np.ascontiguousarray(c[:, [0, 31, 33]].reshape(-1)), DESC).reshape(-1, 3, 64)
+    b = np.maximum(1, x[:, :, 55])
+    cand = np.ascontiguousarray(c[(b[:, 0] == b[:, 2]) & (b[:, 0] != b[:, 1])][:70].reshape(-1))
+    assert len(cand) == 70 * 64
+    off, nodes = wl.gbdt_complete(5, 1000, 8, wl.feature_stats("cfg2"), 0.1)
+    model = ctx.model_create_gbdt(off, nodes, 0.0)
+    (idx, sc), classes = served(ctx, lambda: ctx.select(dev(ks, prob), 130, dev(ks, cand), len(cand), model, 32))
+    assert classes
+    check(prob, cand, (off, nodes, 0.0), 32, idx.cpu().numpy(), sc.cpu().numpy(), range(0, 130, 6))
+
+
 def test_several_planes_of_scores(ks, ctx):
     """More problems than a gigabyte of scores holds (4,224 with this pool, then the rest), and than are
     ordered by counting."""
