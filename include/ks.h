@@ -280,8 +280,9 @@ ks_status ks_score(ks_ctx* ctx, const float* d_features, int64_t rows, const ks_
  * device when it happens): partial lists, a per-call table of 16 x C records of at most 256
  * bytes, and, for a tree model on a batch of 32 problems or more, at most 256 MiB for the
  * tables of per-pair tile rows (larger batches are served in several launches that reuse it),
- * and, for 64 problems or more on a catalogue of 4,096 candidates or more, 0.5 MB per tree and
- * at most 1 GiB of scores for the walk of whole classes of candidates;
+ * and, for batches of more than 100 problems on a catalogue of 4,096 to 2,097,152 candidates with an
+ * ensemble of at most 1,024 trees, 0.46 to 1.1 MB per tree (by the size of the largest tree) and at most
+ * 1 GiB of scores for the walk of whole classes of candidates;
  * KS_ERR_OOM if the workspace cannot be had. d_p and d_c must be 16-byte aligned (each record
  * is fetched with one 128-bit load), else KS_ERR_INVALID_ARG. */
 ks_status ks_select(ks_ctx* ctx, const ks_problem* d_p, int P, const ks_candidate* d_c, int C,

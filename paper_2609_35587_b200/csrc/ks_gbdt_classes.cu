@@ -188,6 +188,13 @@ problem_rows_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, int P, c
 // Rounds that n problems take when a round serves kSlots / s of them.
 __host__ __device__ constexpr int rounds_of(int n, int s) { return (n * s + kSlots - 1) / kSlots; }
 
+// The cost of this walk for `n` problems of one element-type combination, in pairs that their own walks
+// take as long for (see choose_path_kernel).
+__host__ __device__ constexpr int64_t walk_cost(int64_t units, int n) {
+  return units * 13 / 10 * (static_cast<int64_t>(rounds_of(n, 1)) * 900 + 3600);
+}
+__host__ __device__ constexpr bool walk_pays(int64_t cost, int64_t pairs) { return cost + cost / 10 < pairs; }
+
 // Chooses between this path and the per-candidate walk, on the device, where the number of units is
 // known. In clocks of one of two CTAs on an SM, a tree: a candidate's own walk takes 1.0 (52.9 ms for
 // 1,024 x 60,000 pairs and 500 trees); a class 900 for every round of problem slots and 3,600 to be
@@ -198,9 +205,9 @@ __global__ void choose_path_kernel(int64_t pairs, int* counters, int* served) {
   int64_t cost = 0;
   for (int q = 0; q < 16; ++q) {
     const int n = counters[9 + q] - counters[8 + q];
-    if (n > 0) cost += units * 13 / 10 * (static_cast<int64_t>(rounds_of(n, 1)) * 900 + 3600);
+    if (n > 0) cost += walk_cost(units, n);
   }
-  counters[1] = cost + cost / 10 < pairs ? 1 : 0;
+  counters[1] = walk_pays(cost, pairs) ? 1 : 0;
   *served += counters[1];
 }
 
@@ -1234,7 +1241,7 @@ size_t program_bytes(const GbdtModel& g) {
 }
 int batch_problems(int P, int C) {
   const int64_t n = static_cast<int64_t>(kPlaneBytes / (4 * static_cast<size_t>(C))) / kSlots * kSlots;
-  return static_cast<int>(n < P ? (n < kSlots ? kSlots : n) : P);
+  return static_cast<int>(std::min<int64_t>(n, P));  // (classes_apply: at least kSlots fit)
 }
 size_t problem_sort_bytes(int P) {
   size_t bytes = 0;
@@ -1297,11 +1304,14 @@ int class_tree_words(int n_trees, const int64_t* off, const ks_node_host* nodes)
   return (most + 31) / 32 * 32;
 }
 
-// Batches this path may serve (whether it does is decided on the device, where the number of classes
-// is known): enough problems to pay for compiling, enough candidates for classes to have members, and
-// a model whose words fit the compiled form.
+// Batches this path may serve (whether it does is decided on the device, where the number of units is
+// known): enough problems to pay for compiling even if every unit were full (more than 100), enough
+// candidates for classes to have members and few enough for a round of problems' scores to fit the plane,
+// and a model whose words fit the compiled form. A batch refused here costs nothing; one refused on the
+// device has paid for its preparation and for the memory.
 bool classes_apply(const GbdtModel& g, int P, int C, int64_t pairs) {
-  if (!g.fast || P < 64 || C < 4096 || pairs / P < 2048 || C > (1 << 24)) return false;
+  if (!g.fast || P < 1 || C < 4096 || pairs / P < 2048 || C > static_cast<int64_t>(kPlaneBytes / (4 * kSlots))) return false;
+  if (!walk_pays(walk_cost((C + kMembers - 1) / kMembers, P), pairs)) return false;
   if (g.fast_depth < 5 || g.fast_depth > 8 || g.n_trees > kMaxTrees || g.fixed_shift == kNoFixed) return false;
   const int rows = g.n_pair_rows + g.n_prob_rows;
   if (rows > 255 || g.n_pair_rows < 1) return false;

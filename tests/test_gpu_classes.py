@@ -173,6 +173,22 @@ def test_several_planes_of_scores(ks, ctx):
     check(prob, cand, (off, nodes, 0.0), 10, idx.cpu().numpy(), sc.cpu().numpy(), [0, 4223, 4224, 4290, P - 1])
 
 
+@pytest.mark.parametrize("P,C,trees,depth,most", [(96, 20000, 500, 8, 200e6), (130, (1 << 21) + 1, 5, 5, 1.3e9)])
+def test_batches_refused_on_the_host(ks, P, C, trees, depth, most):
+    """Too few problems for any pool, and more candidates than a gigabyte holds the scores of 128 problems
+    for: such a batch reserves no memory for this walk (240 MB of programs, 1.07 GB of scores)."""
+    ctx = ks.Context(DESC, 0)
+    cand, prob = np.resize(wl.candidates_full_grid(1, None), C), wl.problems_batch(2, P, cross_precision=False)
+    off, nodes = wl.gbdt_complete(3, trees, depth, wl.feature_stats("cfg1"), 0.1, "hist256")
+    model, d_p, d_c = ctx.model_create_gbdt(off, nodes, 0.0), dev(ks, prob), dev(ks, cand)
+    out = torch.empty((P, 3), dtype=torch.int32, device="cuda"), torch.empty((P, 3), device="cuda")
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    _, classes = served(ctx, lambda: ctx.select(d_p, P, d_c, C, model, 3, out_idx=out[0], out_score=out[1]))
+    assert not classes and free - torch.cuda.mem_get_info()[0] < most
+    ctx.close()
+
+
 def test_wait_runs_out(ks):
     """A chunk wait that the test hook lets run out is reported, and the next call is clean."""
     ctx = ks.Context(DESC, 0)
