@@ -283,7 +283,10 @@ ks_status ks_score(ks_ctx* ctx, const float* d_features, int64_t rows, const ks_
  * and, for batches of more than 100 problems on a catalogue of 4,096 to 2,097,152 candidates with an
  * ensemble of at most 1,024 trees, 0.46 to 1.1 MB per tree (by the size of the largest tree) and at most
  * 1 GiB of scores for the walk of whole classes of candidates;
- * KS_ERR_OOM if the workspace cannot be had. d_p and d_c must be 16-byte aligned (each record
+ * KS_ERR_OOM if the workspace cannot be had. Where only all of it cannot be had, the call does without the
+ * walk of whole classes, or (a ranker with a layer wider than 256 units or more than two hidden layers) ranks
+ * 2,048 rows at a time with at most 19 MB beside the partial lists; so do the context's later calls of that
+ * size and above. d_p and d_c must be 16-byte aligned (each record
  * is fetched with one 128-bit load), else KS_ERR_INVALID_ARG. */
 ks_status ks_select(ks_ctx* ctx, const ks_problem* d_p, int P, const ks_candidate* d_c, int C,
                     const int64_t* d_seg_offsets, const int32_t* d_seg_index, int64_t pairs,
@@ -403,6 +406,9 @@ ks_status ks_model_describe(const ks_model* model, char* buf, int len);
  * runs out, the kernel sets the status word and returns, and the call reports KS_ERR_TIMEOUT
  * without any fault: the failure path can be tested on a healthy GPU. */
 ks_status ks_debug_set_wait(ks_ctx* ctx, int probe_limit, int starve);
+/* Frees the context's workspace (waits for the device); from then on one of more than `bytes` cannot be
+ * had, as if the device had no more memory (0: no limit). */
+ks_status ks_debug_limit_workspace(ks_ctx* ctx, int64_t bytes);
 /* How many calls of this context the walk of whole classes of candidates has served so far (a tree
  * ensemble on a large batch; the choice falls on the device). Waits for the device; -1 on failure. */
 int64_t ks_debug_class_walks(ks_ctx* ctx);

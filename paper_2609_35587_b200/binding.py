@@ -27,7 +27,8 @@ EXPORTS = ("ks_create", "ks_destroy", "ks_last_cuda_error", "ks_model_create_gbd
            "ks_feature_name", "ks_launch_count", "ks_profile_enable", "ks_profile_last_ms", "ks_device_status", "ks_select_trees_static",
            "ks_enumerate", "ks_valid_catalogue", "ks_remap_indices", "ks_model_describe", "ks_merge_topk", "ks_catalogue_prepare", "ks_catalogue_destroy",
            "ks_select_one_prepared",
-           "ks_debug_set_wait", "ks_debug_bounds_line", "ks_debug_bounds_clear", "ks_debug_walk_floor", "ks_debug_class_walks")
+           "ks_debug_set_wait", "ks_debug_bounds_line", "ks_debug_bounds_clear", "ks_debug_walk_floor", "ks_debug_class_walks",
+           "ks_debug_limit_workspace")
 
 
 class KsError(RuntimeError):
@@ -84,6 +85,7 @@ def _load() -> ctypes.CDLL:
     lib.ks_select_one_prepared.argtypes = [vp, vp, _Problem, i32, vp, vp, vp]
     lib.ks_debug_set_wait.argtypes = [vp, i32, i32]
     lib.ks_debug_walk_floor.argtypes = [vp, vp, i64, vp, i32, vp, vp]
+    lib.ks_debug_limit_workspace.argtypes = [vp, i64]
     lib.ks_debug_class_walks.argtypes = [vp]
     lib.ks_debug_class_walks.restype = i64
     lib.ks_debug_bounds_line.restype = i32
@@ -255,6 +257,10 @@ class Context:
     def debug_set_wait(self, probe_limit: int = 0, starve: bool = False):
         """Test hook: probe budget of the kernels' bounded waits, and the starved-wait mode."""
         self._check(_lib.ks_debug_set_wait(self._h, int(probe_limit), int(starve)), "ks_debug_set_wait")
+
+    def debug_limit_workspace(self, n_bytes: int = 0):
+        """Test hook: frees the workspace; one of more than `n_bytes` cannot be had from then on (0: no limit)."""
+        self._check(_lib.ks_debug_limit_workspace(self._h, int(n_bytes)), "ks_debug_limit_workspace")
 
     def debug_class_walks(self) -> int:
         """How many calls the walk of whole classes has served so far (the choice falls on the device)."""

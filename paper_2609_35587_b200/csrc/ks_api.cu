@@ -50,14 +50,39 @@ ks_status ensure_workspace(ks_ctx* ctx, size_t bytes) {
     ctx->ws_bytes = 0;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFree(workspace)");
   }
-  const size_t want = bytes + (bytes < (size_t(128) << 20) ? bytes / 2 : size_t(64) << 20) + (1u << 20);
-  cudaError_t e = cudaMalloc(&ctx->ws, want);
+  size_t want = bytes + (bytes < (size_t(128) << 20) ? bytes / 2 : size_t(64) << 20) + (1u << 20);
+  cudaError_t e = cudaErrorMemoryAllocation;
+  for (int room = 1; room >= 0 && e == cudaErrorMemoryAllocation; --room) {  // with room to grow, else without
+    if (!room) want = bytes;
+    ctx->ws = nullptr;
+    if (want <= ctx->ws_limit) e = cudaMalloc(&ctx->ws, want);
+    if (e != cudaSuccess) cudaGetLastError();
+  }
   if (e != cudaSuccess) {
     ctx->ws = nullptr;
     return cuda_fail(ctx, e, "cudaMalloc(workspace)");
   }
   ctx->ws_bytes = want;
   return KS_OK;
+}
+
+// The workspace of a call whose size is bytes(lean): what it takes with little of it where all cannot be
+// had (ctx->wait.lean tells the launches). A size once refused is not asked for again.
+template <typename Bytes>
+ks_status size_workspace(ks_ctx* ctx, Bytes bytes) {
+  const size_t all = bytes(false);
+  ctx->wait.lean = 0;
+  if (all <= ctx->ws_bytes) return KS_OK;
+  const size_t less = bytes(true);
+  if (less == all) return ensure_workspace(ctx, all);
+  if (all < ctx->ws_refused) {
+    const ks_status s = ensure_workspace(ctx, all);
+    if (s != KS_ERR_OOM) return s;
+    ctx->ws_refused = all;
+    ctx->err[0] = '\0';
+  }
+  ctx->wait.lean = 1;
+  return ensure_workspace(ctx, less);
 }
 
 }  // namespace
@@ -352,6 +377,17 @@ ks_status ks_debug_set_wait(ks_ctx* ctx, int probe_limit, int starve) {
   return KS_OK;
 }
 
+ks_status ks_debug_limit_workspace(ks_ctx* ctx, int64_t bytes) {
+  if (!ctx || bytes < 0) return KS_ERR_INVALID_ARG;
+  DeviceGuard g(ctx->device);
+  cudaError_t e = cudaFree(ctx->ws);  // (synchronises)
+  ctx->ws = nullptr;
+  ctx->ws_bytes = 0;
+  ctx->ws_refused = SIZE_MAX;
+  ctx->ws_limit = bytes > 0 ? static_cast<size_t>(bytes) : SIZE_MAX;
+  return e == cudaSuccess ? KS_OK : cuda_fail(ctx, e, "ks_debug_limit_workspace");
+}
+
 int64_t ks_debug_class_walks(ks_ctx* ctx) {
   if (!ctx) return -1;
   DeviceGuard g(ctx->device);
@@ -573,7 +609,7 @@ ks_status ks_score(ks_ctx* ctx, const float* d_features, int64_t rows, const ks_
     return e == cudaSuccess ? KS_OK : cuda_fail(ctx, e, "ks_score");
   }
   if (model->kind == 1 && model->mlp.wide) {
-    ks_status s = ensure_workspace(ctx, ks::score_wide_scratch_bytes(model->mlp, rows));
+    ks_status s = size_workspace(ctx, [&](bool lean) { return ks::score_wide_scratch_bytes(model->mlp, rows, lean); });
     if (s != KS_OK) return s;
     cudaError_t e = ks::launch_score_wide(model->mlp, d_features, rows, d_scores, ctx->ws, ctx->d_status,
                                           static_cast<cudaStream_t>(stream), &ctx->launches, &ctx->wait);
@@ -599,7 +635,9 @@ ks_status ks_select(ks_ctx* ctx, const ks_problem* d_p, int P, const ks_candidat
   if (!d_p || !d_topk_idx || !d_topk_score || (pairs > 0 && !d_c)) return KS_ERR_INVALID_ARG;
   if (!aligned16(d_p) || !aligned16(d_c)) return KS_ERR_INVALID_ARG;
   DeviceGuard g(ctx->device);
-  s = ensure_workspace(ctx, ks::select_partial_bytes(*model, P, C, pairs, d_seg_offsets != nullptr, k));
+  s = size_workspace(ctx, [&](bool lean) {
+    return ks::select_partial_bytes(*model, P, C, pairs, d_seg_offsets != nullptr, k, lean);
+  });
   if (s != KS_OK) return s;
   cudaError_t e = ks::launch_select(ctx->desc, *model, d_p, nullptr, P, d_c, C, d_seg_offsets,
                                     d_seg_index, pairs, k, ctx->ws, d_topk_idx, d_topk_score,
@@ -669,8 +707,9 @@ ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int 
 
   // every other model: the general path with one problem; its merge kernel writes the k results
   // straight into the mapped host block, so there is no copy between the kernel and the caller
-  const size_t part = align_up(ks::select_partial_bytes(*model, 1, C, C, false, k));
-  ks_status s = ensure_workspace(ctx, part);
+  ks_status s = size_workspace(ctx, [&](bool lean) {
+    return align_up(ks::select_partial_bytes(*model, 1, C, C, false, k, lean));
+  });
   if (s != KS_OK) return s;
   cudaError_t e = ks::launch_select(ctx->desc, *model, nullptr, &p, 1, d_c, C, nullptr, nullptr, C, k,
                                     ctx->ws, ctx->d_pinned_idx, ctx->d_pinned_score, st, &ctx->launches,
@@ -794,14 +833,14 @@ ks_status ks_select_host(ks_ctx* ctx, const ks_problem* h_p, int P, const ks_can
   if (seg && (h_seg_offsets[0] != 0 || h_seg_offsets[P] != pairs)) return KS_ERR_INVALID_ARG;
   DeviceGuard g(ctx->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const size_t b_part = align_up(ks::select_partial_bytes(*model, P, C, pairs, seg, k));
   const size_t b_p = align_up(sizeof(ks_problem) * P), b_c = align_up(sizeof(ks_candidate) * C);
   const size_t b_so = seg ? align_up(sizeof(int64_t) * (P + 1)) : 0;
   const size_t b_si = seg ? align_up(sizeof(int32_t) * pairs) : 0;
   const size_t b_oi = align_up(sizeof(int32_t) * P * k), b_os = align_up(sizeof(float) * P * k);
-  s = ensure_workspace(ctx, b_part + b_p + b_c + b_so + b_si + b_oi + b_os);
+  const auto part = [&](bool lean) { return align_up(ks::select_partial_bytes(*model, P, C, pairs, seg, k, lean)); };
+  s = size_workspace(ctx, [&](bool lean) { return part(lean) + b_p + b_c + b_so + b_si + b_oi + b_os; });
   if (s != KS_OK) return s;
-  char* q = static_cast<char*>(ctx->ws) + b_part;
+  char* q = static_cast<char*>(ctx->ws) + part(ctx->wait.lean);
   ks_problem* d_p = reinterpret_cast<ks_problem*>(q); q += b_p;
   ks_candidate* d_c = reinterpret_cast<ks_candidate*>(q); q += b_c;
   int64_t* d_so = seg ? reinterpret_cast<int64_t*>(q) : nullptr; q += b_so;

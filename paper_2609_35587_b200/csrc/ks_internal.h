@@ -62,11 +62,12 @@ struct FeatQ {
 
 // What a launch takes from its context: the probe budget of the kernels' bounded waits (0: the
 // default), the test hook that starves a wait (the barrier is armed for more bytes than its copy
-// brings), and the context's device words (kWord...). The words belong to the context and not to the
+// brings), whether it has to do with little workspace, and the context's device words (kWord...). The words belong to the context and not to the
 // process: another context's kernels may run at the same time.
 struct FastWait {
   int limit;
   int starve;
+  int lean;  // the memory for all of the workspace could not be had: without the walk of whole classes, few rows at a time
   int* words;
 };
 
@@ -136,7 +137,9 @@ struct ks_ctx {
   int* d_status = nullptr;  // bounded waits give up; d_status is its device alias
   int64_t launches = 0;
   int select_one_seq = 0;  // sequence number of the last single-problem call
-  ks::FastWait wait{0, 0, nullptr};  // probe budget of bounded device waits (0: default), starve hook (tests), d_words
+  ks::FastWait wait{0, 0, 0, nullptr};  // probe budget of bounded device waits (0: default), starve hook (tests), lean, d_words
+  size_t ws_refused = SIZE_MAX;  // the smallest workspace that could not be had
+  size_t ws_limit = SIZE_MAX;    // test hook: larger ones cannot be had
   char err[256] = {0};
   // optional timing of the dominant kernel of the last ks_select* call (ks_profile_enable)
   bool profile = false;
@@ -323,13 +326,13 @@ cudaError_t build_wide_mlp(MlpModel& m, const uint16_t* const* h_w, const float*
                            const float* h_sigma);
 void free_wide_mlp(MlpModel& m);
 int wide_rank_blocks(int64_t per_problem);
-size_t wide_scratch_bytes(const MlpModel& m, int P, int64_t pairs);
+size_t wide_scratch_bytes(const MlpModel& m, int P, int64_t pairs, bool lean);
 cudaError_t launch_select_wide(const ks_gpu_desc& desc, const MlpModel& m, const ks_problem* d_p,
                                const ks_problem* p_by_value, int P, const ks_candidate* d_c, int C, int nblk,
                                const int64_t* seg_off, const int32_t* seg_idx, int64_t pairs, int k,
                                unsigned long long* partial, void* scratch, int* status, cudaStream_t stream,
                                int64_t* launches, cudaEvent_t ev_begin, const FastWait* wait);
-size_t score_wide_scratch_bytes(const MlpModel& m, int64_t rows);
+size_t score_wide_scratch_bytes(const MlpModel& m, int64_t rows, bool lean);
 cudaError_t launch_score_wide(const MlpModel& m, const float* d_feat, int64_t rows, float* d_scores, void* scratch,
                               int* status, cudaStream_t stream, int64_t* launches, const FastWait* wait);
 
@@ -353,7 +356,7 @@ cudaError_t launch_score_linear(const MlpModel& m, const float* d_feat, int64_t 
 // Fused featurize + score + top-k. `p_by_value` non-null selects the single-problem form.
 // d_partial: workspace for the per-block partial lists and per-call tables, at least
 // select_partial_bytes().
-size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, bool segmented, int k);
+size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, bool segmented, int k, bool lean);
 cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const ks_problem* d_p,
                           const ks_problem* p_by_value, int P, const ks_candidate* d_c, int C,
                           const int64_t* d_seg_off, const int32_t* d_seg_idx, int64_t pairs, int k,

@@ -856,7 +856,7 @@ static int64_t per_problem_rows(int P, int C, int64_t pairs, bool segmented) {
   return segmented ? (P > 0 ? (pairs + P - 1) / P : 0) : C;
 }
 
-size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, bool segmented, int k) {
+size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, bool segmented, int k, bool lean) {
   const int64_t per = per_problem_rows(P, C, pairs, segmented);
   if (model.kind == 0 && model.gbdt.fast) {
     int nblk, rows;
@@ -870,7 +870,7 @@ size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, 
     }
     const size_t memo = (fast_memo_bytes(model.gbdt, P, C) + 255) / 256 * 256;
     // a dense batch is ranked in similarity order of the catalogue (ks_order.cu)
-    const bool classes = memo > 0 && classes_apply(model.gbdt, P, C, pairs);
+    const bool classes = memo > 0 && !lean && classes_apply(model.gbdt, P, C, pairs);
     const size_t order = (memo > 0 && P >= kOrderMinProblems && (!segmented || classes))
                              ? (order_scratch_bytes(C) + 255) / 256 * 256 : 0;
     return part + (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256 + memo + order +
@@ -883,7 +883,7 @@ size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, 
   }
   if (model.kind == 1 && model.mlp.wide) {
     const size_t part = static_cast<size_t>(P) * wide_rank_blocks(per) * k * sizeof(unsigned long long);
-    return (part + 255) / 256 * 256 + wide_scratch_bytes(model.mlp, P, pairs);
+    return (part + 255) / 256 * 256 + wide_scratch_bytes(model.mlp, P, pairs, lean);
   }
   if (model.kind == 1 && model.mlp.h_ridge) {
     const size_t part = static_cast<size_t>(P) * ridge_blocks(P, C, per, segmented) * k * sizeof(unsigned long long);
@@ -928,7 +928,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     // then take similar paths through the trees); the order sits behind the memo
     const int32_t* perm = nullptr;
     ClassCall classes{pairs, nullptr, nullptr};
-    const bool use_classes = memo_mem && classes_apply(model.gbdt, P, C, pairs);
+    const bool use_classes = memo_mem && !wait->lean && classes_apply(model.gbdt, P, C, pairs);
     if (memo_mem && P >= kOrderMinProblems && C > 0 && (!d_seg_off || use_classes)) {
       char* order_mem = static_cast<char*>(memo_mem) + (fast_memo_bytes(model.gbdt, P, C) + 255) / 256 * 256;
       cudaError_t eo = launch_catalogue_order(d_c, C, order_mem, stream, launches);

@@ -72,6 +72,10 @@ constexpr int kSmemWide = 1024 + kStages * kStageBytes + kMaxBiasBytes;
 constexpr int kPairs = 74;                         // CTA pairs the machine holds (148 SMs)
 constexpr int64_t kBatchRows = int64_t{55} * kPairs * kRowsPair;  // rows per launch: whole rounds of all pairs (1.04 M)
 constexpr int64_t kScorePairs = 64 * kBatchRows;  // scores held at a time (267 MB)
+// ... where the memory for that cannot be had (at most 19 MB in all)
+constexpr int64_t kLeanRows = 8 * kRowsPair, kLeanScorePairs = 512 * kLeanRows;
+constexpr int64_t batch_rows(bool lean) { return lean ? kLeanRows : kBatchRows; }
+constexpr int64_t score_pairs(bool lean) { return lean ? kLeanScorePairs : kScorePairs; }
 constexpr int kTileN = 256;
 
 // Parts that the K blocks of a layer are summed in. The tensor core adds to its fp32 accumulator by
@@ -772,9 +776,9 @@ int wide_rank_blocks(int64_t per_problem) {
 }
 
 // problem terms | scores of a round's pairs | operand image of a batch | activations
-size_t wide_scratch_bytes(const MlpModel& m, int P, int64_t pairs) {
-  const int64_t batch = std::min(pairs, kBatchRows);
-  return up(sizeof(ProblemTerms) * static_cast<size_t>(P > 0 ? P : 1)) + up(sizeof(float) * static_cast<size_t>(std::min(pairs, kScorePairs))) +
+size_t wide_scratch_bytes(const MlpModel& m, int P, int64_t pairs, bool lean) {
+  const int64_t batch = std::min(pairs, batch_rows(lean));
+  return up(sizeof(ProblemTerms) * static_cast<size_t>(P > 0 ? P : 1)) + up(sizeof(float) * static_cast<size_t>(std::min(pairs, score_pairs(lean)))) +
          up(image_bytes(*m.wide, batch)) + static_cast<size_t>(act_rows(*m.wide, batch)) * 128 + 1024;
 }
 
@@ -784,13 +788,14 @@ cudaError_t launch_select_wide(const ks_gpu_desc& desc, const MlpModel& m, const
                                unsigned long long* partial, void* scratch, int* status, cudaStream_t stream,
                                int64_t* launches, cudaEvent_t ev_begin, const FastWait* wait) {
   const WideMlp& w = *m.wide;
+  const int64_t batch = batch_rows(wait->lean), round = score_pairs(wait->lean);
   char* q = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(scratch) + 1023) / 1024 * 1024);
   ProblemTerms* terms = reinterpret_cast<ProblemTerms*>(q);
   q += up(sizeof(ProblemTerms) * static_cast<size_t>(P));
   float* scores = reinterpret_cast<float*>(q);
-  q += up(sizeof(float) * static_cast<size_t>(std::min(pairs, kScorePairs)));
+  q += up(sizeof(float) * static_cast<size_t>(std::min(pairs, round)));
   uint8_t* image = reinterpret_cast<uint8_t*>(q);
-  q += up(image_bytes(w, std::min(pairs, kBatchRows)));
+  q += up(image_bytes(w, std::min(pairs, batch)));
   uint8_t* act = reinterpret_cast<uint8_t*>(q);
   ks_problem pv{};
   if (p_by_value) pv = *p_by_value;
@@ -798,10 +803,10 @@ cudaError_t launch_select_wide(const ks_gpu_desc& desc, const MlpModel& m, const
   ++*launches;
   if (ev_begin) cudaEventRecord(ev_begin, stream);
   int64_t first = 0;
-  do {  // a round: the scores of kScorePairs pairs, then their ranking
-    const int64_t round0 = first, round_end = std::min(pairs, round0 + kScorePairs);
-    for (; first < round_end; first += kBatchRows) {
-      const int64_t n = std::min(round_end - first, kBatchRows), padded = (n + kRowsPair - 1) / kRowsPair * kRowsPair;
+  do {  // a round: the scores of so many pairs, then their ranking
+    const int64_t round0 = first, round_end = std::min(pairs, round0 + round);
+    for (; first < round_end; first += batch) {
+      const int64_t n = std::min(round_end - first, batch), padded = (n + kRowsPair - 1) / kRowsPair * kRowsPair;
       const unsigned grid = static_cast<unsigned>((padded + 127) / 128);
       if (w.input.onehot)
         wide_pair_rows_kernel<true><<<grid, 128, 0, stream>>>(desc, terms, P, d_c, C, seg_off, seg_idx, first, n, padded,
@@ -821,18 +826,19 @@ cudaError_t launch_select_wide(const ks_gpu_desc& desc, const MlpModel& m, const
   return cudaGetLastError();
 }
 
-size_t score_wide_scratch_bytes(const MlpModel& m, int64_t rows) {
-  const int64_t batch = std::min(rows, kBatchRows);
+size_t score_wide_scratch_bytes(const MlpModel& m, int64_t rows, bool lean) {
+  const int64_t batch = std::min(rows, batch_rows(lean));
   return up(image_bytes(*m.wide, batch)) + static_cast<size_t>(act_rows(*m.wide, batch)) * 128 + 1024;
 }
 
 cudaError_t launch_score_wide(const MlpModel& m, const float* d_feat, int64_t rows, float* d_scores, void* scratch,
                               int* status, cudaStream_t stream, int64_t* launches, const FastWait* wait) {
   const WideMlp& w = *m.wide;
+  const int64_t batch = batch_rows(wait->lean);
   uint8_t* image = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(scratch) + 1023) / 1024 * 1024);
-  uint8_t* act = image + up(image_bytes(w, std::min(rows, kBatchRows)));
-  for (int64_t first = 0; first < rows; first += kBatchRows) {
-    const int64_t n = std::min(rows - first, kBatchRows), padded = (n + kRowsPair - 1) / kRowsPair * kRowsPair;
+  uint8_t* act = image + up(image_bytes(w, std::min(rows, batch)));
+  for (int64_t first = 0; first < rows; first += batch) {
+    const int64_t n = std::min(rows - first, batch), padded = (n + kRowsPair - 1) / kRowsPair * kRowsPair;
     const unsigned grid = static_cast<unsigned>((padded + 127) / 128);
     const float* x = d_feat + first * KS_F_PAD;
     if (w.input.onehot) wide_given_rows_kernel<true><<<grid, 128, 0, stream>>>(x, n, padded, w.input, image, wait->words + kWordWide);
