@@ -321,6 +321,10 @@ __device__ __forceinline__ void tile_column(const FeatQ& q, float4 x, uint32_t t
 // 64 x 2,048 candidates, 100 trees: 161 -> 120, with the memo in its place 143; four calls of one problem with
 // its 61,140 valid candidates: 900 -> 677).
 constexpr int kTileRows = 128, kTileCols = kPairCols + kCandCols;
+// Thresholds that fit beside 64 columns of a block's rows and the static part (49,152). The walk's own tile
+// geometries hold 376 rows of 127 at most, 47,752.
+constexpr int kTileMaxThr = (227 * 1024 - 3072) / 4 - 64 * kTileRows;
+static_assert(kTileMaxThr >= 376 * kSlice, "every ensemble of the regular geometries");
 
 __global__ void __launch_bounds__(256, 3)
 tile_pairs_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int P,
@@ -1068,7 +1072,8 @@ static std::vector<PartitionCode> partition_codes(int L) {
 // 256 candidates measured slower than one CTA of 512 x 512; two CTAs of 128 x 512 and one CTA of
 // 256 x 1,024 have too few warps). More rows than 376: the general kernel.
 // KS_FAST_GEOMETRY="threads,candidates,buffer KiB" overrides the choice (a tuning aid; a geometry
-// that does not fit is refused).
+// that does not fit is refused). With buffers of 8 KB more rows fit than the kernels that build tiles
+// in front of the walk can stage thresholds for (kTileMaxThr): such an ensemble takes the general kernel.
 struct Geometry {
   int threads, cands, buf_bytes, ctas_per_sm;
 };
@@ -1163,6 +1168,7 @@ cudaError_t build_fast_gbdt(GbdtModel& m, int n_trees, const int64_t* off, const
   }
   Geometry geom{};
   if (n_rows == 0 || !pick_geometry(n_rows, &geom)) return cudaSuccess;  // generic path
+  if (thr_class[0] + thr_class[1] + thr_class[2] > kTileMaxThr) return cudaSuccess;
   if (n_class[0] > kFastMaxProbRows || n_class[1] > kFastMaxCandRec) return cudaSuccess;
   const int NC = geom.cands, threads = geom.threads;
   // rows and thresholds ordered: per-pair, candidate-only, problem-only features
@@ -1752,7 +1758,7 @@ cudaError_t launch_score_fast(const ks_gpu_desc& desc, const GbdtModel& g, const
   a.stream = stream;
   a.fv = make_view(g, wait);
   uint8_t* tiles = static_cast<uint8_t*>(scratch);
-  // (376 rows of 127 thresholds, the most that any geometry holds, take 187 KB)
+  // (at most kTileMaxThr thresholds, 192 KB)
   const size_t smem = sizeof(float) * (64 * kTileRows + g.n_qthr);
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(&tile_rows_kernel), smem);
   if (e != cudaSuccess) return e;

@@ -36,3 +36,30 @@ def test_rows(trees, rows):
     ref = oracle.score_gbdt(x, off, nodes, base)
     assert np.all(np.abs(got - ref) <= 1e-5 * np.maximum(1, np.abs(ref)))
     ctx.close()
+
+
+def test_more_thresholds_than_are_staged(monkeypatch):
+    """Small chunk buffers leave room for 408 rows of 127 thresholds, more than the kernel that builds tiles
+    from rows can hold: such an ensemble (here 400 rows, 50,800 thresholds) takes the general kernel."""
+    from paper_2609_35587_b200 import binding as ks
+    monkeypatch.setenv("KS_FAST_GEOMETRY", "512,512,8")
+    device = torch.device("cuda", 0)
+    prob, cand, _, _ = wl.make_inputs(2, P=2, seg=1)
+    x = oracle.featurize(prob, cand[:300], DESC)
+    off, nodes = wl.gbdt_complete(3, 200, 8, wl.feature_stats("cfg2"), 0.1)
+    nodes = nodes.copy()
+    rng = np.random.default_rng(5)
+    per = np.where(np.arange(63) < 41, 6 * 127, 7 * 127)
+    feat = np.repeat(np.arange(63), per)
+    lo, hi = x[:, :63].min(0), x[:, :63].max(0)
+    thr = np.concatenate([np.linspace(lo[f], hi[f] + 1, n, dtype=np.float64) for f, n in enumerate(per)]).astype(np.float32)
+    split = np.flatnonzero(nodes["feat"] != 0xFFFF)
+    order = rng.permutation(len(split)) % len(feat)
+    nodes["feat"][split], nodes["v"][split] = feat[order], thr[order]
+    ctx = ks.Context(DESC, 0)
+    model = ctx.model_create_gbdt(off, nodes, 0.0)
+    assert "select_generic_kernel" in model.describe()
+    got = ctx.score(ks.to_device(x, device), model).cpu().numpy()
+    ref = oracle.score_gbdt(x, off, nodes, 0.0)
+    assert np.all(np.abs(got - ref) <= 1e-5 * np.maximum(1, np.abs(ref)))
+    ctx.close()
