@@ -196,9 +196,10 @@ __device__ __forceinline__ void tmem_wait(uint32_t (&r)[32]) {
                :
                : "memory");
 }
+// ReLU of both, rounded to bf16; of what is not a number 0 (x > 0 is false; cvt's own .relu keeps it)
 __device__ __forceinline__ uint32_t bf16_relu2(float lo, float hi) {
   uint32_t d;
-  asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+  asm("{\n .reg .b32 t;\n cvt.rn.bf16x2.f32 t, %1, %2;\n max.bf16x2 %0, t, %3;\n}\n" : "=r"(d) : "f"(hi), "f"(lo), "r"(0));
   return d;
 }
 

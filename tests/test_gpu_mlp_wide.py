@@ -146,3 +146,19 @@ def test_sums_as_exact_as_in_sequence(ks, ctx, hidden):
         ref = h64[:, 0]
         wrong += torch.stack([((s - ref) ** 2).sum() / (ref ** 2).sum() for s in (got, h32[:, 0].double())]).cpu()
     assert wrong[0].sqrt() <= 1.2 * wrong[1].sqrt(), wrong.sqrt()
+
+
+@pytest.mark.parametrize("hidden", [[320, 64], [64, 64, 64]])
+def test_infinite_sums(ks, ctx, hidden):
+    """Two units of the first layer are infinite; a unit of the second takes their difference, the others
+    less than their sum. ReLU gives 0 for what is not a number and for minus infinity, as in the oracle."""
+    mlp = make(False, hidden, 3)
+    mlp["biases"][0][:2] = np.inf
+    mlp["weights"][1][:, :2] = 0xBF80  # -1
+    mlp["weights"][1][0, 0] = 0x3F80   # +1
+    prob, cand, _, _ = wl.make_inputs(2, P=1, seg=1)
+    x = oracle.featurize(prob, cand[:200], DESC)
+    ref = oracle.score_mlp(x, mlp)
+    assert np.all(np.isfinite(ref))
+    got = ctx.score(dev(ks, x), ctx.model_create_mlp(mlp)).cpu().numpy()
+    assert np.all(np.abs(got - ref) <= TOL * np.maximum(1, np.abs(ref)))
