@@ -4,6 +4,7 @@
 #include <mutex>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <new>
 #include <vector>
 
@@ -197,6 +198,12 @@ void free_model(ks_model* m) {
   ks::free_ridge(m->mlp);
   delete m;
 }
+
+// Frees a model that is not handed out, also when the host runs out of memory on the way.
+struct ModelOwner {
+  ks_model* m = nullptr;
+  ~ModelOwner() { free_model(m); }
+};
 
 ks_status check_pairs(int P, int C, const void* seg_off, const void* seg_idx, int64_t pairs) {
   if (P < 0 || C < 0 || pairs < 0) return KS_ERR_INVALID_ARG;
@@ -417,44 +424,47 @@ ks_status ks_model_create_gbdt(ks_ctx* ctx, int n_trees, const int64_t* h_tree_o
   if (h_tree_offsets[0] != 0) return KS_ERR_INVALID_ARG;
   const int64_t total = h_tree_offsets[n_trees];
   if (total < 0 || total > (1ll << 31) - 1) return KS_ERR_INVALID_ARG;
-  int max_depth = 0;
-  for (int t = 0; t < n_trees; ++t) {
-    const int64_t lo = h_tree_offsets[t], hi = h_tree_offsets[t + 1];
-    if (hi <= lo) return KS_ERR_INVALID_ARG;
-    const int d = validate_tree(h_nodes + lo, hi - lo);
-    if (d < 0) return KS_ERR_INVALID_ARG;
-    if (d > max_depth) max_depth = d;
-  }
-  std::vector<ks::DevNode> dev(static_cast<size_t>(total));
-  for (int64_t i = 0; i < total; ++i) {
-    dev[i].v = h_nodes[i].thr_or_leaf;
-    dev[i].feat = h_nodes[i].kind == KS_NODE_PARTITION ? static_cast<uint16_t>(h_nodes[i].feat | 0x8000u)
-                                                       : h_nodes[i].feat;
-    dev[i].left = h_nodes[i].feat == 0xFFFF ? 0 : static_cast<uint16_t>(h_nodes[i].left);
-  }
-  std::vector<int> roots(n_trees + 1);
-  for (int t = 0; t <= n_trees; ++t) roots[t] = static_cast<int>(h_tree_offsets[t]);
+  ModelOwner own;
+  try {
+    int max_depth = 0;
+    for (int t = 0; t < n_trees; ++t) {
+      const int64_t lo = h_tree_offsets[t], hi = h_tree_offsets[t + 1];
+      if (hi <= lo) return KS_ERR_INVALID_ARG;
+      const int d = validate_tree(h_nodes + lo, hi - lo);
+      if (d < 0) return KS_ERR_INVALID_ARG;
+      if (d > max_depth) max_depth = d;
+    }
+    std::vector<ks::DevNode> dev(static_cast<size_t>(total));
+    for (int64_t i = 0; i < total; ++i) {
+      dev[i].v = h_nodes[i].thr_or_leaf;
+      dev[i].feat = h_nodes[i].kind == KS_NODE_PARTITION ? static_cast<uint16_t>(h_nodes[i].feat | 0x8000u)
+                                                         : h_nodes[i].feat;
+      dev[i].left = h_nodes[i].feat == 0xFFFF ? 0 : static_cast<uint16_t>(h_nodes[i].left);
+    }
+    std::vector<int> roots(n_trees + 1);
+    for (int t = 0; t <= n_trees; ++t) roots[t] = static_cast<int>(h_tree_offsets[t]);
 
-  DeviceGuard g(ctx->device);
-  ks_model* m = new (std::nothrow) ks_model();
-  if (!m) return KS_ERR_OOM;
-  m->ctx = ctx;
-  m->device = ctx->device;
-  m->kind = 0;
-  m->gbdt.n_trees = n_trees;
-  m->gbdt.max_depth = max_depth;
-  m->gbdt.n_nodes = total;
-  m->gbdt.base = base_score;
-  cudaError_t e = upload(&m->gbdt.d_nodes, dev.data(), dev.size());
-  if (e == cudaSuccess) e = upload(&m->gbdt.d_roots, roots.data(), roots.size());
-  if (e == cudaSuccess) e = ks::build_fast_gbdt(m->gbdt, n_trees, h_tree_offsets, h_nodes);
-  if (e != cudaSuccess) {
-    ks_status s = cuda_fail(ctx, e, "ks_model_create_gbdt");
-    free_model(m);
-    return s;
+    DeviceGuard g(ctx->device);
+    ks_model* m = new (std::nothrow) ks_model();
+    if (!m) return KS_ERR_OOM;
+    own.m = m;
+    m->ctx = ctx;
+    m->device = ctx->device;
+    m->kind = 0;
+    m->gbdt.n_trees = n_trees;
+    m->gbdt.max_depth = max_depth;
+    m->gbdt.n_nodes = total;
+    m->gbdt.base = base_score;
+    cudaError_t e = upload(&m->gbdt.d_nodes, dev.data(), dev.size());
+    if (e == cudaSuccess) e = upload(&m->gbdt.d_roots, roots.data(), roots.size());
+    if (e == cudaSuccess) e = ks::build_fast_gbdt(m->gbdt, n_trees, h_tree_offsets, h_nodes);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "ks_model_create_gbdt");
+    *out_model = m;
+    own.m = nullptr;
+    return KS_OK;
+  } catch (const std::exception&) {  // (the vectors of the repacking)
+    return KS_ERR_OOM;
   }
-  *out_model = m;
-  return KS_OK;
 }
 
 ks_status ks_model_create_mlp(ks_ctx* ctx, int n_layers, const int* h_widths,
@@ -474,25 +484,28 @@ ks_status ks_model_create_mlp(ks_ctx* ctx, int n_layers, const int* h_widths,
   for (int j = 0; j < in0; ++j)
     if (!std::isfinite(h_mu[j]) || !std::isfinite(h_sigma[j]) || h_sigma[j] == 0.0f) return KS_ERR_INVALID_ARG;
 
-  DeviceGuard g(ctx->device);
-  ks_model* m = new (std::nothrow) ks_model();
-  if (!m) return KS_ERR_OOM;
-  m->ctx = ctx;
-  m->device = ctx->device;
-  m->kind = 1;
-  m->mlp.n_layers = n_layers;
-  for (int l = 0; l <= n_layers; ++l) m->mlp.widths[l] = h_widths[l];
-  cudaError_t e = ks::build_fast_mlp(m->mlp, h_w_bf16, h_bias, h_mu, h_sigma);
-  // the resident-weights kernel scores given rows in the ordinal input form only
-  if (e == cudaSuccess && !ks::score_mlp_tc_ok(m->mlp)) e = ks::build_wide_mlp(m->mlp, h_w_bf16, h_bias, h_mu, h_sigma);
-  if (e == cudaSuccess) e = ks::build_ridge(m->mlp, h_w_bf16[0], h_bias[0], h_mu, h_sigma);
-  if (e != cudaSuccess) {
-    ks_status s = cuda_fail(ctx, e, "ks_model_create_mlp");
-    free_model(m);
-    return s;
+  ModelOwner own;
+  try {
+    DeviceGuard g(ctx->device);
+    ks_model* m = new (std::nothrow) ks_model();
+    if (!m) return KS_ERR_OOM;
+    own.m = m;
+    m->ctx = ctx;
+    m->device = ctx->device;
+    m->kind = 1;
+    m->mlp.n_layers = n_layers;
+    for (int l = 0; l <= n_layers; ++l) m->mlp.widths[l] = h_widths[l];
+    cudaError_t e = ks::build_fast_mlp(m->mlp, h_w_bf16, h_bias, h_mu, h_sigma);
+    // the resident-weights kernel scores given rows in the ordinal input form only
+    if (e == cudaSuccess && !ks::score_mlp_tc_ok(m->mlp)) e = ks::build_wide_mlp(m->mlp, h_w_bf16, h_bias, h_mu, h_sigma);
+    if (e == cudaSuccess) e = ks::build_ridge(m->mlp, h_w_bf16[0], h_bias[0], h_mu, h_sigma);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "ks_model_create_mlp");
+    *out_model = m;
+    own.m = nullptr;
+    return KS_OK;
+  } catch (const std::exception&) {  // (the vectors of the repacking)
+    return KS_ERR_OOM;
   }
-  *out_model = m;
-  return KS_OK;
 }
 
 ks_status ks_model_create_static(ks_ctx* ctx, ks_model** out_model) {

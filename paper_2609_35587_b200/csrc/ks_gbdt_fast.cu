@@ -1208,6 +1208,7 @@ cudaError_t build_fast_gbdt(GbdtModel& m, int n_trees, const int64_t* off, const
   std::vector<uint32_t> chunks(static_cast<size_t>(n_chunks) * chunk_words);
   FastTopParams* top = new (std::nothrow) FastTopParams();
   if (!top) return cudaErrorMemoryAllocation;
+  m.h_top = top;  // (freed with the model)
   const uint32_t always_left = 0xFFu;  // row 0, threshold 127: no byte (0x80 | bin) exceeds 0xFF
   for (int ch = 0; ch < n_chunks; ++ch) {
     uint32_t* base = chunks.data() + static_cast<size_t>(ch) * chunk_words;
@@ -1290,13 +1291,9 @@ cudaError_t build_fast_gbdt(GbdtModel& m, int n_trees, const int64_t* off, const
   if (e == cudaSuccess) e = cudaMemcpy(m.d_qthr, table.data(), table.size() * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&m.d_qfeat), sizeof(fq));
   if (e == cudaSuccess) e = cudaMemcpy(m.d_qfeat, fq, sizeof(fq), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    delete top;
-    return e;
-  }
+  if (e != cudaSuccess) return e;
   m.fixed_shift = fixed_point_shift(n_trees, off, nodes);
   m.class_words = class_tree_words(n_trees, off, nodes);
-  m.h_top = top;
   m.top_levels = L;
   m.top_compact = compact;
   m.fast = true;

@@ -738,6 +738,7 @@ cudaError_t build_fast_mlp(MlpModel& m, const uint16_t* const* h_w_in, const flo
   }
   MlpTcParams* prm = new (std::nothrow) MlpTcParams();
   if (!prm) return cudaErrorMemoryAllocation;
+  m.h_tc_params = prm;  // (freed with the model)
   std::memset(prm, 0, sizeof(*prm));
   auto fold = [&](int src, float& scale, float& shift) {
     const double s = 1.0 / static_cast<double>(h_sigma[src]);
@@ -793,13 +794,8 @@ cudaError_t build_fast_mlp(MlpModel& m, const uint16_t* const* h_w_in, const flo
     if (e == cudaSuccess) e = cudaMemcpy(m.d_w1_prob, w1p.data(), w1p.size() * sizeof(float), cudaMemcpyHostToDevice);
     prm->w1_prob = m.d_w1_prob;
   }
-  if (e != cudaSuccess) {
-    delete prm;
-    return e;
-  }
-  m.h_tc_params = prm;
-  m.tc = true;
-  return cudaSuccess;
+  m.tc = e == cudaSuccess;
+  return e;
 }
 
 void free_fast_mlp(MlpModel& m) {
