@@ -173,10 +173,12 @@ def test_several_planes_of_scores(ks, ctx):
     check(prob, cand, (off, nodes, 0.0), 10, idx.cpu().numpy(), sc.cpu().numpy(), [0, 4223, 4224, 4290, P - 1])
 
 
-@pytest.mark.parametrize("P,C,trees,depth,most", [(96, 20000, 500, 8, 200e6), (130, (1 << 21) + 1, 5, 5, 1.3e9)])
+@pytest.mark.parametrize("P,C,trees,depth,most", [(96, 20000, 500, 8, 200e6), (130, (1 << 21) + 1, 5, 5, 1.5e9)])
 def test_batches_refused_on_the_host(ks, P, C, trees, depth, most):
     """Too few problems for any pool, and more candidates than a gigabyte holds the scores of 128 problems
-    for: such a batch reserves no memory for this walk (240 MB of programs, 1.07 GB of scores)."""
+    for: such a batch reserves no memory for this walk (240 MB of programs, 1.07 GB of scores). What it does
+    reserve: 85 MB for 96 problems and half of it to grow; 16 x 2,097,153 records of 32 bytes, their classes and
+    order, 1.4 GB with room."""
     ctx = ks.Context(DESC, 0)
     cand, prob = np.resize(wl.candidates_full_grid(1, None), C), wl.problems_batch(2, P, cross_precision=False)
     off, nodes = wl.gbdt_complete(3, trees, depth, wl.feature_stats("cfg1"), 0.1, "hist256")

@@ -109,7 +109,7 @@ from paper_2609_35587_b200 import binding as ks, workloads as wl
 ctx = ks.Context(wl.gpu_desc(), 0)
 st = wl.feature_stats("cfg1")
 gbdt = wl.gbdt_complete(1, 4000, 8, st, 0.1, "slots128")  # 2 M nodes, 16 MB in the library's form
-mlp = wl.mlp_xavier(1, [64, 1024, 1024, 1024, 1024, 1], st["mu"], st["sigma"])  # a weight image of 6.7 MB
+mlp = wl.mlp_xavier(1, [64, 1024, 1024, 1024, 1024, 1024, 1], st["mu"], st["sigma"])  # a weight image of 8.5 MB
 small = wl.gbdt_complete(1, 3, 4, st, 0.1), wl.mlp_xavier(1, [64, 320, 1], st["mu"], st["sigma"])
 ctx.model_create_gbdt(*small[0]).close(), ctx.model_create_mlp(small[1]).close()
 soft, hard = resource.getrlimit(resource.RLIMIT_AS)
@@ -131,8 +131,10 @@ print("statuses", got)
 def test_host_memory_runs_out(ks):
     """Creating a model where the host has no memory for its repacked form: a status, no exception across
     the C boundary (which would end the process)."""
+    import os
     import subprocess
     import sys
-    r = subprocess.run([sys.executable, "-c", CHILD], capture_output=True, text=True, timeout=120)
+    env = dict(os.environ, MALLOC_MMAP_THRESHOLD_="65536")  # large blocks are new mappings, not reused ones
+    r = subprocess.run([sys.executable, "-c", CHILD], capture_output=True, text=True, timeout=120, env=env)
     assert r.returncode == 0, r.stderr[-2000:]
     assert f"statuses [{ks.KS_ERR_OOM}, {ks.KS_ERR_OOM}]" in r.stdout, r.stdout
