@@ -86,6 +86,7 @@ struct SliceArgs {
   int n_slices;            // 1 = every CTA walks the whole ensemble
   long long pairs;         // rows of the partial-score planes
   float* scores;           // [n_slices][pairs] partial scores
+  int* words;              // the context's device words: the blocks' counters (reset by their last users), kWordWalk
   int32_t* out_idx;        // single-problem form only: [k] final result (device-visible, may be
   float* out_score;        // mapped host memory); null when a merge kernel follows
   const uint8_t* tiles;    // prepared tiles [blocks][rows][NC] (tile_pairs_kernel), or null
@@ -120,11 +121,11 @@ constexpr int kCandThreads = 256;
 template <int kBlockCands>
 __global__ void __launch_bounds__(kCandThreads)
 cand_rows_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, const unsigned* mask_ptr, int combo0,
-                 FastView fv, uint8_t* __restrict__ out, MemoView memo, int thr_cap) {
+                 FastView fv, uint8_t* __restrict__ out, MemoView memo, int thr_cap, int* ctx_words) {
   extern __shared__ __align__(16) float s_cthr[];  // thresholds of the candidate-only features, values, records
   __shared__ FeatQ s_fq[64];
   const int combo = combo0 >= 0 ? combo0 : blockIdx.y, tid = threadIdx.x;
-  if (fv.words && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) fv.words[kWordWalk] = 0;
+  if (ctx_words && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) ctx_words[kWordWalk] = 0;
   if (mask_ptr && !((*mask_ptr >> combo) & 1u)) return;
   const float* T = stage_thresholds(fv, fv.thr_cand0, fv.thr_prob0 - fv.thr_cand0, s_cthr, thr_cap) - fv.thr_cand0;
   if (tid < 64) s_fq[tid] = fv.feat[tid];
@@ -194,7 +195,7 @@ static_assert(sizeof(ProblemTerms) <= 128, "problem record");
 
 __global__ void __launch_bounds__(256)
 pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int n_prob,
-                  const ks_candidate* __restrict__ c, FastView fv, MemoView memo, int thr_cap, const int* path) {
+                  const ks_candidate* __restrict__ c, FastView fv, MemoView memo, int thr_cap, const int* path, int* words) {
   extern __shared__ __align__(16) float s_pthr[];  // thresholds of the per-pair features, then the records
   __shared__ ProblemTerms s_pt;
   __shared__ FeatQ s_fq[64];
@@ -206,7 +207,7 @@ pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem
   // (also) precedes the select kernel, whose CTAs leave at once when the class walk
   // (ks_gbdt_classes.cu) serves the call; that one then writes the partial lists
   const bool skip = path && *path == 1;
-  if (blockIdx.x == 0 && tid == 0) fv.words[kWordWalk] = skip ? kLeaveServed : 0;
+  if (blockIdx.x == 0 && tid == 0) words[kWordWalk] = skip ? kLeaveServed : 0;
   if (skip) return;
   int most = 0;
   for (int q = 0; q < kMemoCombos; ++q) most = max(most, memo.count[q]);
@@ -329,14 +330,14 @@ static_assert(kTileMaxThr >= 376 * kSlice, "every ensemble of the regular geomet
 __global__ void __launch_bounds__(256, 3)
 tile_pairs_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int P,
                   const ks_candidate* __restrict__ c, int C, FastView fv, int W, int groups,
-                  uint8_t* __restrict__ tiles) {
+                  uint8_t* __restrict__ tiles, int* words) {
   extern __shared__ __align__(16) float s_x[];  // [kTileCols][kTileRows], then the thresholds of every feature
   __shared__ ProblemTerms s_pt;
   __shared__ FeatQ s_fq[64];
   __shared__ float s_pf[64];
   float* s_thr = s_x + kTileCols * kTileRows;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (blockIdx.x == 0 && tid == 0) fv.words[kWordWalk] = 0;
+  if (blockIdx.x == 0 && tid == 0) words[kWordWalk] = 0;
   const long long n_items = static_cast<long long>(P) * groups;
   const int begin = static_cast<int>(n_items * blockIdx.x / gridDim.x);
   const int end = static_cast<int>(n_items * (blockIdx.x + 1) / gridDim.x);
@@ -402,12 +403,12 @@ constexpr int kTileWarps = 16;
 
 __global__ void __launch_bounds__(kTileWarps * 32, 2)
 tile_rows_kernel(const float* __restrict__ feat, int64_t rows, FastView fv, uint8_t* __restrict__ tiles, int W,
-                 int groups) {
+                 int groups, int* words) {
   extern __shared__ __align__(16) float s_x[];  // [64][kTileRows], then the thresholds of every feature
   __shared__ FeatQ s_fq[64];
   float* s_thr = s_x + 64 * kTileRows;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (blockIdx.x == 0 && threadIdx.x == 0) fv.words[kWordWalk] = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) words[kWordWalk] = 0;
   stage_thresholds(fv, 0, fv.n_thr, s_thr, fv.n_thr);
   if (threadIdx.x < 64) s_fq[threadIdx.x] = fv.feat[threadIdx.x];
   const uint32_t thr = smem_u32(s_thr);
@@ -713,7 +714,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
       problem_terms(use_value ? p_value : load_problem(p + prob), desc, s_pt);
       problem_columns(s_pt, [&](int col, float v) { s_pfeat[col] = v; });
     }
-    s_abort = *reinterpret_cast<volatile int*>(fv.words + kWordWalk);
+    s_abort = *reinterpret_cast<volatile int*>(sl.words + kWordWalk);
   }
   if (tid < KS_MAX_K) s_list[tid] = 0ull;
   if (!tiles_given && fv.prob_tab) {
@@ -804,7 +805,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
         if (*v_fail || !mbar_wait_bounded(bar, par, fv.wait_limit, v_fail)) {
           if (!*v_fail) {
             s_fail = 1;
-            atomicExch(fv.words + kWordWalk, kLeaveFailed);
+            atomicExch(sl.words + kWordWalk, kLeaveFailed);
             if (status) atomicExch(status, KS_ERR_TIMEOUT);
           }
           break;
@@ -952,7 +953,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
       __threadfence();
       __syncthreads();
       if (tid == 0) {
-        int* cnt = fv.words + static_cast<size_t>(prob) * nblk + chunk;
+        int* cnt = sl.words + static_cast<size_t>(prob) * nblk + chunk;
         s_last = atomicAdd(cnt, 1) == S - 1;
         if (s_last) *cnt = 0;  // nobody else touches this counter again in this launch
       }
@@ -988,7 +989,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     // single-problem form: the last block to finish merges the per-block lists
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(fv.words + nblk, 1) == nblk - 1;
+    if (tid == 0) s_last = atomicAdd(sl.words + nblk, 1) == nblk - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
@@ -1012,7 +1013,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     }
     __syncthreads();
     if (tid == 0) {
-      fv.words[nblk] = 0;
+      sl.words[nblk] = 0;
       if (sl.out_seq) {  // the results are in place: tell the host, which polls this word
         __threadfence_system();
         *reinterpret_cast<volatile int*>(sl.out_seq) = sl.seq;
@@ -1519,7 +1520,7 @@ int staged_floats(int count, size_t* bytes) {
 // combo >= 0: only that type combination; else those of the mask, or all (null).
 static cudaError_t launch_cand_rows(const ks_gpu_desc& desc, const GbdtModel& g, const ks_candidate* d_c, int C,
                                     const unsigned* d_mask, int combo, const FastView& fv, uint8_t* d_rows,
-                                    const MemoView& memo, cudaStream_t stream, int64_t* launches) {
+                                    const MemoView& memo, int* words, cudaStream_t stream, int64_t* launches) {
   const int count = g.thr_prob0 - g.thr_cand0, block = C < 8192 ? 64 : 256;
   const size_t own = static_cast<size_t>(block) * (cand_rec_bytes(g) + 4 + 4 * kCandCols);
   size_t thr = (static_cast<size_t>(count) + 3) / 4 * 16;
@@ -1530,7 +1531,7 @@ static cudaError_t launch_cand_rows(const ks_gpu_desc& desc, const GbdtModel& g,
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
   kernel<<<dim3(std::min((C + block - 1) / block, 2 * kSmCount), combo >= 0 ? 1 : kCombos), kCandThreads, smem, stream>>>(
-      desc, d_c, C, d_mask, combo, fv, d_rows, memo, cap);
+      desc, d_c, C, d_mask, combo, fv, d_rows, memo, cap, words);
   ++*launches;
   return cudaGetLastError();
 }
@@ -1547,7 +1548,7 @@ cudaError_t fast_prepare(const ks_gpu_desc& desc, const GbdtModel& g, const ks_c
     e = memo_clear(memo, stream);
     if (e != cudaSuccess) return e;
   }
-  e = launch_cand_rows(desc, g, d_c, C, nullptr, -1, fv, static_cast<uint8_t*>(d_rows), memo, stream, launches);
+  e = launch_cand_rows(desc, g, d_c, C, nullptr, -1, fv, static_cast<uint8_t*>(d_rows), memo, nullptr, stream, launches);
   if (e != cudaSuccess) return e;
   if (memo.keys) {
     e = memo_compact(memo, stream);
@@ -1656,7 +1657,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     const int resident = std::max<int>(1, std::min<int>(3, 226 * 1024 / (smem + 4096)));
     if (C > 0)
       tile_pairs_kernel<<<std::min(P * groups, resident * kSmCount), 256, smem, stream>>>(
-          desc, d_p, a.pv, a.uv, P, d_c, C, fv, W, groups, slice->tiles);
+          desc, d_p, a.pv, a.uv, P, d_c, C, fv, W, groups, slice->tiles, wait->words);
     else
       e = cudaMemsetAsync(slice->tiles, 0x80, fast_tiles_bytes(g, static_cast<int64_t>(P) * nblk), stream);
     if (e != cudaSuccess) return e;
@@ -1667,7 +1668,8 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
       if (e != cudaSuccess) return e;
     }
     e = launch_cand_rows(desc, g, d_c, C, a.uv ? nullptr : d_mask,
-                         a.uv ? (a.pv.dtype_ab & 3) * 4 + (a.pv.dtype_d & 3) : -1, fv, d_rows, memo, stream, launches);
+                         a.uv ? (a.pv.dtype_ab & 3) * 4 + (a.pv.dtype_d & 3) : -1, fv, d_rows, memo, wait->words, stream,
+                         launches);
     if (e != cudaSuccess) return e;
     if (memo.keys) {
       e = ensure_dynamic_smem(reinterpret_cast<const void*>(&pair_table_kernel), pthr_bytes);
@@ -1681,7 +1683,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     }
   }
   if (C == 0) {  // no kernel in front of the walk: the word that a failed call may have left is cleared here
-    e = cudaMemsetAsync(fv.words + kWordWalk, 0, sizeof(int), stream);
+    e = cudaMemsetAsync(wait->words + kWordWalk, 0, sizeof(int), stream);
     if (e != cudaSuccess) return e;
   }
   e = cudaGetLastError();
@@ -1694,6 +1696,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
   }
 
   a.sl.n_slices = 1;
+  a.sl.words = wait->words;
   if (slice && slice->n_slices > 1) {
     a.sl.n_slices = slice->n_slices;
     a.sl.pairs = slice->pairs;
@@ -1715,7 +1718,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
       const int64_t table_slots = static_cast<int64_t>(kSmCount) * (2 * (pthr_bytes + 4096) <= 227 * 1024 ? 2 : 1);
       pair_table_kernel<<<static_cast<unsigned>(table_items < table_slots ? table_items : table_slots), 256, pthr_bytes,
                           stream>>>(
-          desc, d_p ? d_p + first : nullptr, a.pv, a.uv, n, d_c, fv, memo, pthr_cap, path);
+          desc, d_p ? d_p + first : nullptr, a.pv, a.uv, n, d_c, fv, memo, pthr_cap, path, wait->words);
       ++*launches;
     }
     a.dependent = memo.keys != nullptr;
@@ -1765,13 +1768,14 @@ cudaError_t launch_score_fast(const ks_gpu_desc& desc, const GbdtModel& g, const
     const int W = g.block_cands / 4, groups = nblk * (W / 32);
     const int resident = 2 * (smem + 3072) <= 227 * 1024 ? 2 : 1;
     tile_rows_kernel<<<std::min(groups, resident * kSmCount), kTileWarps * 32, smem, stream>>>(
-        d_feat + first * KS_F_PAD, n, a.fv, tiles, W, groups);
+        d_feat + first * KS_F_PAD, n, a.fv, tiles, W, groups, wait->words);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     a.C = static_cast<int>(n);
     a.nblk = nblk;
     a.sl = SliceArgs{};
     a.sl.n_slices = 1;
+    a.sl.words = wait->words;
     a.sl.tiles = tiles;
     a.sl.score_out = d_scores + first;
     a.sl.repeat = floor_repeat;

@@ -145,7 +145,6 @@ struct FastView {
   int wait_limit, starve;           // probes a chunk wait may take; test hook: arm the barrier for bytes that never come
   int buf_bytes;                    // size of one chunk buffer in shared memory
   float base;
-  int* words;                       // the context's device words (null: a call outside the walk)
   const uint32_t* chunks;      // [n_chunks][chunk_bytes / 4]
   const float* thr;            // [n_thr] sorted thresholds, feature after feature (per-pair features first)
   const FeatQ* feat;           // [64] rows and thresholds of each feature column
@@ -187,7 +186,6 @@ inline FastView make_view(const GbdtModel& g, const FastWait* wait) {
   fv.pair_rec = pair_rec_bytes(g);
   fv.wait_limit = wait && wait->limit > 0 ? wait->limit : kFastWaitLimit;
   fv.starve = wait ? wait->starve : 0;
-  fv.words = wait ? wait->words : nullptr;
   fv.buf_bytes = g.buf_bytes;
   fv.base = g.base;
   fv.chunks = g.d_qnodes;
