@@ -13,8 +13,8 @@
 // layer's A. No CTA waits for another pair. The next layer's first K blocks only need the first
 // column tiles of the layer before, so the epilogue of a layer's last tile runs under the next
 // layer's MMAs.
-// Measured on 16 x 60,000 pairs of the shipped shape (3.4 TFLOP): 4.6 ms a call, of it 4.1 ms in
-// the layers (830 TFLOP/s, 0.59 of cuBLAS's sustained rate); a tile MLP on the CUDA cores took
+// Measured on 16 x 60,000 pairs of the shipped shape (3.4 TFLOP): 4.8 ms a call, of it 4.3 ms in
+// the layers (790 TFLOP/s, 0.56 of cuBLAS's sustained rate); a tile MLP on the CUDA cores took
 // 440 ms. This kernel is the only one for these shapes. What is left of the gap is the operands' way from L2
 // (a K block brings 128 flop a byte, so the sustained rate would need 10.9 TB/s) and the parts that a
 // layer's sums are taken in (see part_count; 3.8 ms a call without them). Taking
@@ -78,19 +78,20 @@ constexpr int64_t batch_rows(bool lean) { return lean ? kLeanRows : kBatchRows; 
 constexpr int64_t score_pairs(bool lean) { return lean ? kLeanScorePairs : kScorePairs; }
 constexpr int kTileN = 256;
 
-// Parts that the K blocks of a layer are summed in. The tensor core adds to its fp32 accumulator by
-// truncation, so that what a long sum loses grows with its length, where additions that round lose the
-// square root of it: with all of 1,024 in one accumulator the scores were 1.66 times as far from 64 bits as
-// with sums in sequence. So an accumulator takes a part of K, and the epilogue adds the parts, which
-// rounds. One part more than the square root of the blocks is no further off than the sequence: rms error
-// of 64-1024-1024-512-256-1 over 320,000 rows 3.8e-4 in sequence, 6.9e-4 in one part, 3.9e-4 in four parts
-// of 16 blocks, 3.6e-4 in six. What a part costs is reading its accumulator: 128 KB an SM from TMEM, some
-// 2,300 clocks, beside the 2,000 to 4,600 that its MMAs and operands take (16 x 60,000 pairs: 3.8 ms in one
-// part, 4.3 in four, 4.6 like this, 4.7 in six).
+// Parts that a layer's K is summed in. The tensor core adds to its fp32 accumulator by truncation, so that
+// what a sum loses grows with the number of its MMAs (16 of K each) and with its size, where additions that
+// round lose the square root of their number: measured, a sum over 64 of K has 1.27 times the error of the
+// same sum in sequence, one over 1,024 1.66 times (as scores, against 64 bits). So an accumulator takes a
+// part of K, and the epilogue adds the parts, which rounds. In the square, p parts of b blocks of 64 lose
+// 1.6 b^3 / p^2 where the sequence loses b^2: p is the smallest with 2 p^2 >= 3 b. What a part costs is
+// reading its accumulator: 128 KB an SM from TMEM, some 2,300 clocks, beside the 2,000 to 4,600 that its
+// MMAs and operands take (16 x 60,000 pairs of the shipped shape: 3.8 ms in one part, 4.8 like this, of it 0.15
+// for the two parts of the first layer; parts cut within a block 5.4). Error of that shape, root mean square
+// over 320,000 rows: 3.8e-4 in sequence, 6.4e-4 in one part, 3.6e-4 like this.
 constexpr int part_count(int kblocks) {
-  int root = 1;
-  while ((root + 1) * (root + 1) <= kblocks) ++root;
-  return root + 1 < kblocks ? root + 1 : kblocks;
+  int p = 1;
+  while (2 * p * p < 3 * kblocks) ++p;
+  return p;
 }
 
 struct WideArgs {
@@ -455,17 +456,25 @@ mlp_wide_kernel(const __grid_constant__ WideArgs a, const __grid_constant__ CUte
                 const uint32_t acc = part & 1u;
                 if (!(ok = wait_ok(bar_read(acc), ((part >> 1) & 1u) ^ 1u))) break;
                 fence_after();
-                const int first = kbs * j / parts, stop = kbs * (j + 1) / parts;
-                for (int kb = first; kb < stop; ++kb, ++it) {
+                // whole blocks, or (a layer of one block) 32 of K
+                const int first = kbs > 1 ? 4 * (kbs * j / parts) : 4 * j / parts;
+                const int stop = kbs > 1 ? 4 * (kbs * (j + 1) / parts) : 4 * (j + 1) / parts;
+                for (int u = first; u < stop; u = (u | 3) + 1) {
                   const int s = static_cast<int>(it % kStages);
-                  if (!(ok = wait_ok(bar_full(s), (it / kStages) & 1u))) break;
-                  fence_after();
+                  if ((u & 3) == 0) {  // (a block that the part before has begun is there)
+                    if (!(ok = wait_ok(bar_full(s), (it / kStages) & 1u))) break;
+                    fence_after();
+                  }
                   const uint64_t da = operand_desc(sbase + s * kStageBytes);
                   const uint64_t db = operand_desc(sbase + s * kStageBytes + kBlockBytes);
 #pragma unroll
                   for (int k16 = 0; k16 < 4; ++k16)  // 32 bytes on in K: two units of the address field
-                    mma_pair(tmem + acc * 256u, da + 2u * k16, db + 2u * k16, idesc, kb > first || k16 > 0);
-                  commit_pair(bar_empty(s));
+                    if (k16 >= (u & 3) && (u & ~3) + k16 < stop)
+                      mma_pair(tmem + acc * 256u, da + 2u * k16, db + 2u * k16, idesc, (u & ~3) + k16 > first);
+                  if ((u | 3) < stop) {
+                    commit_pair(bar_empty(s));
+                    ++it;
+                  }
                 }
                 if (ok) commit_pair(bar_acc(acc));
               }
