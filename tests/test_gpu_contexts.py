@@ -60,9 +60,9 @@ def test_overlapping_contexts(ks):
     serial = {name: f() for name, f in asked.items()}
     torch.cuda.synchronize()
     s_a, s_b = torch.cuda.Stream(), torch.cuda.Stream()
-    n = 48
+    n = 120
     with torch.cuda.stream(s_a):
-        batches = [a.select(d_p, 512, d_c, 60000, model, 10) for _ in range(n)]  # queued, a tenth of a second
+        batches = [a.select(d_p, 512, d_c, 60000, model, 10) for _ in range(n)]  # queued, some tenths of a second
     rounds = 0
     with torch.cuda.stream(s_b):
         while True:
