@@ -376,6 +376,26 @@ __device__ __forceinline__ float ridge_level(const float (&lut)[4], float v) {
   return (code >= 0 && code < 4) ? lut[code] : 0.0f;
 }
 
+// the candidate-only part of the sum, and the resident-block count
+__device__ __forceinline__ float ridge_candidate_sum(const ks_gpu_desc& desc, const RidgeParams& prm, int combo,
+                                                     const ks_candidate& cand, long long& b_eff) {
+  ks_problem fake{};
+  fake.m = fake.n = fake.k = 1;
+  fake.dtype_ab = static_cast<uint8_t>(combo >> 2);
+  fake.dtype_d = static_cast<uint8_t>(combo & 3);
+  ProblemTerms t;
+  problem_terms(fake, desc, t);
+  float s = 0.0f;
+  featurize_pair(t, cand, desc, [&](int col, float v) {
+    if (feat_class(col) != 1) return;
+    s += ridge_term(prm, col, v);
+    if (col == 17) s += ridge_level(prm.lut17, v);
+    if (col == 18) s += ridge_level(prm.lut18, v);
+  });
+  b_eff = resources(t, cand, desc).b_eff;
+  return s;
+}
+
 // per (type combination, candidate): (candidate-only part of the sum, resident-block count)
 __global__ void __launch_bounds__(256)
 ridge_cand_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, const unsigned* mask_ptr,
@@ -384,21 +404,9 @@ ridge_cand_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, c
   if (!((*mask_ptr >> combo) & 1u)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= C) return;
-  ks_problem fake{};
-  fake.m = fake.n = fake.k = 1;
-  fake.dtype_ab = static_cast<uint8_t>(combo >> 2);
-  fake.dtype_d = static_cast<uint8_t>(combo & 3);
-  ProblemTerms t;
-  problem_terms(fake, desc, t);
   const ks_candidate cand = c[i];
-  float s = 0.0f;
-  featurize_pair(t, cand, desc, [&](int col, float v) {
-    if (feat_class(col) != 1) return;
-    s += ridge_term(prm, col, v);
-    if (col == 17) s += ridge_level(prm.lut17, v);
-    if (col == 18) s += ridge_level(prm.lut18, v);
-  });
-  const long long b_eff = resources(t, cand, desc).b_eff;
+  long long b_eff;
+  const float s = ridge_candidate_sum(desc, prm, combo, cand, b_eff);
   out[static_cast<size_t>(combo) * C + i] = make_float2(s, static_cast<float>(b_eff));
   if (memo.keys) memo.cls[static_cast<size_t>(combo) * C + i] = memo_assign(memo, combo, i, cand, b_eff);
 }
@@ -467,7 +475,7 @@ ridge_pair_kernel(ks_gpu_desc desc, const RidgeProblem* __restrict__ problems, c
   }
 }
 
-// the per-pair part in place, for a candidate without a class (out of line: it would cost the kernel
+// the per-pair part in place, for a candidate without a class (out of line: it would cost a kernel
 // half its resident warps)
 __device__ __noinline__ float ridge_pair_in_place(const ks_gpu_desc& desc, const ProblemTerms& t, const ks_candidate* c,
                                                   long long b_eff, const RidgeParams& prm) {
@@ -476,135 +484,328 @@ __device__ __noinline__ float ridge_pair_in_place(const ks_gpu_desc& desc, const
   return pair;
 }
 
-// A block ranks kQ problems against its share of the candidates. What bounds it is the instructions a
-// pair takes, so a candidate is fetched once for the kQ problems, the class sums are gathered from
+// Segmented batches, and batches of few problems: a block ranks one problem against its share of the
+// candidates. What bounds it is the instructions a pair takes, so the class sums are gathered from
 // shared memory, and a warp keeps a running top-k list (one key a lane): a score that does not reach
 // the best k-th score any of the block's warps has seen costs no more than the comparison. (Ranking
-// eight keys a thread from scratch, with sums from L2, took 852 us for 1,024 x 60,000 pairs.)
-constexpr int kRidgeThreads = 512, kRidgeProblems = 4;
+// eight keys a thread from scratch, with sums from L2, took three times as long.)
+constexpr int kRidgeThreads = 512;
 constexpr int kRidgeClasses = 2048;  // classes whose sums are staged; the others are fetched from L2
 // kClasses: with the class tables; without them (few problems) every pair is evaluated in place.
-template <int kQ, bool kClasses>
+template <bool kClasses>
 __global__ void __launch_bounds__(kRidgeThreads, kClasses ? 2 : 1)
 select_ridge_kernel(const __grid_constant__ ks_gpu_desc desc, const RidgeProblem* __restrict__ problems, const ks_candidate* __restrict__ c,
                     PairMap map, const float2* __restrict__ cand_tab, const __grid_constant__ RidgeParams prm, int k,
                     unsigned long long* __restrict__ partial /* [P][nblk][k] */, MemoView memo) {
-  __shared__ float s_tab[kQ][kClasses ? kRidgeClasses : 1];
-  __shared__ ProblemTerms s_pt;  // (without classes, where kQ = 1)
-  __shared__ unsigned s_bar[kQ];  // upper word of a key below which nothing can make the list
+  __shared__ float s_tab[kClasses ? kRidgeClasses : 1];
+  __shared__ ProblemTerms s_pt;  // (without classes)
+  __shared__ unsigned s_bar;     // upper word of a key below which nothing can make the list
   // The upper words of a warp's best key and (for k > 16) its second best, in one 64-bit word: another warp
   // sees both from before or both from after an update, so no candidate counts twice in the bar.
-  __shared__ unsigned long long s_best[kQ][kRidgeThreads / 32];
+  __shared__ unsigned long long s_best[kRidgeThreads / 32];
   __shared__ unsigned long long s_list[kRidgeThreads / 32][32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int group = blockIdx.x / map.nblk, chunk = blockIdx.x % map.nblk;
-  __shared__ int s_combo[kQ];
-  __shared__ float s_sum[kQ];
-  auto prob = [&](int q) { return min(group * kQ + q, map.P - 1); };
-  unsigned long long top[kQ];
-#pragma unroll
-  for (int q = 0; q < kQ; ++q) {
-    const int combo = problems[prob(q)].combo;
-    if (tid == 0) {
-      s_combo[q] = combo;
-      s_sum[q] = problems[prob(q)].sum;
-    }
-    top[q] = 0ull;
-    if (kClasses) {
-      const int n = min(memo.count[combo], kRidgeClasses);
-      const float* src = static_cast<const float*>(memo.tab) + static_cast<size_t>(prob(q)) * kMemoCap;
-      for (int j = tid; j < n; j += kRidgeThreads) s_tab[q][j] = __ldg(src + j);
-    }
+  const int prob = blockIdx.x / map.nblk, chunk = blockIdx.x % map.nblk;
+  const int combo = problems[prob].combo;
+  const float sum = problems[prob].sum;
+  const float* tab = static_cast<const float*>(memo.tab) + static_cast<size_t>(prob) * kMemoCap;
+  unsigned long long top = 0ull;
+  if (kClasses) {
+    const int n = min(memo.count[combo], kRidgeClasses);
+    for (int j = tid; j < n; j += kRidgeThreads) s_tab[j] = __ldg(tab + j);
   }
   if (!kClasses && tid < static_cast<int>(sizeof(ProblemTerms) / 4))
-    reinterpret_cast<uint32_t*>(&s_pt)[tid] = reinterpret_cast<const uint32_t*>(&problems[prob(0)].t)[tid];
-  if (tid < kQ) s_bar[tid] = 0u;
-  if (tid < kQ * kRidgeThreads / 32) (&s_best[0][0])[tid] = 0ull;
+    reinterpret_cast<uint32_t*>(&s_pt)[tid] = reinterpret_cast<const uint32_t*>(&problems[prob].t)[tid];
+  if (tid == 0) s_bar = 0u;
+  if (tid < kRidgeThreads / 32) s_best[tid] = 0ull;
   __syncthreads();
-  int64_t lo, len;  // (per-problem segments: kQ = 1)
-  segment_of(map, prob(0), lo, len);
+  int64_t lo, len;
+  segment_of(map, prob, lo, len);
   const int64_t share = (len + map.nblk - 1) / map.nblk, stop = min(len, share * (chunk + 1));
-  bool mixed = false;  // element types differ among the block's problems
-#pragma unroll
-  for (int q = 1; q < kQ; ++q) mixed |= s_combo[q] != s_combo[0];
-  const float2* tab0 = cand_tab + static_cast<size_t>(s_combo[0]) * map.C;
+  const float2* cand = cand_tab + static_cast<size_t>(combo) * map.C;
   // a candidate's record is fetched one round ahead
   auto row_index = [&](int64_t r) { return r < stop ? pool_index(map, lo, r) : 0; };
   const int64_t r_first = share * chunk + warp * 32 + lane;
   int next_idx = row_index(r_first);
-  float2 next = __ldg(tab0 + next_idx);
+  float2 next = __ldg(cand + next_idx);
   for (int64_t r = r_first; r - lane < stop; r += kRidgeThreads) {
     const bool live = r < stop;
     const int idx = next_idx;
-    float2 t = next;
+    const float2 t = next;
     next_idx = row_index(r + kRidgeThreads);
-    next = __ldg(tab0 + next_idx);
+    next = __ldg(cand + next_idx);
+    const int cls = __float_as_int(t.y);
+    float pair = 0.0f;
+    if (kClasses && cls >= 0) {
+      pair = cls < kRidgeClasses ? s_tab[cls] : __ldg(tab + cls);
+    } else if (kClasses) {
+      pair = ridge_pair_in_place(desc, problems[prob].t, c + idx, -static_cast<long long>(cls), prm);
+    } else {
+      pair_columns<true>(s_pt, load_candidate(c + idx), desc, static_cast<long long>(t.y),
+                         [&](int col, float v) { pair += ridge_term(prm, col, v); });
+    }
+    const float score = ((sum + t.x) + pair) + 0.0f;
+    if (__any_sync(0xFFFFFFFFu, live && sortable(score) >= *const_cast<volatile unsigned*>(&s_bar))) {
+      warp_topk_insert(top, live ? make_key(score, idx) : 0ull, k);
+      // The k-th largest of the warps' best keys bounds the k-th best score from below (each is a
+      // candidate of its own), far better than any one warp's k-th.
+      constexpr int kWarps = kRidgeThreads / 32;
+      volatile unsigned long long* best = s_best;
+      const unsigned mine = static_cast<unsigned>(top >> 32), after = __shfl_sync(0xFFFFFFFFu, mine, 1);
+      if (lane == 0) best[warp] = static_cast<unsigned long long>(mine) << 32 | (k > kWarps ? after : 0u);
+      __syncwarp();
+      const unsigned long long two = lane < kWarps ? best[lane] : 0ull;
+      const unsigned first = static_cast<unsigned>(two >> 32), second = static_cast<unsigned>(two);
+      int ahead = 0, ahead2 = 0;  // of the two: keys that are at least as good
 #pragma unroll
-    for (int q = 0; q < kQ; ++q) {
-      if (q > 0 && mixed) t = __ldg(cand_tab + static_cast<size_t>(s_combo[q]) * map.C + idx);
-      const int cls = __float_as_int(t.y);
-      float pair = 0.0f;
-      if (kClasses && cls >= 0) {
-        pair = cls < kRidgeClasses ? s_tab[q][cls]
-                                   : __ldg(static_cast<const float*>(memo.tab) + static_cast<size_t>(prob(q)) * kMemoCap + cls);
-      } else if (kClasses) {
-        pair = ridge_pair_in_place(desc, problems[prob(q)].t, c + idx, -static_cast<long long>(cls), prm);
-      } else {
-        pair_columns<true>(s_pt, load_candidate(c + idx), desc, static_cast<long long>(t.y),
-                           [&](int col, float v) { pair += ridge_term(prm, col, v); });
-      }
-      const float score = ((s_sum[q] + t.x) + pair) + 0.0f;
-      if (__any_sync(0xFFFFFFFFu, live && sortable(score) >= *const_cast<volatile unsigned*>(&s_bar[q]))) {
-        warp_topk_insert(top[q], live ? make_key(score, idx) : 0ull, k);
-        // The k-th largest of the warps' best keys bounds the k-th best score from below (each is a
-        // candidate of its own), far better than any one warp's k-th.
-        constexpr int kWarps = kRidgeThreads / 32;
-        volatile unsigned long long* best = s_best[q];
-        const unsigned mine = static_cast<unsigned>(top[q] >> 32), after = __shfl_sync(0xFFFFFFFFu, mine, 1);
-        if (lane == 0) best[warp] = static_cast<unsigned long long>(mine) << 32 | (k > kWarps ? after : 0u);
-        __syncwarp();
-        const unsigned long long pair = lane < kWarps ? best[lane] : 0ull;
-        const unsigned first = static_cast<unsigned>(pair >> 32), second = static_cast<unsigned>(pair);
-        int ahead = 0, ahead2 = 0;  // of the two: keys that are at least as good
+      for (int i = 0; i < kWarps; ++i) ahead += __shfl_sync(0xFFFFFFFFu, first, i) >= first;
+      unsigned bar = ahead >= k ? first : 0u;
+      if (k > kWarps) {
 #pragma unroll
-        for (int i = 0; i < kWarps; ++i) ahead += __shfl_sync(0xFFFFFFFFu, first, i) >= first;
-        unsigned bar = ahead >= k ? first : 0u;
-        if (k > kWarps) {
-#pragma unroll
-          for (int i = 0; i < kWarps; ++i) {
-            const unsigned f = __shfl_sync(0xFFFFFFFFu, first, i), s = __shfl_sync(0xFFFFFFFFu, second, i);
-            ahead += s >= first;
-            ahead2 += (f >= second) + (s >= second);
-          }
-          bar = max(ahead >= k ? first : 0u, ahead2 >= k ? second : 0u);
+        for (int i = 0; i < kWarps; ++i) {
+          const unsigned f = __shfl_sync(0xFFFFFFFFu, first, i), s = __shfl_sync(0xFFFFFFFFu, second, i);
+          ahead += s >= first;
+          ahead2 += (f >= second) + (s >= second);
         }
-        bar = __reduce_max_sync(0xFFFFFFFFu, bar);
-        if (lane == 0) atomicMax(&s_bar[q], bar);
+        bar = max(ahead >= k ? first : 0u, ahead2 >= k ? second : 0u);
       }
+      bar = __reduce_max_sync(0xFFFFFFFFu, bar);
+      if (lane == 0) atomicMax(&s_bar, bar);
     }
   }
-#pragma unroll
-  for (int q = 0; q < kQ; ++q) {
+  s_list[warp][lane] = top;
+  __syncthreads();
+  if (warp == 0) {
+    for (int w = 1; w < kRidgeThreads / 32; ++w) warp_topk_insert(top, s_list[w][lane], k);
+    if (lane < k) partial[(static_cast<size_t>(prob) * map.nblk + chunk) * k + lane] = top;
+  }
+}
+
+// ---- dense batches: the classes of the catalogue, their members and their largest sums ----
+//
+// The score ((problem + candidate) + pair) rounds after every addition, and rounding keeps the order: among
+// the members of a class (equal pair part, see ks_memo.cuh) the one with the largest candidate part has the
+// largest score. So a problem ranks its classes by that score first, and only a class whose best
+// member reaches the k-th best of them is looked into: about k classes of 36 members instead of 60,000 pairs.
+// What is not a number or infinite is outside this order: such a class is always looked into.
+//
+// Slots of a combination's table: a power of two above the 10,785 classes of the valid search space. A
+// candidate without a slot (more classes than slots) is kept in a list of its own and always evaluated.
+constexpr int kRidgeCap = 16384;
+struct RidgeClass {  // 32 bytes
+  ks_candidate member;
+  float best;   // largest candidate-only sum of the class; not finite: look into it
+  int b_eff;
+  int first, count;  // its members in the list
+};
+struct RidgeMember {
+  int idx;
+  float sum;  // candidate-only part
+};
+// What a call keeps, per type combination. The first four are cleared in front of a call.
+struct RidgeTables {
+  unsigned* mask;            // combinations in use (with the clearing of the next two)
+  unsigned long long* keys;  // [16][kRidgeCap], 0 = free
+  uint2* stat;               // [16][kRidgeCap + 1] (largest sum as a sortable word, members); the last entry: without a class
+  int* n;                    // [16] (classes, their members)
+  int* rep;                  // [16][kRidgeCap] one member
+  uint2* place;              // [16][C] (slot, place among its members)
+  float* sum;                // [16][C] candidate-only part
+  int* first;                // [16][kRidgeCap] where a slot's members begin in the list (those without a class end it)
+  RidgeClass* cls;           // [16][kRidgeCap]
+  RidgeMember* list;         // [16][C]
+  float* pair;               // [blocks][kRidgeCap] a block's per-pair parts
+};
+
+// A class's largest sum: order-preserving, with everything that is not finite above all.
+__device__ __forceinline__ unsigned ridge_bound_word(float s) { return isfinite(s) ? sortable(s) : 0xFFFFFFFFu; }
+
+// per (type combination, candidate): the candidate-only part of the sum, and its class
+__global__ void __launch_bounds__(256)
+ridge_members_kernel(const __grid_constant__ ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C,
+                     const __grid_constant__ RidgeParams prm, RidgeTables t) {
+  const int combo = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (!((*t.mask >> combo) & 1u) || i >= C) return;
+  const ks_candidate cand = load_candidate(c + i);
+  long long b_eff;
+  const float s = ridge_candidate_sum(desc, prm, combo, cand, b_eff);
+  const size_t at = static_cast<size_t>(combo) * kRidgeCap;
+  const unsigned slot = memo_slot<kRidgeCap>(t.keys + at, t.rep + at, i, cand, b_eff);
+  uint2* stat = t.stat + static_cast<size_t>(combo) * (kRidgeCap + 1) + min(slot, static_cast<unsigned>(kRidgeCap));
+  atomicMax(&stat->x, ridge_bound_word(s));
+  t.place[static_cast<size_t>(combo) * C + i] = make_uint2(slot, atomicAdd(&stat->y, 1u));
+  t.sum[static_cast<size_t>(combo) * C + i] = s;
+}
+
+__device__ __noinline__ float ridge_lone_pair(const ks_gpu_desc& desc, const ProblemTerms& t, const ks_candidate* c,
+                                              const RidgeParams& prm) {
+  return ridge_pair_in_place(desc, t, c, resources(t, load_candidate(c), desc).b_eff, prm);
+}
+
+// Packs the classes of every combination and gives each its part of the list: a thread a slot, two atomic
+// operations a block. (One block for all of a combination's slots took 40 us for 1,700 classes and 100 for 10,785.)
+__global__ void __launch_bounds__(256)
+ridge_classes_kernel(const __grid_constant__ ks_gpu_desc desc, const ks_candidate* __restrict__ c, RidgeTables t) {
+  __shared__ int s_n, s_members, s_cls0, s_first0;
+  const int combo = blockIdx.y, slot = blockIdx.x * 256 + threadIdx.x;
+  if (!((*t.mask >> combo) & 1u)) return;
+  if (threadIdx.x == 0) s_n = s_members = 0;
+  __syncthreads();
+  const uint2 st = t.stat[static_cast<size_t>(combo) * (kRidgeCap + 1) + slot];
+  int j = 0, first = 0;
+  if (st.y != 0u) {
+    j = atomicAdd(&s_n, 1);
+    first = atomicAdd(&s_members, static_cast<int>(st.y));
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && s_n > 0) {
+    s_cls0 = atomicAdd(t.n + 2 * combo, s_n);
+    s_first0 = atomicAdd(t.n + 2 * combo + 1, s_members);
+  }
+  __syncthreads();
+  if (st.y == 0u) return;
+  const size_t at = static_cast<size_t>(combo) * kRidgeCap;
+  ProblemTerms pt;  // the resident-block count depends on the element sizes alone
+  pt.bA = bytes_ab(combo >> 2);
+  pt.bD = bytes_d(combo & 3);
+  RidgeClass r;
+  r.member = load_candidate(c + t.rep[at + slot]);
+  r.best = st.x == 0xFFFFFFFFu ? __uint_as_float(0x7FC00000u) : key_score(static_cast<unsigned long long>(st.x) << 32);
+  r.b_eff = static_cast<int>(resources(pt, r.member, desc).b_eff);
+  r.first = s_first0 + first;
+  r.count = static_cast<int>(st.y);
+  t.first[at + slot] = r.first;
+  t.cls[at + s_cls0 + j] = r;
+}
+
+__global__ void __launch_bounds__(256)
+ridge_list_kernel(int C, RidgeTables t) {
+  const int combo = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (!((*t.mask >> combo) & 1u) || i >= C) return;
+  const size_t at = static_cast<size_t>(combo) * C;
+  const uint2 p = t.place[at + i];
+  const int first = p.x == kNoClass ? C - static_cast<int>(t.stat[static_cast<size_t>(combo) * (kRidgeCap + 1) + kRidgeCap].y)
+                                    : t.first[static_cast<size_t>(combo) * kRidgeCap + p.x];
+  t.list[at + first + p.y] = RidgeMember{i, t.sum[at + i]};
+}
+
+// A block ranks a problem's share y of the classes (gridDim.y shares); blocks take problem after problem.
+// First every thread evaluates its classes and keeps its best one: the k-th largest of these bounds the k-th
+// best score from below (they are candidates of their own). Then the classes that reach it are looked into,
+// a warp a class. What bounds it is the arithmetic of the per-pair columns, once per (problem, class), so the
+// blocks are small: seven of 128 threads an SM serve 1,024 problems in one even round. 1,024 x 60,000 pairs: the
+// whole call 115 us, of it 75 here; every pair added up and compared, from a table of the pair parts, 279.
+constexpr int kRidgeRankThreads = 128, kRidgeRankBlocks = 7;
+__global__ void __launch_bounds__(kRidgeRankThreads, kRidgeRankBlocks)
+ridge_rank_kernel(const __grid_constant__ ks_gpu_desc desc, const RidgeProblem* __restrict__ problems, int P,
+                  const ks_candidate* __restrict__ c, int C, const __grid_constant__ RidgeParams prm, int k, RidgeTables t,
+                  unsigned long long* __restrict__ partial /* [P][gridDim.y][k], or null: the lists are the result */,
+                  int32_t* __restrict__ out_idx, float* __restrict__ out_score) {
+  constexpr int kWarps = kRidgeRankThreads / 32;
+  __shared__ RidgeProblem s_p;
+  __shared__ unsigned long long s_warp[kWarps * KS_MAX_K], s_list[KS_MAX_K];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* pair_of = t.pair + static_cast<size_t>(blockIdx.y * gridDim.x + blockIdx.x) * kRidgeCap;
+  for (int prob = blockIdx.x; prob < P; prob += gridDim.x) {
+    __syncthreads();  // the problem before is finished with
+    static_assert(sizeof(RidgeProblem) % 4 == 0 && sizeof(RidgeProblem) / 4 <= kRidgeRankThreads, "one word a thread");
+    if (tid < static_cast<int>(sizeof(RidgeProblem) / 4))
+      reinterpret_cast<uint32_t*>(&s_p)[tid] = __ldg(reinterpret_cast<const uint32_t*>(problems + prob) + tid);
     __syncthreads();
-    s_list[warp][lane] = top[q];
-    __syncthreads();
-    if (warp == 0 && group * kQ + q < map.P) {
-      unsigned long long mine = top[q];
-      for (int w = 1; w < kRidgeThreads / 32; ++w) warp_topk_insert(mine, s_list[w][lane], k);
-      if (lane < k) partial[(static_cast<size_t>(prob(q)) * map.nblk + chunk) * k + lane] = mine;
+    const int n = t.n[2 * s_p.combo];
+    const int begin = static_cast<int>(static_cast<int64_t>(n) * blockIdx.y / gridDim.y);
+    const int end = static_cast<int>(static_cast<int64_t>(n) * (blockIdx.y + 1) / gridDim.y);
+    const RidgeClass* cls = t.cls + static_cast<size_t>(s_p.combo) * kRidgeCap;
+    const float sum = s_p.sum;
+    unsigned long long best = 0ull;
+    for (int j = begin + tid; j < end; j += kRidgeRankThreads) {
+      const ks_candidate cand = load_candidate(&cls[j].member);
+      float pair = 0.0f;
+      pair_columns<true>(s_p.t, cand, desc, static_cast<long long>(cls[j].b_eff),
+                         [&](int col, float v) { pair += ridge_term(prm, col, v); });
+      pair_of[j] = pair;
+      const float bound = ((sum + cls[j].best) + pair) + 0.0f;
+      if (isfinite(bound)) best = max(best, make_key(bound, j));
+    }
+    unsigned long long one[1] = {best};
+    block_topk<1>(one, k, s_warp, s_list);
+    const unsigned bar = static_cast<unsigned>(s_list[k - 1] >> 32);
+    unsigned long long mine = 0ull;  // the warp's running list
+    const RidgeMember* list = t.list + static_cast<size_t>(s_p.combo) * C;
+    for (int j0 = begin + 32 * warp; j0 < end; j0 += kRidgeRankThreads) {
+      const int j = j0 + lane;
+      float pair = 0.0f;
+      int first = 0, count = 0;
+      bool look = false;
+      if (j < end) {
+        pair = pair_of[j];
+        const float bound = ((sum + cls[j].best) + pair) + 0.0f;
+        look = !isfinite(bound) || sortable(bound) >= bar;
+        if (look) {
+          first = cls[j].first;
+          count = cls[j].count;
+        }
+      }
+      for (unsigned todo = __ballot_sync(0xFFFFFFFFu, look); todo; todo &= todo - 1) {
+        const int src = __ffs(todo) - 1;
+        const int f = __shfl_sync(0xFFFFFFFFu, first, src), m = __shfl_sync(0xFFFFFFFFu, count, src);
+        const float q = __shfl_sync(0xFFFFFFFFu, pair, src);
+        for (int i = lane; i - lane < m; i += 32) {
+          unsigned long long key = 0ull;
+          if (i < m) {
+            const RidgeMember e = list[f + i];
+            key = make_key(((sum + e.sum) + q) + 0.0f, e.idx);
+            if (static_cast<unsigned>(key >> 32) < bar) key = 0ull;
+          }
+          warp_topk_insert(mine, key, k);
+        }
+      }
+    }
+    // candidates without a class: dealt to the blocks and warps like the classes
+    const int lone = static_cast<int>(t.stat[static_cast<size_t>(s_p.combo) * (kRidgeCap + 1) + kRidgeCap].y);
+    const int lone_at = C - lone;
+    for (int i0 = 32 * (blockIdx.y * kWarps + warp); i0 < lone; i0 += 32 * kWarps * gridDim.y) {
+      unsigned long long key = 0ull;
+      if (i0 + lane < lone) {
+        const RidgeMember e = list[lone_at + i0 + lane];
+        key = make_key(((sum + e.sum) + ridge_lone_pair(desc, s_p.t, c + e.idx, prm)) + 0.0f, e.idx);
+      }
+      warp_topk_insert(mine, key, k);
+    }
+    one[0] = mine;
+    block_topk<1>(one, k, s_warp, s_list);
+    if (tid < k) {
+      if (partial) {
+        partial[(static_cast<size_t>(prob) * gridDim.y + blockIdx.y) * k + tid] = s_list[tid];
+      } else {
+        out_idx[static_cast<size_t>(prob) * k + tid] = key_index(s_list[tid]);
+        out_score[static_cast<size_t>(prob) * k + tid] = key_score(s_list[tid]);
+      }
     }
   }
 }
 
-// Problems a block ranks, and blocks per group of problems: as many as fill the machine once (two blocks
-// of 512 threads an SM), with about 512 candidates each at least.
-// Several problems share a block only where the class tables are used: without them the kernel ranks one.
-size_t ridge_memo_bytes(int P, int C);
-static int ridge_group(bool segmented, int P, int C) { return segmented || ridge_memo_bytes(P, C) == 0 ? 1 : kRidgeProblems; }
-static int ridge_blocks(int P, int C, int64_t per_problem, bool segmented) {
-  const int g = ridge_group(segmented, P, C);
-  const int64_t groups = (P + g - 1) / g, most = std::max<int64_t>(1, (per_problem + 511) / 512);
-  return static_cast<int>(std::min(most, std::max<int64_t>(1, 2 * 148 / groups)));
+
+// Blocks a problem of the kernels above takes.
+// Of the class form: as many as the machine holds at once; a block has a thread for each of the valid search
+// space's 10,785 classes then.
+static int ridge_rank_shares(int P) {
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(64, kRidgeRankBlocks * 148 / P)));
+}
+static int ridge_rank_grid(int P) {
+  return static_cast<int>(std::min<int64_t>(P, kRidgeRankBlocks * 148 / ridge_rank_shares(P)));
+}
+// Of the candidate form: as many as fill the machine once (two blocks of 512 threads an SM), with about 512
+// candidates each at least.
+static int ridge_blocks(int P, int64_t per_problem) {
+  const int64_t most = std::max<int64_t>(1, (per_problem + 511) / 512);
+  return static_cast<int>(std::min(most, std::max<int64_t>(1, 2 * 148 / P)));
+}
+// Dense batches go by classes where that many pairs take longer one by one than the class tables do: 60,000
+// grid candidates 55 us whatever the (few) problems, in place 87 for 24 and 106 for 32; 61,140 valid candidates (10,785
+// classes) 89 and 95, in place 88 and 108; 5,000 candidates 52, in place 45 for 64 and 58 for 128.
+static bool ridge_by_classes(int P, int C, bool segmented, bool lean) {
+  return !segmented && !lean && P >= 30 && static_cast<int64_t>(P) * C >= 600000;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -838,10 +1039,33 @@ cudaError_t launch_score_linear(const MlpModel& m, const float* d_feat, int64_t 
 size_t ridge_scratch_bytes(int P, int C) {
   return 256 + (sizeof(float2) * 16 * static_cast<size_t>(C) + 255) / 256 * 256 + (sizeof(RidgeProblem) * static_cast<size_t>(P) + 255) / 256 * 256;
 }
-// classes and the per-(problem, class) sums of the linear scorer (0: not used)
-size_t ridge_memo_bytes(int P, int C) {
-  if (P < kMemoMinProblems || P > kMemoMaxProblems || C < 1) return 0;
+// classes and the per-(problem, class) sums of a segmented batch (0: not used)
+static size_t ridge_memo_bytes(int P, int C, bool segmented) {
+  if (!segmented || P < kMemoMinProblems || P > kMemoMaxProblems || C < 1) return 0;
   return memo_fixed_bytes(C) + sizeof(float) * static_cast<size_t>(P) * kMemoCap;
+}
+// The parts of the class form's memory; `cleared` receives the bytes at its beginning that a call clears.
+static size_t ridge_tables(int P, int C, void* mem, RidgeTables* t, size_t* cleared) {
+  size_t at = 0;
+  const auto take = [&](size_t bytes) {
+    char* q = static_cast<char*>(mem) + at;
+    at += (bytes + 255) / 256 * 256;
+    return q;
+  };
+  const size_t slots = static_cast<size_t>(16) * kRidgeCap, all = static_cast<size_t>(16) * C;
+  t->mask = reinterpret_cast<unsigned*>(take(256));
+  t->keys = reinterpret_cast<unsigned long long*>(take(slots * sizeof(unsigned long long)));
+  t->stat = reinterpret_cast<uint2*>(take((slots + 16) * sizeof(uint2)));
+  t->n = reinterpret_cast<int*>(take(32 * sizeof(int)));
+  *cleared = at;
+  t->rep = reinterpret_cast<int*>(take(slots * sizeof(int)));
+  t->place = reinterpret_cast<uint2*>(take(all * sizeof(uint2)));
+  t->sum = reinterpret_cast<float*>(take(all * sizeof(float)));
+  t->first = reinterpret_cast<int*>(take(slots * sizeof(int)));
+  t->cls = reinterpret_cast<RidgeClass*>(take(slots * sizeof(RidgeClass)));
+  t->list = reinterpret_cast<RidgeMember*>(take(all * sizeof(RidgeMember)));
+  t->pair = reinterpret_cast<float*>(take(static_cast<size_t>(ridge_rank_grid(P)) * ridge_rank_shares(P) * kRidgeCap * sizeof(float)));
+  return at;
 }
 
 static int pick_sub_tiles(int P, int64_t per_problem) {
@@ -886,8 +1110,14 @@ size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, 
     return (part + 255) / 256 * 256 + wide_scratch_bytes(model.mlp, P, pairs, lean);
   }
   if (model.kind == 1 && model.mlp.h_ridge) {
-    const size_t part = static_cast<size_t>(P) * ridge_blocks(P, C, per, segmented) * k * sizeof(unsigned long long);
-    return (part + 255) / 256 * 256 + ridge_scratch_bytes(P, C) + ridge_memo_bytes(P, C);
+    if (ridge_by_classes(P, C, segmented, lean)) {
+      RidgeTables t;
+      size_t cleared;
+      const size_t part = static_cast<size_t>(P) * ridge_rank_shares(P) * k * sizeof(unsigned long long);
+      return (part + 255) / 256 * 256 + ridge_tables(P, C, nullptr, &t, &cleared) + sizeof(RidgeProblem) * static_cast<size_t>(P);
+    }
+    const size_t part = static_cast<size_t>(P) * ridge_blocks(P, per) * k * sizeof(unsigned long long);
+    return (part + 255) / 256 * 256 + ridge_scratch_bytes(P, C) + ridge_memo_bytes(P, C, segmented);
   }
   const int st = pick_sub_tiles(P, per);
   int64_t nblk = (per + static_cast<int64_t>(st) * kBlock - 1) / (static_cast<int64_t>(st) * kBlock);
@@ -968,10 +1198,36 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
   }
   if (model.kind == 1 && model.mlp.h_ridge) {
-    // linear scorer: per-call tables of what a problem, a candidate and a class bring, then the kernel
-    // that adds and ranks
+    const RidgeParams& prm = *model.mlp.h_ridge;
+    ks_problem pv{};
+    if (p_by_value) pv = *p_by_value;
+    if (ridge_by_classes(P, C, d_seg_off != nullptr, wait->lean)) {
+      const int shares = ridge_rank_shares(P);
+      unsigned long long* partial = static_cast<unsigned long long*>(d_partial);
+      char* mem = static_cast<char*>(d_partial) + (static_cast<size_t>(P) * shares * k * sizeof(unsigned long long) + 255) / 256 * 256;
+      RidgeTables t;
+      size_t cleared;
+      RidgeProblem* d_prob = reinterpret_cast<RidgeProblem*>(mem + ridge_tables(P, C, mem, &t, &cleared));
+      cudaError_t e = cudaMemsetAsync(mem, 0, cleared, stream);
+      if (e != cudaSuccess) return e;
+      const dim3 all((C + 255) / 256, 16);
+      ridge_problem_kernel<<<(P + 127) / 128, 128, 0, stream>>>(desc, d_p, pv, p_by_value != nullptr, P, prm, d_prob, t.mask);
+      ridge_members_kernel<<<all, 256, 0, stream>>>(desc, d_c, C, prm, t);
+      ridge_classes_kernel<<<dim3(kRidgeCap / 256, 16), 256, 0, stream>>>(desc, d_c, t);
+      ridge_list_kernel<<<all, 256, 0, stream>>>(C, t);
+      if (ev_begin) cudaEventRecord(ev_begin, stream);
+      ridge_rank_kernel<<<dim3(ridge_rank_grid(P), shares), kRidgeRankThreads, 0, stream>>>(
+          desc, d_prob, P, d_c, C, prm, k, t, shares > 1 ? partial : nullptr, d_topk_idx, d_topk_score);
+      *launches += 5;
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+      if (ev_end) cudaEventRecord(ev_end, stream);
+      return shares > 1 ? launch_merge(partial, P, shares * k, k, d_topk_idx, d_topk_score, stream, launches) : cudaSuccess;
+    }
+    // per-call tables of what a problem, a candidate and (segments) a class bring, then the kernel that adds
+    // and ranks
     PairMap map = make_map(P, C, pairs, d_seg_off, d_seg_idx, kBlock);
-    map.nblk = ridge_blocks(P, C, per, d_seg_off != nullptr);
+    map.nblk = ridge_blocks(P, per);
     unsigned long long* partial = static_cast<unsigned long long*>(d_partial);
     const size_t part_bytes = (static_cast<size_t>(P) * map.nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
     char* mem = static_cast<char*>(d_partial) + part_bytes;
@@ -979,15 +1235,12 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     float2* d_tab = reinterpret_cast<float2*>(mem + 256);
     RidgeProblem* d_prob =
         reinterpret_cast<RidgeProblem*>(mem + 256 + (sizeof(float2) * 16 * static_cast<size_t>(C) + 255) / 256 * 256);
-    const RidgeParams& prm = *model.mlp.h_ridge;
-    ks_problem pv{};
-    if (p_by_value) pv = *p_by_value;
     cudaError_t e = cudaMemsetAsync(d_mask, 0, sizeof(unsigned), stream);
     if (e != cudaSuccess) return e;
     ridge_problem_kernel<<<(P + 127) / 128, 128, 0, stream>>>(desc, d_p, pv, p_by_value != nullptr, P, prm, d_prob, d_mask);
     ++*launches;
     MemoView memo{};
-    if (ridge_memo_bytes(P, C) != 0) {  // (never for a single problem)
+    if (ridge_memo_bytes(P, C, d_seg_off != nullptr) != 0) {  // (never for a single problem)
       memo = memo_view(mem + ridge_scratch_bytes(P, C), C);
       e = memo_clear(memo, stream);
       if (e != cudaSuccess) return e;
@@ -1005,11 +1258,9 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
       }
     }
     if (ev_begin) cudaEventRecord(ev_begin, stream);
-    const int group = ridge_group(d_seg_off != nullptr, P, C);
-    const unsigned blocks = static_cast<unsigned>(static_cast<int64_t>((P + group - 1) / group) * map.nblk);
-    auto kernel = !memo.keys ? &select_ridge_kernel<1, false>
-                  : group == 1 ? &select_ridge_kernel<1, true> : &select_ridge_kernel<kRidgeProblems, true>;
-    kernel<<<blocks, kRidgeThreads, 0, stream>>>(desc, d_prob, d_c, map, d_tab, prm, k, partial, memo);
+    auto kernel = memo.keys ? &select_ridge_kernel<true> : &select_ridge_kernel<false>;
+    kernel<<<static_cast<unsigned>(static_cast<int64_t>(P) * map.nblk), kRidgeThreads, 0, stream>>>(
+        desc, d_prob, d_c, map, d_tab, prm, k, partial, memo);
     ++*launches;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

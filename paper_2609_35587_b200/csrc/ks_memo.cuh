@@ -43,10 +43,11 @@ cudaError_t memo_clear(const MemoView& memo, cudaStream_t stream);
 cudaError_t memo_compact(const MemoView& memo, cudaStream_t stream);
 
 #ifdef __CUDACC__
-// Class of candidate i (of type combination `combo`, resident-block count b_eff), creating the
-// slot when the candidate is the first of its class.
-__device__ __forceinline__ unsigned memo_assign(const MemoView& memo, int combo, int i, const ks_candidate& cand,
-                                                long long b_eff) {
+// Slot of candidate i's class (resident-block count b_eff) in a table of kCap slots, taking a free one when
+// the candidate is the first of its class.
+template <int kCap>
+__device__ __forceinline__ unsigned memo_slot(unsigned long long* keys, int* reps, int i, const ks_candidate& cand,
+                                              long long b_eff) {
   if (!(cand.tile_m < 4096 && cand.tile_n < 4096 && cand.tile_k < 4096 && cand.cluster_m < 32 &&
         cand.cluster_n < 32 && b_eff >= 0 && b_eff < 64))
     return kNoClass;
@@ -55,15 +56,20 @@ __device__ __forceinline__ unsigned memo_assign(const MemoView& memo, int combo,
       (static_cast<unsigned long long>(cand.tile_k) << 24) | (static_cast<unsigned long long>(cand.stages) << 36) |
       (static_cast<unsigned long long>(cand.cluster_m) << 44) | (static_cast<unsigned long long>(cand.cluster_n) << 49) |
       (static_cast<unsigned long long>(b_eff) << 54);
-  unsigned long long* K = memo.keys + static_cast<size_t>(combo) * kMemoCap;
-  unsigned h = static_cast<unsigned>((key * 0x9E3779B97F4A7C15ull) >> 40) & (kMemoCap - 1);
+  unsigned h = static_cast<unsigned>((key * 0x9E3779B97F4A7C15ull) >> 40) & (kCap - 1);
   for (int probe = 0; probe < 64; ++probe) {
-    const unsigned long long prev = atomicCAS(K + h, 0ull, key);
-    if (prev == 0ull) memo.reps[static_cast<size_t>(combo) * kMemoCap + h] = i;  // this thread made the slot
+    const unsigned long long prev = atomicCAS(keys + h, 0ull, key);
+    if (prev == 0ull) reps[h] = i;  // this thread made the slot
     if (prev == 0ull || prev == key) return h;
-    h = (h + 1) & (kMemoCap - 1);
+    h = (h + 1) & (kCap - 1);
   }
   return kNoClass;
+}
+// The same in the walks' tables, for type combination `combo`.
+__device__ __forceinline__ unsigned memo_assign(const MemoView& memo, int combo, int i, const ks_candidate& cand,
+                                                long long b_eff) {
+  const size_t at = static_cast<size_t>(combo) * kMemoCap;
+  return memo_slot<kMemoCap>(memo.keys + at, memo.reps + at, i, cand, b_eff);
 }
 #endif
 

@@ -86,3 +86,37 @@ def test_problems_beyond_the_class_tables(ks, ctx, P, C):
         _, _, ref = oracle.select(prob[p:p + 1], cand, DESC, 5, mlp=mlp, want_scores=True)
         ok, msg = topk_accept(idx[p], sc[p], ref, np.arange(C, dtype=np.int32), 5, 1e-4)
         assert ok, (p, msg)
+
+
+@pytest.mark.parametrize("what,P,C,k", [("plain", 30, 20000, 10), ("plain", 1040, 600, 32), ("valid", 33, 61140, 7),
+                                        ("no class", 40, 15001, 10), ("ties", 32, 18755, 32), ("not finite", 32, 19000, 10),
+                                        ("many", 8200, 80, 3)])
+def test_classes_against_pairs(ks, ctx, what, P, C, k):
+    """A dense batch ranked by classes gives bit for bit what its pairs give one by one: the same pool as a
+    segment of every problem takes the kernel that adds up each pair. Candidates without a class (a
+    tile of 4,096 or more), equal scores everywhere, scores that are not finite; more problems than blocks."""
+    dev = torch.device("cuda", 0)
+    st = wl.feature_stats("cfg2")
+    mlp = wl.mlp_xavier(C, [64, 1], st["mu"], st["sigma"])
+    w = mlp["weights"][0]  # bf16 bits
+    if what == "ties":
+        w[:] = 0
+    if what == "not finite":
+        w[0, 46] = 0x7F80  # +inf on a candidate column: inf, -inf or (0 inf) not a number
+    model = ctx.model_create_mlp(mlp)
+    prob = wl.problems_batch(C, P, cross_precision=True)
+    if what == "valid":
+        rec, _, n = ctx.valid_catalogue(prob[:1], ks.KS_VALID_COUPLED)
+        C, d_c = min(C, n), rec[:min(C, n)].contiguous()
+    else:
+        cand = wl.candidates_full_grid(5, C)
+        if what == "no class":
+            cand["tile_m"][::50] = 4096
+        d_c = ks.to_device(cand, dev)
+    d_p = ks.to_device(prob, dev)
+    idx, sc = ctx.select(d_p, P, d_c, C, model, k)
+    off = torch.arange(P + 1, device=dev, dtype=torch.int64) * C
+    every = torch.arange(C, device=dev, dtype=torch.int32).repeat(P)
+    ridx, rsc = ctx.select(d_p, P, d_c, C, model, k, off, every, P * C)
+    assert torch.equal(idx, ridx)
+    assert torch.equal(sc.view(torch.int32), rsc.view(torch.int32))
