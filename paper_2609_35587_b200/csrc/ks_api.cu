@@ -131,7 +131,7 @@ ks_status read_status(ks_ctx* ctx) {
   const int v = *static_cast<volatile int*>(ctx->h_status);
   if (v != 0) {
     *ctx->h_status = 0;
-    // a failed launch may have left arrival counters of the slice mode behind
+    // a failed launch may have left arrival counters of the split walk behind
     if (ctx->d_words) cudaMemset(ctx->d_words, 0, sizeof(int) * ks::kWordServed);
     return static_cast<ks_status>(v);
   }
@@ -673,24 +673,21 @@ ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int 
   int32_t* pin_idx = static_cast<int32_t*>(ctx->pinned);
   float* pin_sc = reinterpret_cast<float*>(pin_idx + KS_MAX_K);
 
-  // Latency path for a qualifying tree model: the trees are split over several CTAs per
-  // candidate block, the last block writes the k results straight into mapped host memory.
+  // Latency path for a qualifying tree model: the machine's CTAs share out the blocks' trees, the last
+  // block writes the k results straight into mapped host memory.
   if (model->kind == 0 && model->gbdt.fast && C > 0) {
     const int NC = model->gbdt.block_cands;
     const int nblk = (C + NC - 1) / NC;
-    const int S = ks::fast_slices(model->gbdt, nblk);
-    if (S > 1) {
+    if (ks::fast_splits(model->gbdt, nblk)) {
       const size_t b_part = align_up(sizeof(unsigned long long) * nblk * k);
       // scratch of this path: the prepared tiles, one per candidate block (no per-call table)
       const size_t b_scratch = align_up(static_cast<size_t>(nblk) * model->gbdt.n_qrows * NC);
-      const size_t b_scores = align_up(sizeof(float) * static_cast<size_t>(S) * C);
+      const size_t b_scores = align_up(ks::fast_split_bytes(model->gbdt));
       ks_status s = ensure_workspace(ctx, b_part + b_scratch + b_scores);
       if (s != KS_OK) return s;
       char* base = static_cast<char*>(ctx->ws);
-      ks::FastSlice sl;
-      sl.n_slices = S;
-      sl.pairs = C;
-      sl.scores = reinterpret_cast<float*>(base + b_part + b_scratch);
+      ks::FastSplit sl;
+      sl.scores = reinterpret_cast<double*>(base + b_part + b_scratch);
       sl.out_idx = ctx->d_pinned_idx;
       sl.out_score = ctx->d_pinned_score;
       sl.tiles = reinterpret_cast<uint8_t*>(base + b_part);
@@ -711,7 +708,7 @@ ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int 
       }
       if (e != cudaSuccess) return cuda_fail(ctx, e, "ks_select_one");
       s = read_status(ctx);
-      if (s != KS_OK) return s;  // (with the slice mode's counters cleared)
+      if (s != KS_OK) return s;  // (with the split walk's counters cleared)
       std::memcpy(h_topk_idx, pin_idx, k * sizeof(int32_t));
       std::memcpy(h_topk_score, pin_sc, k * sizeof(float));
       return KS_OK;
@@ -749,13 +746,12 @@ ks_status ks_catalogue_prepare(ks_ctx* ctx, const ks_candidate* d_c, int C, cons
   const ks::GbdtModel& g = model->gbdt;
   if (model->kind == 0 && g.fast && C > 0) {
     const int nblk = (C + g.block_cands - 1) / g.block_cands;
-    const int S = ks::fast_slices(g, nblk);
     const size_t b_memo = ks::fast_prepared_memo_bytes(g, C);
-    if (S > 1 && b_memo > 0) {
+    if (ks::fast_splits(g, nblk) && b_memo > 0) {
       DeviceGuard guard(ctx->device);
       const size_t b_rows = align_up(ks::fast_prepared_rows_bytes(g, C));
       const size_t b_part = align_up(sizeof(unsigned long long) * nblk * KS_MAX_K);
-      const size_t b_scores = align_up(sizeof(float) * static_cast<size_t>(S) * C);
+      const size_t b_scores = align_up(ks::fast_split_bytes(g));
       cat->off_memo = b_rows;
       cat->off_part = b_rows + align_up(b_memo);
       cat->off_scores = cat->off_part + b_part;
@@ -775,7 +771,6 @@ ks_status ks_catalogue_prepare(ks_ctx* ctx, const ks_candidate* d_c, int C, cons
         return cuda_fail(ctx, e, "ks_catalogue_prepare");
       }
       cat->nblk = nblk;
-      cat->slices = S;
       cat->prepared = true;
     }
   }
@@ -805,10 +800,8 @@ ks_status ks_select_one_prepared(ks_ctx* ctx, const ks_catalogue* cat, ks_proble
   float* pin_sc = reinterpret_cast<float*>(pin_idx + KS_MAX_K);
   char* base = static_cast<char*>(cat->d_mem);
   const ks::GbdtModel& gm = cat->model->gbdt;
-  ks::FastSlice sl{};
-  sl.n_slices = cat->slices;
-  sl.pairs = cat->C;
-  sl.scores = reinterpret_cast<float*>(base + cat->off_scores);
+  ks::FastSplit sl{};
+  sl.scores = reinterpret_cast<double*>(base + cat->off_scores);
   sl.out_idx = ctx->d_pinned_idx;
   sl.out_score = ctx->d_pinned_score;
   sl.tiles = nullptr;

@@ -834,13 +834,7 @@ __device__ bool compile_class(const ClassArgs& a, ClassShared& sh, BuildShared* 
 // suspended by the barrier itself, not put to sleep for a fixed time.
 __device__ __forceinline__ bool chunk_wait(uint32_t bar, uint32_t parity, int limit, volatile int* fail) {
   for (int i = 0; i < limit; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
+    if (mbar_try_wait(bar, parity)) return true;
     if ((i & 63) == 63 && *fail) return false;
   }
   return false;

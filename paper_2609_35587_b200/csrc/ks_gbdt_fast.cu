@@ -27,8 +27,8 @@
 //   (see MemoView).
 //
 // Other entries into the same walk
-//   single-problem call: the trees are split over several CTAs per candidate block (slices),
-//   the tiles are built once by tile_pairs_kernel; scoring call (ks_score): tiles are quantised
+//   few candidate blocks (a single problem, a short list): the machine's CTAs share out the trees of all
+//   blocks evenly (split walk); scoring call (ks_score): tiles are quantised
 //   from given feature rows by tile_rows_kernel and the scores are stored instead of ranked.
 //
 // Kernel (an item = one problem x up to NC candidates; a CTA of THREADS threads serves one item,
@@ -78,23 +78,45 @@ constexpr int kNBuf = 2;                // buffers of a ring (four of 8 KB and t
 // shared memory map (byte offsets from the dynamic shared base): the rings' chunk buffers, then the tile
 constexpr int kOffBuf0 = 0;
 
-// Slice mode (single-problem latency call): the trees are split over n_slices CTAs per
-// candidate block. Every CTA stores its partial scores; the last CTA to arrive for a block
-// (atomic counter, nobody waits) adds the slices in a fixed order and ranks the block; the
-// last block overall merges the lists and writes the final result.
-struct SliceArgs {
-  int n_slices;            // 1 = every CTA walks the whole ensemble
-  long long pairs;         // rows of the partial-score planes
-  float* scores;           // [n_slices][pairs] partial scores
-  int* words;              // the context's device words: the blocks' counters (reset by their last users), kWordWalk
-  int32_t* out_idx;        // single-problem form only: [k] final result (device-visible, may be
-  float* out_score;        // mapped host memory); null when a merge kernel follows
-  const uint8_t* tiles;    // prepared tiles [blocks][rows][NC] (tile_pairs_kernel), or null
-  int* out_seq;            // single-problem form: receives `seq` once the k results are written
+// Split walk: where there are too few candidate blocks for whole rounds of the machine's CTAs, the blocks'
+// trees lie on one line, block after block, and every CTA takes an equal stretch of it. A stretch's ends fall
+// inside blocks: such a part's sums go to memory, and the last CTA to arrive at a block (atomic counter,
+// nobody waits) adds its parts in order and ranks it. In a single-problem call the last block overall
+// merges the lists and writes the final result. Where a block is cut depends on where it lies, a
+// candidate's score must not (equal candidates tie, whatever their places): a chunk's trees are added up in
+// 32 bits, in a fixed order, and the chunks' sums in 64, where their order leaves no trace in the result.
+//
+// The line is measured in trees, a block's beginning with `fill` trees' worth for its tile; a CTA that starts
+// inside a block fills its tile too, but that holds for nearly all of them. Trees are dealt in units of
+// one chunk a ring. CTA c begins at the unit that holds point c * total / gridDim.x.
+struct SplitArgs {
+  int units;            // of a block; 0: CTAs take whole blocks
+  int unit, fill;       // trees of a unit, and what filling a tile counts for
+  long long blocks;
+  double* scores;       // [CTAs][2][NC]: sums of a CTA's first and last part
+  int* words;           // the context's device words: arrival counters, by the first CTA of a block (reset by their last users), kWordWalk
+  int32_t* out_idx;     // single-problem form only: [k] final result (device-visible, may be
+  float* out_score;     // mapped host memory); null when a merge kernel follows
+  const uint8_t* tiles; // prepared tiles [blocks][rows][NC] (tile_pairs_kernel, tile_rows_kernel), or null
+  int* out_seq;         // single-problem form: receives `seq` once the k results are written
   int seq;
-  float* score_out;        // scoring call (ks_score): the scores of the block's rows go here, no ranking
-  int repeat;              // floor measurement only: passes over the resident chunks
+  float* score_out;     // scoring call (ks_score): the scores of the block's rows go here, no ranking
+  int repeat;           // floor measurement only: passes over the resident chunks
 };
+__host__ __device__ __forceinline__ long long split_block(const SplitArgs& s) { return s.fill + static_cast<long long>(s.units) * s.unit; }
+// first unit (of all blocks') of CTA c of n
+__host__ __device__ __forceinline__ long long split_start(const SplitArgs& s, long long c, long long n) {
+  const long long len = split_block(s), x = c * (s.blocks * len) / n, block = x / len, in = x - block * len - s.fill;
+  return block * s.units + (in > 0 ? in / s.unit : 0);
+}
+// the CTAs that hold the first and the last unit of a block: the largest c whose start is not behind it
+__host__ __device__ __forceinline__ int split_first(const SplitArgs& s, long long block, long long n) {
+  const long long len = split_block(s);
+  return static_cast<int>(((block * len + s.fill + s.unit) * n - 1) / (s.blocks * len));
+}
+__host__ __device__ __forceinline__ int split_last(const SplitArgs& s, long long block, long long n) {
+  return static_cast<int>(((block + 1) * split_block(s) * n - 1) / (s.blocks * split_block(s)));
+}
 
 // ------------------------------------------------------------------------------------------
 // candidate-only rows, once per call
@@ -317,7 +339,7 @@ __device__ __forceinline__ void tile_column(const FeatQ& q, float4 x, uint32_t t
 // Slots past the catalogue get the last candidate's bytes (they are not ranked). Also clears the abort flag
 // (this kernel precedes the select kernel). What bounds it is the latency of the columns' divisions and of
 // the searches. One problem x 61,140 candidates, 500 trees: 29 us, where a thread that wrote its candidate's
-// bytes one by one took 72. Every split walk of a dense batch takes its tiles from here: left to the slices,
+// bytes one by one took 72. Every split walk of a dense batch takes its tiles from here: left to the parts of a block,
 // each computed the per-pair columns again (10 problems x 934 candidates, 326 trees: 125 -> 48 us the whole call;
 // 64 x 2,048 candidates, 100 trees: 161 -> 120, with the memo in its place 143; four calls of one problem with
 // its 61,140 valid candidates: 900 -> 677).
@@ -337,6 +359,7 @@ tile_pairs_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem
   __shared__ float s_pf[64];
   float* s_thr = s_x + kTileCols * kTileRows;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the walk waits for this grid before it reads the tiles)
   if (blockIdx.x == 0 && tid == 0) words[kWordWalk] = 0;
   const long long n_items = static_cast<long long>(P) * groups;
   const int begin = static_cast<int>(n_items * blockIdx.x / gridDim.x);
@@ -408,6 +431,7 @@ tile_rows_kernel(const float* __restrict__ feat, int64_t rows, FastView fv, uint
   __shared__ FeatQ s_fq[64];
   float* s_thr = s_x + 64 * kTileRows;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the walk waits for this grid before it reads the tiles)
   if (blockIdx.x == 0 && threadIdx.x == 0) words[kWordWalk] = 0;
   stage_thresholds(fv, 0, fv.n_thr, s_thr, fv.n_thr);
   if (threadIdx.x < 64) s_fq[threadIdx.x] = fv.feat[threadIdx.x];
@@ -576,6 +600,13 @@ __device__ __noinline__ void fill_tile(const ks_gpu_desc& desc, const ProblemTer
 // the kernel
 // ------------------------------------------------------------------------------------------
 
+// Bounded wait for a tile that is copied in one piece: the thread is suspended by the barrier itself.
+__device__ __forceinline__ bool tile_wait(uint32_t bar, uint32_t parity, int limit) {
+  for (int i = 0; i < limit; ++i)
+    if (mbar_try_wait(bar, parity)) return true;
+  return false;
+}
+
 // bytes of `a` where the top bit of the matching byte of `m` is set, else bytes of `b`
 __device__ __forceinline__ uint32_t byte_select(uint32_t m, uint32_t a, uint32_t b) {
   const uint32_t f = __byte_perm(m, 0u, 0xBA98u);  // top bit of every byte replicated over the byte
@@ -622,18 +653,20 @@ __device__ __forceinline__ uint32_t path_step(uint32_t a, uint32_t cb_r, uint32_
 // levels' constants travel as one 32-bit word per node (row offset << 8 | j + 1) instead of a
 // (row offset, replicated j + 1) pair, so that twice as many trees keep their word-wise levels.
 // THREADS threads rank NC candidates: NC / 4 words times THREADS / (NC / 4) tree groups.
+// kSplit: the CTAs share out the blocks' trees (SplitArgs); a form of its own, since what it keeps slowed the
+// other by 2 %.
 // kFloor (measurement only): the walk without its chunk rings. Every tree group's first kNBuf
 // chunks are copied once and stay resident; the group walks them again and again (sl.repeat
 // times as many chunk walks as it has chunks), never waits, releases or refills, so the time per
 // pass is that of the gather and instruction stream of the walk alone, at the occupancy and tile
 // size of the real kernel.
-template <int L, int NP, bool kCompact, int THREADS, int NC, bool kFloor = false>
+template <int L, int NP, bool kCompact, int THREADS, int NC, bool kSplit, bool kFloor = false>
 __global__ void __launch_bounds__(THREADS, THREADS <= 256 ? 2 : 1)
 select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value,
                    const ks_candidate* __restrict__ c, int P, int C, int nblk, int rows_per_cta,
                    const int64_t* __restrict__ seg_off, const int32_t* __restrict__ seg_idx, FastView fv,
                    int k, unsigned long long* __restrict__ partial, int* __restrict__ status,
-                   SliceArgs sl, int n_items, const __grid_constant__ FastTopParams top) {
+                   SplitArgs sl, int n_items, const __grid_constant__ FastTopParams top) {
   constexpr int W = NC / 4;        // words per tile row = lane slots
   constexpr int G = THREADS / W;   // tree groups
   constexpr int RG = ring_count(G);  // chunk rings
@@ -643,40 +676,36 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
   __shared__ ProblemTerms s_pt;
   __shared__ unsigned long long s_warp[THREADS / 32 * KS_MAX_K];
   __shared__ unsigned long long s_list[KS_MAX_K];
-  __shared__ __align__(8) unsigned long long s_bar[kNBuf * RG];  // [ring][buffer]
+  __shared__ __align__(8) unsigned long long s_bar[kNBuf * RG + 1];  // [ring][buffer], then the tile's
   __shared__ FeatQ s_fq[64];
   __shared__ uint8_t s_pbin[kFastMaxProbRows];
   __shared__ float s_pfeat[64];
-  __shared__ int s_fail, s_last, s_done[kNBuf * RG], s_abort, s_pending[kNBuf * RG];
+  __shared__ int s_fail, s_last, s_done[kNBuf * RG], s_abort, s_pending[kNBuf * RG], s_parts[3];
   // the classes of the candidates whose candidate-only rows the tile holds (one-CTA forms only:
   // there a CTA serves one candidate block for many problems in a row, see below)
   __shared__ unsigned s_cid[THREADS > 256 && NC == 1024 ? NC : 1];
 
   const int tid = threadIdx.x;
   const int kOffTile = kNBuf * RG * fv.buf_bytes;  // every ring has kNBuf buffers
-  const int S = sl.n_slices;
   const uint32_t sbase = smem_u32(smem);
   const uint32_t bar0 = smem_u32(&s_bar[0]);  // barrier of buffer b: bar0 + 8 b
   const bool tiles_given = sl.tiles != nullptr;  // the tiles were built in front: no feature work here
   if (tid == 0) {
-    for (int b = 0; b < kNBuf * RG; ++b) mbar_init(bar0 + 8u * b, 1);
+    for (int b = 0; b <= kNBuf * RG; ++b) mbar_init(bar0 + 8u * b, 1);
     s_fail = 0;
     for (int b = 0; b < kNBuf * RG; ++b) s_done[b] = s_pending[b] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid < 64) s_fq[tid] = fv.feat[tid];
   __syncthreads();
-  // everything above is independent of the kernel in front (the per-problem tables): when this
-  // grid was launched as its programmatic dependent, wait for that grid here
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   uint32_t phases = 0;  // bit b: parity of buffer b's barrier
   const int word = tid % W, grp = tid / W;
   volatile int* v_fail = &s_fail;
 
-  // An item is one (problem, candidate block, tree slice). The batch form of a geometry that holds one CTA per SM is
+  // An item is one (problem, candidate block). The batch form of a geometry that holds one CTA per SM is
   // launched with one CTA per SM, so that a CTA's set-up and the gap between two CTAs are paid
-  // once, not per item; everything else (two CTAs per SM, which hide each other's gaps; tree
-  // slices and scoring, which leave an item early) is launched with one CTA per item.
+  // once, not per item; so is a split walk, whose CTAs take parts of items. Two CTAs per SM hide each
+  // other's gaps: there a batch is launched with one CTA per item.
   // A CTA (of the 1,024-candidate forms) that serves many items of a dense batch takes a run of
   // consecutive items in the order (candidate block, problem): successive items then are the same
   // candidates for another problem, and while the element types stay the same their
@@ -684,15 +713,27 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
   // batches in the benchmark; compiled with this path it ran them 2 % slower, so it keeps the
   // plain order.)
   const int grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
-  const bool block_major = NC == 1024 && grid < n_items && !seg_off && S == 1;
+  constexpr bool split = kSplit;
+  const bool block_major = NC == 1024 && grid < n_items && !seg_off && !tiles_given;
   const int per_cta = (n_items + grid - 1) / grid;
-  const int first_item = block_major ? cta * per_cta : cta, item_step = block_major ? 1 : grid;
-  const int last_item = block_major ? (first_item + per_cta < n_items ? first_item + per_cta : n_items) : n_items;
+  long long unit = split ? split_start(sl, cta, grid) : 0;  // a split walk: the next unit
+  const long long unit_first = unit, unit_end = split ? split_start(sl, cta + 1, grid) : 0;
+  int first_item = block_major ? cta * per_cta : cta, item_step = block_major ? 1 : grid;
+  int last_item = block_major ? (first_item + per_cta < n_items ? first_item + per_cta : n_items) : n_items;
+  if (split) {
+    first_item = static_cast<int>(unit / sl.units);
+    item_step = 1;
+    last_item = static_cast<int>((unit_end + sl.units - 1) / sl.units);
+  }
   int held_chunk = -1, held_combo = -1;  // what the tile's candidate-only rows belong to
+  uint32_t tile_phase = 0;
+  // everything above is independent of the kernel in front (the per-problem tables): when this
+  // grid was launched as its programmatic dependent, wait for that grid here
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll 1
   for (int item = first_item; item < last_item; item += item_step) {
-  const int prob = block_major ? item % P : item / (nblk * S);
-  const int chunk = block_major ? item / P : (item / S) % nblk, slice = item % S;
+  const int prob = block_major ? item % P : item / nblk;
+  const int chunk = block_major ? item / P : item % nblk;
   // rows of this problem: lo = where its scores sit in per-row arrays; lo_idx = where its pool
   // indices start in seg_idx (per-problem segments, or - without offsets - one ranking order of
   // the whole catalogue shared by every problem)
@@ -706,8 +747,15 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     len = C;
   }
   // chunks of the ensemble this CTA walks
-  const int ch_begin = static_cast<int>(static_cast<int64_t>(fv.n_chunks) * slice / S);
-  const int ch_end = static_cast<int>(static_cast<int64_t>(fv.n_chunks) * (slice + 1) / S);
+  int ch_begin = 0, ch_end = fv.n_chunks;
+  const bool first_part = unit == unit_first;
+  if (split) {
+    const long long block0 = static_cast<long long>(item) * sl.units;
+    ch_begin = static_cast<int>(unit - block0) * RG;
+    unit = unit_end < block0 + sl.units ? unit_end : block0 + sl.units;
+    ch_end = static_cast<int>(unit - block0) * RG < fv.n_chunks ? static_cast<int>(unit - block0) * RG : fv.n_chunks;
+  }
+  const bool whole = ch_begin == 0 && ch_end == fv.n_chunks;
   __syncthreads();  // the item before this one is finished with the shared state
   if (tid == 0) {
     if (!tiles_given && !fv.prob_tab) {
@@ -726,7 +774,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
   __syncthreads();
   if (s_abort) {  // a wait ran out in an earlier CTA of this call, which fails, or the class walk serves the call: leave at once
     if (s_abort == kLeaveFailed && tid == 0 && status) atomicExch(status, KS_ERR_TIMEOUT);
-    if (tid < k && slice == 0 && partial) partial[(static_cast<size_t>(prob) * nblk + chunk) * k + tid] = 0ull;
+    if (tid < k && partial) partial[(static_cast<size_t>(prob) * nblk + chunk) * k + tid] = 0ull;
     return;
   }
   if (!tiles_given && !fv.prob_tab && tid < KS_F && feat_class(tid) == 0) {
@@ -736,17 +784,47 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
              [&](int row, uint8_t b) { s_pbin[KS_IDX(row - first, kFastMaxProbRows)] = b; });
   }
 
+  bool ranked = !sl.score_out;
   for (int64_t start = static_cast<int64_t>(chunk) * rows_per_cta; start < len;
        start += static_cast<int64_t>(nblk) * rows_per_cta) {
     const int64_t stop = (start + rows_per_cta < len) ? start + rows_per_cta : len;
     // ---- phase A ---------------------------------------------------------------------------------
     __syncthreads();
-    if (sl.tiles) {
-      // the block's tile was built once for all the CTAs that share it
-      const uint4* src =
-          reinterpret_cast<const uint4*>(sl.tiles + (static_cast<size_t>(prob) * nblk + chunk) * fv.n_rows * NC);
-      uint4* dst = reinterpret_cast<uint4*>(smem + kOffTile);
-      for (int i = tid; i < fv.n_rows * (NC / 16); i += THREADS) dst[i] = __ldcg(src + i);
+    // The first chunks are on their way while the tile is filled, where the fill leaves the chunk buffers alone.
+    const auto start_rings = [&] {
+      // ring g takes the chunks ch_begin + g, ch_begin + g + RG, ... through its own buffers
+      for (int g = 0; g < RG; ++g)
+        for (int b = 0; b < kNBuf && ch_begin + g + b * RG < ch_end; ++b) {
+          const int rb = g * kNBuf + b;
+          // test hook: a barrier armed for more bytes than its copy brings never completes
+          mbar_expect_tx(bar0 + 8u * rb, fv.chunk_bytes + (fv.starve ? 16 : 0));
+          bulk_copy_g2s(sbase + kOffBuf0 + rb * fv.buf_bytes,
+                        reinterpret_cast<const char*>(fv.chunks) + static_cast<size_t>(ch_begin + g + b * RG) * fv.chunk_bytes,
+                        fv.chunk_bytes, bar0 + 8u * rb);
+          s_pending[rb] = 1;
+        }
+    };
+    const bool early = tiles_given || fv.pair_class;
+    if (early && tid == 0) {
+      fence_async_proxy();
+      if (tiles_given) {
+        // the block's tile was built in front, in one piece
+        const uint32_t bar = bar0 + 8u * (kNBuf * RG), bytes = static_cast<uint32_t>(fv.n_rows) * NC;
+        asm volatile("fence.proxy.async.global;" ::: "memory");  // (written by ordinary stores of the kernel in front)
+        mbar_expect_tx(bar, bytes);
+        bulk_copy_g2s(sbase + kOffTile, sl.tiles + (static_cast<size_t>(prob) * nblk + chunk) * bytes, bytes, bar);
+      }
+      start_rings();
+    }
+    bool tile_late = false;
+    if (tiles_given) {
+      if (!tile_wait(bar0 + 8u * (kNBuf * RG), tile_phase, fv.wait_limit)) {
+        tile_late = true;
+        s_fail = 1;
+        atomicExch(sl.words + kWordWalk, kLeaveFailed);
+        if (status) atomicExch(status, KS_ERR_TIMEOUT);
+      }
+      tile_phase ^= 1u;
     } else {
       // thresholds of the per-pair features: into the idle chunk buffers when they fit
       const float* T = stage_thresholds(fv, 0, fv.thr_cand0, reinterpret_cast<float*>(smem + kOffBuf0),
@@ -762,21 +840,12 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     __syncthreads();  // tile complete; the threshold table is no longer needed
 
     // ---- phase B ---------------------------------------------------------------------------------
-    if (tid == 0) {
+    if (!early && tid == 0) {
       fence_async_proxy();
-      // ring g takes the chunks ch_begin + g, ch_begin + g + RG, ... through its own buffers
-      for (int g = 0; g < RG; ++g)
-        for (int b = 0; b < kNBuf && ch_begin + g + b * RG < ch_end; ++b) {
-          const int rb = g * kNBuf + b;
-          // test hook: a barrier armed for more bytes than its copy brings never completes
-          mbar_expect_tx(bar0 + 8u * rb, fv.chunk_bytes + (fv.starve ? 16 : 0));
-          bulk_copy_g2s(sbase + kOffBuf0 + rb * fv.buf_bytes,
-                        reinterpret_cast<const char*>(fv.chunks) + static_cast<size_t>(ch_begin + g + b * RG) * fv.chunk_bytes,
-                        fv.chunk_bytes, bar0 + 8u * rb);
-          s_pending[rb] = 1;
-        }
+      start_rings();
     }
     float score[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    double sums[4] = {0.0, 0.0, 0.0, 0.0};  // split walk: of the chunks' sums
     const uint32_t cb = sbase + kOffTile + word * 4;
     const int tpc = fv.tpc, grp_trees = (tpc + GPR - 1) / GPR;
     const int np = NP >= 0 ? NP : fv.depth - L;
@@ -880,6 +949,13 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
           score[r] += lds_f32(a[r]);
         }
       }
+      if (split) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          sums[r] += static_cast<double>(score[r]);
+          score[r] = 0.0f;
+        }
+      }
       // Release the buffer without a block-wide barrier: every warp of the group counts itself
       // out, and the last one to leave refills the buffer (nobody waits; warps may run a chunk ahead).
       __syncwarp();
@@ -903,11 +979,12 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     if (*v_fail) {
       // The call has failed. Before this CTA gives its shared memory back, give the copies that
       // may still be in flight the time to land (bounded again); the test hook's copies land in
-      // full although their barriers never complete, so there a short pause stands in for it.
+      // full although their barriers never complete, so there a short pause stands in for it (and so it does
+      // for a tile whose wait ran out).
       if (word == 0 && grp % GPR == 0) {  // one thread per ring, for its ring's buffers (it knows their parities)
         for (int b = 0; b < kNBuf; ++b) {
           if (!s_pending[ring * kNBuf + b]) continue;
-          if (fv.starve) {
+          if (fv.starve || tile_late) {
             for (int i = 0; i < 64; ++i) __nanosleep(kSleepNs);
           } else {
             mbar_wait_bounded(bar0 + 8u * (ring * kNBuf + b), (phases >> b) & 1u, fv.wait_limit, &s_abort /* stays 0 */);
@@ -915,24 +992,73 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
         }
       }
       __syncthreads();
-      if (tid < k && slice == 0 && partial) partial[(static_cast<size_t>(prob) * nblk + chunk) * k + tid] = 0ull;
+      if (tid < k && partial) partial[(static_cast<size_t>(prob) * nblk + chunk) * k + tid] = 0ull;
       return;
     }
 
     // ---- phase C ---------------------------------------------------------------------------------
-    float* s_part = reinterpret_cast<float*>(smem + kOffBuf0);  // [G - 1][4][W], buffers are idle now
-    if (grp > 0) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r) s_part[((grp - 1) * 4 + r) * W + word] = score[r];
-    }
-    __syncthreads();
-    // this thread's sum over the groups, in a fixed order
+    // this thread's sum over the groups, in a fixed order; the buffers are idle now
     float total[4];
+    if (split) {
+      double* s_part = reinterpret_cast<double*>(smem + kOffBuf0);  // [G - 1][4][W]
+      if (grp > 0) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      total[r] = score[r];
-      if (grp == 0)
-        for (int g = 1; g < G; ++g) total[r] += s_part[((g - 1) * 4 + r) * W + word];
+        for (int r = 0; r < 4; ++r) s_part[((grp - 1) * 4 + r) * W + word] = sums[r];
+      }
+      __syncthreads();
+      if (grp == 0) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          for (int g = 1; g < G; ++g) sums[r] += s_part[((g - 1) * 4 + r) * W + word];
+      }
+      if (!whole) {
+        // publish this part's sums, let the last arrival finish the block
+        double2* to = reinterpret_cast<double2*>(sl.scores + (2 * static_cast<size_t>(cta) + (first_part ? 0 : 1)) * NC + 4 * word);
+        if (grp == 0) {
+          __stcg(to, make_double2(sums[0], sums[1]));
+          __stcg(to + 1, make_double2(sums[2], sums[3]));
+        }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+          const int c0 = split_first(sl, item, grid), n = split_last(sl, item, grid) - c0 + 1;
+          s_parts[0] = c0;
+          s_parts[1] = n;
+          s_parts[2] = split_start(sl, c0, grid) < static_cast<long long>(item) * sl.units ? 1 : 0;  // its last part
+          s_last = atomicAdd(sl.words + c0, 1) == n - 1;
+          if (s_last) sl.words[c0] = 0;  // nobody else touches this counter again in this launch
+        }
+        __syncthreads();
+        if (!s_last) {
+          ranked = false;
+          continue;
+        }
+        __threadfence();
+        if (grp == 0) {
+          const double* from = sl.scores + 2 * static_cast<size_t>(s_parts[0]) * NC + 4 * word;
+          sums[0] = sums[1] = sums[2] = sums[3] = 0.0;
+          for (int q = 0; q < s_parts[1]; ++q) {
+            const double2* p2 = reinterpret_cast<const double2*>(from + (2 * q + (q == 0 ? s_parts[2] : 0)) * NC);
+            const double2 u = __ldcg(p2), v = __ldcg(p2 + 1);
+            sums[0] += u.x; sums[1] += u.y; sums[2] += v.x; sums[3] += v.y;
+          }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) total[r] = static_cast<float>(sums[r]);
+    } else {
+      float* s_part = reinterpret_cast<float*>(smem + kOffBuf0);  // [G - 1][4][W]
+      if (grp > 0) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) s_part[((grp - 1) * 4 + r) * W + word] = score[r];
+      }
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        total[r] = score[r];
+        if (grp == 0)
+          for (int g = 1; g < G; ++g) total[r] += s_part[((g - 1) * 4 + r) * W + word];
+      }
     }
     if (sl.score_out) {
       // scoring call: the scores are the result (same order of additions as the ranking path)
@@ -943,24 +1069,6 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
       }
       continue;
     }
-    if (S > 1) {
-      // slice mode: publish this CTA's partial scores, let the last arrival finish the block
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int64_t row = start + 4 * word + r;
-        if (grp == 0 && row < stop) __stcg(sl.scores + static_cast<size_t>(slice) * sl.pairs + lo + row, total[r]);
-      }
-      __threadfence();
-      __syncthreads();
-      if (tid == 0) {
-        int* cnt = sl.words + static_cast<size_t>(prob) * nblk + chunk;
-        s_last = atomicAdd(cnt, 1) == S - 1;
-        if (s_last) *cnt = 0;  // nobody else touches this counter again in this launch
-      }
-      __syncthreads();
-      if (!s_last) return;
-      __threadfence();
-    }
     unsigned long long keys[5];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -968,30 +1076,23 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
       // byte r of word `word` is row 4 word + r of the block
       const int64_t row = start + 4 * word + r;
       if (grp == 0 && row < stop) {
-        float s;
-        if (S > 1) {
-          s = fv.base;
-          for (int q = 0; q < S; ++q) s += __ldcg(sl.scores + static_cast<size_t>(q) * sl.pairs + lo + row);
-        } else {
-          s = fv.base + total[r];
-        }
-        keys[r] = make_key(s + 0.0f, seg_idx ? seg_idx[lo_idx + row] : static_cast<int>(row));
+        keys[r] = make_key((fv.base + total[r]) + 0.0f, seg_idx ? seg_idx[lo_idx + row] : static_cast<int>(row));
       }
     }
     keys[4] = tid < k ? s_list[tid] : 0ull;
     __syncthreads();
     block_topk<5>(keys, k, s_warp, s_list);
   }
-  if (sl.score_out) return;
+  if (!ranked) continue;
   if (tid < k)
     partial[KS_IDX((static_cast<size_t>(prob) * nblk + chunk) * k + tid, static_cast<size_t>(P) * nblk * k)] = s_list[tid];
-  if (S > 1 && sl.out_idx) {
+  if (sl.out_idx) {
     // single-problem form: the last block to finish merges the per-block lists
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(sl.words + nblk, 1) == nblk - 1;
+    if (tid == 0) s_last = atomicAdd(sl.words + kMaxShares, 1) == nblk - 1;
     __syncthreads();
-    if (!s_last) return;
+    if (!s_last) continue;
     __threadfence();
     // the whole CTA ranks the nblk * k keys (each key is read once)
     const int n_keys = nblk * k;
@@ -1013,7 +1114,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     }
     __syncthreads();
     if (tid == 0) {
-      sl.words[nblk] = 0;
+      sl.words[kMaxShares] = 0;
       if (sl.out_seq) {  // the results are in place: tell the host, which polls this word
         __threadfence_system();
         *reinterpret_cast<volatile int*>(sl.out_seq) = sl.seq;
@@ -1193,6 +1294,8 @@ cudaError_t build_fast_gbdt(GbdtModel& m, int n_trees, const int64_t* off, const
   const int group_buf = geom.buf_bytes / rings / 16 * 16;
   int tpc = group_buf / (per_tree_words * 4) / gpr * gpr;
   if (tpc < gpr) return cudaSuccess;
+  // (eight trees a thread are enough to hide a chunk's beginning and end; more only make a split walk's units coarse)
+  tpc = std::min(tpc, 8 * gpr);
   if (tpc > (n_trees + G - 1) / G * gpr) tpc = (n_trees + G - 1) / G * gpr;  // a small ensemble: one short chunk per ring
   const int n_chunks = (n_trees + tpc - 1) / tpc;
   const int chunk_words = (tpc * per_tree_words + 3) / 4 * 4;  // bulk copies move multiples of 16 bytes
@@ -1327,7 +1430,7 @@ void free_fast_gbdt(GbdtModel& m) {
 
 // Blocks per problem: full tiles of the model's block size. A block's cost does not depend on how
 // many of its slots are live, so an under-filled machine is filled by splitting the trees over
-// several CTAs per block (slices) rather than by shorter blocks.
+// several CTAs per block (split walk) rather than by shorter blocks.
 void fast_tiling(const GbdtModel& g, int P, int64_t per_problem, int* nblk, int* rows_per_cta) {
   int64_t n = (per_problem + g.block_cands - 1) / g.block_cands;
   if (n < 1) n = 1;
@@ -1387,27 +1490,31 @@ size_t fast_memo_bytes(const GbdtModel& g, int P, int C) {
   return memo_fixed_bytes(C) + static_cast<size_t>(batch) * (static_cast<size_t>(kMemoCap) * pair_rec_bytes(g) + kProbRec);
 }
 
-// Slice count of the single-problem call: the trees are split over S CTAs per candidate block.
-// A CTA costs its tile fill (about 0.15 of a whole-ensemble walk of its block) plus 1 / S of that
-// walk, and blocks x S CTAs run in waves of the CTAs the machine holds at once: the S with the
-// shortest estimated makespan wins.
-int fast_slices(const GbdtModel& g, int64_t blocks) {
-  if (blocks < 1) blocks = 1;
-  if (blocks > kMaxSliceBlocks) return 1;
-  const int64_t slots = static_cast<int64_t>(g.ctas_per_sm) * kSmCount;
-  if (blocks >= slots) return 1;  // the machine is full without slices
-  int best = 1;
-  double best_cost = 1e30;
-  for (int s = 1; s <= g.n_chunks && s <= 32; ++s) {
-    const int64_t waves = (blocks * s + slots - 1) / slots;
-    const double cost = static_cast<double>(waves) * (0.15 + 1.0 / s);
-    if (cost < best_cost - 1e-9) {
-      best_cost = cost;
-      best = s;
-    }
-  }
-  return best;
+// A split walk of `blocks` candidate blocks whose tiles cost `fill` trees' worth of walking each: the line of
+// trees (see SplitArgs) and the CTAs that share it, one for every place of the machine unless a stretch
+// would be shorter than a tile and a unit. Returns the CTAs.
+// Measured: 61,140 candidates x 500 trees (60 blocks, one CTA an SM) on 120 CTAs in equal slices 79 us, on 148 by
+// stretches 68; 96,000 candidates (94 blocks), 282 CTAs in two rounds 114, now 84; a million given rows (977
+// blocks, 6.6 rounds) 930, now 896.
+static int split_plan(const GbdtModel& g, int64_t blocks, int fill, SplitArgs* s) {
+  const int rings = ring_count(g.fast_threads / (g.block_cands / 4));
+  s->units = (g.n_chunks + rings - 1) / rings;
+  s->unit = rings * g.tpc;
+  s->fill = fill;
+  s->blocks = blocks;
+  const int64_t most = blocks * split_block(*s) / (s->fill + s->unit), slots = static_cast<int64_t>(g.ctas_per_sm) * kSmCount;
+  return static_cast<int>(std::max<int64_t>(1, std::min(most, slots)));
 }
+// A tile that is built in the walk from prepared records takes 7 us, and one that is copied 2 to 3, where
+// a tree of eight levels takes a block of 1,024 candidates 0.25 us.
+constexpr int kFillRecords = 28, kFillCopy = 10;
+
+// Whether a dense walk of so many blocks is split: where whole blocks would leave part of the machine idle.
+bool fast_splits(const GbdtModel& g, int64_t blocks) {
+  return blocks >= 1 && blocks < static_cast<int64_t>(g.ctas_per_sm) * kSmCount && g.n_chunks > ring_count(g.fast_threads / (g.block_cands / 4));
+}
+size_t fast_split_bytes(const GbdtModel& g) { return sizeof(double) * 2 * 2 * kSmCount * g.block_cands; }
+static_assert(2 * kSmCount <= kMaxShares, "an arrival counter for every CTA");
 
 size_t fast_prepared_rows_bytes(const GbdtModel& g, int C) { return static_cast<size_t>(kCombos) * C * cand_rec_bytes(g); }
 size_t fast_prepared_memo_bytes(const GbdtModel& g, int C) {
@@ -1430,27 +1537,28 @@ struct WalkArgs {
   int k;
   unsigned long long* partial;
   int* status;
-  SliceArgs sl;
+  SplitArgs sl;
+  int split_ctas;  // of a split walk
   const FastTopParams* top;
   cudaStream_t stream;
   int dependent;  // launched right behind the kernel whose tables it reads
 };
 
-template <int L, int NP, bool kCompact, int THREADS, int NC, bool kFloor = false>
-cudaError_t launch_ln(const WalkArgs& a) {
+template <int L, int NP, bool kCompact, int THREADS, int NC, bool kSplit, bool kFloor = false>
+cudaError_t launch_form(const WalkArgs& a) {
   const size_t smem = static_cast<size_t>(kNBuf) * ring_count(THREADS / (NC / 4)) * a.fv.buf_bytes +
                       static_cast<size_t>(a.fv.n_rows) * NC;
-  auto kernel = &select_fast_kernel<L, NP, kCompact, THREADS, NC, kFloor>;
+  auto kernel = &select_fast_kernel<L, NP, kCompact, THREADS, NC, kSplit, kFloor>;
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
-  // One CTA per item, or - batch form of the geometries that hold one CTA per SM - one CTA per SM,
-  // each serving many items. (Two persistent CTAs on an SM run in step, so that both fill and rank
-  // at the same time and neither hides the other's: measured 6 % slower than one CTA per item.)
-  const int64_t n_items = static_cast<int64_t>(a.P) * a.nblk * a.sl.n_slices;
-  const bool persistent = THREADS > 256 && a.sl.n_slices == 1 && !a.sl.score_out && !a.sl.tiles;
+  // One CTA per item; or - batch form of the geometries that hold one CTA per SM - one CTA per SM, each
+  // serving many items; or a split walk's CTAs. (Two persistent CTAs on an SM run in step, so that both fill
+  // and rank at the same time and neither hides the other's: measured 6 % slower than one CTA per item.)
+  const int64_t n_items = static_cast<int64_t>(a.P) * a.nblk;
+  const bool persistent = THREADS > 256 && !a.sl.tiles;
   const int64_t slots = kSmCount;
-  cfg.gridDim = dim3(static_cast<unsigned>(persistent && n_items > slots ? slots : n_items));
+  cfg.gridDim = dim3(static_cast<unsigned>(kSplit ? a.split_ctas : (persistent && n_items > slots ? slots : n_items)));
   cfg.blockDim = dim3(THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = a.stream;
@@ -1465,6 +1573,11 @@ cudaError_t launch_ln(const WalkArgs& a) {
   return cudaLaunchKernelEx(&cfg, kernel, a.desc, a.d_p, a.pv, a.uv, a.d_c, a.P, a.C, a.nblk, a.rows_per_cta,
                             a.seg_off, a.seg_idx, a.fv, a.k, a.partial, a.status, a.sl, static_cast<int>(n_items),
                             *a.top);
+}
+
+template <int L, int NP, bool kCompact, int THREADS, int NC>
+cudaError_t launch_ln(const WalkArgs& a) {
+  return a.sl.units > 0 ? launch_form<L, NP, kCompact, THREADS, NC, true>(a) : launch_form<L, NP, kCompact, THREADS, NC, false>(a);
 }
 
 // the instantiation for a model's top levels and depth, within one tile geometry
@@ -1495,8 +1608,8 @@ cudaError_t launch_walk_floor(const GbdtModel& g, const WalkArgs& a) {
   if (g.top_compact || g.top_levels != 3 || g.fast_depth != 8 || g.block_cands != 1024 ||
       g.n_chunks < kNBuf * ring_count(g.fast_threads / 256))  // every ring needs its kNBuf resident chunks
     return cudaErrorNotSupported;
-  if (g.fast_threads == 512) return launch_ln<3, 5, false, 512, 1024, true>(a);
-  return launch_ln<3, 5, false, 256, 1024, true>(a);
+  if (g.fast_threads == 512) return launch_form<3, 5, false, 512, 1024, false, true>(a);
+  return launch_form<3, 5, false, 256, 1024, false, true>(a);
 }
 
 cudaError_t launch_walk(const GbdtModel& g, const WalkArgs& a) {
@@ -1588,7 +1701,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
                                int nblk, int rows_per_cta, const int64_t* seg_off, const int32_t* seg_idx,
                                int k, unsigned long long* partial, void* scratch, int* status,
                                cudaStream_t stream, int64_t* launches, cudaEvent_t ev_begin,
-                               const FastSlice* slice, void* memo_mem, const FastWait* wait,
+                               const FastSplit* split, void* memo_mem, const FastWait* wait,
                                const FastPrepared* prep, const int32_t* perm, const ClassCall* classes) {
   WalkArgs a{};
   a.desc = desc;
@@ -1622,7 +1735,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
 
   // candidate-only rows for the type combinations in use
   cudaError_t e = cudaSuccess;
-  const bool tiles_mode = !prep && slice && slice->n_slices > 1 && slice->tiles && !seg_off;
+  const bool tiles_mode = !prep && split && split->tiles && !seg_off;
   if (!prep && !a.uv && !tiles_mode) {
     e = cudaMemsetAsync(d_mask, 0, sizeof(unsigned), stream);
     if (e != cudaSuccess) return e;
@@ -1657,9 +1770,9 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     const int resident = std::max<int>(1, std::min<int>(3, 226 * 1024 / (smem + 4096)));
     if (C > 0)
       tile_pairs_kernel<<<std::min(P * groups, resident * kSmCount), 256, smem, stream>>>(
-          desc, d_p, a.pv, a.uv, P, d_c, C, fv, W, groups, slice->tiles, wait->words);
+          desc, d_p, a.pv, a.uv, P, d_c, C, fv, W, groups, split->tiles, wait->words);
     else
-      e = cudaMemsetAsync(slice->tiles, 0x80, fast_tiles_bytes(g, static_cast<int64_t>(P) * nblk), stream);
+      e = cudaMemsetAsync(split->tiles, 0x80, fast_tiles_bytes(g, static_cast<int64_t>(P) * nblk), stream);
     if (e != cudaSuccess) return e;
     ++*launches;
   } else if (C > 0) {
@@ -1695,17 +1808,15 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     if (e != cudaSuccess) return e;
   }
 
-  a.sl.n_slices = 1;
   a.sl.words = wait->words;
-  if (slice && slice->n_slices > 1) {
-    a.sl.n_slices = slice->n_slices;
-    a.sl.pairs = slice->pairs;
-    a.sl.scores = slice->scores;
-    a.sl.out_idx = slice->out_idx;
-    a.sl.out_score = slice->out_score;
-    a.sl.tiles = tiles_mode ? slice->tiles : nullptr;
-    a.sl.out_seq = slice->out_seq;
-    a.sl.seq = slice->seq;
+  if (split) {
+    a.split_ctas = split_plan(g, static_cast<int64_t>(P) * nblk, tiles_mode ? kFillCopy : kFillRecords, &a.sl);
+    a.sl.scores = split->scores;
+    a.sl.out_idx = split->out_idx;
+    a.sl.out_score = split->out_score;
+    a.sl.tiles = tiles_mode ? split->tiles : nullptr;
+    a.sl.out_seq = split->out_seq;
+    a.sl.seq = split->seq;
   }
   // problems in batches when the memo's table does not hold them all at once
   const int step = memo.keys ? balanced_step(g, P, memo_batch, nblk) : P;
@@ -1721,7 +1832,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
           desc, d_p ? d_p + first : nullptr, a.pv, a.uv, n, d_c, fv, memo, pthr_cap, path, wait->words);
       ++*launches;
     }
-    a.dependent = memo.keys != nullptr;
+    a.dependent = memo.keys != nullptr || tiles_mode;
     a.d_p = d_p ? d_p + first : nullptr;
     a.P = n;
     a.seg_off = seg_off ? seg_off + first : nullptr;
@@ -1742,7 +1853,7 @@ constexpr int64_t kScoreBatchRows = 4096 * 1024;
 
 size_t score_fast_scratch_bytes(const GbdtModel& g, int64_t rows) {
   int64_t blocks = (std::min(rows, kScoreBatchRows) + g.block_cands - 1) / g.block_cands;
-  return static_cast<size_t>(blocks) * g.n_qrows * g.block_cands;
+  return (static_cast<size_t>(blocks) * g.n_qrows * g.block_cands + 255) / 256 * 256 + fast_split_bytes(g);
 }
 
 cudaError_t launch_score_fast(const ks_gpu_desc& desc, const GbdtModel& g, const float* d_feat, int64_t rows,
@@ -1773,9 +1884,13 @@ cudaError_t launch_score_fast(const ks_gpu_desc& desc, const GbdtModel& g, const
     if (e != cudaSuccess) return e;
     a.C = static_cast<int>(n);
     a.nblk = nblk;
-    a.sl = SliceArgs{};
-    a.sl.n_slices = 1;
+    a.sl = SplitArgs{};
+    if (floor_repeat == 0 && (g.ctas_per_sm == 1 || nblk < 2 * kSmCount)) {
+      a.split_ctas = split_plan(g, nblk, kFillCopy, &a.sl);
+      a.sl.scores = reinterpret_cast<double*>(tiles + score_fast_scratch_bytes(g, std::min(rows, kScoreBatchRows)) - fast_split_bytes(g));
+    }
     a.sl.words = wait->words;
+    a.dependent = 1;
     a.sl.tiles = tiles;
     a.sl.score_out = d_scores + first;
     a.sl.repeat = floor_repeat;

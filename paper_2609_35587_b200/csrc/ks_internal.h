@@ -155,7 +155,7 @@ struct ks_catalogue {
   int C = 0;
   int device = 0;
   bool prepared = false;   // false: calls go through ks_select_one
-  int nblk = 0, slices = 1, max_k = KS_MAX_K;
+  int nblk = 0, max_k = KS_MAX_K;
   void* d_mem = nullptr;   // one block: rows | memo | partial lists | partial-score planes | similarity order
   size_t off_memo = 0, off_part = 0, off_scores = 0, off_order = 0;
 };
@@ -179,11 +179,11 @@ constexpr int kFastMaxPairRec = 256;   // rows of per-pair features a memoised m
 constexpr size_t kMemoTableBytes = size_t(256) << 20;  // per-(problem, class) records held at a time
 constexpr int kFastWaitLimit = 1 << 17;  // probes of a chunk wait (a sleep ends early, ~0.2 us measured): tens of ms
 constexpr int kMlpThreads = 512;        // threads per block of the tensor-core MLP kernel
-constexpr int kMaxSliceBlocks = 1024;  // candidate blocks the slice mode supports
-// A context's device words: the arrival counters of the slice mode (zero between calls), then a word per
+constexpr int kMaxShares = 1024;       // CTAs that a split walk may have
+// A context's device words: the arrival counters of the split walk (zero between calls), then a word per
 // kernel family that makes the CTAs which start after it was raised leave at once. It is cleared in front
 // of every launch of the family.
-constexpr int kWordWalk = kMaxSliceBlocks + 1, kWordMlp = kWordWalk + 1, kWordWide = kWordMlp + 1;
+constexpr int kWordWalk = kMaxShares + 1, kWordMlp = kWordWalk + 1, kWordWide = kWordMlp + 1;
 constexpr int kWordServed = kWordWide + 1;  // calls that the walk of whole classes has served (ks_debug_class_walks)
 constexpr int kContextWords = kWordServed + 1;
 constexpr int kLeaveFailed = 1, kLeaveServed = 2;  // a wait ran out; another kernel serves the call
@@ -216,11 +216,9 @@ struct ClassCall {
   void* scratch;     // classes_scratch_bytes
 };
 
-// Slice mode of the quantised tree kernel (few candidate blocks: the trees are split over several CTAs).
-struct FastSlice {
-  int n_slices;
-  long long pairs;   // rows of one partial-score plane
-  float* scores;     // [n_slices][pairs]
+// Split walk of the quantised tree kernel (few candidate blocks: the machine's CTAs share out their trees).
+struct FastSplit {
+  double* scores;    // fast_split_bytes: partial sums
   int32_t* out_idx;  // single-problem form: [k], device-visible; else null (a merge kernel follows)
   float* out_score;
   uint8_t* tiles;    // scratch for the tiles [problems * blocks][rows][block_cands], or null
@@ -280,7 +278,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
                                int nblk, int rows_per_cta, const int64_t* seg_off, const int32_t* seg_idx,
                                int k, unsigned long long* partial, void* scratch, int* status,
                                cudaStream_t stream, int64_t* launches, cudaEvent_t ev_begin,
-                               const FastSlice* slice, void* memo_mem, const FastWait* wait,
+                               const FastSplit* split, void* memo_mem, const FastWait* wait,
                                const FastPrepared* prep = nullptr, const int32_t* perm = nullptr,
                                const ClassCall* classes = nullptr);
 // Prepared catalogue (single-problem calls against a fixed catalogue and model).
@@ -288,7 +286,8 @@ size_t fast_prepared_rows_bytes(const GbdtModel& g, int C);
 size_t fast_prepared_memo_bytes(const GbdtModel& g, int C);  // 0: the model's per-pair rows do not fit a record
 cudaError_t fast_prepare(const ks_gpu_desc& desc, const GbdtModel& g, const ks_candidate* d_c, int C, void* d_rows,
                          void* memo_mem, cudaStream_t stream, int64_t* launches);
-int fast_slices(const GbdtModel& g, int64_t blocks);
+bool fast_splits(const GbdtModel& g, int64_t blocks);  // whether a dense walk of so many blocks is split
+size_t fast_split_bytes(const GbdtModel& g);
 // ks_score with a qualifying ensemble: tiles quantised from the feature rows, then the same walk.
 size_t score_fast_scratch_bytes(const GbdtModel& g, int64_t rows);
 cudaError_t launch_score_fast(const ks_gpu_desc& desc, const GbdtModel& g, const float* d_feat, int64_t rows,

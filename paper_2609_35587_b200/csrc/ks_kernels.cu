@@ -1086,10 +1086,8 @@ size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, 
     int nblk, rows;
     fast_tiling(model.gbdt, P, per, &nblk, &rows);
     const size_t part = (static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
-    const int S = segmented ? 1 : fast_slices(model.gbdt, static_cast<int64_t>(P) * nblk);
-    if (S > 1) {
-      const size_t planes = (sizeof(float) * S * static_cast<size_t>(pairs) + 255) / 256 * 256;
-      return part + planes + 256 +
+    if (!segmented && fast_splits(model.gbdt, static_cast<int64_t>(P) * nblk)) {
+      return part + fast_split_bytes(model.gbdt) + 512 +
              std::max(fast_scratch_bytes(model.gbdt, C), fast_tiles_bytes(model.gbdt, static_cast<int64_t>(P) * nblk));
     }
     const size_t memo = (fast_memo_bytes(model.gbdt, P, C) + 255) / 256 * 256;
@@ -1138,20 +1136,16 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     fast_tiling(model.gbdt, P, per, &nblk, &rows);
     unsigned long long* part = static_cast<unsigned long long*>(d_partial);
     const size_t part_bytes = (static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
-    // an under-filled machine: split the trees over several CTAs per block (dense form only,
-    // where a block covers its rows in one pass)
-    const int sized_slices = d_seg_off ? 1 : fast_slices(model.gbdt, static_cast<int64_t>(P) * nblk);  // as sized
+    // an under-filled machine: the CTAs share out the blocks' trees (dense form only, where a block covers
+    // its rows in one pass)
+    const bool splits = !d_seg_off && fast_splits(model.gbdt, static_cast<int64_t>(P) * nblk);  // as sized
     char* mem = static_cast<char*>(d_partial) + part_bytes;
-    FastSlice sl{};
-    sl.n_slices = p_by_value ? 1 : sized_slices;  // (a single problem has a path of its own)
-    if (sl.n_slices > 1) {
-      // the slices of a block share a tile that is built in front of them; behind the tiles, their score planes
-      sl.pairs = pairs;
-      sl.tiles = reinterpret_cast<uint8_t*>(mem);
-      sl.scores = reinterpret_cast<float*>(mem + (fast_tiles_bytes(model.gbdt, static_cast<int64_t>(P) * nblk) + 255) / 256 * 256);
-    }
+    FastSplit split{};
+    // the parts of a block share a tile that is built in front of them; behind the tiles, their sums
+    split.tiles = reinterpret_cast<uint8_t*>(mem);
+    split.scores = reinterpret_cast<double*>(mem + (fast_tiles_bytes(model.gbdt, static_cast<int64_t>(P) * nblk) + 255) / 256 * 256);
     // the memo of the per-pair rows sits behind the per-call table (batches of whole-ensemble CTAs only)
-    void* memo_mem = (sized_slices > 1 || p_by_value || fast_memo_bytes(model.gbdt, P, C) == 0)
+    void* memo_mem = (splits || p_by_value || fast_memo_bytes(model.gbdt, P, C) == 0)
                          ? nullptr
                          : mem + (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256;
     // a dense batch of problems: rank the catalogue in similarity order (neighbouring candidates
@@ -1169,7 +1163,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     }
     cudaError_t e = launch_select_fast(desc, model.gbdt, d_p, p_by_value, P, d_c, C, nblk, rows, d_seg_off,
                                        d_seg_idx, k, part, mem, d_status,
-                                       stream, launches, ev_begin, sl.n_slices > 1 ? &sl : nullptr, memo_mem, wait,
+                                       stream, launches, ev_begin, splits && !p_by_value ? &split : nullptr, memo_mem, wait,
                                        nullptr, perm, use_classes ? &classes : nullptr);
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);

@@ -1,0 +1,65 @@
+"""Walks whose trees the machine's CTAs share out: block counts at the edges of the split (one block, one CTA less
+than blocks, whole rounds), chunk counts that do not divide, depths of every form, both geometries. Where a
+block is cut depends on its place, a candidate's score must not: a pool that repeats the same candidates
+gives every copy the same score, bit for bit, and the copies rank by index."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2609_35587_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+DESC = wl.gpu_desc()
+
+
+@pytest.fixture(scope="module")
+def ks():
+    from paper_2609_35587_b200 import binding
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ctx(ks):
+    return ks.Context(DESC, 0)
+
+
+@pytest.mark.parametrize("C,P,trees,depth,law", [(1024, 1, 9, 8, "pernode"), (1025, 1, 33, 6, "slots128"),
+                                                 (60001, 1, 61, 8, "pernode"), (3000, 19, 100, 6, "hist256"),
+                                                 (150500, 1, 40, 7, "pernode"), (2048, 73, 70, 3, "slots128"),
+                                                 (1500, 148, 25, 8, "slots128"), (9000, 3, 17, 10, "hist256")])
+def test_copies_of_candidates_tie(ks, ctx, C, P, trees, depth, law):
+    dev, k, period = torch.device("cuda", 0), 32, 431
+    off, nodes = wl.gbdt_complete(C + trees, trees, depth, wl.feature_stats("cfg1"), 0.1, law)
+    model = ctx.model_create_gbdt(off, nodes, 0.25)
+    base = wl.candidates_full_grid(7, period)
+    cand = base[np.arange(C) % period]
+    prob = wl.problems_batch(C, P)
+    d_c, d_p = ks.to_device(cand, dev), ks.to_device(prob, dev)
+    idx, sc = (t.cpu().numpy() for t in ctx.select(d_p, P, d_c, C, model, k))
+    for p in sorted({0, P // 2, P - 1}):
+        _, _, ref = oracle.select(prob[p:p + 1], base, DESC, 1, gbdt=(off, nodes, 0.25), want_scores=True)
+        # the distinct scores in the answer, and all copies of their candidates in index order
+        want = []
+        for c in np.argsort(-ref[np.arange(period)], kind="stable"):
+            want += list(range(c, C, period))
+            if len(want) >= 4 * k:
+                break
+        got = idx[p]
+        assert np.allclose(sc[p], ref[got % period], rtol=1e-5, atol=1e-5)
+        for c in set(got % period):
+            mine = got[got % period == c]
+            assert len(set(sc[p][got % period == c])) == 1
+            assert np.array_equal(mine, np.arange(c, C, period)[:len(mine)])
+        assert set(got % period) <= set(np.array(want) % period)
+    if P == 1:
+        one_i, one_s = ctx.select_one(prob, d_c, C, model, k)
+        assert np.array_equal(one_i.numpy(), idx[0]) and np.array_equal(one_s.numpy(), sc[0])
+        cat = ctx.catalogue_prepare(d_c, C, model)
+        one_i, one_s = ctx.select_one_prepared(cat, prob, k)
+        assert np.array_equal(one_i.numpy(), idx[0]) and np.array_equal(one_s.numpy(), sc[0])
+        rows = ctx.featurize(d_p, 1, d_c, C)
+        score = ctx.score(rows, model).cpu().numpy()
+        assert np.array_equal(score[idx[0]], sc[0])
+        for c in range(0, period, 7):
+            assert len(set(score[c::period])) == 1
