@@ -276,7 +276,7 @@ ks_status ks_create(ks_ctx** out_ctx, int cuda_device, const ks_gpu_desc* desc) 
     return KS_ERR_OOM;
   }
   ctx->wait.words = ctx->d_words;
-  ks_status s = ensure_workspace(ctx, 1u << 20);
+  ks_status s = ensure_workspace(ctx, 16u << 20);  // (what calls of one or a few problems take)
   // status word in mapped pinned host memory: kernels write it through d_status, the host
   // reads h_status after a synchronisation without issuing a copy
   if (s == KS_OK && (cudaHostAlloc(reinterpret_cast<void**>(&ctx->h_status), sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
@@ -678,10 +678,10 @@ ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int 
   if (model->kind == 0 && model->gbdt.fast && C > 0) {
     const int NC = model->gbdt.block_cands;
     const int nblk = (C + NC - 1) / NC;
-    if (ks::fast_splits(model->gbdt, nblk)) {
+    if (ks::fast_splits(model->gbdt, 1, nblk, true)) {
       const size_t b_part = align_up(sizeof(unsigned long long) * nblk * k);
       // scratch of this path: the prepared tiles, one per candidate block (no per-call table)
-      const size_t b_scratch = align_up(static_cast<size_t>(nblk) * model->gbdt.n_qrows * NC);
+      const size_t b_scratch = ks::fast_tiles_bytes(model->gbdt, 1, nblk);
       const size_t b_scores = align_up(ks::fast_split_bytes(model->gbdt));
       ks_status s = ensure_workspace(ctx, b_part + b_scratch + b_scores);
       if (s != KS_OK) return s;
@@ -747,7 +747,7 @@ ks_status ks_catalogue_prepare(ks_ctx* ctx, const ks_candidate* d_c, int C, cons
   if (model->kind == 0 && g.fast && C > 0) {
     const int nblk = (C + g.block_cands - 1) / g.block_cands;
     const size_t b_memo = ks::fast_prepared_memo_bytes(g, C);
-    if (ks::fast_splits(g, nblk) && b_memo > 0) {
+    if (ks::fast_splits(g, 1, nblk, true) && b_memo > 0) {
       DeviceGuard guard(ctx->device);
       const size_t b_rows = align_up(ks::fast_prepared_rows_bytes(g, C));
       const size_t b_part = align_up(sizeof(unsigned long long) * nblk * KS_MAX_K);

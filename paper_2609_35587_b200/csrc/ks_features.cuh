@@ -107,7 +107,9 @@ __device__ __forceinline__ float log2_dim(unsigned v) {
   return __double2float_rn(log2(static_cast<double>(v)));
 }
 
-__device__ inline void problem_terms(const ks_problem& p, const ks_gpu_desc& h, ProblemTerms& t) {
+// kLogs false: without the logarithms (columns 0 to 2), for kernels that have other threads evaluate them.
+template <bool kLogs = true>
+__device__ __forceinline__ void problem_terms(const ks_problem& p, const ks_gpu_desc& h, ProblemTerms& t) {
   t.M = p.m; t.N = p.n; t.K = p.k;
   t.dtype_ab = p.dtype_ab & 3;
   t.dtype_d = p.dtype_d & 3;
@@ -120,9 +122,11 @@ __device__ inline void problem_terms(const ks_problem& p, const ks_gpu_desc& h, 
   t.bytesA = t.bA * M * K;
   t.bytesB = t.bA * K * N;
   t.Q_epi = t.bD * M * N + (t.has_bias ? t.bD * M : 0);
-  t.log2m = log2_dim(t.M);
-  t.log2n = log2_dim(t.N);
-  t.log2k = log2_dim(t.K);
+  if (kLogs) {
+    t.log2m = log2_dim(t.M);
+    t.log2n = log2_dim(t.N);
+    t.log2k = log2_dim(t.K);
+  }
   t.i_problem = __fdiv_rn(F64i(2 * M * N * K), F64i(t.bytesA + t.bytesB + t.Q_epi));
   t.ws_frac_l2 = __fdiv_rn(F64i(t.bytesA + t.bytesB), F64i(static_cast<long long>(h.l2_bytes)));
   t.f_traffic_epi = F64i(t.Q_epi);

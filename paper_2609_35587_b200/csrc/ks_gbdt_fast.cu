@@ -49,6 +49,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
+#include <climits>
 #include <cstring>
 #include <limits>
 #include <new>
@@ -92,30 +93,39 @@ constexpr int kOffBuf0 = 0;
 struct SplitArgs {
   int units;            // of a block; 0: CTAs take whole blocks
   int unit, fill;       // trees of a unit, and what filling a tile counts for
-  long long blocks;
+  int blocks;
+  int step, rest;       // total / CTAs, and the remainder
   double* scores;       // [CTAs][2][NC]: sums of a CTA's first and last part
   int* words;           // the context's device words: arrival counters, by the first CTA of a block (reset by their last users), kWordWalk
   int32_t* out_idx;     // single-problem form only: [k] final result (device-visible, may be
   float* out_score;     // mapped host memory); null when a merge kernel follows
-  const uint8_t* tiles; // prepared tiles [blocks][rows][NC] (tile_pairs_kernel, tile_rows_kernel), or null
+  const uint8_t* tiles; // tiles built in front: [blocks][rows][NC] (tile_rows_kernel), or the per-pair rows alone (tile_pairs_kernel)
+  const uint8_t* cand_tiles;  // the candidate-only rows of the latter, or null
   int* out_seq;         // single-problem form: receives `seq` once the k results are written
   int seq;
   float* score_out;     // scoring call (ks_score): the scores of the block's rows go here, no ranking
   int repeat;           // floor measurement only: passes over the resident chunks
 };
-__host__ __device__ __forceinline__ long long split_block(const SplitArgs& s) { return s.fill + static_cast<long long>(s.units) * s.unit; }
+// (32 bits hold a launch's trees, see split_fits)
+__host__ __device__ __forceinline__ int split_block(const SplitArgs& s) { return s.fill + s.units * s.unit; }
 // first unit (of all blocks') of CTA c of n
-__host__ __device__ __forceinline__ long long split_start(const SplitArgs& s, long long c, long long n) {
-  const long long len = split_block(s), x = c * (s.blocks * len) / n, block = x / len, in = x - block * len - s.fill;
+__host__ __device__ __forceinline__ int split_start(const SplitArgs& s, int c, int n) {
+  const int len = split_block(s), x = c * s.step + c * s.rest / n, block = x / len, in = x - block * len - s.fill;
   return block * s.units + (in > 0 ? in / s.unit : 0);
 }
-// the CTAs that hold the first and the last unit of a block: the largest c whose start is not behind it
-__host__ __device__ __forceinline__ int split_first(const SplitArgs& s, long long block, long long n) {
-  const long long len = split_block(s);
-  return static_cast<int>(((block * len + s.fill + s.unit) * n - 1) / (s.blocks * len));
+// (a n - 1) / total; in 32 bits where they hold the product, as a division in 64 takes half a microsecond
+__host__ __device__ __forceinline__ int split_quotient(int a, int n, int total) {
+  if (total < (1 << 21)) return static_cast<int>((static_cast<unsigned>(a) * static_cast<unsigned>(n) - 1u) / static_cast<unsigned>(total));
+  return static_cast<int>((static_cast<long long>(a) * n - 1) / total);
 }
-__host__ __device__ __forceinline__ int split_last(const SplitArgs& s, long long block, long long n) {
-  return static_cast<int>(((block + 1) * split_block(s) * n - 1) / (s.blocks * split_block(s)));
+// the CTAs that hold the first and the last unit of a block: the largest c whose start is not behind it
+__host__ __device__ __forceinline__ int split_first(const SplitArgs& s, int block, int n) {
+  const int len = split_block(s);
+  return split_quotient(block * len + s.fill + s.unit, n, s.blocks * len);
+}
+__host__ __device__ __forceinline__ int split_last(const SplitArgs& s, int block, int n) {
+  const int len = split_block(s);
+  return split_quotient((block + 1) * len, n, s.blocks * len);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -188,22 +198,22 @@ cand_rows_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, co
   }
 }
 
-// Packs the occupied slots of every type combination's table (one block per combination), so
-// that the per-problem kernel runs full warps over classes only. `keys` then holds a slot's place.
-__global__ void __launch_bounds__(1024)
+// Packs the occupied slots of every type combination's table, so that the per-problem kernel runs full
+// warps over classes only. `keys` then holds a slot's place. A thread a slot, an atomic operation a warp
+// (one block for all of a combination's slots took 7 us for half as many).
+__global__ void __launch_bounds__(256)
 memo_compact_kernel(MemoView memo) {
-  __shared__ int s_n;
-  const int combo = blockIdx.x;
-  if (threadIdx.x == 0) s_n = 0;
-  __syncthreads();
-  for (int slot = threadIdx.x; slot < kMemoCap; slot += 1024)
-    if (memo.keys[static_cast<size_t>(combo) * kMemoCap + slot] != 0ull) {
-      const int j = atomicAdd(&s_n, 1);
-      memo.dense[static_cast<size_t>(combo) * kMemoCap + j] = slot;
-      memo.keys[static_cast<size_t>(combo) * kMemoCap + slot] = j;  // (the key is not needed any more)
-    }
-  __syncthreads();
-  if (threadIdx.x == 0) memo.count[combo] = s_n;
+  const int combo = blockIdx.y, slot = blockIdx.x * 256 + threadIdx.x, lane = threadIdx.x & 31;
+  unsigned long long& key = memo.keys[static_cast<size_t>(combo) * kMemoCap + slot];
+  const bool used = key != 0ull;
+  const unsigned all = __ballot_sync(0xFFFFFFFFu, used);
+  if (all == 0u) return;
+  int first = 0;
+  if (lane == 0) first = atomicAdd(memo.count + combo, __popc(all));
+  const int j = __shfl_sync(0xFFFFFFFFu, first, 0) + __popc(all & ((1u << lane) - 1u));
+  if (!used) return;
+  memo.dense[static_cast<size_t>(combo) * kMemoCap + j] = slot;
+  key = j;  // (the key is not needed any more)
 }
 
 // Per problem: the tile bytes of the per-pair rows of every class, from the class's member, plus
@@ -332,31 +342,47 @@ __device__ __forceinline__ void tile_column(const FeatQ& q, float4 x, uint32_t t
   }
 }
 
+// What a walk copies its tiles from: the per-pair rows of every (problem, candidate block), the candidate-only
+// rows of every block once per type combination in use (at the first problem that has it), and every problem's
+// record (problem-only rows, then that first problem).
+struct PairTiles {
+  uint8_t* pair;  // [P][blocks][pair rows][NC]
+  uint8_t* cand;  // [P][blocks][candidate rows][NC]
+  uint8_t* prob;  // [P][kProbRec]
+};
+inline PairTiles pair_tiles(const GbdtModel& g, int P, int nblk, uint8_t* mem) {
+  const auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+  PairTiles t;
+  t.pair = mem;
+  t.cand = t.pair + up(static_cast<size_t>(P) * nblk * g.n_pair_rows * g.block_cands);
+  t.prob = t.cand + up(static_cast<size_t>(P) * nblk * g.n_cand_rows * g.block_cands);
+  return t;
+}
+
 // An item is 128 candidates (32 words of a tile) of one problem; a block takes a run of items, so that the
-// thresholds are staged once and a problem's terms evaluated once or twice. Half of the threads
-// compute the per-pair columns of a candidate each, the other half the candidate-only ones; then a warp takes
-// every eighth column, four candidates a lane, and stores whole lines, in the layout phase A would produce.
+// thresholds are staged once and a problem's terms evaluated once or twice. Two threads share a
+// candidate's columns; then a warp takes every eighth column, four candidates a lane, and stores whole
+// lines, in the layout phase A would produce. The first problem of a type combination also brings the
+// candidate-only columns, for all that have it, and the first item of a problem its problem-only rows.
 // Slots past the catalogue get the last candidate's bytes (they are not ranked). Also clears the abort flag
-// (this kernel precedes the select kernel). What bounds it is the latency of the columns' divisions and of
-// the searches. One problem x 61,140 candidates, 500 trees: 29 us, where a thread that wrote its candidate's
-// bytes one by one took 72. Every split walk of a dense batch takes its tiles from here: left to the parts of a block,
-// each computed the per-pair columns again (10 problems x 934 candidates, 326 trees: 125 -> 48 us the whole call;
-// 64 x 2,048 candidates, 100 trees: 161 -> 120, with the memo in its place 143; four calls of one problem with
-// its 61,140 valid candidates: 900 -> 677).
+// (this kernel precedes the select kernel). What bounds it is the issue of the searches beside the
+// latency of the columns' divisions. One problem x 61,140 candidates, 500 trees: 18 us (21 with the candidate-only columns
+// for every problem, four searches of the problem-only ones in every lane and a last item for some blocks; a thread that
+// wrote its candidate's bytes one by one took 72); 64 x 2,048: 30 -> 16.
 constexpr int kTileRows = 128, kTileCols = kPairCols + kCandCols;
 // Thresholds that fit beside 64 columns of a block's rows and the static part (49,152). The walk's own tile
 // geometries hold 376 rows of 127 at most, 47,752.
 constexpr int kTileMaxThr = (227 * 1024 - 3072) / 4 - 64 * kTileRows;
 static_assert(kTileMaxThr >= 376 * kSlice, "every ensemble of the regular geometries");
 
-__global__ void __launch_bounds__(256, 3)
-tile_pairs_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int P,
-                  const ks_candidate* __restrict__ c, int C, FastView fv, int W, int groups,
-                  uint8_t* __restrict__ tiles, int* words) {
+__global__ void __launch_bounds__(256, 4)
+tile_pairs_kernel(const __grid_constant__ ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int P,
+                  const ks_candidate* __restrict__ c, int C, FastView fv, int W, int groups, PairTiles tiles, int* words) {
   extern __shared__ __align__(16) float s_x[];  // [kTileCols][kTileRows], then the thresholds of every feature
   __shared__ ProblemTerms s_pt;
   __shared__ FeatQ s_fq[64];
   __shared__ float s_pf[64];
+  __shared__ int s_first;
   float* s_thr = s_x + kTileCols * kTileRows;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the walk waits for this grid before it reads the tiles)
@@ -364,48 +390,81 @@ tile_pairs_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem
   const long long n_items = static_cast<long long>(P) * groups;
   const int begin = static_cast<int>(n_items * blockIdx.x / gridDim.x);
   const int end = static_cast<int>(n_items * (blockIdx.x + 1) / gridDim.x);
+  // A problem's terms and columns (the logarithms by threads of their own), and the first problem of its combination.
+  // Between two barriers.
   const auto evaluate = [&](int prob) {
-    problem_terms(use_value ? p_value : load_problem(p + prob), desc, s_pt);
-    problem_columns(s_pt, [&](int col, float v) { s_pf[col] = v; });
+    if (tid < 128 && (tid & 31) == 0) {
+      const ks_problem pr = use_value ? p_value : load_problem(p + prob);
+      if (tid == 0) {
+        problem_terms<false>(pr, desc, s_pt);
+        problem_columns(s_pt, [&](int col, float v) { if (col > 2) s_pf[col] = v; });
+      } else {
+        s_pf[warp - 1] = log2_dim(warp == 1 ? pr.m : (warp == 2 ? pr.n : pr.k));
+      }
+    } else if (tid >= 128) {
+      const ks_problem pr = use_value ? p_value : load_problem(p + prob);
+      int first = prob;
+      if (!use_value)
+        for (int q = tid - 128; q < first; q += 128) {
+          const ks_problem other = load_problem(p + q);
+          if ((other.dtype_ab & 3) == (pr.dtype_ab & 3) && (other.dtype_d & 3) == (pr.dtype_d & 3)) first = q;
+        }
+      first = __reduce_min_sync(0xFFFFFFFFu, first);
+      if (lane == 0) atomicMin(&s_first, first);
+    }
   };
   int held = begin / groups;
-  if (tid == 0 && begin < end) evaluate(held);  // while the other warps stage
-  stage_thresholds(fv, 0, fv.n_thr, s_thr, fv.n_thr);
+  if (tid == 0) s_first = INT_MAX;
   if (tid < 64) s_fq[tid] = fv.feat[tid];
+  __syncthreads();
+  if (begin < end) evaluate(held);
+  stage_thresholds(fv, 0, fv.n_thr, s_thr, fv.n_thr);
   const uint32_t thr = smem_u32(s_thr);
   for (int item = begin; item < end; ++item) {
     const int prob = item / groups, g = item - prob * groups;
     __syncthreads();  // the columns of the item before have been read
     if (prob != held) {
-      if (tid == 0) evaluate(prob);
+      if (tid == 0) s_first = INT_MAX;
+      __syncthreads();
+      evaluate(prob);
       held = prob;
       __syncthreads();
     }
+    if (g == 0) {
+      uint8_t* rec = tiles.prob + static_cast<size_t>(prob) * kProbRec;
+      if (tid < KS_F && feat_class(tid) == 0) {
+        const FeatQ& q = s_fq[tid];
+        const int first = fv.n_pair_rows + fv.n_cand_rows;
+        quantise(q, s_thr + q.thr0, s_pf[tid], false, [&](int row, uint8_t b) { rec[KS_IDX(row - first, kFastMaxProbRows)] = b; });
+      }
+      if (tid == 64) *reinterpret_cast<int*>(rec + kFastMaxProbRows) = s_first;
+    }
+    const bool with_cand = s_first == prob;
     const int row = tid % kTileRows;
     const ks_candidate cand = load_candidate(c + min(g * kTileRows + row, C - 1));
-    if (tid < kTileRows) {
-      const long long b_eff = resources(s_pt, cand, desc).b_eff;
-      pair_columns<true>(s_pt, cand, desc, b_eff, [&](int col, float v) { s_x[pair_slot(col) * kTileRows + row] = v; });
-    } else {
-      featurize_pair(s_pt, cand, desc, [&](int col, float v) {
+    const long long b_eff = resources(s_pt, cand, desc).b_eff;
+    if (tid < kTileRows)
+      pair_columns<true>(s_pt, cand, desc, b_eff, [&](int col, float v) { if (col <= 32) s_x[pair_slot(col) * kTileRows + row] = v; });
+    else
+      pair_columns<true>(s_pt, cand, desc, b_eff, [&](int col, float v) { if (col > 32) s_x[pair_slot(col) * kTileRows + row] = v; });
+    if (with_cand) {
+      const auto put = [&](int col, float v) {
         if (col < KS_F && feat_class(col) == 1) s_x[(kPairCols + cand_slot(col)) * kTileRows + row] = v;
-      });
+      };
+      if (tid < kTileRows) featurize_pair(s_pt, cand, desc, [&](int col, float v) { if (col <= 49) put(col, v); });
+      else featurize_pair(s_pt, cand, desc, [&](int col, float v) { if (col > 49) put(col, v); });
     }
     __syncthreads();
-    const int in_block = g * 32 / W;
-    uint32_t* out = reinterpret_cast<uint32_t*>(tiles) +
-                    (static_cast<size_t>(prob) * (groups * 32 / W) + in_block) * fv.n_rows * W + (g * 32 - in_block * W) + lane;
+    const int in_block = g * 32 / W, word = g * 32 - in_block * W + lane;
+    const size_t block = static_cast<size_t>(prob) * (groups * 32 / W) + in_block;
+    uint32_t* pair_out = reinterpret_cast<uint32_t*>(tiles.pair) + block * fv.n_pair_rows * W + word;
+    // (rows are counted over the whole tile: the candidate-only ones follow the per-pair ones)
+    uint32_t* cand_out = reinterpret_cast<uint32_t*>(tiles.cand) + block * fv.n_cand_rows * W + word - static_cast<ptrdiff_t>(fv.n_pair_rows) * W;
 #pragma unroll 1
-    for (int col = warp; col < KS_F; col += 8) {
-      const int cls = feat_class(col);
-      float4 x;
-      if (cls == 0) {
-        x.x = x.y = x.z = x.w = s_pf[col];
-      } else {
-        const int slot = cls == 2 ? pair_slot(col) : kPairCols + cand_slot(col);
-        x = *reinterpret_cast<const float4*>(s_x + slot * kTileRows + 4 * lane);
-      }
-      tile_column(s_fq[col], x, thr, fv.n_rows, W, out);
+    for (int slot = warp; slot < (with_cand ? kTileCols : kPairCols); slot += 8) {
+      const bool is_pair = slot < kPairCols;
+      const float4 x = *reinterpret_cast<const float4*>(s_x + slot * kTileRows + 4 * lane);
+      tile_column(s_fq[is_pair ? pair_col(slot) : cand_col(slot - kPairCols)], x, thr, fv.n_rows, W, is_pair ? pair_out : cand_out);
     }
   }
 }
@@ -716,14 +775,14 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
   constexpr bool split = kSplit;
   const bool block_major = NC == 1024 && grid < n_items && !seg_off && !tiles_given;
   const int per_cta = (n_items + grid - 1) / grid;
-  long long unit = split ? split_start(sl, cta, grid) : 0;  // a split walk: the next unit
-  const long long unit_first = unit, unit_end = split ? split_start(sl, cta + 1, grid) : 0;
+  int unit = split ? split_start(sl, cta, grid) : 0;  // a split walk: the next unit
+  const int unit_first = unit, unit_end = split ? split_start(sl, cta + 1, grid) : 0;
   int first_item = block_major ? cta * per_cta : cta, item_step = block_major ? 1 : grid;
   int last_item = block_major ? (first_item + per_cta < n_items ? first_item + per_cta : n_items) : n_items;
   if (split) {
-    first_item = static_cast<int>(unit / sl.units);
+    first_item = unit / sl.units;
     item_step = 1;
-    last_item = static_cast<int>((unit_end + sl.units - 1) / sl.units);
+    last_item = (unit_end + sl.units - 1) / sl.units;
   }
   int held_chunk = -1, held_combo = -1;  // what the tile's candidate-only rows belong to
   uint32_t tile_phase = 0;
@@ -750,22 +809,22 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
   int ch_begin = 0, ch_end = fv.n_chunks;
   const bool first_part = unit == unit_first;
   if (split) {
-    const long long block0 = static_cast<long long>(item) * sl.units;
-    ch_begin = static_cast<int>(unit - block0) * RG;
+    const int block0 = item * sl.units;
+    ch_begin = (unit - block0) * RG;
     unit = unit_end < block0 + sl.units ? unit_end : block0 + sl.units;
-    ch_end = static_cast<int>(unit - block0) * RG < fv.n_chunks ? static_cast<int>(unit - block0) * RG : fv.n_chunks;
+    ch_end = (unit - block0) * RG < fv.n_chunks ? (unit - block0) * RG : fv.n_chunks;
   }
   const bool whole = ch_begin == 0 && ch_end == fv.n_chunks;
   __syncthreads();  // the item before this one is finished with the shared state
   if (tid == 0) {
-    if (!tiles_given && !fv.prob_tab) {
+    if (!fv.prob_tab && !tiles_given) {
       problem_terms(use_value ? p_value : load_problem(p + prob), desc, s_pt);
       problem_columns(s_pt, [&](int col, float v) { s_pfeat[col] = v; });
     }
     s_abort = *reinterpret_cast<volatile int*>(sl.words + kWordWalk);
   }
   if (tid < KS_MAX_K) s_list[tid] = 0ull;
-  if (!tiles_given && fv.prob_tab) {
+  if (fv.prob_tab) {
     const uint8_t* rec = fv.prob_tab + static_cast<size_t>(prob) * kProbRec;
     for (int i = tid; i < fv.n_prob_rows; i += THREADS) s_pbin[i] = __ldcg(rec + i);
     if (tid < static_cast<int>(sizeof(ProblemTerms) / 4))
@@ -808,16 +867,30 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     if (early && tid == 0) {
       fence_async_proxy();
       if (tiles_given) {
-        // the block's tile was built in front, in one piece
-        const uint32_t bar = bar0 + 8u * (kNBuf * RG), bytes = static_cast<uint32_t>(fv.n_rows) * NC;
+        // the block's tile was built in front, in one piece or two
+        const uint32_t bar = bar0 + 8u * (kNBuf * RG);
+        const uint32_t bytes = static_cast<uint32_t>(sl.cand_tiles ? fv.n_pair_rows : fv.n_rows) * NC;
+        const uint32_t more = sl.cand_tiles ? static_cast<uint32_t>(fv.n_cand_rows) * NC : 0u;
         asm volatile("fence.proxy.async.global;" ::: "memory");  // (written by ordinary stores of the kernel in front)
-        mbar_expect_tx(bar, bytes);
-        bulk_copy_g2s(sbase + kOffTile, sl.tiles + (static_cast<size_t>(prob) * nblk + chunk) * bytes, bytes, bar);
+        mbar_expect_tx(bar, bytes + more);
+        if (bytes) bulk_copy_g2s(sbase + kOffTile, sl.tiles + (static_cast<size_t>(prob) * nblk + chunk) * bytes, bytes, bar);
+        // (the record's terms are the first problem of the combination here)
+        if (more) {
+          const size_t first = KS_IDX(*reinterpret_cast<const int*>(&s_pt), P);
+          bulk_copy_g2s(sbase + kOffTile + bytes, sl.cand_tiles + (first * nblk + chunk) * more, more, bar);
+        }
       }
       start_rings();
     }
     bool tile_late = false;
     if (tiles_given) {
+      if (sl.cand_tiles) {  // problem-only rows: one byte for the whole row
+        unsigned char* dst = smem + kOffTile + static_cast<size_t>(fv.n_pair_rows + fv.n_cand_rows) * NC;
+        for (int i = tid; i < fv.n_prob_rows * (NC / 16); i += THREADS) {
+          const uint32_t b = s_pbin[i / (NC / 16)] * 0x01010101u;
+          reinterpret_cast<uint4*>(dst)[i] = make_uint4(b, b, b, b);
+        }
+      }
       if (!tile_wait(bar0 + 8u * (kNBuf * RG), tile_phase, fv.wait_limit)) {
         tile_late = true;
         s_fail = 1;
@@ -1024,7 +1097,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
           const int c0 = split_first(sl, item, grid), n = split_last(sl, item, grid) - c0 + 1;
           s_parts[0] = c0;
           s_parts[1] = n;
-          s_parts[2] = split_start(sl, c0, grid) < static_cast<long long>(item) * sl.units ? 1 : 0;  // its last part
+          s_parts[2] = split_start(sl, c0, grid) < item * sl.units ? 1 : 0;  // its last part
           s_last = atomicAdd(sl.words + c0, 1) == n - 1;
           if (s_last) sl.words[c0] = 0;  // nobody else touches this counter again in this launch
         }
@@ -1035,12 +1108,22 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
         }
         __threadfence();
         if (grp == 0) {
+          // parts 0 .. n - 1: the first CTA's first or last one, the others' first
           const double* from = sl.scores + 2 * static_cast<size_t>(s_parts[0]) * NC + 4 * word;
+          const int n = s_parts[1], second = s_parts[2] * NC;
           sums[0] = sums[1] = sums[2] = sums[3] = 0.0;
-          for (int q = 0; q < s_parts[1]; ++q) {
-            const double2* p2 = reinterpret_cast<const double2*>(from + (2 * q + (q == 0 ? s_parts[2] : 0)) * NC);
-            const double2 u = __ldcg(p2), v = __ldcg(p2 + 1);
-            sums[0] += u.x; sums[1] += u.y; sums[2] += v.x; sums[3] += v.y;
+          for (int q0 = 0; q0 < n; q0 += 4) {
+            double2 u[4], v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const double2* p2 = reinterpret_cast<const double2*>(from + 2 * static_cast<size_t>(q0 + q) * NC + (q0 + q == 0 ? second : 0));
+              u[q] = q0 + q < n ? __ldcg(p2) : make_double2(0.0, 0.0);
+              v[q] = q0 + q < n ? __ldcg(p2 + 1) : make_double2(0.0, 0.0);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              sums[0] += u[q].x; sums[1] += u[q].y; sums[2] += v[q].x; sums[3] += v[q].y;
+            }
           }
         }
       }
@@ -1294,8 +1377,9 @@ cudaError_t build_fast_gbdt(GbdtModel& m, int n_trees, const int64_t* off, const
   const int group_buf = geom.buf_bytes / rings / 16 * 16;
   int tpc = group_buf / (per_tree_words * 4) / gpr * gpr;
   if (tpc < gpr) return cudaSuccess;
-  // (eight trees a thread are enough to hide a chunk's beginning and end; more only make a split walk's units coarse)
-  tpc = std::min(tpc, 8 * gpr);
+  // At least sixteen chunks a ring, so that a split walk's units are not coarse, but no fewer than eight trees a thread, which
+  // hide a chunk's beginning and end (100 trees of depth 6 in chunks of 32: 64 x 2,048 from host memory 122 us, of 8 112).
+  tpc = std::min(tpc, std::max(8, n_trees / (16 * rings)) * gpr);
   if (tpc > (n_trees + G - 1) / G * gpr) tpc = (n_trees + G - 1) / G * gpr;  // a small ensemble: one short chunk per ring
   const int n_chunks = (n_trees + tpc - 1) / tpc;
   const int chunk_words = (tpc * per_tree_words + 3) / 4 * 4;  // bulk copies move multiples of 16 bytes
@@ -1439,18 +1523,17 @@ void fast_tiling(const GbdtModel& g, int P, int64_t per_problem, int* nblk, int*
   *rows_per_cta = g.block_cands;
 }
 
-size_t fast_tiles_bytes(const GbdtModel& g, int64_t blocks) {
-  return static_cast<size_t>(blocks) * g.n_qrows * g.block_cands;
+size_t fast_tiles_bytes(const GbdtModel& g, int P, int nblk) {
+  return reinterpret_cast<size_t>(pair_tiles(g, P, nblk, nullptr).prob) + static_cast<size_t>(P) * kProbRec;
 }
 
 size_t fast_scratch_bytes(const GbdtModel& g, int C) {
   return 256 + static_cast<size_t>(kCombos) * C * cand_rec_bytes(g);
 }
 
-// Memo of the per-pair rows (see MemoView): worth its per-problem table only for a batch of
-// problems (7 problems x 61,140 candidates with it: 537 -> 693 us, of which 100 go to finding the classes)
-// and only where the walk is not split, since a split walk takes whole tiles (see tile_pairs_kernel). The
-// table is held for at most `fast_memo_batch` problems at a time (256 MiB of
+// Memo of the per-pair rows (see MemoView): for every dense batch that is not split (a split walk takes whole
+// tiles, see tile_pairs_kernel) and for segmented batches of 32 problems or more. The
+// table is held for at most `fast_memo_batch` problems at a time (512 MiB of
 // records); a larger call is served batch by batch. 0 = not used.
 size_t memo_fixed_bytes(int C) {
   return static_cast<size_t>(kMemoCombos) * kMemoCap * (sizeof(unsigned long long) + 2 * sizeof(int)) + 256 +
@@ -1469,30 +1552,32 @@ MemoView memo_view(void* mem, int C) {
   return v;
 }
 cudaError_t memo_clear(const MemoView& memo, cudaStream_t stream) {
-  return cudaMemsetAsync(memo.keys, 0, static_cast<size_t>(kMemoCombos) * kMemoCap * sizeof(unsigned long long), stream);
+  // (the counts lie behind the keys)
+  return cudaMemsetAsync(memo.keys, 0, static_cast<size_t>(kMemoCombos) * (kMemoCap * sizeof(unsigned long long) + sizeof(int)), stream);
 }
 cudaError_t memo_compact(const MemoView& memo, cudaStream_t stream) {
-  memo_compact_kernel<<<kMemoCombos, 1024, 0, stream>>>(memo);
+  memo_compact_kernel<<<dim3(kMemoCap / 256, kMemoCombos), 256, 0, stream>>>(memo);
   return cudaGetLastError();
 }
 
-int fast_memo_batch(const GbdtModel& g, int P) {
-  if (P < kMemoMinProblems || g.n_pair_rows < 1 || g.n_pair_rows > kFastMaxPairRec) return 0;
+int fast_memo_batch(const GbdtModel& g, int P, bool segmented, bool lean) {
+  if (P < (segmented || lean ? kMemoMinProblems : kMemoMinDense) || g.n_pair_rows < 1 || g.n_pair_rows > kFastMaxPairRec) return 0;
   const size_t per_problem = static_cast<size_t>(kMemoCap) * pair_rec_bytes(g);
   int64_t batch = static_cast<int64_t>(kMemoTableBytes / per_problem);
   if (batch < kMemoMinProblems) batch = kMemoMinProblems;
+  if (lean) batch = kMemoMinProblems / 2;
   return static_cast<int>(batch < P ? batch : P);
 }
 
-size_t fast_memo_bytes(const GbdtModel& g, int P, int C) {
-  const int batch = fast_memo_batch(g, P);
+size_t fast_memo_bytes(const GbdtModel& g, int P, int C, bool segmented, bool lean) {
+  const int batch = fast_memo_batch(g, P, segmented, lean);
   if (batch == 0 || C < 1) return 0;
   return memo_fixed_bytes(C) + static_cast<size_t>(batch) * (static_cast<size_t>(kMemoCap) * pair_rec_bytes(g) + kProbRec);
 }
 
 // A split walk of `blocks` candidate blocks whose tiles cost `fill` trees' worth of walking each: the line of
 // trees (see SplitArgs) and the CTAs that share it, one for every place of the machine unless a stretch
-// would be shorter than a tile and a unit. Returns the CTAs.
+// would be shorter than a tile and a unit. Returns the CTAs; without units, whole blocks do as well.
 // Measured: 61,140 candidates x 500 trees (60 blocks, one CTA an SM) on 120 CTAs in equal slices 79 us, on 148 by
 // stretches 68; 96,000 candidates (94 blocks), 282 CTAs in two rounds 114, now 84; a million given rows (977
 // blocks, 6.6 rounds) 930, now 896.
@@ -1501,17 +1586,54 @@ static int split_plan(const GbdtModel& g, int64_t blocks, int fill, SplitArgs* s
   s->units = (g.n_chunks + rings - 1) / rings;
   s->unit = rings * g.tpc;
   s->fill = fill;
-  s->blocks = blocks;
-  const int64_t most = blocks * split_block(*s) / (s->fill + s->unit), slots = static_cast<int64_t>(g.ctas_per_sm) * kSmCount;
-  return static_cast<int>(std::max<int64_t>(1, std::min(most, slots)));
+  s->blocks = static_cast<int>(blocks);
+  const auto deal = [&](int64_t ctas) {
+    const int64_t total = blocks * split_block(*s);
+    s->step = static_cast<int>(total / ctas);
+    s->rest = static_cast<int>(total % ctas);
+    return static_cast<int>(ctas);
+  };
+  const int64_t len = split_block(*s), slots = static_cast<int64_t>(g.ctas_per_sm) * kSmCount;
+  // Whole rounds that are nearly full are left as they are (293 blocks of 300,000 given rows: split 4 % slower).
+  const int64_t rounds = (blocks + slots - 1) / slots;
+  if (rounds > 1 && 20 * blocks >= 19 * rounds * slots) {
+    s->units = 0;
+    return 0;
+  }
+  // The last CTA of a block reads all its parts, 0.1 us each: 32 at most (one block of 1,000 trees: 125 parts 93 us the
+  // whole call, 32 parts 80).
+  constexpr int64_t kParts = 32;
+  const int64_t most = std::max<int64_t>(1, std::min({blocks * len / (fill + s->unit), slots, kParts * blocks}));
+  // Stretches that end where blocks do spare the second tile and the second part of most CTAs (some 4 us):
+  // an equal number of CTAs a block, where that keeps nearly all of them busy.
+  const int64_t each = std::min<int64_t>({slots / blocks, s->units, kParts});
+  if (each >= 1) {
+    const int64_t aligned = (s->units + each - 1) / each * s->unit;
+    const int64_t shared = (blocks * len / most - fill + s->unit - 1) / s->unit * s->unit + fill + 16;
+    if (aligned <= shared) {
+      s->fill = 0;
+      return deal(blocks * each);
+    }
+  }
+  return deal(most);
 }
 // A tile that is built in the walk from prepared records takes 7 us, and one that is copied 2 to 3, where
 // a tree of eight levels takes a block of 1,024 candidates 0.25 us.
 constexpr int kFillRecords = 28, kFillCopy = 10;
 
-// Whether a dense walk of so many blocks is split: where whole blocks would leave part of the machine idle.
-bool fast_splits(const GbdtModel& g, int64_t blocks) {
-  return blocks >= 1 && blocks < static_cast<int64_t>(g.ctas_per_sm) * kSmCount && g.n_chunks > ring_count(g.fast_threads / (g.block_cands / 4));
+// Whether a dense walk of so many blocks is split: where whole blocks would leave part of the machine idle,
+// in the only round of CTAs or in the last of a few. Measured against whole blocks that fill their tiles in
+// the walk (500 trees, 256 bins): 7 problems x 61,140 valid candidates (420 blocks) 533 -> 455 us, 31 x 61,140 (1,860) 2,117 ->
+// 1,900, 64 x 9,000 grid candidates (576) 695 -> 595. From 32 problems on a catalogue in similarity order with class
+// records is the alternative: 100 x 9,000 (900 blocks) 1,110 -> 934, 32 x 60,000 (1,888) 1,879 -> 1,959. A problem looks through those
+// before it for its type combination, so there may not be very many.
+constexpr int kSplitBlocks = 13 * kSmCount, kSplitBlocksMemo = 8 * kSmCount, kSplitProblems = 512;
+static bool split_fits(const GbdtModel& g, int64_t blocks) {  // (a line of trees is counted in 32 bits)
+  return blocks * (static_cast<int64_t>(g.n_chunks + 2) * g.tpc + 64) < int64_t{1} << 30;
+}
+bool fast_splits(const GbdtModel& g, int P, int nblk, bool one_round) {
+  const int64_t blocks = static_cast<int64_t>(P) * nblk;
+  return split_fits(g, blocks) && P >= 1 && P <= kSplitProblems && blocks < (one_round ? g.ctas_per_sm * kSmCount : P < kMemoMinProblems ? kSplitBlocks : kSplitBlocksMemo) && g.n_chunks > ring_count(g.fast_threads / (g.block_cands / 4));
 }
 size_t fast_split_bytes(const GbdtModel& g) { return sizeof(double) * 2 * 2 * kSmCount * g.block_cands; }
 static_assert(2 * kSmCount <= kMaxShares, "an arrival counter for every CTA");
@@ -1723,7 +1845,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
   fv.cand_rows = d_rows;
   if (!seg_off && perm) a.seg_idx = perm;  // dense form ranked in the given order of the catalogue
   MemoView memo{};
-  int memo_batch = (memo_mem && !p_by_value && C > 0) ? fast_memo_batch(g, P) : 0;
+  int memo_batch = (memo_mem && !p_by_value && C > 0) ? fast_memo_batch(g, P, seg_off != nullptr, wait->lean) : 0;
   if (memo_batch > 0) memo = memo_view(memo_mem, C);
   if (prep) {  // prepared catalogue: candidate-only rows and classes were made once, for every type combination
     fv.cand_rows = prep->cand_rows;
@@ -1767,13 +1889,18 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     e = ensure_dynamic_smem(reinterpret_cast<const void*>(&tile_pairs_kernel), smem);
     if (e != cudaSuccess) return e;
     const int W = g.block_cands / 4, groups = nblk * (W / 32);
-    const int resident = std::max<int>(1, std::min<int>(3, 226 * 1024 / (smem + 4096)));
-    if (C > 0)
+    const int resident = std::max<int>(1, std::min<int>(4, 226 * 1024 / (smem + 4096)));
+    const PairTiles tiles = pair_tiles(g, P, nblk, split->tiles);
+    if (C > 0) {
       tile_pairs_kernel<<<std::min(P * groups, resident * kSmCount), 256, smem, stream>>>(
-          desc, d_p, a.pv, a.uv, P, d_c, C, fv, W, groups, split->tiles, wait->words);
-    else
-      e = cudaMemsetAsync(split->tiles, 0x80, fast_tiles_bytes(g, static_cast<int64_t>(P) * nblk), stream);
+          desc, d_p, a.pv, a.uv, P, d_c, C, fv, W, groups, tiles, wait->words);
+    } else {  // (nobody is ranked: any bytes with the top bit, and an index in range)
+      e = cudaMemsetAsync(split->tiles, 0x80, tiles.prob - split->tiles, stream);
+      if (e == cudaSuccess) e = cudaMemsetAsync(tiles.prob, 0, static_cast<size_t>(P) * kProbRec, stream);
+    }
     if (e != cudaSuccess) return e;
+    fv.prob_tab = tiles.prob;
+    a.sl.cand_tiles = tiles.cand;
     ++*launches;
   } else if (C > 0) {
     if (memo.keys) {
@@ -1810,11 +1937,10 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
 
   a.sl.words = wait->words;
   if (split) {
-    a.split_ctas = split_plan(g, static_cast<int64_t>(P) * nblk, tiles_mode ? kFillCopy : kFillRecords, &a.sl);
     a.sl.scores = split->scores;
     a.sl.out_idx = split->out_idx;
     a.sl.out_score = split->out_score;
-    a.sl.tiles = tiles_mode ? split->tiles : nullptr;
+    a.sl.tiles = tiles_mode ? split->tiles : nullptr;  // (per-pair rows first)
     a.sl.out_seq = split->out_seq;
     a.sl.seq = split->seq;
   }
@@ -1837,6 +1963,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     a.P = n;
     a.seg_off = seg_off ? seg_off + first : nullptr;
     a.partial = partial + static_cast<size_t>(first) * nblk * k;
+    if (split) a.split_ctas = split_plan(g, static_cast<int64_t>(n) * nblk, tiles_mode ? kFillCopy : kFillRecords, &a.sl);
     e = launch_walk(g, a);
     ++*launches;
     if (e != cudaSuccess) return e;
@@ -1885,7 +2012,7 @@ cudaError_t launch_score_fast(const ks_gpu_desc& desc, const GbdtModel& g, const
     a.C = static_cast<int>(n);
     a.nblk = nblk;
     a.sl = SplitArgs{};
-    if (floor_repeat == 0 && (g.ctas_per_sm == 1 || nblk < 2 * kSmCount)) {
+    if (floor_repeat == 0 && (g.ctas_per_sm == 1 || nblk < 2 * kSmCount) && split_fits(g, nblk)) {
       a.split_ctas = split_plan(g, nblk, kFillCopy, &a.sl);
       a.sl.scores = reinterpret_cast<double*>(tiles + score_fast_scratch_bytes(g, std::min(rows, kScoreBatchRows)) - fast_split_bytes(g));
     }

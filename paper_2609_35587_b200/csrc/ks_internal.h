@@ -67,7 +67,7 @@ struct FeatQ {
 struct FastWait {
   int limit;
   int starve;
-  int lean;  // the memory for all of the workspace could not be had: without the walk of whole classes, few rows at a time
+  int lean;  // the memory for all of the workspace could not be had: without the walk of whole classes, few rows or problems at a time
   int* words;
 };
 
@@ -176,7 +176,7 @@ constexpr int kFastMaxDepth = 10;
 constexpr int kFastMaxProbRows = 256;  // rows of problem-only features
 constexpr int kFastMaxCandRec = 256;   // rows of candidate-only features (bytes of a per-call record)
 constexpr int kFastMaxPairRec = 256;   // rows of per-pair features a memoised model may have
-constexpr size_t kMemoTableBytes = size_t(256) << 20;  // per-(problem, class) records held at a time
+constexpr size_t kMemoTableBytes = size_t(512) << 20;  // per-(problem, class) records held at a time
 constexpr int kFastWaitLimit = 1 << 17;  // probes of a chunk wait (a sleep ends early, ~0.2 us measured): tens of ms
 constexpr int kMlpThreads = 512;        // threads per block of the tensor-core MLP kernel
 constexpr int kMaxShares = 1024;       // CTAs that a split walk may have
@@ -221,7 +221,7 @@ struct FastSplit {
   double* scores;    // fast_split_bytes: partial sums
   int32_t* out_idx;  // single-problem form: [k], device-visible; else null (a merge kernel follows)
   float* out_score;
-  uint8_t* tiles;    // scratch for the tiles [problems * blocks][rows][block_cands], or null
+  uint8_t* tiles;    // fast_tiles_bytes of scratch for tiles that are built in front of the walk, or null
   int* out_seq;      // single-problem form: device-visible word that receives `seq` after the results
   int seq;
 };
@@ -270,8 +270,8 @@ cudaError_t launch_remap_indices(int32_t* d_idx, long long n, const int32_t* d_m
 // Quantised tree path: blocks per problem for `per_problem` rows, and the launch itself.
 void fast_tiling(const GbdtModel& g, int P, int64_t per_problem, int* nblk, int* rows_per_cta);
 size_t fast_scratch_bytes(const GbdtModel& g, int C);  // per-call table of candidate-only rows
-size_t fast_tiles_bytes(const GbdtModel& g, int64_t blocks);  // the tiles of that many (problem, candidate block) pairs
-size_t fast_memo_bytes(const GbdtModel& g, int P, int C);  // memo of the per-pair rows (0: not used)
+size_t fast_tiles_bytes(const GbdtModel& g, int P, int nblk);  // tiles of a dense walk, built in front of it
+size_t fast_memo_bytes(const GbdtModel& g, int P, int C, bool segmented, bool lean);  // memo of the per-pair rows (0: not used)
 void free_fast_gbdt(GbdtModel& m);
 cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, const ks_problem* d_p,
                                const ks_problem* p_by_value, int P, const ks_candidate* d_c, int C,
@@ -286,7 +286,8 @@ size_t fast_prepared_rows_bytes(const GbdtModel& g, int C);
 size_t fast_prepared_memo_bytes(const GbdtModel& g, int C);  // 0: the model's per-pair rows do not fit a record
 cudaError_t fast_prepare(const ks_gpu_desc& desc, const GbdtModel& g, const ks_candidate* d_c, int C, void* d_rows,
                          void* memo_mem, cudaStream_t stream, int64_t* launches);
-bool fast_splits(const GbdtModel& g, int64_t blocks);  // whether a dense walk of so many blocks is split
+// whether a dense walk of P problems with so many blocks each is split (`one_round`: only where they are fewer than the machine's CTAs)
+bool fast_splits(const GbdtModel& g, int P, int nblk, bool one_round);
 size_t fast_split_bytes(const GbdtModel& g);
 // ks_score with a qualifying ensemble: tiles quantised from the feature rows, then the same walk.
 size_t score_fast_scratch_bytes(const GbdtModel& g, int64_t rows);

@@ -1080,17 +1080,22 @@ static int64_t per_problem_rows(int P, int C, int64_t pairs, bool segmented) {
   return segmented ? (P > 0 ? (pairs + P - 1) / P : 0) : C;
 }
 
+// Dense walks that are split: few blocks, and not for the walk of whole classes to serve.
+static bool select_splits(const GbdtModel& g, int P, int C, int64_t pairs, int nblk, bool segmented, bool lean) {
+  return !segmented && fast_splits(g, P, nblk, lean) && (lean || !classes_apply(g, P, C, pairs));
+}
+
 size_t select_partial_bytes(const ks_model& model, int P, int C, int64_t pairs, bool segmented, int k, bool lean) {
   const int64_t per = per_problem_rows(P, C, pairs, segmented);
   if (model.kind == 0 && model.gbdt.fast) {
     int nblk, rows;
     fast_tiling(model.gbdt, P, per, &nblk, &rows);
     const size_t part = (static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
-    if (!segmented && fast_splits(model.gbdt, static_cast<int64_t>(P) * nblk)) {
+    if (select_splits(model.gbdt, P, C, pairs, nblk, segmented, lean)) {
       return part + fast_split_bytes(model.gbdt) + 512 +
-             std::max(fast_scratch_bytes(model.gbdt, C), fast_tiles_bytes(model.gbdt, static_cast<int64_t>(P) * nblk));
+             std::max(fast_scratch_bytes(model.gbdt, C), fast_tiles_bytes(model.gbdt, P, nblk));
     }
-    const size_t memo = (fast_memo_bytes(model.gbdt, P, C) + 255) / 256 * 256;
+    const size_t memo = (fast_memo_bytes(model.gbdt, P, C, segmented, lean) + 255) / 256 * 256;
     // a dense batch is ranked in similarity order of the catalogue (ks_order.cu)
     const bool classes = memo > 0 && !lean && classes_apply(model.gbdt, P, C, pairs);
     const size_t order = (memo > 0 && P >= kOrderMinProblems && (!segmented || classes))
@@ -1138,14 +1143,14 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     const size_t part_bytes = (static_cast<size_t>(P) * nblk * k * sizeof(unsigned long long) + 255) / 256 * 256;
     // an under-filled machine: the CTAs share out the blocks' trees (dense form only, where a block covers
     // its rows in one pass)
-    const bool splits = !d_seg_off && fast_splits(model.gbdt, static_cast<int64_t>(P) * nblk);  // as sized
+    const bool splits = select_splits(model.gbdt, P, C, pairs, nblk, d_seg_off != nullptr, wait->lean);  // as sized
     char* mem = static_cast<char*>(d_partial) + part_bytes;
     FastSplit split{};
     // the parts of a block share a tile that is built in front of them; behind the tiles, their sums
     split.tiles = reinterpret_cast<uint8_t*>(mem);
-    split.scores = reinterpret_cast<double*>(mem + (fast_tiles_bytes(model.gbdt, static_cast<int64_t>(P) * nblk) + 255) / 256 * 256);
+    split.scores = reinterpret_cast<double*>(mem + fast_tiles_bytes(model.gbdt, P, nblk));
     // the memo of the per-pair rows sits behind the per-call table (batches of whole-ensemble CTAs only)
-    void* memo_mem = (splits || p_by_value || fast_memo_bytes(model.gbdt, P, C) == 0)
+    void* memo_mem = (splits || p_by_value || fast_memo_bytes(model.gbdt, P, C, d_seg_off != nullptr, wait->lean) == 0)
                          ? nullptr
                          : mem + (fast_scratch_bytes(model.gbdt, C) + 255) / 256 * 256;
     // a dense batch of problems: rank the catalogue in similarity order (neighbouring candidates
@@ -1154,7 +1159,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     ClassCall classes{pairs, nullptr, nullptr};
     const bool use_classes = memo_mem && !wait->lean && classes_apply(model.gbdt, P, C, pairs);
     if (memo_mem && P >= kOrderMinProblems && C > 0 && (!d_seg_off || use_classes)) {
-      char* order_mem = static_cast<char*>(memo_mem) + (fast_memo_bytes(model.gbdt, P, C) + 255) / 256 * 256;
+      char* order_mem = static_cast<char*>(memo_mem) + (fast_memo_bytes(model.gbdt, P, C, d_seg_off != nullptr, wait->lean) + 255) / 256 * 256;
       cudaError_t eo = launch_catalogue_order(d_c, C, order_mem, stream, launches);
       if (eo != cudaSuccess) return eo;
       if (!d_seg_off) perm = reinterpret_cast<const int32_t*>(order_mem);

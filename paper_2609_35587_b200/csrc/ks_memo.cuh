@@ -20,8 +20,8 @@
 namespace ks {
 
 constexpr int kMemoCombos = 16;  // dtype_ab x dtype_d
-constexpr int kMemoCap = 8192;   // slots per type combination (a power of two)
-constexpr int kMemoMinProblems = 32;
+constexpr int kMemoCap = 16384;  // slots per type combination: a power of two above the 10,785 classes of the valid search space
+constexpr int kMemoMinProblems = 32, kMemoMinDense = 3;  // (segmented and dense batches)
 constexpr int kMemoMaxProblems = 8192;
 constexpr unsigned kNoClass = 0xFFFFFFFFu;
 
@@ -61,7 +61,7 @@ __device__ __forceinline__ unsigned memo_slot(unsigned long long* keys, int* rep
     const unsigned long long prev = atomicCAS(keys + h, 0ull, key);
     if (prev == 0ull) reps[h] = i;  // this thread made the slot
     if (prev == 0ull || prev == key) return h;
-    h = (h + 1) & (kCap - 1);
+    h = (h + probe + 1) & (kCap - 1);  // (steps of 1, 2, 3, ...: no clusters)
   }
   return kNoClass;
 }
