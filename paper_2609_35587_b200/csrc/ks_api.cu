@@ -746,24 +746,22 @@ ks_status ks_catalogue_prepare(ks_ctx* ctx, const ks_candidate* d_c, int C, cons
   const ks::GbdtModel& g = model->gbdt;
   if (model->kind == 0 && g.fast && C > 0) {
     const int nblk = (C + g.block_cands - 1) / g.block_cands;
-    const size_t b_memo = ks::fast_prepared_memo_bytes(g, C);
-    if (ks::fast_splits(g, 1, nblk, true) && b_memo > 0) {
+    if (ks::fast_splits(g, 1, nblk, true)) {
       DeviceGuard guard(ctx->device);
-      const size_t b_rows = align_up(ks::fast_prepared_rows_bytes(g, C));
+      const size_t b_rows = ks::fast_prepared_rows_bytes(g, nblk);
       const size_t b_part = align_up(sizeof(unsigned long long) * nblk * KS_MAX_K);
       const size_t b_scores = align_up(ks::fast_split_bytes(g));
-      cat->off_memo = b_rows;
-      cat->off_part = b_rows + align_up(b_memo);
+      cat->off_call = b_rows;
+      cat->off_part = b_rows + align_up(ks::fast_prepared_call_bytes(g, nblk));
       cat->off_scores = cat->off_part + b_part;
       cat->off_order = cat->off_scores + b_scores;
       cudaError_t e = cudaMalloc(&cat->d_mem, cat->off_order + ks::order_scratch_bytes(C));
-      if (e == cudaSuccess)
-        e = ks::fast_prepare(ctx->desc, g, d_c, C, cat->d_mem, static_cast<char*>(cat->d_mem) + cat->off_memo,
-                             static_cast<cudaStream_t>(stream), &ctx->launches);
       // the catalogue is ranked in similarity order (neighbouring candidates take similar paths)
+      int* order = reinterpret_cast<int*>(static_cast<char*>(cat->d_mem) + cat->off_order);
       if (e == cudaSuccess)
-        e = ks::launch_catalogue_order(d_c, C, static_cast<char*>(cat->d_mem) + cat->off_order,
-                                       static_cast<cudaStream_t>(stream), &ctx->launches);
+        e = ks::launch_catalogue_order(d_c, C, order, static_cast<cudaStream_t>(stream), &ctx->launches);
+      if (e == cudaSuccess)
+        e = ks::fast_prepare(ctx->desc, g, d_c, C, nblk, cat->d_mem, order, static_cast<cudaStream_t>(stream), &ctx->launches);
       if (e == cudaSuccess) e = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
       if (e != cudaSuccess) {
         cudaFree(cat->d_mem);
@@ -808,7 +806,7 @@ ks_status ks_select_one_prepared(ks_ctx* ctx, const ks_catalogue* cat, ks_proble
   int* h_seq = reinterpret_cast<int*>(pin_sc + KS_MAX_K);
   sl.out_seq = reinterpret_cast<int*>(ctx->d_pinned_score + KS_MAX_K);
   sl.seq = ++ctx->select_one_seq;
-  ks::FastPrepared prep{reinterpret_cast<const uint8_t*>(base), base + cat->off_memo};
+  ks::FastPrepared prep{reinterpret_cast<const uint8_t*>(base), reinterpret_cast<uint8_t*>(base + cat->off_call)};
   cudaError_t e = ks::launch_select_fast(ctx->desc, gm, nullptr, &p, 1, cat->d_c, cat->C, cat->nblk, gm.block_cands,
                                          nullptr, nullptr, k, reinterpret_cast<unsigned long long*>(base + cat->off_part),
                                          nullptr, ctx->d_status, st, &ctx->launches, nullptr, &sl, nullptr, &ctx->wait,

@@ -226,7 +226,7 @@ constexpr int kProbRec = kFastMaxProbRows + 128;  // problem-only rows, then the
 static_assert(sizeof(ProblemTerms) <= 128, "problem record");
 
 __global__ void __launch_bounds__(256)
-pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int n_prob,
+pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, int n_prob,
                   const ks_candidate* __restrict__ c, FastView fv, MemoView memo, int thr_cap, const int* path, int* words) {
   extern __shared__ __align__(16) float s_pthr[];  // thresholds of the per-pair features, then the records
   __shared__ ProblemTerms s_pt;
@@ -257,7 +257,7 @@ pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem
   for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
     const int prob = item / class_blocks, j = (item % class_blocks) * 256 + tid;
     const bool first_block = item % class_blocks == 0;
-    const ks_problem pr = use_value ? p_value : load_problem(p + prob);
+    const ks_problem pr = load_problem(p + prob);
     const int combo = (pr.dtype_ab & 3) * 4 + (pr.dtype_d & 3);
     const int n_classes = memo.count[combo];
     __syncthreads();  // the previous item's terms are no longer read (and the staging is complete)
@@ -364,7 +364,9 @@ inline PairTiles pair_tiles(const GbdtModel& g, int P, int nblk, uint8_t* mem) {
 // candidate's columns; then a warp takes every eighth column, four candidates a lane, and stores whole
 // lines, in the layout phase A would produce. The first problem of a type combination also brings the
 // candidate-only columns, for all that have it, and the first item of a problem its problem-only rows.
-// Slots past the catalogue get the last candidate's bytes (they are not ranked). Also clears the abort flag
+// Two more forms serve a prepared catalogue, whose candidates are taken in `order`: without `tiles.pair` the candidate-only
+// rows of all 16 type combinations, once; without `tiles.cand` a call's per-pair rows and record, which then names the
+// combination. Slots past the catalogue get the last candidate's bytes (they are not ranked). Also clears the abort flag
 // (this kernel precedes the select kernel). What bounds it is the issue of the searches beside the
 // latency of the columns' divisions. One problem x 61,140 candidates, 500 trees: 18 us (21 with the candidate-only columns
 // for every problem, four searches of the problem-only ones in every lane and a last item for some blocks; a thread that
@@ -377,7 +379,8 @@ static_assert(kTileMaxThr >= 376 * kSlice, "every ensemble of the regular geomet
 
 __global__ void __launch_bounds__(256, 4)
 tile_pairs_kernel(const __grid_constant__ ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value, int P,
-                  const ks_candidate* __restrict__ c, int C, FastView fv, int W, int groups, PairTiles tiles, int* words) {
+                  const ks_candidate* __restrict__ c, int C, const int* __restrict__ order, FastView fv, int W, int groups,
+                  PairTiles tiles, int* words) {
   extern __shared__ __align__(16) float s_x[];  // [kTileCols][kTileRows], then the thresholds of every feature
   __shared__ ProblemTerms s_pt;
   __shared__ FeatQ s_fq[64];
@@ -386,15 +389,24 @@ tile_pairs_kernel(const __grid_constant__ ks_gpu_desc desc, const ks_problem* __
   float* s_thr = s_x + kTileCols * kTileRows;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the walk waits for this grid before it reads the tiles)
-  if (blockIdx.x == 0 && tid == 0) words[kWordWalk] = 0;
+  if (words && blockIdx.x == 0 && tid == 0) words[kWordWalk] = 0;
+  const bool cand_only = !tiles.pair, prepared = !tiles.cand;
   const long long n_items = static_cast<long long>(P) * groups;
   const int begin = static_cast<int>(n_items * blockIdx.x / gridDim.x);
   const int end = static_cast<int>(n_items * (blockIdx.x + 1) / gridDim.x);
   // A problem's terms and columns (the logarithms by threads of their own), and the first problem of its combination.
   // Between two barriers.
+  const auto fetch = [&](int prob) {
+    ks_problem pr = use_value ? p_value : load_problem(p + prob);
+    if (cand_only) {  // "problem" stands for a type combination
+      pr.dtype_ab = static_cast<uint8_t>(prob >> 2);
+      pr.dtype_d = static_cast<uint8_t>(prob & 3);
+    }
+    return pr;
+  };
   const auto evaluate = [&](int prob) {
     if (tid < 128 && (tid & 31) == 0) {
-      const ks_problem pr = use_value ? p_value : load_problem(p + prob);
+      const ks_problem pr = fetch(prob);
       if (tid == 0) {
         problem_terms<false>(pr, desc, s_pt);
         problem_columns(s_pt, [&](int col, float v) { if (col > 2) s_pf[col] = v; });
@@ -402,8 +414,8 @@ tile_pairs_kernel(const __grid_constant__ ks_gpu_desc desc, const ks_problem* __
         s_pf[warp - 1] = log2_dim(warp == 1 ? pr.m : (warp == 2 ? pr.n : pr.k));
       }
     } else if (tid >= 128) {
-      const ks_problem pr = use_value ? p_value : load_problem(p + prob);
-      int first = prob;
+      const ks_problem pr = fetch(prob);
+      int first = prepared ? (pr.dtype_ab & 3) * 4 + (pr.dtype_d & 3) : prob;
       if (!use_value)
         for (int q = tid - 128; q < first; q += 128) {
           const ks_problem other = load_problem(p + q);
@@ -430,7 +442,7 @@ tile_pairs_kernel(const __grid_constant__ ks_gpu_desc desc, const ks_problem* __
       held = prob;
       __syncthreads();
     }
-    if (g == 0) {
+    if (g == 0 && !cand_only) {
       uint8_t* rec = tiles.prob + static_cast<size_t>(prob) * kProbRec;
       if (tid < KS_F && feat_class(tid) == 0) {
         const FeatQ& q = s_fq[tid];
@@ -439,11 +451,13 @@ tile_pairs_kernel(const __grid_constant__ ks_gpu_desc desc, const ks_problem* __
       }
       if (tid == 64) *reinterpret_cast<int*>(rec + kFastMaxProbRows) = s_first;
     }
-    const bool with_cand = s_first == prob;
-    const int row = tid % kTileRows;
-    const ks_candidate cand = load_candidate(c + min(g * kTileRows + row, C - 1));
+    const bool with_cand = s_first == prob && !prepared;
+    const int row = tid % kTileRows, place = min(g * kTileRows + row, C - 1);
+    const ks_candidate cand = load_candidate(c + (order ? __ldg(order + place) : place));
     const long long b_eff = resources(s_pt, cand, desc).b_eff;
-    if (tid < kTileRows)
+    if (cand_only)
+      ;
+    else if (tid < kTileRows)
       pair_columns<true>(s_pt, cand, desc, b_eff, [&](int col, float v) { if (col <= 32) s_x[pair_slot(col) * kTileRows + row] = v; });
     else
       pair_columns<true>(s_pt, cand, desc, b_eff, [&](int col, float v) { if (col > 32) s_x[pair_slot(col) * kTileRows + row] = v; });
@@ -461,7 +475,7 @@ tile_pairs_kernel(const __grid_constant__ ks_gpu_desc desc, const ks_problem* __
     // (rows are counted over the whole tile: the candidate-only ones follow the per-pair ones)
     uint32_t* cand_out = reinterpret_cast<uint32_t*>(tiles.cand) + block * fv.n_cand_rows * W + word - static_cast<ptrdiff_t>(fv.n_pair_rows) * W;
 #pragma unroll 1
-    for (int slot = warp; slot < (with_cand ? kTileCols : kPairCols); slot += 8) {
+    for (int slot = warp + (cand_only ? kPairCols : 0); slot < (with_cand ? kTileCols : kPairCols); slot += 8) {
       const bool is_pair = slot < kPairCols;
       const float4 x = *reinterpret_cast<const float4*>(s_x + slot * kTileRows + 4 * lane);
       tile_column(s_fq[is_pair ? pair_col(slot) : cand_col(slot - kPairCols)], x, thr, fv.n_rows, W, is_pair ? pair_out : cand_out);
@@ -876,7 +890,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
         if (bytes) bulk_copy_g2s(sbase + kOffTile, sl.tiles + (static_cast<size_t>(prob) * nblk + chunk) * bytes, bytes, bar);
         // (the record's terms are the first problem of the combination here)
         if (more) {
-          const size_t first = KS_IDX(*reinterpret_cast<const int*>(&s_pt), P);
+          const size_t first = KS_IDX(*reinterpret_cast<const int*>(&s_pt), P > kCombos ? P : kCombos);
           bulk_copy_g2s(sbase + kOffTile + bytes, sl.cand_tiles + (first * nblk + chunk) * more, more, bar);
         }
       }
@@ -1575,13 +1589,17 @@ size_t fast_memo_bytes(const GbdtModel& g, int P, int C, bool segmented, bool le
   return memo_fixed_bytes(C) + static_cast<size_t>(batch) * (static_cast<size_t>(kMemoCap) * pair_rec_bytes(g) + kProbRec);
 }
 
-// A split walk of `blocks` candidate blocks whose tiles cost `fill` trees' worth of walking each: the line of
+// Copying a tile takes 2 to 3 us, where a tree of eight levels takes a block of 1,024 candidates 0.25 us.
+constexpr int kFillCopy = 10;
+
+// A split walk of `blocks` candidate blocks: the line of
 // trees (see SplitArgs) and the CTAs that share it, one for every place of the machine unless a stretch
 // would be shorter than a tile and a unit. Returns the CTAs; without units, whole blocks do as well.
 // Measured: 61,140 candidates x 500 trees (60 blocks, one CTA an SM) on 120 CTAs in equal slices 79 us, on 148 by
 // stretches 68; 96,000 candidates (94 blocks), 282 CTAs in two rounds 114, now 84; a million given rows (977
 // blocks, 6.6 rounds) 930, now 896.
-static int split_plan(const GbdtModel& g, int64_t blocks, int fill, SplitArgs* s) {
+static int split_plan(const GbdtModel& g, int64_t blocks, SplitArgs* s) {
+  const int fill = kFillCopy;
   const int rings = ring_count(g.fast_threads / (g.block_cands / 4));
   s->units = (g.n_chunks + rings - 1) / rings;
   s->unit = rings * g.tpc;
@@ -1617,10 +1635,6 @@ static int split_plan(const GbdtModel& g, int64_t blocks, int fill, SplitArgs* s
   }
   return deal(most);
 }
-// A tile that is built in the walk from prepared records takes 7 us, and one that is copied 2 to 3, where
-// a tree of eight levels takes a block of 1,024 candidates 0.25 us.
-constexpr int kFillRecords = 28, kFillCopy = 10;
-
 // Whether a dense walk of so many blocks is split: where whole blocks would leave part of the machine idle,
 // in the only round of CTAs or in the last of a few. Measured against whole blocks that fill their tiles in
 // the walk (500 trees, 256 bins): 7 problems x 61,140 valid candidates (420 blocks) 533 -> 455 us, 31 x 61,140 (1,860) 2,117 ->
@@ -1638,10 +1652,12 @@ bool fast_splits(const GbdtModel& g, int P, int nblk, bool one_round) {
 size_t fast_split_bytes(const GbdtModel& g) { return sizeof(double) * 2 * 2 * kSmCount * g.block_cands; }
 static_assert(2 * kSmCount <= kMaxShares, "an arrival counter for every CTA");
 
-size_t fast_prepared_rows_bytes(const GbdtModel& g, int C) { return static_cast<size_t>(kCombos) * C * cand_rec_bytes(g); }
-size_t fast_prepared_memo_bytes(const GbdtModel& g, int C) {
-  if (g.n_pair_rows < 1 || g.n_pair_rows > kFastMaxPairRec || C < 1) return 0;
-  return memo_fixed_bytes(C) + static_cast<size_t>(kMemoCap) * pair_rec_bytes(g) + kProbRec;
+// A prepared catalogue: the candidate-only rows of its tiles for every type combination, and a call's scratch.
+size_t fast_prepared_rows_bytes(const GbdtModel& g, int nblk) {
+  return (static_cast<size_t>(kCombos) * nblk * g.n_cand_rows * g.block_cands + 255) / 256 * 256;
+}
+size_t fast_prepared_call_bytes(const GbdtModel& g, int nblk) {
+  return (static_cast<size_t>(nblk) * g.n_pair_rows * g.block_cands + 255) / 256 * 256 + kProbRec;
 }
 
 namespace {
@@ -1771,26 +1787,30 @@ static cudaError_t launch_cand_rows(const ks_gpu_desc& desc, const GbdtModel& g,
   return cudaGetLastError();
 }
 
-// Prepared catalogue: the candidate-only rows of every candidate under every element-type
-// combination, and the candidates' classes, computed once for a (catalogue, model) pair.
-cudaError_t fast_prepare(const ks_gpu_desc& desc, const GbdtModel& g, const ks_candidate* d_c, int C, void* d_rows,
-                         void* memo_mem, cudaStream_t stream, int64_t* launches) {
-  FastView fv = make_view(g, nullptr);
-  MemoView memo{};
-  if (memo_mem) memo = memo_view(memo_mem, C);
-  cudaError_t e = cudaSuccess;
-  if (memo.keys) {
-    e = memo_clear(memo, stream);
-    if (e != cudaSuccess) return e;
-  }
-  e = launch_cand_rows(desc, g, d_c, C, nullptr, -1, fv, static_cast<uint8_t*>(d_rows), memo, nullptr, stream, launches);
+// The tile kernel in one of its forms, see there.
+static cudaError_t launch_tile_pairs(const ks_gpu_desc& desc, const GbdtModel& g, const ks_problem* d_p, const ks_problem& pv, int uv,
+                                     int P, const ks_candidate* d_c, int C, const int* order, int nblk, const PairTiles& tiles,
+                                     int* words, cudaStream_t stream, int64_t* launches) {
+  const size_t smem = sizeof(float) * (kTileCols * kTileRows + g.n_qthr);
+  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(&tile_pairs_kernel), smem);
   if (e != cudaSuccess) return e;
-  if (memo.keys) {
-    e = memo_compact(memo, stream);
-    if (e != cudaSuccess) return e;
-    ++*launches;
-  }
+  const int W = g.block_cands / 4, groups = nblk * (W / 32);
+  const int resident = std::max<int>(1, std::min<int>(4, 226 * 1024 / (smem + 4096)));
+  tile_pairs_kernel<<<std::min(P * groups, resident * kSmCount), 256, smem, stream>>>(
+      desc, d_p, pv, uv, P, d_c, C, order, make_view(g, nullptr), W, groups, tiles, words);
+  ++*launches;
   return cudaGetLastError();
+}
+
+// Prepared catalogue: the candidate-only rows of its tiles, in the catalogue's order, for every type combination,
+// computed once for a (catalogue, model) pair.
+cudaError_t fast_prepare(const ks_gpu_desc& desc, const GbdtModel& g, const ks_candidate* d_c, int C, int nblk, void* d_rows,
+                         const int* order, cudaStream_t stream, int64_t* launches) {
+  if (g.n_cand_rows == 0) return cudaSuccess;
+  ks_problem any{};
+  any.m = any.n = any.k = 1;
+  return launch_tile_pairs(desc, g, nullptr, any, 1, kCombos, d_c, C, order, nblk, PairTiles{nullptr, static_cast<uint8_t*>(d_rows), nullptr},
+                           nullptr, stream, launches);
 }
 
 // Problems per launch when a call is served in batches of at most `cap`. In the launch form
@@ -1847,14 +1867,6 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
   MemoView memo{};
   int memo_batch = (memo_mem && !p_by_value && C > 0) ? fast_memo_batch(g, P, seg_off != nullptr, wait->lean) : 0;
   if (memo_batch > 0) memo = memo_view(memo_mem, C);
-  if (prep) {  // prepared catalogue: candidate-only rows and classes were made once, for every type combination
-    fv.cand_rows = prep->cand_rows;
-    if (prep->memo_mem) {
-      memo = memo_view(prep->memo_mem, C);
-      memo_batch = 1;
-    }
-  }
-
   // candidate-only rows for the type combinations in use
   cudaError_t e = cudaSuccess;
   const bool tiles_mode = !prep && split && split->tiles && !seg_off;
@@ -1877,23 +1889,15 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     pthr_bytes = thr_part + rec_bytes + 16;
   }
   if (prep) {
-    if (memo.keys) {
-      e = ensure_dynamic_smem(reinterpret_cast<const void*>(&pair_table_kernel), pthr_bytes);
-      if (e != cudaSuccess) return e;
-      fv.pair_class = memo.cls;
-      fv.pair_tab = static_cast<const uint8_t*>(memo.tab);
-      fv.prob_tab = fv.pair_tab + static_cast<size_t>(kMemoCap) * pair_rec_bytes(g);
-    }
-  } else if (tiles_mode) {
-    const size_t smem = sizeof(float) * (kTileCols * kTileRows + g.n_qthr);
-    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&tile_pairs_kernel), smem);
+    const PairTiles tiles{prep->call, nullptr, prep->call + fast_prepared_call_bytes(g, nblk) - kProbRec};
+    e = launch_tile_pairs(desc, g, d_p, a.pv, a.uv, P, d_c, C, perm, nblk, tiles, wait->words, stream, launches);
     if (e != cudaSuccess) return e;
-    const int W = g.block_cands / 4, groups = nblk * (W / 32);
-    const int resident = std::max<int>(1, std::min<int>(4, 226 * 1024 / (smem + 4096)));
+    fv.prob_tab = tiles.prob;
+    a.sl.cand_tiles = prep->cand_rows;
+  } else if (tiles_mode) {
     const PairTiles tiles = pair_tiles(g, P, nblk, split->tiles);
     if (C > 0) {
-      tile_pairs_kernel<<<std::min(P * groups, resident * kSmCount), 256, smem, stream>>>(
-          desc, d_p, a.pv, a.uv, P, d_c, C, fv, W, groups, tiles, wait->words);
+      e = launch_tile_pairs(desc, g, d_p, a.pv, a.uv, P, d_c, C, nullptr, nblk, tiles, wait->words, stream, launches);
     } else {  // (nobody is ranked: any bytes with the top bit, and an index in range)
       e = cudaMemsetAsync(split->tiles, 0x80, tiles.prob - split->tiles, stream);
       if (e == cudaSuccess) e = cudaMemsetAsync(tiles.prob, 0, static_cast<size_t>(P) * kProbRec, stream);
@@ -1901,7 +1905,6 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     if (e != cudaSuccess) return e;
     fv.prob_tab = tiles.prob;
     a.sl.cand_tiles = tiles.cand;
-    ++*launches;
   } else if (C > 0) {
     if (memo.keys) {
       e = memo_clear(memo, stream);
@@ -1940,7 +1943,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     a.sl.scores = split->scores;
     a.sl.out_idx = split->out_idx;
     a.sl.out_score = split->out_score;
-    a.sl.tiles = tiles_mode ? split->tiles : nullptr;  // (per-pair rows first)
+    a.sl.tiles = prep ? prep->call : split->tiles;  // (per-pair rows first)
     a.sl.out_seq = split->out_seq;
     a.sl.seq = split->seq;
   }
@@ -1955,15 +1958,15 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
       const int64_t table_slots = static_cast<int64_t>(kSmCount) * (2 * (pthr_bytes + 4096) <= 227 * 1024 ? 2 : 1);
       pair_table_kernel<<<static_cast<unsigned>(table_items < table_slots ? table_items : table_slots), 256, pthr_bytes,
                           stream>>>(
-          desc, d_p ? d_p + first : nullptr, a.pv, a.uv, n, d_c, fv, memo, pthr_cap, path, wait->words);
+          desc, d_p + first, n, d_c, fv, memo, pthr_cap, path, wait->words);
       ++*launches;
     }
-    a.dependent = memo.keys != nullptr || tiles_mode;
+    a.dependent = memo.keys != nullptr || tiles_mode || prep;
     a.d_p = d_p ? d_p + first : nullptr;
     a.P = n;
     a.seg_off = seg_off ? seg_off + first : nullptr;
     a.partial = partial + static_cast<size_t>(first) * nblk * k;
-    if (split) a.split_ctas = split_plan(g, static_cast<int64_t>(n) * nblk, tiles_mode ? kFillCopy : kFillRecords, &a.sl);
+    if (split) a.split_ctas = split_plan(g, static_cast<int64_t>(n) * nblk, &a.sl);
     e = launch_walk(g, a);
     ++*launches;
     if (e != cudaSuccess) return e;
@@ -2013,7 +2016,7 @@ cudaError_t launch_score_fast(const ks_gpu_desc& desc, const GbdtModel& g, const
     a.nblk = nblk;
     a.sl = SplitArgs{};
     if (floor_repeat == 0 && (g.ctas_per_sm == 1 || nblk < 2 * kSmCount) && split_fits(g, nblk)) {
-      a.split_ctas = split_plan(g, nblk, kFillCopy, &a.sl);
+      a.split_ctas = split_plan(g, nblk, &a.sl);
       a.sl.scores = reinterpret_cast<double*>(tiles + score_fast_scratch_bytes(g, std::min(rows, kScoreBatchRows)) - fast_split_bytes(g));
     }
     a.sl.words = wait->words;

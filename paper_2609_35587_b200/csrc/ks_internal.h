@@ -156,8 +156,8 @@ struct ks_catalogue {
   int device = 0;
   bool prepared = false;   // false: calls go through ks_select_one
   int nblk = 0, max_k = KS_MAX_K;
-  void* d_mem = nullptr;   // one block: rows | memo | partial lists | partial-score planes | similarity order
-  size_t off_memo = 0, off_part = 0, off_scores = 0, off_order = 0;
+  void* d_mem = nullptr;   // one block: candidate-only rows | a call's rows | partial lists | partial sums | similarity order
+  size_t off_call = 0, off_part = 0, off_scores = 0, off_order = 0;
 };
 
 struct ks_model {
@@ -228,8 +228,8 @@ struct FastSplit {
 
 // What a prepared catalogue hands to the quantised tree kernel instead of per-call work.
 struct FastPrepared {
-  const uint8_t* cand_rows;  // [16 type combinations][C][record] candidate-only rows
-  void* memo_mem;            // class tables and ids of every combination + one problem's record table, or null
+  const uint8_t* cand_rows;  // [16 type combinations][blocks][candidate-only rows][block_cands], in the catalogue's order
+  uint8_t* call;             // fast_prepared_call_bytes: per-pair rows and record of a call's problem
 };
 
 // Similarity order of a catalogue (ks_order.cu): positions sorted so that neighbours differ in as
@@ -282,10 +282,10 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
                                const FastPrepared* prep = nullptr, const int32_t* perm = nullptr,
                                const ClassCall* classes = nullptr);
 // Prepared catalogue (single-problem calls against a fixed catalogue and model).
-size_t fast_prepared_rows_bytes(const GbdtModel& g, int C);
-size_t fast_prepared_memo_bytes(const GbdtModel& g, int C);  // 0: the model's per-pair rows do not fit a record
-cudaError_t fast_prepare(const ks_gpu_desc& desc, const GbdtModel& g, const ks_candidate* d_c, int C, void* d_rows,
-                         void* memo_mem, cudaStream_t stream, int64_t* launches);
+size_t fast_prepared_rows_bytes(const GbdtModel& g, int nblk);
+size_t fast_prepared_call_bytes(const GbdtModel& g, int nblk);
+cudaError_t fast_prepare(const ks_gpu_desc& desc, const GbdtModel& g, const ks_candidate* d_c, int C, int nblk, void* d_rows,
+                         const int* order, cudaStream_t stream, int64_t* launches);
 // whether a dense walk of P problems with so many blocks each is split (`one_round`: only where they are fewer than the machine's CTAs)
 bool fast_splits(const GbdtModel& g, int P, int nblk, bool one_round);
 size_t fast_split_bytes(const GbdtModel& g);
