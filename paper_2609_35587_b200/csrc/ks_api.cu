@@ -138,6 +138,14 @@ ks_status read_status(ks_ctx* ctx) {
   return KS_OK;
 }
 
+// Waits for a word of mapped host memory that the call's last kernel writes behind its results (HostNotice).
+// Not seen within a few milliseconds (a failed launch never writes it), it waits the regular way.
+cudaError_t wait_for_word(const int* word, int seq, cudaStream_t stream) {
+  for (int spin = 0; spin < (1 << 22); ++spin)
+    if (*static_cast<const volatile int*>(word) == seq) return cudaSuccess;
+  return cudaStreamSynchronize(stream);
+}
+
 inline size_t align_up(size_t v, size_t a = 256) { return (v + a - 1) / a * a; }
 
 template <typename T>
@@ -549,9 +557,16 @@ ks_status ks_valid_catalogue(ks_ctx* ctx, const ks_problem* problem, unsigned fl
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ks_status s = ensure_workspace(ctx, ks::valid_catalogue_scratch_bytes(C));
   if (s != KS_OK) return s;
+  // where records or ids are written, the kernel that writes them tells the host the count when it is done
+  int* h_word = static_cast<int*>(ctx->pinned) + 2 * KS_MAX_K + 1;
+  const bool told = h_count && C > 0 && (d_out || d_out_index);
+  ks::HostNotice notice{reinterpret_cast<int*>(ctx->d_pinned_idx) + 2 * KS_MAX_K + 1, told ? ++ctx->host_seq : 0};
   cudaError_t e = ks::launch_valid_catalogue(ctx->desc, *problem, flags, d_candidates, C, ctx->ws, d_out,
-                                             d_out_index, d_count, st, &ctx->launches);
-  if (e == cudaSuccess && h_count) {
+                                             d_out_index, d_count, st, &ctx->launches, ctx->d_words, told ? &notice : nullptr);
+  if (e == cudaSuccess && told) {
+    e = wait_for_word(h_word, notice.seq, st);
+    if (e == cudaSuccess) *h_count = *static_cast<volatile int*>(h_word + 1);
+  } else if (e == cudaSuccess && h_count) {
     e = cudaMemcpyAsync(h_count, d_count, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   }
@@ -695,17 +710,12 @@ ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int 
       // returns a few microseconds before the stream reports completion
       int* h_seq = reinterpret_cast<int*>(pin_sc + KS_MAX_K);
       sl.out_seq = reinterpret_cast<int*>(ctx->d_pinned_score + KS_MAX_K);
-      sl.seq = ++ctx->select_one_seq;
+      sl.seq = ++ctx->host_seq;
       cudaError_t e = ks::launch_select_fast(ctx->desc, model->gbdt, nullptr, &p, 1, d_c, C, nblk, NC,
                                              nullptr, nullptr, k, reinterpret_cast<unsigned long long*>(base),
                                              base + b_part, ctx->d_status, st, &ctx->launches, nullptr, &sl, nullptr,
                                              &ctx->wait);
-      if (e == cudaSuccess) {
-        bool seen = false;
-        for (int spin = 0; spin < (1 << 22) && !seen; ++spin) seen = *static_cast<volatile int*>(h_seq) == sl.seq;
-        // not seen within a few milliseconds (a failed launch never writes it): wait the regular way
-        if (!seen) e = cudaStreamSynchronize(st);
-      }
+      if (e == cudaSuccess) e = wait_for_word(h_seq, sl.seq, st);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "ks_select_one");
       s = read_status(ctx);
       if (s != KS_OK) return s;  // (with the split walk's counters cleared)
@@ -721,10 +731,11 @@ ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int 
     return align_up(ks::select_partial_bytes(*model, 1, C, C, false, k, lean));
   });
   if (s != KS_OK) return s;
+  const ks::HostNotice notice{reinterpret_cast<int*>(ctx->d_pinned_score + KS_MAX_K), ++ctx->host_seq};
   cudaError_t e = ks::launch_select(ctx->desc, *model, nullptr, &p, 1, d_c, C, nullptr, nullptr, C, k,
                                     ctx->ws, ctx->d_pinned_idx, ctx->d_pinned_score, st, &ctx->launches,
-                                    ctx->d_status, nullptr, nullptr, &ctx->wait);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+                                    ctx->d_status, nullptr, nullptr, &ctx->wait, &notice);
+  if (e == cudaSuccess) e = wait_for_word(reinterpret_cast<int*>(pin_sc + KS_MAX_K), notice.seq, st);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "ks_select_one");
   std::memcpy(h_topk_idx, pin_idx, k * sizeof(int32_t));
   std::memcpy(h_topk_score, pin_sc, k * sizeof(float));
@@ -805,17 +816,13 @@ ks_status ks_select_one_prepared(ks_ctx* ctx, const ks_catalogue* cat, ks_proble
   sl.tiles = nullptr;
   int* h_seq = reinterpret_cast<int*>(pin_sc + KS_MAX_K);
   sl.out_seq = reinterpret_cast<int*>(ctx->d_pinned_score + KS_MAX_K);
-  sl.seq = ++ctx->select_one_seq;
+  sl.seq = ++ctx->host_seq;
   ks::FastPrepared prep{reinterpret_cast<const uint8_t*>(base), reinterpret_cast<uint8_t*>(base + cat->off_call)};
   cudaError_t e = ks::launch_select_fast(ctx->desc, gm, nullptr, &p, 1, cat->d_c, cat->C, cat->nblk, gm.block_cands,
                                          nullptr, nullptr, k, reinterpret_cast<unsigned long long*>(base + cat->off_part),
                                          nullptr, ctx->d_status, st, &ctx->launches, nullptr, &sl, nullptr, &ctx->wait,
                                          &prep, reinterpret_cast<const int32_t*>(base + cat->off_order));
-  if (e == cudaSuccess) {
-    bool seen = false;
-    for (int spin = 0; spin < (1 << 22) && !seen; ++spin) seen = *static_cast<volatile int*>(h_seq) == sl.seq;
-    if (!seen) e = cudaStreamSynchronize(st);  // a failed launch never writes the word: wait the regular way
-  }
+  if (e == cudaSuccess) e = wait_for_word(h_seq, sl.seq, st);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "ks_select_one_prepared");
   ks_status s = read_status(ctx);
   if (s != KS_OK) return s;

@@ -110,7 +110,9 @@ template <bool kScatter>
 __global__ void __launch_bounds__(kCatThreads)
 valid_kernel(const __grid_constant__ ks_gpu_desc desc, ValidArgs args, const ks_candidate* __restrict__ d_c,
              int C, int* __restrict__ block_sums, ks_candidate* __restrict__ out_c,
-             int32_t* __restrict__ out_index) {
+             int32_t* __restrict__ out_index, const int32_t* d_count, int* arrivals, HostNotice notice) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (the second pass is the dependent of the scan)
   __shared__ int s_warp[kCatThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long base = static_cast<long long>(blockIdx.x) * kCatTile + threadIdx.x * kCatPerThread;
@@ -153,6 +155,16 @@ valid_kernel(const __grid_constant__ ks_gpu_desc desc, ValidArgs args, const ks_
       ++pos;
     }
   }
+  if (!notice.word) return;
+  // the last block to finish tells the host the count, which waits for it
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  __threadfence();
+  if (atomicAdd(arrivals, 1) != static_cast<int>(gridDim.x) - 1) return;
+  *arrivals = 0;
+  notice.word[1] = *d_count;
+  __threadfence_system();
+  *static_cast<volatile int*>(notice.word) = notice.seq;
 }
 
 // One block: block_sums[0..n) -> exclusive prefix in place; the grand total goes to d_count.
@@ -160,6 +172,8 @@ __global__ void __launch_bounds__(1024) scan_block_sums_kernel(int* __restrict__
                                                                int32_t* __restrict__ d_count) {
   __shared__ int s_warp[32];
   __shared__ int s_carry;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (the dependent of the counting pass)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_carry = 0;
   __syncthreads();
@@ -222,7 +236,7 @@ size_t valid_catalogue_scratch_bytes(int C) {
 cudaError_t launch_valid_catalogue(const ks_gpu_desc& desc, const ks_problem& p, unsigned flags,
                                    const ks_candidate* d_c, int C, void* d_scratch, ks_candidate* d_out,
                                    int32_t* d_out_index, int32_t* d_count, cudaStream_t stream,
-                                   int64_t* launches) {
+                                   int64_t* launches, int* words, const HostNotice* notice) {
   if (C == 0) return cudaMemsetAsync(d_count, 0, sizeof(int32_t), stream);
   ValidArgs a;
   const int dab = p.dtype_ab & 3, dd = p.dtype_d & 3;
@@ -235,14 +249,33 @@ cudaError_t launch_valid_catalogue(const ks_gpu_desc& desc, const ks_problem& p,
   a.flags = flags;
   const int nblk = (C + kCatTile - 1) / kCatTile;
   int* sums = static_cast<int*>(d_scratch);
-  valid_kernel<false><<<nblk, kCatThreads, 0, stream>>>(desc, a, d_c, C, sums, nullptr, nullptr);
-  scan_block_sums_kernel<<<1, 1024, 0, stream>>>(sums, nblk, d_count);
+  // each of the three is launched as the dependent of the one in front
+  cudaLaunchConfig_t cfg{};
+  cfg.stream = stream;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.gridDim = dim3(nblk);
+  cfg.blockDim = dim3(kCatThreads);
+  const HostNotice none{nullptr, 0};
+  const int32_t* count = d_count;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, &valid_kernel<false>, desc, a, d_c, C, sums, static_cast<ks_candidate*>(nullptr),
+                                     static_cast<int32_t*>(nullptr), count, static_cast<int*>(nullptr), none);
+  if (e != cudaSuccess) return e;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(1024);
+  e = cudaLaunchKernelEx(&cfg, &scan_block_sums_kernel, sums, nblk, d_count);
+  if (e != cudaSuccess) return e;
   *launches += 2;
   if (d_out || d_out_index) {
-    valid_kernel<true><<<nblk, kCatThreads, 0, stream>>>(desc, a, d_c, C, sums, d_out, d_out_index);
+    cfg.gridDim = dim3(nblk);
+    cfg.blockDim = dim3(kCatThreads);
+    e = cudaLaunchKernelEx(&cfg, &valid_kernel<true>, desc, a, d_c, C, sums, d_out, d_out_index, count, words, notice ? *notice : none);
     ++*launches;
   }
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_remap_indices(int32_t* d_idx, long long n, const int32_t* d_map, int map_len,

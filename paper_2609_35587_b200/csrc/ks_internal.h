@@ -136,7 +136,7 @@ struct ks_ctx {
   int* h_status = nullptr;  // status word (mapped pinned host memory) set by kernels whose
   int* d_status = nullptr;  // bounded waits give up; d_status is its device alias
   int64_t launches = 0;
-  int select_one_seq = 0;  // sequence number of the last single-problem call
+  int host_seq = 0;  // sequence number of the last call whose end the host polls for
   ks::FastWait wait{0, 0, 0, nullptr};  // probe budget of bounded device waits (0: default), starve hook (tests), lean, d_words
   size_t ws_refused = SIZE_MAX;  // the smallest workspace that could not be had
   size_t ws_limit = SIZE_MAX;    // test hook: larger ones cannot be had
@@ -226,6 +226,13 @@ struct FastSplit {
   int seq;
 };
 
+// A word of mapped host memory that receives `seq` once a call's results lie beside it: the host polls it and is
+// back some 5 us before the stream reports completion.
+struct HostNotice {
+  int* word;  // device-visible
+  int seq;
+};
+
 // What a prepared catalogue hands to the quantised tree kernel instead of per-call work.
 struct FastPrepared {
   const uint8_t* cand_rows;  // [16 type combinations][blocks][candidate-only rows][block_cands], in the catalogue's order
@@ -263,7 +270,7 @@ size_t valid_catalogue_scratch_bytes(int C);
 cudaError_t launch_valid_catalogue(const ks_gpu_desc& desc, const ks_problem& p, unsigned flags,
                                    const ks_candidate* d_c, int C, void* d_scratch, ks_candidate* d_out,
                                    int32_t* d_out_index, int32_t* d_count, cudaStream_t stream,
-                                   int64_t* launches);
+                                   int64_t* launches, int* words, const HostNotice* notice);
 cudaError_t launch_remap_indices(int32_t* d_idx, long long n, const int32_t* d_map, int map_len,
                                  cudaStream_t stream, int64_t* launches);
 
@@ -362,6 +369,6 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                           const int64_t* d_seg_off, const int32_t* d_seg_idx, int64_t pairs, int k,
                           void* d_partial, int32_t* d_topk_idx, float* d_topk_score,
                           cudaStream_t stream, int64_t* launches, int* d_status,
-                          cudaEvent_t ev_begin, cudaEvent_t ev_end, const FastWait* wait);
+                          cudaEvent_t ev_begin, cudaEvent_t ev_end, const FastWait* wait, const HostNotice* notice = nullptr);
 
 }  // namespace ks

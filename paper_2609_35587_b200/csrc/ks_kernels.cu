@@ -818,7 +818,8 @@ static bool ridge_by_classes(int P, int C, bool segmented, bool lean) {
 template <int kWarps>
 __global__ void __launch_bounds__(kBlock)
 topk_merge_kernel(const unsigned long long* __restrict__ partial, int P, int n_keys, int k,
-                  int32_t* __restrict__ out_idx, float* __restrict__ out_score) {
+                  int32_t* __restrict__ out_idx, float* __restrict__ out_score, HostNotice notice) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched as the dependent of the kernel in front)
   __shared__ unsigned long long s_list[kWarps][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int prob = kWarps == 1 ? blockIdx.x * (kBlock / 32) + warp : blockIdx.x, part = kWarps == 1 ? 0 : warp;
@@ -842,18 +843,30 @@ topk_merge_kernel(const unsigned long long* __restrict__ partial, int P, int n_k
     out_idx[static_cast<size_t>(prob) * k + lane] = key_index(mine);
     out_score[static_cast<size_t>(prob) * k + lane] = key_score(mine);
   }
+  if (notice.word) {  // (a single problem)
+    __threadfence_system();
+    __syncwarp();
+    if (lane == 0) *static_cast<volatile int*>(notice.word) = notice.seq;
+  }
 }
 
 // A block per problem while that leaves the machine room, else a warp.
 static cudaError_t launch_merge(const unsigned long long* partial, int P, int n_keys, int k, int32_t* d_topk_idx,
-                                float* d_topk_score, cudaStream_t stream, int64_t* launches) {
+                                float* d_topk_score, cudaStream_t stream, int64_t* launches, const HostNotice* notice = nullptr) {
   constexpr int kPer = kBlock / 32;
-  if (P <= 8 * 148 && n_keys > 128)
-    topk_merge_kernel<kPer><<<P, kBlock, 0, stream>>>(partial, P, n_keys, k, d_topk_idx, d_topk_score);
-  else
-    topk_merge_kernel<1><<<(P + kPer - 1) / kPer, kBlock, 0, stream>>>(partial, P, n_keys, k, d_topk_idx, d_topk_score);
+  const bool blocks = P <= 8 * 148 && n_keys > 128;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(blocks ? P : (P + kPer - 1) / kPer);
+  cfg.blockDim = dim3(kBlock);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   if (launches) ++*launches;
-  return cudaGetLastError();
+  return cudaLaunchKernelEx(&cfg, blocks ? &topk_merge_kernel<kPer> : &topk_merge_kernel<1>, partial, P, n_keys, k, d_topk_idx,
+                            d_topk_score, notice ? *notice : HostNotice{nullptr, 0});
 }
 
 // Merge of ranked lists (the exchange step of a candidate-split selection): per problem, n
@@ -1133,7 +1146,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                           const int64_t* d_seg_off, const int32_t* d_seg_idx, int64_t pairs, int k,
                           void* d_partial, int32_t* d_topk_idx, float* d_topk_score,
                           cudaStream_t stream, int64_t* launches, int* d_status, cudaEvent_t ev_begin,
-                          cudaEvent_t ev_end, const FastWait* wait) {
+                          cudaEvent_t ev_end, const FastWait* wait, const HostNotice* notice) {
   if (P == 0) return cudaSuccess;
   const int64_t per = per_problem_rows(P, C, pairs, d_seg_off != nullptr);
   if (model.kind == 0 && model.gbdt.fast) {
@@ -1172,7 +1185,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                                        nullptr, perm, use_classes ? &classes : nullptr);
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
+    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice);
   }
   if (model.kind == 1 && model.mlp.tc) {
     const int nblk = mlp_tc_blocks_per_problem(P, per);
@@ -1183,7 +1196,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                                          launches, ev_begin, wait);
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
+    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice);
   }
   if (model.kind == 1 && model.mlp.wide) {
     const int nblk = wide_rank_blocks(per);
@@ -1194,7 +1207,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                                        ev_begin, wait);
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
+    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice);
   }
   if (model.kind == 1 && model.mlp.h_ridge) {
     const RidgeParams& prm = *model.mlp.h_ridge;
@@ -1264,7 +1277,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
+    return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice);
   }
   const int st = pick_sub_tiles(P, per);
   const PairMap map = make_map(P, C, pairs, d_seg_off, d_seg_idx, st * kBlock);
@@ -1289,7 +1302,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (ev_end) cudaEventRecord(ev_end, stream);
-  return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, launches);
+  return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice);
 }
 
 

@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(kCandThreads)
 mlp_cand_cols_kernel(ks_gpu_desc desc, const ks_candidate* __restrict__ c, int C, const unsigned* mask_ptr,
                      int combo0, const __grid_constant__ MlpTcParams prm, uint8_t* __restrict__ out) {
   const int combo = combo0 >= 0 ? combo0 : blockIdx.y;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the select kernel waits for this grid before it reads anything)
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *prm.leave = 0;
   if (mask_ptr && !((*mask_ptr >> combo) & 1u)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -364,6 +365,7 @@ select_mlp_tc_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_prob
   __shared__ int s_fail, s_abort;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (tid == 0) s_abort = *reinterpret_cast<volatile int*>(prm.leave);
   __syncthreads();
   if (s_abort) {  // a wait ran out in an earlier CTA of this call: it fails, leave at once
@@ -387,7 +389,7 @@ select_mlp_tc_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_prob
                  bar_f1 = smem_u32(&s_bar[6]), bar_a1 = smem_u32(&s_bar[7]), bar_x1 = smem_u32(&s_bar[8]),
                  bar_b1 = smem_u32(&s_bar[9]);
 
-  if (tid == 0 && !kRows) {
+  if (tid == 64 && !kRows) {  // (beside the barriers and the weights, which the first thread sees to)
     problem_terms(use_value ? p_value : p[prob], desc, s_pt);
     pair_fast_terms(s_pt, desc, s_pf);
     ks_candidate dummy{};
@@ -849,21 +851,23 @@ cudaError_t launch_select_mlp_tc(const ks_gpu_desc& desc, const MlpModel& m, con
   if (ev_begin) cudaEventRecord(ev_begin, stream);
   const unsigned grid = static_cast<unsigned>(static_cast<int64_t>(P) * nblk);
   const uint8_t* image = reinterpret_cast<const uint8_t*>(m.d_tc_image);
-  if (m.h_tc_params->onehot) {
-    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&select_mlp_tc_kernel<1>), kSmemBytes);
-    if (e != cudaSuccess) return e;
-    select_mlp_tc_kernel<1><<<grid, kT, kSmemBytes, stream>>>(desc, d_p, pv, uv, d_c, P, C, nblk, seg_off, seg_idx, image,
-                                                              d_cols, k, partial, status, nullptr, nullptr,
-                                                              *m.h_tc_params);
-  } else {
-    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&select_mlp_tc_kernel<0>), kSmemBytes);
-    if (e != cudaSuccess) return e;
-    select_mlp_tc_kernel<0><<<grid, kT, kSmemBytes, stream>>>(desc, d_p, pv, uv, d_c, P, C, nblk, seg_off, seg_idx, image,
-                                                              d_cols, k, partial, status, nullptr, nullptr,
-                                                              *m.h_tc_params);
-  }
+  auto kernel = m.h_tc_params->onehot ? &select_mlp_tc_kernel<1> : &select_mlp_tc_kernel<0>;
+  e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), kSmemBytes);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kT);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr{};  // the dependent of the table kernel: 2.5 us less between the two
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = C > 0 && !ev_begin ? 1 : 0;
   ++*launches;
-  return cudaGetLastError();
+  return cudaLaunchKernelEx(&cfg, kernel, desc, d_p, pv, uv, d_c, P, C, nblk, seg_off, seg_idx, image,
+                            static_cast<const uint8_t*>(d_cols), k, partial, status, static_cast<const float*>(nullptr),
+                            static_cast<float*>(nullptr), *m.h_tc_params);
 }
 
 // ks_score on the tensor-core kernel (ordinal input form): one CTA per SM, each with an equal
