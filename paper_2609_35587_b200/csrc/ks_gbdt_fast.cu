@@ -728,18 +728,28 @@ __device__ __forceinline__ uint32_t path_step(uint32_t a, uint32_t cb_r, uint32_
 // THREADS threads rank NC candidates: NC / 4 words times THREADS / (NC / 4) tree groups.
 // kSplit: the CTAs share out the blocks' trees (SplitArgs); a form of its own, since what it keeps slowed the
 // other by 2 %.
+// kShared: the top levels come from the chunk in shared memory, not from the parameters. That takes three more
+// shared-memory wavefronts and seven more instructions a tree (5 % of the walk), but a launch costs the host 7 us
+// where 28 KB of parameters make it 21; see takes_shared_top.
 // kFloor (measurement only): the walk without its chunk rings. Every tree group's first kNBuf
 // chunks are copied once and stay resident; the group walks them again and again (sl.repeat
 // times as many chunk walks as it has chunks), never waits, releases or refills, so the time per
 // pass is that of the gather and instruction stream of the walk alone, at the occupancy and tile
 // size of the real kernel.
-template <int L, int NP, bool kCompact, int THREADS, int NC, bool kSplit, bool kFloor = false>
+template <bool kShared>
+struct TopArg {
+  FastTopParams p;
+};
+template <>
+struct TopArg<true> {};
+
+template <int L, int NP, bool kCompact, int THREADS, int NC, bool kSplit, bool kShared = false, bool kFloor = false>
 __global__ void __launch_bounds__(THREADS, THREADS <= 256 ? 2 : 1)
 select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_problem p_value, int use_value,
                    const ks_candidate* __restrict__ c, int P, int C, int nblk, int rows_per_cta,
                    const int64_t* __restrict__ seg_off, const int32_t* __restrict__ seg_idx, FastView fv,
                    int k, unsigned long long* __restrict__ partial, int* __restrict__ status,
-                   SplitArgs sl, int n_items, const __grid_constant__ FastTopParams top) {
+                   SplitArgs sl, int n_items, const __grid_constant__ TopArg<kShared> top) {
   constexpr int W = NC / 4;        // words per tile row = lane slots
   constexpr int G = THREADS / W;   // tree groups
   constexpr int RG = ring_count(G);  // chunk rings
@@ -985,8 +995,18 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
           // A tile byte is 0x80 | bin and a node constant (j + 1) in every byte, so byte r of
           // d[n] keeps its top bit iff candidate r goes right at node n; no byte borrows.
           uint32_t d[kTop > 0 ? kTop : 1];
-          if (kCompact) {
-            const uint32_t* tw = reinterpret_cast<const uint32_t*>(top.w) +
+          if constexpr (kShared) {
+            // (the nodes of a level lie side by side, aligned since a chunk's trees are a multiple of four). A node's low
+            // byte is v = 0x80 | j: byte r of tile + 0x7F.. - v.. is 0x80 + bin - (j + 1), as below.
+            uint32_t n[7];
+            n[0] = lds_u32(buf + 4u * t);
+            lds_u64(buf + 4u * tpc + 8u * t, n[1], n[2]);
+            lds_u128(buf + 12u * tpc + 16u * t, n[3], n[4], n[5], n[6]);
+#pragma unroll
+            for (int i = 0; i < 7; ++i)
+              d[i] = lds_u32(cb + static_cast<uint32_t>(KS_IDX(n[i] >> 8, fv.n_rows * NC))) + 0x7F7F7F7Fu - __byte_perm(n[i], 0u, 0u);
+          } else if constexpr (kCompact) {
+            const uint32_t* tw = reinterpret_cast<const uint32_t*>(top.p.w) +
                                  static_cast<size_t>(KS_IDX(ch * tpc + t, 2 * kFastTopPairs / (kTop > 0 ? kTop : 1))) * kTop;
 #pragma unroll
             for (int n = 0; n < kTop; ++n) {
@@ -994,7 +1014,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
               d[n] = lds_u32(cb + static_cast<uint32_t>(KS_IDX(v >> 8, fv.n_rows * NC))) - __byte_perm(v, 0u, 0u);
             }
           } else {
-            const uint2* tw = top.w + static_cast<size_t>(KS_IDX(ch * tpc + t, kFastTopPairs / (kTop > 0 ? kTop : 1))) * kTop;
+            const uint2* tw = top.p.w + static_cast<size_t>(KS_IDX(ch * tpc + t, kFastTopPairs / (kTop > 0 ? kTop : 1))) * kTop;
 #pragma unroll
             for (int n = 0; n < kTop; ++n)
               d[n] = lds_u32(cb + static_cast<uint32_t>(KS_IDX(tw[n].x, fv.n_rows * NC))) - tw[n].y;
@@ -1682,11 +1702,11 @@ struct WalkArgs {
   int dependent;  // launched right behind the kernel whose tables it reads
 };
 
-template <int L, int NP, bool kCompact, int THREADS, int NC, bool kSplit, bool kFloor = false>
+template <int L, int NP, bool kCompact, int THREADS, int NC, bool kSplit, bool kShared = false, bool kFloor = false>
 cudaError_t launch_form(const WalkArgs& a) {
   const size_t smem = static_cast<size_t>(kNBuf) * ring_count(THREADS / (NC / 4)) * a.fv.buf_bytes +
                       static_cast<size_t>(a.fv.n_rows) * NC;
-  auto kernel = &select_fast_kernel<L, NP, kCompact, THREADS, NC, kSplit, kFloor>;
+  auto kernel = &select_fast_kernel<L, NP, kCompact, THREADS, NC, kSplit, kShared, kFloor>;
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
@@ -1710,18 +1730,41 @@ cudaError_t launch_form(const WalkArgs& a) {
   cfg.numAttrs = a.dependent ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, a.desc, a.d_p, a.pv, a.uv, a.d_c, a.P, a.C, a.nblk, a.rows_per_cta,
                             a.seg_off, a.seg_idx, a.fv, a.k, a.partial, a.status, a.sl, static_cast<int>(n_items),
-                            *a.top);
+                            *reinterpret_cast<const TopArg<kShared>*>(a.top));
 }
 
 template <int L, int NP, bool kCompact, int THREADS, int NC>
 cudaError_t launch_ln(const WalkArgs& a) {
-  return a.sl.units > 0 ? launch_form<L, NP, kCompact, THREADS, NC, true>(a) : launch_form<L, NP, kCompact, THREADS, NC, false>(a);
+  return launch_form<L, NP, kCompact, THREADS, NC, false>(a);
+}
+
+// Split walks take the top levels from the chunk where the launch would keep the GPU waiting, i.e. behind the tiles
+// of few blocks (10 to 14 us): 500 candidates, 500 trees, prepared 46.5 -> 42 us, 60,000 95.5 -> 97.5. And where the
+// parameters hold fewer than three levels of the ensemble.
+bool takes_shared_top(const GbdtModel& g, const WalkArgs& a) {
+  if (g.fast_depth < 3 || g.tpc % 4 != 0) return false;
+  return g.top_levels < 3 || g.top_compact || (!a.sl.score_out && a.sl.blocks < 50);
 }
 
 // the instantiation for a model's top levels and depth, within one tile geometry
 template <int THREADS, int NC>
 cudaError_t launch_walk_geom(const GbdtModel& g, const WalkArgs& a) {
   const int L = g.top_levels, np = g.fast_depth - L;
+  if (a.sl.units > 0) {
+    if (takes_shared_top(g, a)) {
+      if (g.fast_depth == 8) return launch_form<3, 5, false, THREADS, NC, true, true>(a);
+      if (g.fast_depth == 7) return launch_form<3, 4, false, THREADS, NC, true, true>(a);
+      if (g.fast_depth == 6) return launch_form<3, 3, false, THREADS, NC, true, true>(a);
+      return launch_form<3, -1, false, THREADS, NC, true, true>(a);
+    }
+    if (L == 3 && !g.top_compact) {
+      if (np == 5) return launch_form<3, 5, false, THREADS, NC, true>(a);
+      if (np == 4) return launch_form<3, 4, false, THREADS, NC, true>(a);
+      if (np == 3) return launch_form<3, 3, false, THREADS, NC, true>(a);
+      return launch_form<3, -1, false, THREADS, NC, true>(a);
+    }
+    return launch_form<0, -1, false, THREADS, NC, true>(a);
+  }
   if (g.top_compact) {
     if (np == 5) return launch_ln<3, 5, true, THREADS, NC>(a);
     if (np == 4) return launch_ln<3, 4, true, THREADS, NC>(a);
@@ -1746,8 +1789,8 @@ cudaError_t launch_walk_floor(const GbdtModel& g, const WalkArgs& a) {
   if (g.top_compact || g.top_levels != 3 || g.fast_depth != 8 || g.block_cands != 1024 ||
       g.n_chunks < kNBuf * ring_count(g.fast_threads / 256))  // every ring needs its kNBuf resident chunks
     return cudaErrorNotSupported;
-  if (g.fast_threads == 512) return launch_form<3, 5, false, 512, 1024, false, true>(a);
-  return launch_form<3, 5, false, 256, 1024, false, true>(a);
+  if (g.fast_threads == 512) return launch_form<3, 5, false, 512, 1024, false, false, true>(a);
+  return launch_form<3, 5, false, 256, 1024, false, false, true>(a);
 }
 
 cudaError_t launch_walk(const GbdtModel& g, const WalkArgs& a) {
