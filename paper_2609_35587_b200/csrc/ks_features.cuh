@@ -209,41 +209,65 @@ __device__ __forceinline__ Resources resources(const ProblemTerms& t, const ks_c
 // The columns that depend on both the problem and the candidate (sections "Work Decomposition
 // and Wave Quantization", "Memory Behavior", "Pipeline Balance"), given the candidate's
 // effective resident-block count b_eff.
+//
+// What bounds the kernels that evaluate them by the million is the issue of this arithmetic, and most of it is
+// 64-bit: divisions by emulation, conversions at a quarter of the 32-bit rate. Counts of tiles and clusters fit 32 bits
+// where there are fewer than 2^15 tiles a side (same integers, same roundings); else the 64-bit form below.
 template <bool kExact, typename Put>
 __device__ __forceinline__ void pair_columns(const ProblemTerms& t, const ks_candidate& c, const ks_gpu_desc& h,
                                              long long b_eff, Put put) {
   const int TM = c.tile_m, TN = c.tile_n, TK = c.tile_k, S = c.stages;
   const int cM = c.cluster_m, cN = c.cluster_n;
   const int bA = t.bA;
-  const long long n_m = cdiv_u32(t.M, TM), n_n = cdiv_u32(t.N, TN), n_k = cdiv_u32(t.K, TK);
-  const long long n_tiles = n_m * n_n;
-  put(23, F64i(n_m));
-  put(24, F64i(n_n));
-  put(25, F64i(n_k));
-  put(26, F64i(n_tiles));
-  put(27, fdiv<kExact>(F64i(n_m * TM - t.M), F64i(t.M)));
-  put(28, fdiv<kExact>(F64i(n_n * TN - t.N), F64i(t.N)));
-  put(29, fdiv<kExact>(F64i(n_tiles), F64i(h.num_sms)));
-  const long long resident = static_cast<long long>(h.num_sms) * b_eff;
-  const long long waves = cdiv_fit(n_tiles, resident);
-  put(30, F64i(waves));
-  const float eta = fdiv<kExact>(F64i(n_tiles), F64i(waves * resident));
+  const unsigned m = cdiv_u32(t.M, TM), n = cdiv_u32(t.N, TN), k = cdiv_u32(t.K, TK);
+  const float f_m = __uint2float_rn(m), f_n = __uint2float_rn(n), f_k = __uint2float_rn(k);
+  const unsigned sms = h.num_sms;
+  // tiles, waves, tiles that fit those waves, tiles of whole clusters less tiles
+  float f_tiles, f_waves, f_slots, f_waste;
+  long long g_m, g_n;  // clusters a side: ceil(M / (c T)) = ceil(ceil(M / T) / c)
+  if ((m | n) < (1u << 15) && b_eff < 64 && sms < (1u << 16)) {
+    const unsigned tiles = m * n, resident = sms * static_cast<unsigned>(b_eff);
+    const unsigned waves = cdiv_u32(tiles, resident), a = cdiv_u32(m, cM), b = cdiv_u32(n, cN);
+    f_tiles = __uint2float_rn(tiles);
+    f_waves = __uint2float_rn(waves);
+    f_slots = __uint2float_rn(waves * resident);
+    f_waste = F64i(static_cast<long long>(a) * b * cM * cN - tiles);
+    g_m = a;
+    g_n = b;
+  } else {
+    const long long n_tiles = static_cast<long long>(m) * n, resident = static_cast<long long>(sms) * b_eff;
+    const long long waves = cdiv_fit(n_tiles, resident);
+    g_m = cdiv_fit(m, cM);
+    g_n = cdiv_fit(n, cN);
+    f_tiles = F64i(n_tiles);
+    f_waves = F64i(waves);
+    f_slots = F64i(waves * resident);
+    f_waste = F64i(g_m * g_n * cM * cN - n_tiles);
+  }
+  put(23, f_m);
+  put(24, f_n);
+  put(25, f_k);
+  put(26, f_tiles);
+  put(27, fdiv<kExact>(__uint2float_rn(m * TM - t.M), __uint2float_rn(t.M)));
+  put(28, fdiv<kExact>(__uint2float_rn(n * TN - t.N), __uint2float_rn(t.N)));
+  put(29, fdiv<kExact>(f_tiles, __uint2float_rn(sms)));
+  put(30, f_waves);
+  const float eta = fdiv<kExact>(f_tiles, f_slots);
   put(31, eta);
   put(32, fmaxf(0.0f, __fsub_rn(1.0f, eta)));
-  const long long n_c = cdiv_fit(t.M, static_cast<long long>(cM) * TM) * cdiv_fit(t.N, static_cast<long long>(cN) * TN);
-  put(33, fdiv<kExact>(F64i(n_c * cM * cN - n_tiles), F64i(n_tiles)));
-  put(34, fdiv<kExact>(F64i(n_m), F64i(cM)));
-  put(35, fdiv<kExact>(F64i(n_n), F64i(cN)));
-  put(36, F32i(cM > n_m || cN > n_n));
-  const long long restream = n_n * t.bytesA + n_m * t.bytesB;
-  put(39, fdiv<kExact>(F64i(restream), F64i(t.bytesA + t.bytesB)));
+  put(33, fdiv<kExact>(f_waste, f_tiles));
+  put(34, fdiv<kExact>(f_m, F32i(cM)));
+  put(35, fdiv<kExact>(f_n, F32i(cN)));
+  put(36, F32i(static_cast<unsigned>(cM) > m || static_cast<unsigned>(cN) > n));
+  const float f_restream = F64i(n * t.bytesA + m * t.bytesB);
+  put(39, fdiv<kExact>(f_restream, F64i(t.bytesA + t.bytesB)));
   const float fl2 = F64i(static_cast<long long>(h.l2_bytes));
   put(41, fdiv<kExact>(F64i(static_cast<long long>(bA) * TM * t.K), fl2));
   put(42, fdiv<kExact>(F64i(static_cast<long long>(bA) * TN * t.K), fl2));
-  put(43, F64i(restream));
-  put(44, F64i(cdiv_fit(n_n, cN) * t.bytesA + cdiv_fit(n_m, cM) * t.bytesB));
-  put(60, fdiv<kExact>(F64i(min(static_cast<long long>(S), n_k)), F32i(S)));
-  put(61, fdiv<kExact>(F64i(n_k), F32i(S)));
+  put(43, f_restream);
+  put(44, F64i(g_n * t.bytesA + g_m * t.bytesB));
+  put(60, fdiv<kExact>(__uint2float_rn(min(static_cast<unsigned>(S), k)), F32i(S)));
+  put(61, fdiv<kExact>(f_k, F32i(S)));
 }
 
 // ---- per-pair columns for consumers that round them to bf16 ------------------------------------
