@@ -135,7 +135,7 @@ __device__ __forceinline__ void problem_terms(const ks_problem& p, const ks_gpu_
 
 // a / b rounded up for non-negative operands; takes the 32-bit path when both fit (same value)
 __device__ __forceinline__ long long cdiv_fit(long long a, long long b) {
-  if (((a | b) >> 32) == 0)
+  if (((a + b) >> 32) == 0)  // (the sum that is divided has to fit, too)
     return static_cast<long long>(cdiv_u32(static_cast<unsigned>(a), static_cast<unsigned>(b)));
   return cdiv_i64(a, b);
 }
