@@ -212,8 +212,9 @@ __device__ __forceinline__ Resources resources(const ProblemTerms& t, const ks_c
 //
 // What bounds the kernels that evaluate them by the million is the issue of this arithmetic, and most of it is
 // 64-bit: divisions by emulation, conversions at a quarter of the 32-bit rate. Counts of tiles and clusters fit 32 bits
-// where there are fewer than 2^15 tiles a side (same integers, same roundings); else the 64-bit form below.
-template <bool kExact, typename Put>
+// where there are fewer than 2^15 tiles a side (same integers, same roundings); else, and without kNarrow, the 64-bit
+// form below.
+template <bool kExact, bool kNarrow = true, typename Put>
 __device__ __forceinline__ void pair_columns(const ProblemTerms& t, const ks_candidate& c, const ks_gpu_desc& h,
                                              long long b_eff, Put put) {
   const int TM = c.tile_m, TN = c.tile_n, TK = c.tile_k, S = c.stages;
@@ -225,7 +226,7 @@ __device__ __forceinline__ void pair_columns(const ProblemTerms& t, const ks_can
   // tiles, waves, tiles that fit those waves, tiles of whole clusters less tiles
   float f_tiles, f_waves, f_slots, f_waste;
   long long g_m, g_n;  // clusters a side: ceil(M / (c T)) = ceil(ceil(M / T) / c)
-  if ((m | n) < (1u << 15) && b_eff < 64 && sms < (1u << 16)) {
+  if (kNarrow && (m | n) < (1u << 15) && b_eff < 64 && sms < (1u << 16)) {
     const unsigned tiles = m * n, resident = sms * static_cast<unsigned>(b_eff);
     const unsigned waves = cdiv_u32(tiles, resident), a = cdiv_u32(m, cM), b = cdiv_u32(n, cN);
     f_tiles = __uint2float_rn(tiles);

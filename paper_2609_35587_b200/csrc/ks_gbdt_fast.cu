@@ -2004,7 +2004,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
           desc, d_p + first, n, d_c, fv, memo, pthr_cap, path, wait->words);
       ++*launches;
     }
-    a.dependent = memo.keys != nullptr || tiles_mode || prep;
+    a.dependent = memo.keys != nullptr || ((tiles_mode || prep) && !ev_begin);  // (no event stands between the two)
     a.d_p = d_p ? d_p + first : nullptr;
     a.P = n;
     a.seg_off = seg_off ? seg_off + first : nullptr;

@@ -852,7 +852,7 @@ topk_merge_kernel(const unsigned long long* __restrict__ partial, int P, int n_k
 
 // A block per problem while that leaves the machine room, else a warp.
 static cudaError_t launch_merge(const unsigned long long* partial, int P, int n_keys, int k, int32_t* d_topk_idx,
-                                float* d_topk_score, cudaStream_t stream, int64_t* launches, const HostNotice* notice = nullptr) {
+                                float* d_topk_score, cudaStream_t stream, int64_t* launches, const HostNotice* notice = nullptr, bool timed = false) {
   constexpr int kPer = kBlock / 32;
   const bool blocks = P <= 8 * 148 && n_keys > 128;
   cudaLaunchConfig_t cfg{};
@@ -863,7 +863,7 @@ static cudaError_t launch_merge(const unsigned long long* partial, int P, int n_
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = timed ? 0 : 1;  // (an event stands between it and the kernel in front)
   if (launches) ++*launches;
   return cudaLaunchKernelEx(&cfg, blocks ? &topk_merge_kernel<kPer> : &topk_merge_kernel<1>, partial, P, n_keys, k, d_topk_idx,
                             d_topk_score, notice ? *notice : HostNotice{nullptr, 0});
@@ -1185,7 +1185,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                                        nullptr, perm, use_classes ? &classes : nullptr);
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice);
+    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice, ev_end != nullptr);
   }
   if (model.kind == 1 && model.mlp.tc) {
     const int nblk = mlp_tc_blocks_per_problem(P, per);
@@ -1196,7 +1196,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                                          launches, ev_begin, wait);
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice);
+    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice, ev_end != nullptr);
   }
   if (model.kind == 1 && model.mlp.wide) {
     const int nblk = wide_rank_blocks(per);
@@ -1207,7 +1207,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
                                        ev_begin, wait);
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice);
+    return launch_merge(part, P, nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice, ev_end != nullptr);
   }
   if (model.kind == 1 && model.mlp.h_ridge) {
     const RidgeParams& prm = *model.mlp.h_ridge;
@@ -1234,7 +1234,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;
       if (ev_end) cudaEventRecord(ev_end, stream);
-      return shares > 1 ? launch_merge(partial, P, shares * k, k, d_topk_idx, d_topk_score, stream, launches) : cudaSuccess;
+      return shares > 1 ? launch_merge(partial, P, shares * k, k, d_topk_idx, d_topk_score, stream, launches, nullptr, ev_end != nullptr) : cudaSuccess;
     }
     // per-call tables of what a problem, a candidate and (segments) a class bring, then the kernel that adds
     // and ranks
@@ -1277,7 +1277,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (ev_end) cudaEventRecord(ev_end, stream);
-    return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice);
+    return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice, ev_end != nullptr);
   }
   const int st = pick_sub_tiles(P, per);
   const PairMap map = make_map(P, C, pairs, d_seg_off, d_seg_idx, st * kBlock);
@@ -1302,7 +1302,7 @@ cudaError_t launch_select(const ks_gpu_desc& desc, const ks_model& model, const 
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (ev_end) cudaEventRecord(ev_end, stream);
-  return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice);
+  return launch_merge(partial, P, map.nblk * k, k, d_topk_idx, d_topk_score, stream, launches, notice, ev_end != nullptr);
 }
 
 

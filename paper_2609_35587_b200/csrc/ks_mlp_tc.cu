@@ -543,8 +543,9 @@ select_mlp_tc_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_prob
         };
         // single-precision evaluation (the values are rounded to bf16 next); the exact
         // 64-bit form only for tile counts beyond its range
+        // (the fallback without its 32-bit form: the two together in this loop cost the kernel 1.6 %)
         if (!pair_columns_bf16(s_pt, s_pf, cand, desc, w[15] & 0xFFFFu, put))
-          pair_columns<false>(s_pt, cand, desc, static_cast<long long>(w[15] & 0xFFFFu), put);
+          pair_columns<false, false>(s_pt, cand, desc, static_cast<long long>(w[15] & 0xFFFFu), put);
         // positions 0..28 came from the table; 29..49 are the per-pair columns
         w[14] = (w[14] & 0xFFFFu) | (pack_bf16(0.0f, x[29]) & 0xFFFF0000u);
 #pragma unroll
