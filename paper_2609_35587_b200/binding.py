@@ -254,8 +254,9 @@ class Context:
     def device_status(self) -> int:
         return int(_lib.ks_device_status(self._h))
 
-    def debug_set_wait(self, probe_limit: int = 0, starve: bool = False):
-        """Test hook: probe budget of the kernels' bounded waits, and the starved-wait mode."""
+    def debug_set_wait(self, probe_limit: int = 0, starve: int = 0):
+        """Test hook: probe budget of the kernels' bounded waits, and the starved-wait mode (1, or 2 for every
+        other block of the tree kernel)."""
         self._check(_lib.ks_debug_set_wait(self._h, int(probe_limit), int(starve)), "ks_debug_set_wait")
 
     def debug_limit_workspace(self, n_bytes: int = 0):

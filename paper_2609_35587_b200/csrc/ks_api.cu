@@ -388,7 +388,7 @@ ks_status ks_model_describe(const ks_model* model, char* buf, int len) {
 ks_status ks_debug_set_wait(ks_ctx* ctx, int probe_limit, int starve) {
   if (!ctx || probe_limit < 0) return KS_ERR_INVALID_ARG;
   ctx->wait.limit = probe_limit;
-  ctx->wait.starve = starve != 0;
+  ctx->wait.starve = starve == ks::kStarveOdd ? starve : starve != 0 ? ks::kStarveAll : 0;
   return KS_OK;
 }
 
@@ -559,14 +559,16 @@ ks_status ks_valid_catalogue(ks_ctx* ctx, const ks_problem* problem, unsigned fl
   if (s != KS_OK) return s;
   // where records or ids are written, the kernel that writes them tells the host the count when it is done
   int* h_word = static_cast<int*>(ctx->pinned) + 2 * KS_MAX_K + 1;
-  const bool told = h_count && C > 0 && (d_out || d_out_index);
+  bool told = h_count && C > 0 && (d_out || d_out_index);
   ks::HostNotice notice{reinterpret_cast<int*>(ctx->d_pinned_idx) + 2 * KS_MAX_K + 1, told ? ++ctx->host_seq : 0};
   cudaError_t e = ks::launch_valid_catalogue(ctx->desc, *problem, flags, d_candidates, C, ctx->ws, d_out,
                                              d_out_index, d_count, st, &ctx->launches, ctx->d_words, told ? &notice : nullptr);
   if (e == cudaSuccess && told) {
     e = wait_for_word(h_word, notice.seq, st);
-    if (e == cudaSuccess) *h_count = *static_cast<volatile int*>(h_word + 1);
-  } else if (e == cudaSuccess && h_count) {
+    told = *static_cast<volatile int*>(h_word) == notice.seq;
+    if (e == cudaSuccess && told) *h_count = *static_cast<volatile int*>(h_word + 1);
+  }
+  if (e == cudaSuccess && h_count && !told) {
     e = cudaMemcpyAsync(h_count, d_count, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   }

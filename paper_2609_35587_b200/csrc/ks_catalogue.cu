@@ -161,7 +161,6 @@ valid_kernel(const __grid_constant__ ks_gpu_desc desc, ValidArgs args, const ks_
   if (threadIdx.x != 0) return;
   __threadfence();
   if (atomicAdd(arrivals, 1) != static_cast<int>(gridDim.x) - 1) return;
-  *arrivals = 0;
   notice.word[1] = *d_count;
   __threadfence_system();
   *static_cast<volatile int*>(notice.word) = notice.seq;
@@ -169,7 +168,7 @@ valid_kernel(const __grid_constant__ ks_gpu_desc desc, ValidArgs args, const ks_
 
 // One block: block_sums[0..n) -> exclusive prefix in place; the grand total goes to d_count.
 __global__ void __launch_bounds__(1024) scan_block_sums_kernel(int* __restrict__ block_sums, int n,
-                                                               int32_t* __restrict__ d_count) {
+                                                               int32_t* __restrict__ d_count, int* arrivals) {
   __shared__ int s_warp[32];
   __shared__ int s_carry;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -205,7 +204,10 @@ __global__ void __launch_bounds__(1024) scan_block_sums_kernel(int* __restrict__
     if (threadIdx.x == 1023) s_carry = carry + s_warp[31];
     __syncthreads();
   }
-  if (threadIdx.x == 0) *d_count = s_carry;
+  if (threadIdx.x == 0) {
+    *d_count = s_carry;
+    if (arrivals) *arrivals = 0;  // of the second pass, which waits for this kernel
+  }
 }
 
 __global__ void remap_indices_kernel(int32_t* __restrict__ idx, long long n, const int32_t* __restrict__ map,
@@ -266,13 +268,15 @@ cudaError_t launch_valid_catalogue(const ks_gpu_desc& desc, const ks_problem& p,
   cfg.numAttrs = 1;
   cfg.gridDim = dim3(1);
   cfg.blockDim = dim3(1024);
-  e = cudaLaunchKernelEx(&cfg, &scan_block_sums_kernel, sums, nblk, d_count);
+  int* arrivals = notice ? words + kWordValid : nullptr;
+  e = cudaLaunchKernelEx(&cfg, &scan_block_sums_kernel, sums, nblk, d_count, arrivals);
   if (e != cudaSuccess) return e;
   *launches += 2;
   if (d_out || d_out_index) {
     cfg.gridDim = dim3(nblk);
     cfg.blockDim = dim3(kCatThreads);
-    e = cudaLaunchKernelEx(&cfg, &valid_kernel<true>, desc, a, d_c, C, sums, d_out, d_out_index, count, words, notice ? *notice : none);
+    e = cudaLaunchKernelEx(&cfg, &valid_kernel<true>, desc, a, d_c, C, sums, d_out, d_out_index, count, arrivals,
+                           notice ? *notice : none);
     ++*launches;
   }
   return e;

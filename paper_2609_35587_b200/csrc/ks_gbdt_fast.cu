@@ -873,6 +873,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     const int64_t stop = (start + rows_per_cta < len) ? start + rows_per_cta : len;
     // ---- phase A ---------------------------------------------------------------------------------
     __syncthreads();
+    const bool starved = fv.starve == kStarveAll || (fv.starve == kStarveOdd && (cta & 1));
     // The first chunks are on their way while the tile is filled, where the fill leaves the chunk buffers alone.
     const auto start_rings = [&] {
       // ring g takes the chunks ch_begin + g, ch_begin + g + RG, ... through its own buffers
@@ -880,7 +881,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
         for (int b = 0; b < kNBuf && ch_begin + g + b * RG < ch_end; ++b) {
           const int rb = g * kNBuf + b;
           // test hook: a barrier armed for more bytes than its copy brings never completes
-          mbar_expect_tx(bar0 + 8u * rb, fv.chunk_bytes + (fv.starve ? 16 : 0));
+          mbar_expect_tx(bar0 + 8u * rb, fv.chunk_bytes + (starved ? 16 : 0));
           bulk_copy_g2s(sbase + kOffBuf0 + rb * fv.buf_bytes,
                         reinterpret_cast<const char*>(fv.chunks) + static_cast<size_t>(ch_begin + g + b * RG) * fv.chunk_bytes,
                         fv.chunk_bytes, bar0 + 8u * rb);
@@ -1072,7 +1073,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
           s_pending[rb] = 0;
           if (ch + kNBuf * RG < ch_end && !*v_fail) {
             fence_async_proxy();
-            mbar_expect_tx(bar, fv.chunk_bytes + (fv.starve ? 16 : 0));
+            mbar_expect_tx(bar, fv.chunk_bytes + (starved ? 16 : 0));
             bulk_copy_g2s(buf, reinterpret_cast<const char*>(fv.chunks) +
                                    static_cast<size_t>(KS_IDX(ch + kNBuf * RG, fv.n_chunks)) * fv.chunk_bytes,
                           fv.chunk_bytes, bar);
@@ -1091,7 +1092,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
       if (word == 0 && grp % GPR == 0) {  // one thread per ring, for its ring's buffers (it knows their parities)
         for (int b = 0; b < kNBuf; ++b) {
           if (!s_pending[ring * kNBuf + b]) continue;
-          if (fv.starve || tile_late) {
+          if (starved || tile_late) {
             for (int i = 0; i < 64; ++i) __nanosleep(kSleepNs);
           } else {
             mbar_wait_bounded(bar0 + 8u * (ring * kNBuf + b), (phases >> b) & 1u, fv.wait_limit, &s_abort /* stays 0 */);

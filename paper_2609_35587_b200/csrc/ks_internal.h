@@ -66,7 +66,7 @@ struct FeatQ {
 // process: another context's kernels may run at the same time.
 struct FastWait {
   int limit;
-  int starve;
+  int starve;  // kStarve..., 0: none
   int lean;  // the memory for all of the workspace could not be had: without the walk of whole classes, few rows or problems at a time
   int* words;
 };
@@ -184,8 +184,10 @@ constexpr int kMaxShares = 1024;       // CTAs that a split walk may have
 // kernel family that makes the CTAs which start after it was raised leave at once. It is cleared in front
 // of every launch of the family.
 constexpr int kWordWalk = kMaxShares + 1, kWordMlp = kWordWalk + 1, kWordWide = kWordMlp + 1;
-constexpr int kWordServed = kWordWide + 1;  // calls that the walk of whole classes has served (ks_debug_class_walks)
+constexpr int kWordValid = kWordWide + 1;   // arrival counter of ks_valid_catalogue, cleared by the call itself
+constexpr int kWordServed = kWordValid + 1;  // calls that the walk of whole classes has served (ks_debug_class_walks)
 constexpr int kContextWords = kWordServed + 1;
+constexpr int kStarveAll = 1, kStarveOdd = 2;  // test hook: barriers that never complete, of all CTAs or of every other one
 constexpr int kLeaveFailed = 1, kLeaveServed = 2;  // a wait ran out; another kernel serves the call
 
 // Levels of the categorical field held by feature column `col` (0: not a level-code column):

@@ -103,6 +103,30 @@ def test_tensor_core_kernel_wait_runs_out(ks):
     ctx.close()
 
 
+@pytest.mark.parametrize("C", [300, 20000])
+def test_valid_catalogue_after_a_failed_walk(ks, C):
+    """A split walk of which every other block's waits run out leaves arrival counters behind until the status
+    is read. The count of valid candidates, which the last block of a pass tells the host, is its own all the same."""
+    ctx = ks.Context(DESC, 0)
+    w = wl.make_workload(1, P=1, C=1000, trees=200)
+    model = ctx.model_create_gbdt(*w.gbdt)
+    pool = dev(ks, oracle.enumerate_candidates(150000, C, wl.CANDIDATE_DT))
+    want = {f: len(oracle.valid_catalogue(w.problems[:1], DESC, f, pool.cpu().numpy().view(wl.CANDIDATE_DT).reshape(-1),
+                                          dtype=wl.CANDIDATE_DT)[0]) for f in (0, 1)}
+    assert want[0] != want[1]
+    assert ctx.valid_catalogue(w.problems[:1], 1, pool, C)[2] == want[1]
+    ctx.debug_set_wait(2000, 2)
+    ctx.select(dev(ks, w.problems), 1, dev(ks, w.candidates), 1000, model, w.k)
+    ctx.debug_set_wait(0, 0)
+    for f in (0, 1, 0):
+        out, _, n = ctx.valid_catalogue(w.problems[:1], f, pool, C)
+        assert n == want[f]
+    assert ctx.device_status() == ks.KS_ERR_TIMEOUT  # (of the walk)
+    hi, hs = ctx.select_one(w.problems[:1], dev(ks, w.candidates), 1000, model, w.k)
+    assert_matches_oracle(w, hi.numpy()[None], hs.numpy()[None], 1e-5)
+    ctx.close()
+
+
 CHILD = """
 import resource, numpy as np
 from paper_2609_35587_b200 import binding as ks, workloads as wl
