@@ -85,7 +85,9 @@ constexpr int kOffBuf0 = 0;
 // nobody waits) adds its parts in order and ranks it. In a single-problem call the last block overall
 // merges the lists and writes the final result. Where a block is cut depends on where it lies, a
 // candidate's score must not (equal candidates tie, whatever their places): a chunk's trees are added up in
-// 32 bits, in a fixed order, and the chunks' sums in 64, where their order leaves no trace in the result.
+// floats, in a fixed order, and the chunks' sums as doubles that are multiples of one power of two (`grid`, see
+// sum_grid), so that every sum of them is exact, in any order. An ensemble whose leaves spread too far for that has
+// no grid: all blocks are cut alike then.
 //
 // The line is measured in trees, a block's beginning with `fill` trees' worth for its tile; a CTA that starts
 // inside a block fills its tile too, but that holds for nearly all of them. Trees are dealt in units of
@@ -95,6 +97,7 @@ struct SplitArgs {
   int unit, fill;       // trees of a unit, and what filling a tile counts for
   int blocks;
   int step, rest;       // total / CTAs, and the remainder
+  double grid;          // added and subtracted, it rounds a chunk's sum to a multiple of its lowest bit; or 0
   double* scores;       // [CTAs][2][NC]: sums of a CTA's first and last part
   int* words;           // the context's device words: arrival counters, by the first CTA of a block (reset by their last users), kWordWalk
   int32_t* out_idx;     // single-problem form only: [k] final result (device-visible, may be
@@ -1060,7 +1063,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
       if (split) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          sums[r] += static_cast<double>(score[r]);
+          sums[r] += __dsub_rn(__dadd_rn(static_cast<double>(score[r]), sl.grid), sl.grid);
           score[r] = 0.0f;
         }
       }
@@ -1332,6 +1335,30 @@ static bool pick_geometry(int n_rows, Geometry* out) {
   return false;
 }
 
+// What rounds a chunk's sum to a multiple of u, a power of two of which no sum of one leaf a tree has more than
+// 2^51: 1.5 * 2^52 u. Sums of such multiples are exact. The rounding, at most B 2^-52 with B the sum of the trees' largest
+// leaves, is none where every leaf is a multiple of u already; it is far below the last bit of any float score where the
+// leaves are of one scale (`even`: fixed_point_shift's B <= 200 V, so at most V 2^-44 a chunk where a float holds V to
+// 2^-25). Else 0.
+static double sum_grid(int n_trees, const int64_t* off, const ks_node_host* nodes, bool even) {
+  double largest = 0.0;
+  int low = INT_MAX, e = 0;  // exponent of the lowest bit of any leaf
+  for (int t = 0; t < n_trees; ++t) {
+    float top = 0.0f;
+    for (int64_t i = off[t]; i < off[t + 1]; ++i) {
+      const float v = std::fabs(nodes[i].thr_or_leaf);
+      if (nodes[i].feat != 0xFFFF || v == 0.0f) continue;
+      top = std::max(top, v);
+      uint32_t digits = static_cast<uint32_t>(std::ldexp(std::frexp(v, &e), 24));
+      for (e -= 24; !(digits & 1u); digits >>= 1) ++e;
+      low = std::min(low, e);
+    }
+    largest += top;
+  }
+  std::frexp(1.001 * largest, &e);  // (< 2^e; a chunk's float sum rounds up by less than a thousandth)
+  return even || low >= e - 51 ? std::ldexp(1.5, e + 1) : 0.0;
+}
+
 cudaError_t build_fast_gbdt(GbdtModel& m, int n_trees, const int64_t* off, const ks_node_host* nodes) {
   m.fast = false;
   if (n_trees < 1 || m.max_depth < 1 || m.max_depth > kFastMaxDepth) return cudaSuccess;
@@ -1516,6 +1543,7 @@ cudaError_t build_fast_gbdt(GbdtModel& m, int n_trees, const int64_t* off, const
   if (e == cudaSuccess) e = cudaMemcpy(m.d_qfeat, fq, sizeof(fq), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return e;
   m.fixed_shift = fixed_point_shift(n_trees, off, nodes);
+  m.sum_grid = sum_grid(n_trees, off, nodes, m.fixed_shift != kNoFixed);
   m.class_words = class_tree_words(n_trees, off, nodes);
   m.top_levels = L;
   m.top_compact = compact;
@@ -1644,15 +1672,20 @@ static int split_plan(const GbdtModel& g, int64_t blocks, SplitArgs* s) {
   constexpr int64_t kParts = 32;
   const int64_t most = std::max<int64_t>(1, std::min({blocks * len / (fill + s->unit), slots, kParts * blocks}));
   // Stretches that end where blocks do spare the second tile and the second part of most CTAs (some 4 us):
-  // an equal number of CTAs a block, where that keeps nearly all of them busy.
+  // an equal number of CTAs a block, where that keeps nearly all of them busy, or where the sums ask for it.
+  s->grid = g.sum_grid;
   const int64_t each = std::min<int64_t>({slots / blocks, s->units, kParts});
   if (each >= 1) {
     const int64_t aligned = (s->units + each - 1) / each * s->unit;
     const int64_t shared = (blocks * len / most - fill + s->unit - 1) / s->unit * s->unit + fill + 16;
-    if (aligned <= shared) {
+    if (aligned <= shared || g.sum_grid == 0.0) {
       s->fill = 0;
       return deal(blocks * each);
     }
+  }
+  if (g.sum_grid == 0.0) {
+    s->units = 0;
+    return 0;
   }
   return deal(most);
 }
@@ -1668,6 +1701,7 @@ static bool split_fits(const GbdtModel& g, int64_t blocks) {  // (a line of tree
 }
 bool fast_splits(const GbdtModel& g, int P, int nblk, bool one_round) {
   const int64_t blocks = static_cast<int64_t>(P) * nblk;
+  one_round |= g.sum_grid == 0.0;  // (blocks that are all cut alike share one round of CTAs)
   return split_fits(g, blocks) && P >= 1 && P <= kSplitProblems && blocks < (one_round ? g.ctas_per_sm * kSmCount : P < kMemoMinProblems ? kSplitBlocks : kSplitBlocksMemo) && g.n_chunks > ring_count(g.fast_threads / (g.block_cands / 4));
 }
 size_t fast_split_bytes(const GbdtModel& g) { return sizeof(double) * 2 * 2 * kSmCount * g.block_cands; }

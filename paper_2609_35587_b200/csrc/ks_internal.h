@@ -95,6 +95,7 @@ struct GbdtModel {
   FastTopParams* h_top = nullptr;  // host copy, passed by value at every launch
   int tpc = 0;                 // trees per chunk
   int n_chunks = 0;
+  double sum_grid = 0.0;       // rounds the sums that a split walk adds up (see there), 0: none
   int fixed_shift = kNoFixed;  // leaf values as integers, and the words of the largest tree compiled for
   int class_words = 0;         // one candidate (ks_gbdt_classes.cu)
   int chunk_bytes = 0;

@@ -26,7 +26,7 @@ def ctx(ks):
 
 @pytest.mark.parametrize("C,P,trees,depth,law", [(1024, 1, 9, 8, "pernode"), (1025, 1, 33, 6, "slots128"),
                                                  (60001, 1, 61, 8, "pernode"), (3000, 19, 100, 6, "hist256"),
-                                                 (150500, 1, 40, 7, "pernode"), (2048, 73, 70, 3, "slots128"),
+                                                 (150500, 1, 40, 7, "pernode"), (100500, 1, 130, 8, "hist256"), (2048, 73, 70, 3, "slots128"),
                                                  (1500, 148, 25, 8, "slots128"), (9000, 3, 17, 10, "hist256")])
 def test_copies_of_candidates_tie(ks, ctx, C, P, trees, depth, law):
     dev, k, period = torch.device("cuda", 0), 32, 431
@@ -53,13 +53,41 @@ def test_copies_of_candidates_tie(ks, ctx, C, P, trees, depth, law):
             assert np.array_equal(mine, np.arange(c, C, period)[:len(mine)])
         assert set(got % period) <= set(np.array(want) % period)
     if P == 1:
-        one_i, one_s = ctx.select_one(prob, d_c, C, model, k)
-        assert np.array_equal(one_i.numpy(), idx[0]) and np.array_equal(one_s.numpy(), sc[0])
-        cat = ctx.catalogue_prepare(d_c, C, model)
-        one_i, one_s = ctx.select_one_prepared(cat, prob, k)
-        assert np.array_equal(one_i.numpy(), idx[0]) and np.array_equal(one_s.numpy(), sc[0])
-        rows = ctx.featurize(d_p, 1, d_c, C)
-        score = ctx.score(rows, model).cpu().numpy()
-        assert np.array_equal(score[idx[0]], sc[0])
-        for c in range(0, period, 7):
-            assert len(set(score[c::period])) == 1
+        entries_agree(ks, ctx, model, prob, d_p, d_c, C, k, idx[0], sc[0], period)
+
+
+def entries_agree(ks, ctx, model, prob, d_p, d_c, C, k, idx, sc, period):
+    """The single calls and the scoring call give the answer of ks_select, and copies one score."""
+    one_i, one_s = ctx.select_one(prob, d_c, C, model, k)
+    assert np.array_equal(one_i.numpy(), idx) and np.array_equal(one_s.numpy(), sc)
+    cat = ctx.catalogue_prepare(d_c, C, model)
+    one_i, one_s = ctx.select_one_prepared(cat, prob, k)
+    assert np.array_equal(one_i.numpy(), idx) and np.array_equal(one_s.numpy(), sc)
+    rows = ctx.featurize(d_p, 1, d_c, C)
+    score = ctx.score(rows, model).cpu().numpy()
+    assert np.array_equal(score[idx], sc)
+    for c in range(period):
+        assert len(set(score[c::period])) == 1
+
+
+@pytest.mark.parametrize("C,trees,depth,law,huge", [(60001, 250, 8, "pernode", ()), (60001, 250, 8, "pernode", (1e20, 1e16, 1e12, 1e9)),
+                                                    (100500, 130, 8, "slots128", (3e37, 1e9)), (9000, 300, 6, "hist256", (1e12,))])
+def test_copies_tie_whatever_the_leaves(ks, ctx, C, trees, depth, law, huge):
+    """Leaves of one scale over ten binades, and huge ones that cancel over the trees, where every order of
+    additions has a sum of its own: blocks that are cut at different places, and blocks that are cut alike."""
+    dev, k, period = torch.device("cuda", 0), 32, 431
+    off, nodes = wl.gbdt_complete(C + trees, trees, depth, wl.feature_stats("cfg1"), 0.1, law)
+    rng = np.random.default_rng(trees)
+    leaf = nodes["feat"] == 0xFFFF
+    nodes["v"][leaf] *= np.exp2(rng.integers(-5, 6, int(leaf.sum()))).astype(np.float32)
+    at = rng.permutation(trees)[:2 * len(huge)].reshape(-1, 2)
+    for h, (up, down) in zip(huge, at):
+        nodes["v"][off[up]:off[up + 1]][leaf[off[up]:off[up + 1]]] = h
+        nodes["v"][off[down]:off[down + 1]][leaf[off[down]:off[down + 1]]] = -h
+    model = ctx.model_create_gbdt(off, nodes, 0.25)
+    cand = wl.candidates_full_grid(7, period)[np.arange(C) % period]
+    prob = wl.problems_batch(C, 1)
+    d_c, d_p = ks.to_device(cand, dev), ks.to_device(prob, dev)
+    idx, sc = (t.cpu().numpy() for t in ctx.select(d_p, 1, d_c, C, model, k))
+    assert np.all(np.diff(sc[0]) <= 0)
+    entries_agree(ks, ctx, model, prob, d_p, d_c, C, k, idx[0], sc[0], period)
