@@ -388,7 +388,7 @@ ks_status ks_model_describe(const ks_model* model, char* buf, int len) {
 ks_status ks_debug_set_wait(ks_ctx* ctx, int probe_limit, int starve) {
   if (!ctx || probe_limit < 0) return KS_ERR_INVALID_ARG;
   ctx->wait.limit = probe_limit;
-  ctx->wait.starve = starve == ks::kStarveOdd ? starve : starve != 0 ? ks::kStarveAll : 0;
+  ctx->wait.starve = starve == ks::kStarveOdd || starve == ks::kStarveTiles ? starve : starve != 0 ? ks::kStarveAll : 0;
   return KS_OK;
 }
 

@@ -676,11 +676,14 @@ __device__ __noinline__ void fill_tile(const ks_gpu_desc& desc, const ProblemTer
 // the kernel
 // ------------------------------------------------------------------------------------------
 
-// Bounded wait for a tile that is copied in one piece: the thread is suspended by the barrier itself.
-__device__ __forceinline__ bool tile_wait(uint32_t bar, uint32_t parity, int limit) {
-  for (int i = 0; i < limit; ++i)
-    if (mbar_try_wait(bar, parity)) return true;
-  return false;
+// Bounded wait for a tile that is copied in one piece: the thread is suspended by the barrier itself, for as long as the
+// hardware sees fit, so the bound is a time: half a microsecond a probe of `limit`. (To sleep here as mbar_wait_bounded
+// does costs a single call 2 us of 96.)
+__device__ __forceinline__ bool tile_wait(uint32_t bar, uint32_t parity, int limit, volatile int* fail) {
+  const long long begin = clock64(), most = static_cast<long long>(limit) * 1000;
+  while (!mbar_try_wait(bar, parity))
+    if (*fail || clock64() - begin > most) return false;
+  return true;
 }
 
 // bytes of `a` where the top bit of the matching byte of `m` is set, else bytes of `b`
@@ -900,7 +903,7 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
         const uint32_t bytes = static_cast<uint32_t>(sl.cand_tiles ? fv.n_pair_rows : fv.n_rows) * NC;
         const uint32_t more = sl.cand_tiles ? static_cast<uint32_t>(fv.n_cand_rows) * NC : 0u;
         asm volatile("fence.proxy.async.global;" ::: "memory");  // (written by ordinary stores of the kernel in front)
-        mbar_expect_tx(bar, bytes + more);
+        mbar_expect_tx(bar, bytes + more + (fv.starve == kStarveTiles ? 16 : 0));  // (test hook, as below)
         if (bytes) bulk_copy_g2s(sbase + kOffTile, sl.tiles + (static_cast<size_t>(prob) * nblk + chunk) * bytes, bytes, bar);
         // (the record's terms are the first problem of the combination here)
         if (more) {
@@ -919,11 +922,13 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
           reinterpret_cast<uint4*>(dst)[i] = make_uint4(b, b, b, b);
         }
       }
-      if (!tile_wait(bar0 + 8u * (kNBuf * RG), tile_phase, fv.wait_limit)) {
+      if (!tile_wait(bar0 + 8u * (kNBuf * RG), tile_phase, fv.wait_limit, v_fail)) {
         tile_late = true;
-        s_fail = 1;
-        atomicExch(sl.words + kWordWalk, kLeaveFailed);
-        if (status) atomicExch(status, KS_ERR_TIMEOUT);
+        if (!*v_fail) {
+          s_fail = 1;
+          atomicExch(sl.words + kWordWalk, kLeaveFailed);
+          if (status) atomicExch(status, KS_ERR_TIMEOUT);
+        }
       }
       tile_phase ^= 1u;
     } else {
@@ -1090,17 +1095,16 @@ select_fast_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, ks_proble
     if (*v_fail) {
       // The call has failed. Before this CTA gives its shared memory back, give the copies that
       // may still be in flight the time to land (bounded again); the test hook's copies land in
-      // full although their barriers never complete, so there a short pause stands in for it (and so it does
-      // for a tile whose wait ran out).
+      // full although their barriers never complete, so there a short pause stands in for it.
+      const auto let_land = [&](uint32_t bar, uint32_t parity, bool hooked) {
+        if (!hooked) mbar_wait_bounded(bar, parity, fv.wait_limit, &s_abort /* stays 0 */);
+        else
+          for (int i = 0; i < 64; ++i) __nanosleep(kSleepNs);
+      };
       if (word == 0 && grp % GPR == 0) {  // one thread per ring, for its ring's buffers (it knows their parities)
-        for (int b = 0; b < kNBuf; ++b) {
-          if (!s_pending[ring * kNBuf + b]) continue;
-          if (starved || tile_late) {
-            for (int i = 0; i < 64; ++i) __nanosleep(kSleepNs);
-          } else {
-            mbar_wait_bounded(bar0 + 8u * (ring * kNBuf + b), (phases >> b) & 1u, fv.wait_limit, &s_abort /* stays 0 */);
-          }
-        }
+        for (int b = 0; b < kNBuf; ++b)
+          if (s_pending[ring * kNBuf + b]) let_land(bar0 + 8u * (ring * kNBuf + b), (phases >> b) & 1u, starved);
+        if (tile_late && ring == 0) let_land(bar0 + 8u * (kNBuf * RG), tile_phase ^ 1u, fv.starve == kStarveTiles);
       }
       __syncthreads();
       if (tid < k && partial) partial[(static_cast<size_t>(prob) * nblk + chunk) * k + tid] = 0ull;

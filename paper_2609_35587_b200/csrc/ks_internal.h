@@ -188,7 +188,7 @@ constexpr int kWordWalk = kMaxShares + 1, kWordMlp = kWordWalk + 1, kWordWide = 
 constexpr int kWordValid = kWordWide + 1;   // arrival counter of ks_valid_catalogue, cleared by the call itself
 constexpr int kWordServed = kWordValid + 1;  // calls that the walk of whole classes has served (ks_debug_class_walks)
 constexpr int kContextWords = kWordServed + 1;
-constexpr int kStarveAll = 1, kStarveOdd = 2;  // test hook: barriers that never complete, of all CTAs or of every other one
+constexpr int kStarveAll = 1, kStarveOdd = 2, kStarveTiles = 3;  // test hook: barriers that never complete: the chunks', those of every other CTA, the tiles'
 constexpr int kLeaveFailed = 1, kLeaveServed = 2;  // a wait ran out; another kernel serves the call
 
 // Levels of the categorical field held by feature column `col` (0: not a level-code column):

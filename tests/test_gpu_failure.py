@@ -31,24 +31,29 @@ def assert_matches_oracle(w, idx, sc, tol):
     assert np.all(np.abs(sc - rsc) <= tol * np.maximum(1, np.abs(rsc)))
 
 
-@pytest.mark.parametrize("law", ["slots128", "pernode"])
-def test_tree_kernel_wait_runs_out(ks, law):
+@pytest.mark.parametrize("law,starve", [("slots128", 1), ("pernode", 1), ("slots128", 3), ("pernode", 3)])
+def test_tree_kernel_wait_runs_out(ks, law, starve):
+    """With 1 the first chunk of every walk does not arrive, with 3 the tile of every split walk."""
     ctx = ks.Context(DESC, 0)
     w = wl.make_workload(1, P=3, C=2500, trees=60, law=law)
     model = ctx.model_create_gbdt(*w.gbdt)
     assert "select_fast_kernel" in model.describe()
     d_p, d_c = dev(ks, w.problems), dev(ks, w.candidates)
-    ctx.debug_set_wait(2000, True)
+    cat = ctx.catalogue_prepare(d_c, 2500, model)
+    ctx.debug_set_wait(2000, starve)
     # asynchronous batch call: the status word tells
     ctx.select(d_p, 3, d_c, 2500, model, w.k)
     assert ctx.device_status() == ks.KS_ERR_TIMEOUT
     assert ctx.device_status() == ks.KS_OK          # reported once, then cleared
-    # host-buffer call and single-problem call (tree slices) report it themselves
+    # host-buffer call and single-problem calls report it themselves
     with pytest.raises(ks.KsError) as e:
         ctx.select_host(w.problems, 3, w.candidates, 2500, model, w.k)
     assert e.value.status == ks.KS_ERR_TIMEOUT
     with pytest.raises(ks.KsError) as e:
         ctx.select_one(w.problems[:1], d_c, 2500, model, w.k)
+    assert e.value.status == ks.KS_ERR_TIMEOUT
+    with pytest.raises(ks.KsError) as e:
+        ctx.select_one_prepared(cat, w.problems[:1], w.k)
     assert e.value.status == ks.KS_ERR_TIMEOUT
     # scoring call on the same walk
     x = oracle.featurize(w.problems[:1], w.candidates, DESC)
@@ -60,6 +65,8 @@ def test_tree_kernel_wait_runs_out(ks, law):
     assert ctx.device_status() == ks.KS_OK
     assert_matches_oracle(w, idx.cpu().numpy(), sc.cpu().numpy(), 1e-5)
     hi, hs = ctx.select_one(w.problems[1:2], d_c, 2500, model, w.k)
+    assert np.array_equal(hi.numpy(), idx[1].cpu().numpy())
+    hi, hs = ctx.select_one_prepared(cat, w.problems[1:2], w.k)
     assert np.array_equal(hi.numpy(), idx[1].cpu().numpy())
     s = ctx.score(dev(ks, x), model).cpu().numpy()
     rs = oracle.score_gbdt(x, *w.gbdt)
