@@ -227,8 +227,10 @@ ks_status ks_enumerate(ks_ctx* ctx, int64_t first, int64_t count, ks_candidate* 
  *                 input order
  *   d_out_index   device, capacity C, or NULL: their positions in the input (= ids)
  *   d_count       device, one int32: how many are valid
- *   h_count       host, or NULL; when given the call copies the count there and waits for the
- *                 stream, otherwise it is asynchronous on `stream`
+ *   h_count       host, or NULL; when given the call returns with the count there, d_out,
+ *                 d_out_index and d_count written and everything in front of it on `stream` done
+ *                 (cudaStreamQuery may answer cudaErrorNotReady for some microseconds more),
+ *                 otherwise it is asynchronous on `stream`
  * Entries of d_out / d_out_index past the count are left untouched. Uses the context's
  * workspace (calls on one context must not overlap). */
 ks_status ks_valid_catalogue(ks_ctx* ctx, const ks_problem* problem, unsigned flags,
@@ -278,13 +280,16 @@ ks_status ks_score(ks_ctx* ctx, const float* d_features, int64_t rows, const ks_
  * `pairs` as in ks_featurize. The call
  * sizes the context's workspace (owned by the context, grown on demand, which synchronises the
  * device when it happens): partial lists, a per-call table of 16 x C records of at most 256
- * bytes, and, for a tree model on a batch of 32 problems or more, at most 256 MiB for the
- * tables of per-pair tile rows (larger batches are served in several launches that reuse it),
+ * bytes, and, for a tree model on a dense batch of 3 problems or more or a segmented one of 32, at most 512 MiB
+ * for the tables of per-pair tile rows (larger batches are served in several launches that reuse it), or, where
+ * the machine's CTAs share out the trees of few candidate blocks, the blocks' tiles (at most 188 KiB for each of
+ * 1,924 blocks), for a linear scorer 14 MiB, 320 bytes a candidate and 64 KiB for each of at most 1,036 blocks,
  * and, for batches of more than 100 problems on a catalogue of 4,096 to 2,097,152 candidates with an
  * ensemble of at most 1,024 trees, 0.46 to 1.1 MB per tree (by the size of the largest tree) and at most
  * 1 GiB of scores for the walk of whole classes of candidates;
  * KS_ERR_OOM if the workspace cannot be had. Where only all of it cannot be had, the call does without the
- * walk of whole classes, or (a ranker with a layer wider than 256 units or more than two hidden layers) ranks
+ * walk of whole classes, without tiles in front of more blocks than the machine holds at once, with the class tables of 16
+ * problems at a time, without the linear scorer's classes, or (a ranker with a layer wider than 256 units or more than two hidden layers) ranks
  * 2,048 rows at a time with at most 19 MB beside the partial lists; so do the context's later calls of that
  * size and above. d_p and d_c must be 16-byte aligned (each record
  * is fetched with one 128-bit load), else KS_ERR_INVALID_ARG. */
@@ -295,7 +300,10 @@ ks_status ks_select(ks_ctx* ctx, const ks_problem* d_p, int P, const ks_candidat
 
 /* Latency form of ks_select for one problem passed by value against the dense pool
  * d_c[0..C): h_topk_idx / h_topk_score ([k], host memory, pinned for best latency) are
- * valid when the call returns (it synchronises `stream`). */
+ * valid when the call returns. It waits for a word that its last kernel writes behind the results, so
+ * everything in front of it on `stream` is done then, but cudaStreamQuery may answer
+ * cudaErrorNotReady for some microseconds more; where that word does not come (an error of this or of
+ * earlier work), the call synchronises `stream` and reports it. */
 ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int C,
                         const ks_model* model, int k, int32_t* h_topk_idx,
                         float* h_topk_score, void* stream);
@@ -303,11 +311,9 @@ ks_status ks_select_one(ks_ctx* ctx, ks_problem p, const ks_candidate* d_c, int 
 /* A candidate catalogue prepared for a stream of single-problem calls with one model (the
  * dynamic-selection setting: problems arrive one at a time, the catalogue and the ranker stay).
  * Everything about a call that depends only on (catalogue, model) is computed here, once: for a
- * tree ensemble on the quantised path, every candidate's quantised candidate-only columns under
- * each of the 16 element-type combinations and the classes of candidates that look alike to
- * the per-pair columns. ks_select_one_prepared then evaluates the per-pair columns once per class
- * for the problem at hand and runs the fused walk + top-k: two launches per call instead of
- * building the candidates' tiles anew. The handle owns its device memory (a few hundred bytes
+ * tree ensemble on the quantised path, the candidate-only rows of the catalogue's tiles under
+ * each of the 16 element-type combinations, in similarity order. ks_select_one_prepared then builds
+ * the per-pair rows for the problem at hand and runs the fused walk + top-k: two launches per call. The handle owns its device memory (a few hundred bytes
  * per candidate), refers to d_c and the model (both must outlive it and stay unchanged) and
  * belongs to the context. For models the quantised path does not serve, the handle is a plain
  * reference and ks_select_one_prepared is ks_select_one. Synchronises `stream`. */
@@ -414,6 +420,9 @@ ks_status ks_debug_limit_workspace(ks_ctx* ctx, int64_t bytes);
 /* How many calls of this context the walk of whole classes of candidates has served so far (a tree
  * ensemble on a large batch; the choice falls on the device). Waits for the device; -1 on failure. */
 int64_t ks_debug_class_walks(ks_ctx* ctx);
+/* How many walks this context has launched whose trees the machine's CTAs share out (few candidate blocks: ks_select,
+ * ks_select_one, ks_score with a tree ensemble); -1 without a context. */
+int64_t ks_debug_split_walks(const ks_ctx* ctx);
 /* Measurement aid, no counterpart in the paper: the tree walk of ks_score stripped of everything
  * but its gather and instruction stream, to measure the floor that stream sets for the tree
  * kernel. Tiles are built from the `rows` feature rows (device, [rows][64] floats) exactly as

@@ -3,7 +3,7 @@
 // only through (T_M, T_N, T_K, S, c_M, c_N) and its resident-block count, and a cross-product
 // catalogue holds far fewer such classes than candidates (the schedules and the instruction
 // shape do not enter). Per call every candidate is given its class: a slot of a hash table per
-// element-type combination, filled with atomicCAS and linear probing; the slot also remembers
+// element-type combination, filled with atomicCAS and triangular probing (steps of 1, 2, 3, ...); the slot also remembers
 // one member. Whatever depends on (problem, per-pair columns) can then be evaluated once per
 // (problem, class) from the member and looked up per pair. A candidate whose fields do not fit
 // the key, or whose probe sequence runs out (more classes than slots), has no class and is
