@@ -28,6 +28,7 @@ EXPORTS = ("ks_create", "ks_destroy", "ks_last_cuda_error", "ks_model_create_gbd
            "ks_enumerate", "ks_valid_catalogue", "ks_remap_indices", "ks_model_describe", "ks_merge_topk", "ks_catalogue_prepare", "ks_catalogue_destroy",
            "ks_select_one_prepared",
            "ks_debug_set_wait", "ks_debug_bounds_line", "ks_debug_bounds_clear", "ks_debug_walk_floor", "ks_debug_class_walks",
+           "ks_debug_split_walks",
            "ks_debug_limit_workspace")
 
 
@@ -88,6 +89,8 @@ def _load() -> ctypes.CDLL:
     lib.ks_debug_limit_workspace.argtypes = [vp, i64]
     lib.ks_debug_class_walks.argtypes = [vp]
     lib.ks_debug_class_walks.restype = i64
+    lib.ks_debug_split_walks.argtypes = [vp]
+    lib.ks_debug_split_walks.restype = i64
     lib.ks_debug_bounds_line.restype = i32
     lib.ks_debug_bounds_clear.restype = None
     for name in EXPORTS:
@@ -266,6 +269,10 @@ class Context:
     def debug_class_walks(self) -> int:
         """How many calls the walk of whole classes has served so far (the choice falls on the device)."""
         return int(_lib.ks_debug_class_walks(self._h))
+
+    def debug_split_walks(self) -> int:
+        """How many split walks have been launched so far."""
+        return int(_lib.ks_debug_split_walks(self._h))
 
     def profile_enable(self, on: bool = True):
         self._check(_lib.ks_profile_enable(self._h, int(on)), "ks_profile_enable")

@@ -126,7 +126,8 @@ cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes) {
 
 namespace {
 
-// Reads (and clears) the device status word; the stream must have been synchronised.
+// Reads (and clears) the device status word, once the call's last kernel has told that it is done or the stream has been
+// synchronised (every kernel that may raise it ends before that).
 ks_status read_status(ks_ctx* ctx) {
   const int v = *static_cast<volatile int*>(ctx->h_status);
   if (v != 0) {
@@ -402,6 +403,8 @@ ks_status ks_debug_limit_workspace(ks_ctx* ctx, int64_t bytes) {
   ctx->ws_limit = bytes > 0 ? static_cast<size_t>(bytes) : SIZE_MAX;
   return e == cudaSuccess ? KS_OK : cuda_fail(ctx, e, "ks_debug_limit_workspace");
 }
+
+int64_t ks_debug_split_walks(const ks_ctx* ctx) { return ctx ? ctx->split_walks : -1; }
 
 int64_t ks_debug_class_walks(ks_ctx* ctx) {
   if (!ctx) return -1;

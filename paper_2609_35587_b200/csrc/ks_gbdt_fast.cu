@@ -2049,6 +2049,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
     a.seg_off = seg_off ? seg_off + first : nullptr;
     a.partial = partial + static_cast<size_t>(first) * nblk * k;
     if (split) a.split_ctas = split_plan(g, static_cast<int64_t>(n) * nblk, &a.sl);
+    if (a.sl.units > 0) ++*wait->splits;
     e = launch_walk(g, a);
     ++*launches;
     if (e != cudaSuccess) return e;
@@ -2101,6 +2102,7 @@ cudaError_t launch_score_fast(const ks_gpu_desc& desc, const GbdtModel& g, const
       a.split_ctas = split_plan(g, nblk, &a.sl);
       a.sl.scores = reinterpret_cast<double*>(tiles + score_fast_scratch_bytes(g, std::min(rows, kScoreBatchRows)) - fast_split_bytes(g));
     }
+    if (a.sl.units > 0) ++*wait->splits;
     a.sl.words = wait->words;
     a.dependent = 1;
     a.sl.tiles = tiles;

@@ -69,6 +69,7 @@ struct FastWait {
   int starve;  // kStarve..., 0: none
   int lean;  // the memory for all of the workspace could not be had: without the walk of whole classes, few rows or problems at a time
   int* words;
+  int64_t* splits;  // counts the launches of split walks (ks_debug_split_walks)
 };
 
 constexpr int kNoFixed = INT32_MIN;
@@ -138,7 +139,8 @@ struct ks_ctx {
   int* d_status = nullptr;  // bounded waits give up; d_status is its device alias
   int64_t launches = 0;
   int host_seq = 0;  // sequence number of the last call whose end the host polls for
-  ks::FastWait wait{0, 0, 0, nullptr};  // probe budget of bounded device waits (0: default), starve hook (tests), lean, d_words
+  int64_t split_walks = 0;
+  ks::FastWait wait{0, 0, 0, nullptr, &split_walks};  // probe budget of bounded device waits (0: default), starve hook (tests), lean, d_words
   size_t ws_refused = SIZE_MAX;  // the smallest workspace that could not be had
   size_t ws_limit = SIZE_MAX;    // test hook: larger ones cannot be had
   char err[256] = {0};
@@ -156,7 +158,7 @@ struct ks_catalogue {
   int C = 0;
   int device = 0;
   bool prepared = false;   // false: calls go through ks_select_one
-  int nblk = 0, max_k = KS_MAX_K;
+  int nblk = 0;
   void* d_mem = nullptr;   // one block: candidate-only rows | a call's rows | partial lists | partial sums | similarity order
   size_t off_call = 0, off_part = 0, off_scores = 0, off_order = 0;
 };
