@@ -28,18 +28,21 @@ def main() -> int:
     cases.append(("cfg2 pernode segments", wl.make_workload(2, P=3, seg=1100, law="pernode"), 10))
     cases.append(("cfg2 memo", wl.make_workload(2, P=40, seg=90, trees=30, depth=6), 10))
     # more (problem, candidate block) items than SMs: the launch form in which a CTA serves many items
-    cases.append(("many items", wl.make_workload(1, P=90, C=2100, trees=24, depth=8, law="pernode"), 10))
+    # (and more blocks than a split walk takes)
+    cases.append(("many items", wl.make_workload(1, P=400, C=2100, trees=24, depth=8, law="pernode"), 10))
     for name, w, k in cases:
         model = ctx.model_create_gbdt(*w.gbdt)
         assert "select_fast_kernel" in model.describe(), (name, model.describe())
         P, C = len(w.problems), len(w.candidates)
         d_so = None if w.seg_offsets is None else ks.to_device(w.seg_offsets, dev)
         d_si = None if w.seg_index is None else ks.to_device(w.seg_index, dev)
+        splits = ctx.debug_split_walks()
         idx, sc = ctx.select(ks.to_device(w.problems, dev), P, ks.to_device(w.candidates, dev), C, model, k,
                              d_so, d_si, w.pairs)
+        assert name != "many items" or ctx.debug_split_walks() == splits
         torch.cuda.synchronize()
         idx, sc = idx.cpu().numpy(), sc.cpu().numpy()
-        for i in range(P):
+        for i in range(0, P, 1 if P < 100 else 5):
             if w.seg_offsets is None:
                 pool = np.arange(C, dtype=np.int32)
                 so = si = None

@@ -27,7 +27,7 @@ def calls(ks, ctx):
     dev = torch.device("cuda", 0)
     put = lambda a: ks.to_device(a, dev)
     cand = wl.candidates_full_grid(2, 20000)
-    prob = wl.problems_batch(5, 48, cross_precision=False)
+    prob = wl.problems_batch(5, 64, cross_precision=False)
     d_p, d_c = put(prob), put(cand)
     model = trees(ctx, 3, 60, 8)
     rows = ctx.featurize(d_p, 4, d_c, 3000, pairs=12000)
@@ -39,7 +39,7 @@ def calls(ks, ctx):
     cat = ctx.catalogue_prepare(d_c, 20000, model)
     host = lambda pair: tuple(t.cpu().numpy().copy() for t in pair)
     return {
-        "dense": lambda: host(ctx.select(d_p, 48, d_c, 20000, model, 10)),
+        "dense": lambda: host(ctx.select(d_p, 64, d_c, 20000, model, 10)),
         "segments": lambda: host(ctx.select(d_p, 48, d_c, 20000, model, 10, so, si, si.numel())),
         "split": lambda: host(ctx.select(d_p, 3, d_c, 20000, model, 10)),
         "one": lambda: host(ctx.select_one(prob[7:8], d_c, 20000, model, 10)),
@@ -57,7 +57,13 @@ def test_overlapping_contexts(ks):
     d_p, d_c, model = ks.to_device(prob, dev), ks.to_device(cand, dev), trees(a, 1, 100, 8)
     alone = [t.clone() for t in a.select(d_p, 512, d_c, 60000, model, 10)]
     asked = calls(ks, b)
-    serial = {name: f() for name, f in asked.items()}
+    serial, split = {}, set()
+    for name, f in asked.items():
+        before = b.debug_split_walks()
+        serial[name] = f()
+        if b.debug_split_walks() > before:
+            split.add(name)
+    assert split == {"split", "one", "prepared", "rows"}
     torch.cuda.synchronize()
     s_a, s_b = torch.cuda.Stream(), torch.cuda.Stream()
     n = 120

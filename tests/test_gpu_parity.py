@@ -572,8 +572,8 @@ def test_select_tile_geometries(ks, ctx, case):
     quantile-per-node ensembles of config 1 (<= 156 rows: one CTA of 512 threads x 1,024
     candidates with 32 KB chunk buffers), the quantile-per-node ensemble of config 2 (<= 376 rows:
     one CTA of 512 threads x 512 candidates), and an ensemble with a continuous threshold at every node of 3,000 trees (more
-    rows than any geometry holds: the general kernel). Each: a batch (ks_select), the single-problem call (tree slices
-    over prepared tiles), the scoring call on given feature rows, and a batch of 33 problems or
+    rows than any geometry holds: the general kernel). Each: a batch (ks_select), the single-problem call (a split walk
+    over tiles built in front), the scoring call on given feature rows, and a batch of 33 problems or
     more that takes the per-(problem, class) memo."""
     if case == "continuous":
         prob, cand, _, _ = wl.make_inputs(1, P=3, C=2500)
@@ -633,19 +633,20 @@ def test_select_forced_tile_geometry(ks, ctx, geometry, monkeypatch):
 @pytest.mark.parametrize("geometry,segments", [("512,1024,32", False), ("512,512,16", False), ("512,512,32", True)])
 def test_select_more_items_than_sms(ks, ctx, geometry, segments, monkeypatch):
     """The one-CTA-per-SM geometries launch one CTA per SM and let it serve many (problem,
-    candidate block) items: here 330 to 660 items, not a multiple of the 148 CTAs, so that some
-    CTAs take one item more than others, with a ragged last block per problem; dense catalogue
-    (ranked in similarity order) and per-problem segments."""
+    candidate block) items: here 330 to 2,400 items, not a multiple of the 148 CTAs, so that some
+    CTAs take one item more than others, with a ragged last block per problem; per-problem segments
+    and a dense catalogue (ranked in similarity order, and enough problems that the walk is not split)."""
     monkeypatch.setenv("KS_FAST_GEOMETRY", geometry)
     if segments:
         w = wl.make_workload(2, P=110, seg=1300, trees=24, depth=8, law="pernode")
     else:
-        w = wl.make_workload(1, P=110, C=2700, trees=24, depth=8, law="pernode")
+        w = wl.make_workload(1, P=400, C=2700, trees=24, depth=8, law="pernode")
     model = ctx.model_create_gbdt(*w.gbdt)
     t, c, _ = geometry.split(",")
     assert f"threads={t} block={c}" in model.describe(), model.describe()
+    splits = ctx.debug_split_walks()
     idx, sc = run_select(ks, ctx, w, model)
-    check_select(w, idx, sc, TOL_GBDT, sample=range(0, 110, 2))
+    check_select(w, idx, sc, TOL_GBDT, sample=range(0, len(w.problems), 2 if segments else 7))
     idx2, sc2 = run_select(ks, ctx, w, model)     # the barriers' parities carry over from call to call
     assert np.array_equal(idx, idx2) and np.array_equal(sc, sc2)
     if not segments:
@@ -654,18 +655,19 @@ def test_select_more_items_than_sms(ks, ctx, geometry, segments, monkeypatch):
         rng = np.random.default_rng(11)
         w.problems = w.problems.copy()
         kinds = [(0, 0), (1, 1), (2, 1), (3, 3)]       # (dtype_ab, dtype_d)
-        pick = np.repeat(rng.integers(0, 4, 40), rng.integers(1, 6, 40))[:110]
+        pick = np.repeat(rng.integers(0, 4, 160), rng.integers(1, 6, 160))[:400]
         w.problems["dtype_ab"] = [kinds[i][0] for i in pick]
         w.problems["dtype_d"] = [kinds[i][1] for i in pick]
         idx, sc = run_select(ks, ctx, w, model)
-        check_select(w, idx, sc, TOL_GBDT, sample=range(0, 110, 3))
+        check_select(w, idx, sc, TOL_GBDT, sample=range(0, 400, 5))
+    assert ctx.debug_split_walks() == splits
 
 
 @pytest.mark.parametrize("law", ["slots128", "pernode"])
 def test_select_one_prepared_catalogue(ks, ctx, law):
-    """The single-problem call against a prepared catalogue (candidate-only rows and classes made
+    """The single-problem call against a prepared catalogue (the candidate-only rows of its tiles made
     once per catalogue and model): every call must give the oracle's ranking and the same result
-    as the unprepared call; mixed element types use different slices of the prepared tables; a
+    as the unprepared call; mixed element types use different parts of the prepared tables; a
     model the quantised path does not serve goes through the plain call."""
     w = wl.make_workload(3, P=12, C=7000, law=law)
     probs = w.problems.copy()
@@ -678,7 +680,7 @@ def test_select_one_prepared_catalogue(ks, ctx, law):
     cat = ctx.catalogue_prepare(d_c, C, model)
     n0 = ctx.launch_count()
     hi, hs = ctx.select_one_prepared(cat, probs[:1], 10)
-    assert ctx.launch_count() - n0 == 2   # the per-class table of the problem, then the fused walk + top-k
+    assert ctx.launch_count() - n0 == 2   # the per-pair rows of the problem's tiles, then the fused walk + top-k
     for i in range(len(probs)):
         hi, hs = ctx.select_one_prepared(cat, probs[i:i + 1], 10)
         hi, hs = hi.numpy().copy(), hs.numpy().copy()
@@ -692,7 +694,7 @@ def test_select_one_prepared_catalogue(ks, ctx, law):
     pi, ps = ctx.select_one(probs[2:3], d_c, C, model, 10)
     assert np.array_equal(ci.numpy(), pi.numpy())
     cat.close()
-    # other k, a tiny pool (a single block: no slices, plain call), and an MLP
+    # other k, a tiny pool (a single block), and an MLP
     small = ctx.catalogue_prepare(d_c, 40, model)
     hi, hs = ctx.select_one_prepared(small, probs[:1], 32)
     pi, ps = ctx.select_one(probs[:1], d_c, 40, model, 32)
@@ -739,7 +741,7 @@ def test_merge_topk_of_candidate_shares(ks, ctx):
 
 
 def test_select_memo_table_in_batches(ks, ctx):
-    """The per-(problem, class) table holds 256 MiB of records; a batch of more problems than that
+    """The per-(problem, class) table holds 512 MiB of records; a batch of more problems than that
     is served in several launches that reuse it (here 80-byte records: 409 problems at a time)."""
     w = wl.make_workload(1, P=900, C=300, law="pernode")
     model = ctx.model_create_gbdt(*w.gbdt)
@@ -766,19 +768,22 @@ def test_select_pair_row_memo_paths(ks, ctx):
     model = ctx.model_create_gbdt(*w.gbdt)
     idx, sc = run_select(ks, ctx, w, model)
     check_select(w, idx, sc, TOL_GBDT)
-    # more distinct classes than slots: 12,000 different tile shapes
-    i = np.arange(12000)
-    big = np.zeros(12000, wl.CANDIDATE_DT)
+    # more distinct classes than slots (16,384), and too many blocks for a split walk
+    n = 20000
+    i = np.arange(n)
+    big = np.zeros(n, wl.CANDIDATE_DT)
     big["tile_m"], big["tile_n"], big["tile_k"] = 16 * (1 + i % 16), 8 * (1 + (i // 16) % 32), 16 * (1 + (i // 512) % 32)
     big["instr_n"], big["instr_m"], big["instr_k"] = big["tile_n"], 64, 16
     big["stages"], big["cluster_m"], big["cluster_n"] = 2 + i % 3, 1 + (i // 7) % 2, 1
     big["kernel_sched"], big["epi_sched"], big["tile_sched"] = i % 4, i % 3, i % 2
-    assert len(np.unique(big[["tile_m", "tile_n", "tile_k", "stages", "cluster_m"]])) > 8192
-    w1 = wl.make_workload(1, P=33, C=10, trees=12, depth=5)
+    assert len(np.unique(big[["tile_m", "tile_n", "tile_k", "stages", "cluster_m"]])) == n
+    w1 = wl.make_workload(1, P=62, C=10, trees=12, depth=5)
     wb = wl.Workload("memo_overflow", DESC, w1.problems, big, 10, gbdt=w1.gbdt)
     model = ctx.model_create_gbdt(*w1.gbdt)
+    splits = ctx.debug_split_walks()
     idx, sc = run_select(ks, ctx, wb, model)
-    check_select(wb, idx, sc, TOL_GBDT)
+    assert ctx.debug_split_walks() == splits
+    check_select(wb, idx, sc, TOL_GBDT, sample=range(0, 62, 6))
     # segments over the pool
     ws = wl.make_workload(2, P=48, seg=700, trees=20, depth=5)
     model = ctx.model_create_gbdt(*ws.gbdt)

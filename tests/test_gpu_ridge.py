@@ -1,6 +1,6 @@
-"""The linear scorer's kernels at the sizes where they can go wrong: with the class tables (32 problems or
-more, four of them a block) and without, a last group of fewer than four problems, element types that
-change within a group, more classes than are staged (2,048) and more than there are slots (8,192), small
+"""The linear scorer's kernels at the sizes where they can go wrong: dense batches ranked by classes (30 problems
+and 600,000 pairs or more) and pair by pair, segments with the class tables, element types that change from problem
+to problem, more classes than are staged (2,048) and more than there are slots (16,384), small
 and ragged pools, k = 1, 10 and 32. The sums run in the same order as the oracle's problem, candidate and
 pair parts do not, so scores agree to 1e-4 as in the other tests of this scorer."""
 import numpy as np
@@ -68,8 +68,8 @@ def test_merge_of_partial_lists(ks, ctx, P, n):
 
 @pytest.mark.parametrize("P,C", [(8192, 300), (8193, 300), (8195, 70), (40, 0), (31, 0)])
 def test_problems_beyond_the_class_tables(ks, ctx, P, C):
-    """The class tables serve 32 to 8,192 problems and a pool that is not empty; four problems share a block
-    only with them. An empty pool gives empty lists."""
+    """More problems than blocks, on pools small enough to be ranked pair by pair and on either side of 600,000
+    pairs. An empty pool gives empty lists."""
     dev = torch.device("cuda", 0)
     st = wl.feature_stats("cfg2")
     mlp = wl.mlp_xavier(2, [64, 1], st["mu"], st["sigma"])
@@ -89,12 +89,13 @@ def test_problems_beyond_the_class_tables(ks, ctx, P, C):
 
 
 @pytest.mark.parametrize("what,P,C,k", [("plain", 30, 20000, 10), ("plain", 1040, 600, 32), ("valid", 33, 61140, 7),
-                                        ("no class", 40, 15001, 10), ("ties", 32, 18755, 32), ("not finite", 32, 19000, 10),
+                                        ("no class", 40, 15001, 10), ("full", 32, 20000, 10), ("ties", 32, 18755, 32), ("not finite", 32, 19000, 10),
                                         ("many", 8200, 80, 3)])
 def test_classes_against_pairs(ks, ctx, what, P, C, k):
     """A dense batch ranked by classes gives bit for bit what its pairs give one by one: the same pool as a
     segment of every problem takes the kernel that adds up each pair. Candidates without a class (a
-    tile of 4,096 or more), equal scores everywhere, scores that are not finite; more problems than blocks."""
+    tile of 4,096 or more, or more classes than slots: there both kernels evaluate some in place, so the oracle is
+    asked too), equal scores everywhere, scores that are not finite; more problems than blocks."""
     dev = torch.device("cuda", 0)
     st = wl.feature_stats("cfg2")
     mlp = wl.mlp_xavier(C, [64, 1], st["mu"], st["sigma"])
@@ -112,6 +113,11 @@ def test_classes_against_pairs(ks, ctx, what, P, C, k):
         cand = wl.candidates_full_grid(5, C)
         if what == "no class":
             cand["tile_m"][::50] = 4096
+        if what == "full":  # 20,000 classes
+            i = np.arange(C)
+            cand["tile_m"], cand["tile_n"] = 16 * (1 + i % 16), 8 * (1 + i // 16 % 32)
+            cand["tile_k"], cand["stages"] = 16 * (1 + i // 512 % 32), 2 + i // 16384
+            cand["cluster_m"] = cand["cluster_n"] = 1
         d_c = ks.to_device(cand, dev)
     d_p = ks.to_device(prob, dev)
     idx, sc = ctx.select(d_p, P, d_c, C, model, k)
@@ -120,3 +126,8 @@ def test_classes_against_pairs(ks, ctx, what, P, C, k):
     ridx, rsc = ctx.select(d_p, P, d_c, C, model, k, off, every, P * C)
     assert torch.equal(idx, ridx)
     assert torch.equal(sc.view(torch.int32), rsc.view(torch.int32))
+    if what == "full":
+        for p in (0, P - 1):
+            _, _, ref = oracle.select(prob[p:p + 1], cand, DESC, k, mlp=mlp, want_scores=True)
+            ok, msg = topk_accept(idx[p].cpu().numpy(), sc[p].cpu().numpy(), ref, np.arange(C, dtype=np.int32), k, 1e-4)
+            assert ok, (p, msg)

@@ -1,6 +1,6 @@
 """Batches of tree ensembles against small catalogues, which are ordered by counting (up to 8,192 candidates,
-with many equal keys), and the first size that is sorted, each ranked by the candidates' own walks (the orders as
-the walk of whole classes uses them: test_gpu_classes.py). Scores agree to the tolerance of the other tests of tree ensembles."""
+with many equal keys), and the first size that is sorted, each ranked by the candidates' own walks over whole blocks
+(a split walk takes no order; the orders as the walk of whole classes uses them: test_gpu_classes.py). Scores agree to the tolerance of the other tests of tree ensembles."""
 import numpy as np
 import pytest
 import torch
@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 DESC = wl.gpu_desc()
 
 
-@pytest.mark.parametrize("P,C", [(320, 15), (320, 1000), (300, 4097), (70, 8191), (70, 8192), (70, 8193), (4097, 4200)])
+@pytest.mark.parametrize("P,C", [(520, 15), (520, 1000), (300, 4097), (150, 8191), (150, 8192), (150, 8193), (4097, 4200)])
 def test_small_catalogue(P, C):
     from paper_2609_35587_b200 import binding as ks
     dev = torch.device("cuda", 0)
@@ -24,7 +24,7 @@ def test_small_catalogue(P, C):
     ctx = ks.Context(DESC, 0)
     model = ctx.model_create_gbdt(off, nodes, 0.5)
     idx, sc = ctx.select(ks.to_device(prob, dev), P, ks.to_device(cand, dev), C, model, 10)
-    assert ctx.debug_class_walks() == 0
+    assert ctx.debug_class_walks() == 0 and ctx.debug_split_walks() == 0
     idx, sc = idx.cpu().numpy(), sc.cpu().numpy()
     pool = np.arange(C, dtype=np.int32)
     for p in (0, P // 2, P - 1):

@@ -1,6 +1,6 @@
 """Calls whose whole workspace cannot be had (a hook stands in for a full device): a batch for the walk of
-whole classes goes to the candidates' own walks, a wide ranker takes few rows at a time, and what cannot do
-with less is refused. The answers agree with those with all of the workspace, and with the oracle."""
+whole classes goes to the candidates' own walks, a split walk of several rounds of blocks walks whole blocks, the linear
+scorer ranks pair by pair, a wide ranker takes few rows at a time, and what cannot do with less is refused. The answers agree with those with all of the workspace, and with the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -63,6 +63,56 @@ def test_trees(ks, ctx):
     ctx.debug_limit_workspace(0)
     after = host(ctx.select(*args))
     assert ctx.debug_class_walks() == 2 and np.array_equal(after[1], full[1])
+
+
+@pytest.mark.parametrize("P,C", [(9, 60000), (40, 25000)])
+def test_split_walk(ks, ctx, P, C):
+    """531 and 1,000 blocks: the tiles in front take some 30 MB, the rows of the candidates beside them or the class
+    records of a few problems a fraction of that."""
+    dev = torch.device("cuda", 0)
+    prob, cand = wl.problems_batch(3, P, cross_precision=False), wl.candidates_full_grid(1, C)
+    gbdt = (*wl.gbdt_complete(4, 60, 6, wl.feature_stats("cfg1"), 0.1, "slots128"), 0.0)
+    model = ctx.model_create_gbdt(*gbdt)
+    args = ks.to_device(prob, dev), P, ks.to_device(cand, dev), C, model, 10
+    full = host(ctx.select(*args))
+    assert ctx.debug_split_walks() == 1
+    need = 2
+    while True:  # the least that the call does with
+        ctx.debug_limit_workspace(need * MB)
+        try:
+            got = host(ctx.select(*args))
+            break
+        except ks.KsError as e:
+            assert e.status == ks.KS_ERR_OOM
+            need += 2
+    assert ctx.debug_split_walks() == 1
+    for idx, sc in (full, got):
+        for p in (0, P // 2, P - 1):
+            _, _, ref = oracle.select(prob[p:p + 1], cand, DESC, 10, gbdt=gbdt, want_scores=True)
+            ok, msg = topk_accept(idx[p], sc[p], ref, np.arange(C, dtype=np.int32), 10, 1e-5)
+            assert ok, (p, msg)
+    ctx.debug_limit_workspace(0)
+    after = host(ctx.select(*args))
+    assert ctx.debug_split_walks() == 2 and np.array_equal(after[1], full[1])
+
+
+def test_linear_scorer(ks, ctx):
+    """Ranked by classes the call takes some 40 MB, pair by pair 7; the answers are the same bits."""
+    dev = torch.device("cuda", 0)
+    st = wl.feature_stats("cfg2")
+    model = ctx.model_create_mlp(wl.mlp_xavier(3, [64, 1], st["mu"], st["sigma"]))
+    args = ks.to_device(wl.problems_batch(3, 40), dev), 40, ks.to_device(wl.candidates_full_grid(1, 50001), dev), 50001, model, 10
+    full = host(ctx.select(*args))
+    n = ctx.launch_count()
+    ctx.debug_limit_workspace(16 * MB)
+    less = host(ctx.select(*args))
+    launches = ctx.launch_count() - n
+    ctx.debug_limit_workspace(0)
+    n = ctx.launch_count()
+    again = host(ctx.select(*args))
+    assert launches < ctx.launch_count() - n  # (tables of classes)
+    for a, b, c in zip(full, less, again):
+        assert np.array_equal(a, b) and np.array_equal(a, c)
 
 
 @pytest.mark.parametrize("onehot", [False, True])
