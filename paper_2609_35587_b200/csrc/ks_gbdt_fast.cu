@@ -1445,7 +1445,18 @@ cudaError_t build_fast_gbdt(GbdtModel& m, int n_trees, const int64_t* off, const
   if (tpc < gpr) return cudaSuccess;
   // At least sixteen chunks a ring, so that a split walk's units are not coarse, but no fewer than eight trees a thread, which
   // hide a chunk's beginning and end (100 trees of depth 6 in chunks of 32: 64 x 2,048 from host memory 122 us, of 8 112).
-  tpc = std::min(tpc, std::max(8, n_trees / (16 * rings)) * gpr);
+  // A multiple of four a thread, by which the walk is unrolled, and no more padding than the top levels' constants have
+  // room for (500 trees of depth 6, 128 slots, in chunks of 31, 527 with the padding, whose constants take the compact form:
+  // 31 x 62,000 2,070 us and 300 x 3,900 1,231; in chunks of 28 1,434 and 987).
+  const auto top_form = [&](int t) {
+    const int64_t pairs = static_cast<int64_t>((n_trees + t - 1) / t) * t * 7;
+    return pairs <= kFastTopPairs ? 2 : pairs <= 2 * kFastTopPairs ? 1 : 0;
+  };
+  for (int t = std::max(8, n_trees / (16 * rings) / 4 * 4); t >= 8; t -= 4)
+    if (t * gpr < tpc && top_form(t * gpr) >= top_form(tpc)) {
+      tpc = t * gpr;
+      break;
+    }
   if (tpc > (n_trees + G - 1) / G * gpr) tpc = (n_trees + G - 1) / G * gpr;  // a small ensemble: one short chunk per ring
   const int n_chunks = (n_trees + tpc - 1) / tpc;
   const int chunk_words = (tpc * per_tree_words + 3) / 4 * 4;  // bulk copies move multiples of 16 bytes

@@ -88,3 +88,14 @@ def test_copies_tie_whatever_the_leaves(ks, ctx, C, trees, depth, law, huge):
     idx, sc = (t.cpu().numpy() for t in ctx.select(d_p, 1, d_c, C, model, k))
     assert np.all(np.diff(sc[0]) <= 0)
     entries_agree(ks, ctx, model, prob, d_p, d_c, C, k, idx[0], sc[0], period)
+
+
+@pytest.mark.parametrize("trees", [129, 300, 500, 505, 509, 512, 513, 916])
+@pytest.mark.parametrize("law", ["slots128", "hist256"])
+def test_chunks_keep_the_unroll_and_the_top_levels(ks, ctx, trees, law):
+    """A chunk's trees are a multiple of four a thread, and padding to whole chunks leaves the top levels of up to 512
+    trees in the form that holds them twice as fast."""
+    model = ctx.model_create_gbdt(*wl.gbdt_complete(trees, trees, 6, wl.feature_stats("cfg1"), 0.1, law), 0.0)
+    told = dict(w.split("=") for w in model.describe().split()[1:])
+    assert int(told["chunk_trees"]) % 4 == 0, told
+    assert told["top_levels"] == ("3" if trees <= 512 else "3c"), told
