@@ -410,9 +410,9 @@ ks_status ks_model_describe(const ks_model* model, char* buf, int len);
  * `starve` != 0 makes the tree kernel arm each chunk barrier for 16 bytes more than its copy
  * brings, and the tensor-core kernel skip the copy of its weight image, so that the first wait
  * runs out, the kernel sets the status word and returns, and the call reports KS_ERR_TIMEOUT
- * without any fault: the failure path can be tested on a healthy GPU. With `starve` == 2 only every
- * other block of the tree kernel's grid does so, and the others finish their parts; with 3 the barriers
- * of tiles that were built in front of the walk are armed so, and not those of the chunks. */
+ * without any fault: the failure path can be tested on a healthy GPU. Where the trees are shared out among the
+ * CTAs (ks_debug_split_walks), `starve` == 2 makes only every other block of the grid do so, and the others finish their
+ * parts, and 3 arms the barriers of the tiles in front so, and not those of the chunks. */
 ks_status ks_debug_set_wait(ks_ctx* ctx, int probe_limit, int starve);
 /* Frees the context's workspace (waits for the device); from then on one of more than `bytes` cannot be
  * had, as if the device had no more memory (0: no limit). */

@@ -258,7 +258,7 @@ class Context:
         return int(_lib.ks_device_status(self._h))
 
     def debug_set_wait(self, probe_limit: int = 0, starve: int = 0):
-        """Test hook: probe budget of the kernels' bounded waits, and the starved-wait mode (1; 2: every
+        """Test hook: probe budget of the kernels' bounded waits, and the starved-wait mode (1; of split walks 2: every
         other block of the tree kernel; 3: its tiles instead of its chunks)."""
         self._check(_lib.ks_debug_set_wait(self._h, int(probe_limit), int(starve)), "ks_debug_set_wait")
 
