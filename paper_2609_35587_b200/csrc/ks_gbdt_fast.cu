@@ -230,7 +230,8 @@ static_assert(sizeof(ProblemTerms) <= 128, "problem record");
 
 __global__ void __launch_bounds__(256)
 pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, int n_prob,
-                  const ks_candidate* __restrict__ c, FastView fv, MemoView memo, int thr_cap, const int* path, int* words) {
+                  const ks_candidate* __restrict__ c, FastView fv, MemoView memo, int thr_cap, const int* path, int* words, int C,
+                  int most_classes) {
   extern __shared__ __align__(16) float s_pthr[];  // thresholds of the per-pair features, then the records
   __shared__ ProblemTerms s_pt;
   __shared__ FeatQ s_fq[64];
@@ -245,7 +246,15 @@ pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, int n_prob
   if (blockIdx.x == 0 && tid == 0) words[kWordWalk] = skip ? kLeaveServed : 0;
   if (skip) return;
   int most = 0;
-  for (int q = 0; q < kMemoCombos; ++q) most = max(most, memo.count[q]);
+  for (int q = 0; q < kMemoCombos; ++q) {
+    const int n = memo.count[q];
+    if (n <= most_classes) {
+      most = max(most, n);
+    } else {
+      // a type combination of too many classes: its candidates have none for the walk, which evaluates their columns in place
+      for (int i = blockIdx.x * 256 + tid; i < C; i += gridDim.x * 256) memo.cls[static_cast<size_t>(q) * C + i] = kNoClass;
+    }
+  }
   // An item is (block of 256 classes, problem); the blocks of the grid deal the items among
   // themselves, so that the work is even whatever the number of classes. The item of class
   // block 0 also writes its problem's own record (problem-only rows and terms).
@@ -281,7 +290,7 @@ pair_table_kernel(ks_gpu_desc desc, const ks_problem* __restrict__ p, int n_prob
       if (tid < static_cast<int>(sizeof(ProblemTerms) / 4))
         reinterpret_cast<uint32_t*>(out + kFastMaxProbRows)[tid] = reinterpret_cast<const uint32_t*>(&s_pt)[tid];
     }
-    if (j >= n_classes) continue;
+    if (j >= n_classes || n_classes > most_classes) continue;
     if (max_thr < 0) {
       max_thr = 0;
 #pragma unroll
@@ -655,7 +664,7 @@ __device__ __noinline__ void fill_tile(const ks_gpu_desc& desc, const ProblemTer
       else scatter_vectors(q[j], 16 * (v - cand_vecs), fv.n_pair_rows, word0, NC);
     }
   }
-  // candidates without a record (no memo in this call, or a class table that was full): their
+  // candidates without a record (no memo in this call, no class, or a class table that was full): their
   // per-pair columns are computed here, after the word stores that cover their bytes
   if (!__syncthreads_or(lone)) return;
   if (!lone) return;
@@ -2043,6 +2052,12 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
   }
   // problems in batches when the memo's table does not hold them all at once
   const int step = memo.keys ? balanced_step(g, P, memo_batch, nblk) : P;
+  // A table that holds more classes than a problem has candidates is evaluated for nothing: the tiles of a short segment
+  // are filled in place then. Up to 4,096 classes a problem's table is done sooner, spread over the machine,
+  // than a block fills its tile. Mixed types, 500 trees of depth 8 (200, 256 bins): 300 segments of 700
+  // out of 61,085 valid candidates (10,785 classes) 1,955 -> 707 us (1,328 -> 403), 1,000 of 300 6,016 -> 1,937 (3,864 ->
+  // 786); out of 60,000 grid ones, with records 732 (410) and in place 680 (329), but 32 x 700 244 (151) and 267 (149).
+  const int most_classes = seg_off ? std::max(4096, nblk * rows_per_cta) : kMemoCap;
   for (int first = 0; first < P; first += step) {
     const int n = P - first < step ? P - first : step;
     if (memo.keys) {
@@ -2052,7 +2067,7 @@ cudaError_t launch_select_fast(const ks_gpu_desc& desc, const GbdtModel& g, cons
       const int64_t table_slots = static_cast<int64_t>(kSmCount) * (2 * (pthr_bytes + 4096) <= 227 * 1024 ? 2 : 1);
       pair_table_kernel<<<static_cast<unsigned>(table_items < table_slots ? table_items : table_slots), 256, pthr_bytes,
                           stream>>>(
-          desc, d_p + first, n, d_c, fv, memo, pthr_cap, path, wait->words);
+          desc, d_p + first, n, d_c, fv, memo, pthr_cap, path, wait->words, C, most_classes);
       ++*launches;
     }
     a.dependent = memo.keys != nullptr || ((tiles_mode || prep) && !ev_begin);  // (no event stands between the two)

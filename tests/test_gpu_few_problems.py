@@ -45,3 +45,40 @@ def test_select(P, C, trees, depth, k, segmented):
         ok, msg = topk_accept(idx[p], sc[p], ref, seg, k, TOL)
         assert ok, (p, msg)
     ctx.close()
+
+
+@pytest.mark.parametrize("P,length,law", [(40, 300, "pernode"), (70, 4096, "hist256"), (33, 4097, "slots128"), (33, 700, "slots128")])
+def test_short_segments_of_many_classes(P, length, law):
+    """Segments shorter than the classes of the pool (more than 4,096 for a type combination), whose problems have no class
+    records: the same bits as a batch too small for records, and the oracle's ranking."""
+    from paper_2609_35587_b200 import binding as ks
+    dev = torch.device("cuda", 0)
+    ctx = ks.Context(DESC, 0)
+    prob = wl.problems_batch(P, P, cross_precision=True)
+    rec, _, n = ctx.valid_catalogue(prob[:1], ks.KS_VALID_COUPLED)
+    d_c = rec[torch.arange(30000, device=dev) * n // 30000].contiguous()
+    cand = d_c.cpu().numpy().view(wl.CANDIDATE_DT).reshape(-1)
+    assert len(np.unique(cand[["tile_m", "tile_n", "tile_k", "stages", "cluster_m", "cluster_n"]])) > 4097
+    gbdt = (*wl.gbdt_complete(3, 40, 7, wl.feature_stats("cfg2"), 0.1, law), 0.1)
+    model = ctx.model_create_gbdt(*gbdt)
+    rng = np.random.default_rng(P)
+    si = np.concatenate([np.sort(rng.choice(len(cand), length, replace=False)) for _ in range(P)]).astype(np.int32)
+    so = (np.arange(P + 1) * length).astype(np.int64)
+
+    def ranked(first, count):
+        part = si[first * length:(first + count) * length]
+        idx, sc = ctx.select(ks.to_device(prob[first:first + count], dev), count, d_c, len(cand), model, 10,
+                             ks.to_device(so[:count + 1], dev), ks.to_device(part, dev), len(part))
+        return idx.cpu().numpy(), sc.cpu().numpy()
+
+    idx, sc = ranked(0, P)
+    for first, count in ((0, 3), (P - 20, 20)):  # (records: 32 problems or more)
+        some = ranked(first, count)
+        assert np.array_equal(some[0], idx[first:first + count]) and np.array_equal(some[1], sc[first:first + count])
+    for p in (0, P - 1):
+        seg = si[so[p]:so[p + 1]]
+        _, _, ref = oracle.select(prob[p:p + 1], cand, DESC, 10, gbdt=gbdt, want_scores=True,
+                                  seg_off=np.array([0, length], np.int64), seg_idx=seg)
+        ok, msg = topk_accept(idx[p], sc[p], ref, seg, 10, TOL)
+        assert ok, (p, msg)
+    ctx.close()
