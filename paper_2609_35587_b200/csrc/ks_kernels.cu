@@ -803,9 +803,11 @@ static int ridge_blocks(int P, int64_t per_problem) {
 }
 // Dense batches go by classes where that many pairs take longer one by one than the class tables do: 60,000
 // grid candidates 55 us whatever the (few) problems, in place 87 for 24 and 106 for 32; 61,140 valid candidates (10,785
-// classes) 89 and 95, in place 88 and 108; 5,000 candidates 52, in place 45 for 64 and 58 for 128.
+// classes) 89 and 95, in place 88 and 108; 5,000 candidates 52, in place 45 for 64 and 58 for 128. Valid candidates are
+// less alike: 30 x 20,000 of them 73 us, in place 54, 30 x 45,000 84 and 82 (mixed types 99 and 87), 30 x 60,000 86 and 99 (102 and
+// 109), so batches of fewer than 32 problems go by classes from there on.
 static bool ridge_by_classes(int P, int C, bool segmented, bool lean) {
-  return !segmented && !lean && P >= 30 && static_cast<int64_t>(P) * C >= 600000;
+  return !segmented && !lean && P >= 30 && static_cast<int64_t>(P) * C >= (P < 32 ? 1800000 : 600000);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -88,7 +88,7 @@ def test_problems_beyond_the_class_tables(ks, ctx, P, C):
         assert ok, (p, msg)
 
 
-@pytest.mark.parametrize("what,P,C,k", [("plain", 30, 20000, 10), ("plain", 1040, 600, 32), ("valid", 33, 61140, 7),
+@pytest.mark.parametrize("what,P,C,k", [("plain", 30, 60000, 10), ("plain", 1040, 600, 32), ("valid", 33, 61140, 7),
                                         ("no class", 40, 15001, 10), ("full", 32, 20000, 10), ("ties", 32, 18755, 32), ("not finite", 32, 19000, 10),
                                         ("many", 8200, 80, 3)])
 def test_classes_against_pairs(ks, ctx, what, P, C, k):
@@ -131,3 +131,15 @@ def test_classes_against_pairs(ks, ctx, what, P, C, k):
             _, _, ref = oracle.select(prob[p:p + 1], cand, DESC, k, mlp=mlp, want_scores=True)
             ok, msg = topk_accept(idx[p].cpu().numpy(), sc[p].cpu().numpy(), ref, np.arange(C, dtype=np.int32), k, 1e-4)
             assert ok, (p, msg)
+
+
+@pytest.mark.parametrize("P,C,classes", [(31, 58064, False), (31, 58065, True), (32, 18749, False), (32, 18750, True)])
+def test_which_batches_go_by_classes(ks, ctx, P, C, classes):
+    """Five kernels and the merge, or pair by pair three and the merge."""
+    dev = torch.device("cuda", 0)
+    st = wl.feature_stats("cfg2")
+    model = ctx.model_create_mlp(wl.mlp_xavier(2, [64, 1], st["mu"], st["sigma"]))
+    args = ks.to_device(wl.problems_batch(P, P), dev), P, ks.to_device(wl.candidates_full_grid(3, C), dev), C, model, 10
+    n = ctx.launch_count()
+    ctx.select(*args)
+    assert ctx.launch_count() - n == (6 if classes else 4)
