@@ -1620,7 +1620,8 @@ size_t fast_scratch_bytes(const GbdtModel& g, int C) {
 }
 
 // Memo of the per-pair rows (see MemoView): for every dense batch that is not split (a split walk takes whole
-// tiles, see tile_pairs_kernel) and for segmented batches of 32 problems or more. The
+// tiles, see tile_pairs_kernel) and for segmented batches of 32 problems or more. (Dense batches of 3 to 31 problems come here from
+// 1,924 blocks on: 16 x 150,000 grid candidates, 500 trees, 2,802 us without records, 2,240 with; 50 trees 760 and 469.) The
 // table is held for at most `fast_memo_batch` problems at a time (512 MiB of
 // records); a larger call is served batch by batch. 0 = not used.
 size_t memo_fixed_bytes(int C) {
@@ -1718,8 +1719,13 @@ static int split_plan(const GbdtModel& g, int64_t blocks, SplitArgs* s) {
 // in the only round of CTAs or in the last of a few. Measured against whole blocks that fill their tiles in
 // the walk (500 trees, 256 bins): 7 problems x 61,140 valid candidates (420 blocks) 533 -> 455 us, 31 x 61,140 (1,860) 2,117 ->
 // 1,900, 64 x 9,000 grid candidates (576) 695 -> 595. From 32 problems on a catalogue in similarity order with class
-// records is the alternative: 100 x 9,000 (900 blocks) 1,110 -> 934, 32 x 60,000 (1,888) 1,879 -> 1,959. A problem looks through those
-// before it for its type combination, so there may not be very many.
+// records is the alternative: 100 x 9,000 (900 blocks) 1,110 -> 934, 32 x 60,000 (1,888) 1,879 -> 1,959. Which of the two wins up
+// to eight rounds was measured at 50, 200, 500 and 1,000 trees of depth 6 to 8 under the three laws: split walks, on grid pools 0.51
+// to 0.99 of the time with records (full rounds of 592 and 888 blocks 1.01 to 1.02), on the valid pool, whose classes hold
+// few members, 0.28 to 0.85; only 500 trees of depth 8 with a threshold of its own at every node lose at 1,152 grid blocks
+// (1,215 -> 1,281 us; 1,855 -> 1,254 at the same size on the valid pool). A problem looks through those
+// before it for its type combination, so there may not be very many. A single call of more blocks than the machine
+// holds at once keeps whole blocks (310,000 candidates, 500 trees 610 us): its tiles would be 43 MB and more of workspace.
 constexpr int kSplitBlocks = 13 * kSmCount, kSplitBlocksMemo = 8 * kSmCount, kSplitProblems = 512;
 static bool split_fits(const GbdtModel& g, int64_t blocks) {  // (a line of trees is counted in 32 bits)
   return blocks * (static_cast<int64_t>(g.n_chunks + 2) * g.tpc + 64) < int64_t{1} << 30;
