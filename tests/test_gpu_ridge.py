@@ -143,3 +143,38 @@ def test_which_batches_go_by_classes(ks, ctx, P, C, classes):
     n = ctx.launch_count()
     ctx.select(*args)
     assert ctx.launch_count() - n == (6 if classes else 4)
+
+
+@pytest.mark.parametrize("P,length,onehot", [(40, 300, False), (33, 4096, True), (33, 4097, False), (64, 11000, False)])
+def test_short_segments_of_many_classes(ks, ctx, P, length, onehot):
+    """Segments shorter than the pool's classes are added up pair by pair, longer ones from the class sums: the bits of
+    batches too small for class tables either way."""
+    dev = torch.device("cuda", 0)
+    st = wl.feature_stats("cfg2")
+    mu, sg = wl.onehot_stats(st["mu"], st["sigma"]) if onehot else (st["mu"], st["sigma"])
+    mlp = wl.mlp_xavier(P, [80 if onehot else 64, 1], mu, sg)
+    model = ctx.model_create_mlp(mlp)
+    prob = wl.problems_batch(P, P, cross_precision=True)
+    rec, _, n = ctx.valid_catalogue(prob[:1], ks.KS_VALID_COUPLED)
+    d_c = rec[:n].contiguous()
+    rng = np.random.default_rng(P)
+    si = np.concatenate([np.sort(rng.choice(n, length, replace=False)) for _ in range(P)]).astype(np.int32)
+
+    def ranked(first, count):
+        part = si[first * length:(first + count) * length]
+        so = (np.arange(count + 1) * length).astype(np.int64)
+        idx, sc = ctx.select(ks.to_device(prob[first:first + count], dev), count, d_c, n, model, 10,
+                             ks.to_device(so, dev), ks.to_device(part, dev), len(part))
+        return idx.cpu().numpy(), sc.cpu().numpy()
+
+    idx, sc = ranked(0, P)
+    for first, count in ((0, 31), (P - 5, 5)):
+        some = ranked(first, count)
+        assert np.array_equal(some[0], idx[first:first + count]) and np.array_equal(some[1], sc[first:first + count])
+    cand = d_c.cpu().numpy().view(wl.CANDIDATE_DT).reshape(-1)
+    for p in (0, P - 1):
+        seg = si[p * length:(p + 1) * length]
+        _, _, ref = oracle.select(prob[p:p + 1], cand, DESC, 10, mlp=mlp, want_scores=True,
+                                  seg_off=np.array([0, length], np.int64), seg_idx=seg)
+        ok, msg = topk_accept(idx[p], sc[p], ref, seg, 10, 1e-4)
+        assert ok, (p, msg)
